@@ -308,9 +308,11 @@ def adjoint_phases(sv, w, prob, theta, out, info, flush, stream, reps, step=None
     sv.sv_phase_timing(False)
     torch.cuda.synchronize()
     n, I = w.n_qubits, w.n_instances
-    state = I * (8 << n)
+    # states the passes moved: two instances of a real problem share one
+    states = sv.sv_last_adjoint_states()
+    state = states * (8 << n)
     last = sv.sv_last_adjoint_info()
-    nbytes = last["reverse_bytes"]
+    nbytes = last["reverse_bytes"] // I * states
     peak, src = measured_hbm_gbs()
     achieved = nbytes / (ph["reverse_ms"] * 1e-3) / 1e9
     # the gradient's own forward passes (the same relabeling plan), 16 B per
@@ -321,7 +323,8 @@ def adjoint_phases(sv, w, prob, theta, out, info, flush, stream, reps, step=None
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "traffic": traffic,
             "kernel": f"k_tile_rev x {info['n_passes']} reverse tile passes of "
-                      f"2^{info['tile_bits']} amplitudes ({w.name}: {I} states of {n} qubits; "
+                      f"2^{info['tile_bits']} amplitudes ({w.name}: {states} states of {n} "
+                      f"qubits for {I} instances; "
                       "psi and lambda read and lambda written per pass, psi written "
                       "unless the next pass restarts from a stored state)",
             "reverse_ms": ph["reverse_ms"], "bytes_per_reverse": nbytes,

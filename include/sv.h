@@ -421,13 +421,21 @@ sv_status sv_last_phase_ms(float *forward_ms, float *h_ms, float *reverse_ms);
 /* What the last adjoint gradient of states in device memory (sv_grad_adjoint,
  * sv_grad_adjoint_host or sv_grad_ddcl on the tile path of the current
  * device) did: the checkpoint interval it used (1, 2 or 4) and the
- * algorithmic bytes of its reverse tile passes (per pass psi, or its stored
- * state, and lambda read, lambda written, and psi written unless the next
- * reverse pass restarts from a stored state; summed over the call's chunks
- * of instances).  Both are 0 after an adjoint that ran on chip.  Host-only:
+ * algorithmic bytes of its reverse tile passes (per instance and pass psi,
+ * or its stored state, and lambda read, lambda written, and psi written
+ * unless the next reverse pass restarts from a stored state; summed over the
+ * instances, see sv_last_adjoint_states).  Both are 0 after an adjoint that ran on chip.  Host-only:
  * reads values the host recorded when it launched the passes.  Any
  * out-pointer may be NULL. */
 sv_status sv_last_adjoint_info(int32_t *checkpoint_every, int64_t *reverse_bytes);
+
+/* How many states in device memory that adjoint swept: one per instance, or
+ * half as many (rounded up) when the instances' amplitudes are all real (Ry,
+ * X, H, CNOT and CZ gates, Ry encodings, an observable without odd Y counts)
+ * and two instances share one complex state.  The passes then move that share
+ * of reverse_bytes, which counts a state per instance.  0 after an adjoint
+ * that ran on chip. */
+sv_status sv_last_adjoint_states(int32_t *states);
 
 /* ------------------------------------------------------------- autotune */
 

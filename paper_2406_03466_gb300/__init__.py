@@ -85,7 +85,7 @@ EXPORTED = ("sv_alloc", "sv_free", "sv_state_info", "sv_apply_circuit_batch",
             "sv_grad_adjoint_multi", "sv_grad_ddcl", "sv_grad_ddcl_param_shift",
             "sv_grad_param_shift_host", "sv_grad_adjoint_host", "sv_param_shift_energies_range", "sv_sample",
             "sv_param_shift_combine",
-            "sv_last_phase_ms", "sv_last_adjoint_info", "sv_status_string",
+            "sv_last_phase_ms", "sv_last_adjoint_info", "sv_last_adjoint_states", "sv_status_string",
             "sv_last_error",
             "sv_sync_status", "sv_shutdown", "sv_version")
 
@@ -126,6 +126,7 @@ def _load():
     lib.sv_phase_timing.argtypes = [I32]
     lib.sv_last_phase_ms.argtypes = [P(ctypes.c_float)] * 3
     lib.sv_last_adjoint_info.argtypes = [P(ctypes.c_int32), P(ctypes.c_int64)]
+    lib.sv_last_adjoint_states.argtypes = [P(I32)]
     lib.sv_status_string.argtypes = [I32]
     lib.sv_status_string.restype = ctypes.c_char_p
     lib.sv_last_error.restype = ctypes.c_char_p
@@ -592,6 +593,14 @@ def sv_last_adjoint_info() -> dict:
     _check(_lib.sv_last_adjoint_info(ctypes.byref(every), ctypes.byref(nbytes)),
            "sv_last_adjoint_info")
     return {"checkpoint_every": every.value, "reverse_bytes": nbytes.value}
+
+
+def sv_last_adjoint_states() -> int:
+    """States in device memory the last adjoint swept (two instances of a real
+    problem share one; 0 after an on-chip adjoint)."""
+    n = ctypes.c_int32()
+    _check(_lib.sv_last_adjoint_states(ctypes.byref(n)), "sv_last_adjoint_states")
+    return n.value
 
 
 def sv_status_string(status: int) -> str:

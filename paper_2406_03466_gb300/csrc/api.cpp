@@ -69,6 +69,7 @@ struct Packer {
 struct PlanEntry {
     std::vector<sv_gate> gates;  // exact key check against hash collisions
     int n = 0, n_params = 0, input_dim = 0;
+    bool real = false;  // every group's matrix is real
     HostProgram host;
     std::vector<TilePass> tiles;  // tile plans: one kernel descriptor per pass
     DeviceBuf buf;
@@ -123,6 +124,7 @@ struct DeviceCtx {
     // the algorithmic bytes of its reverse tile passes.
     int last_every = 0;
     int64_t last_rev_bytes = 0;
+    int last_states = 0;  // states it swept (two real circuits share one)
     // Uneven batches: one instantiated graph per configuration, and the
     // stream the captures run on.
     std::unordered_map<uint64_t, std::unique_ptr<struct MultiGraph>> graphs;
@@ -245,6 +247,8 @@ sv_status get_plan(DeviceCtx *ctx, const sv_circuit &c, int R, bool fuse, sv_dty
     e->n_params = c.n_params;
     e->input_dim = c.input_dim;
     const HostProgram &h = e->host;
+    e->real = true;
+    for (const Group &g : h.groups) e->real = e->real && g.real;
     Packer pk;
     size_t o_st = pk.add(h.stages.data(), h.stages.size() * sizeof(Stage));
     size_t o_op = pk.add(h.ops.data(), h.ops.size() * sizeof(Op));
@@ -632,20 +636,30 @@ sv_status get_hplan(ObsEntry *obs, int n, sv_dtype dt, HPlanEntry **out,
 int64_t tile_blocks(const DeviceCtx *ctx, int64_t tiles);
 
 // E[r] = <psi_r|H|psi_r> for n_rows states (and lam = H psi unless lam is
-// null) by tile passes.
+// null) by tile passes.  pair: the rows lie two to a state.
 sv_status h_tiles(DeviceCtx *ctx, ObsEntry *obs, int n, sv_dtype dt, int n_rows, const void *psi,
-                  void *lam, double *E, cudaStream_t st, const std::vector<int> *layout = nullptr) {
+                  void *lam, double *E, cudaStream_t st, const std::vector<int> *layout = nullptr,
+                  bool pair = false) {
     HPlanEntry *hp = nullptr;
     sv_status s = get_hplan(obs, n, dt, &hp, layout);
     if (s != SV_OK) return s;
     SV_CUDA(cudaMemsetAsync(E, 0, sizeof(double) * (size_t)n_rows, st));
+    const int n_states = pair ? (n_rows + 1) / 2 : n_rows;
     for (const HPass &P : hp->passes) {
-        const int64_t tiles = (int64_t)n_rows << P.n_tile_bits;
-        cudaError_t e = launch_tile_h(dt == SV_C128, P, n, n_rows, psi, lam, E,
-                                      tile_blocks(ctx, tiles), st);
+        const int64_t tiles = (int64_t)n_states << P.n_tile_bits;
+        cudaError_t e = launch_tile_h(dt == SV_C128, P, n, n_states, psi, lam, E,
+                                      tile_blocks(ctx, tiles), st, pair ? n_rows : 0);
         if (e != cudaSuccess) return cuda_fail(e, "H tile pass");
     }
     return SV_OK;
+}
+
+// Whether the slots of an energy or gradient call share states two by two:
+// real matrices and a real observable keep every amplitude real, so a pair
+// costs what one complex state costs.  One slot alone gains nothing; the
+// tensor-core blocks are complex.
+bool real_pairs(const PlanEntry *pe, const ObsEntry *obs, int n_slots, bool tc) {
+    return n_slots >= 2 && !tc && pe->real && obs && obs->dev.real;
 }
 
 bool wants_tiles(int n, sv_dtype dt, const sv_plan_opts *o) {
@@ -722,16 +736,18 @@ int64_t tile_blocks(const DeviceCtx *ctx, int64_t tiles) {
 
 // Forward tile passes of `pe` over src.n_slots states (|ref> first when init).
 // After pass i with (i + 1) % every == 0 (and not the last pass) the states
-// are copied to checkpoint (i + 1) / every - 1 of `ck`.
+// are copied to checkpoint (i + 1) / every - 1 of `ck`.  pair: real slots
+// two to a state.
 sv_status tiles_forward(DeviceCtx *ctx, const PlanEntry *pe, int R, sv_dtype dt,
                         const SlotSource &src, void *states, void *mats, bool init, void *ck,
-                        int every, cudaStream_t st, bool tc = false) {
+                        int every, cudaStream_t st, bool tc = false, bool pair = false) {
     const int c128 = dt == SV_C128, n = pe->n, G = pe->dev.n_groups;
-    const size_t sbytes = ((size_t)src.n_slots << n) * (c128 ? 16 : 8);
-    cudaError_t e = launch_group_mats(c128, pe->dev, src, mats, st);
+    const int n_states = pair ? (src.n_slots + 1) / 2 : src.n_slots;
+    const size_t sbytes = ((size_t)n_states << n) * (c128 ? 16 : 8);
+    cudaError_t e = launch_group_mats(c128, pe->dev, src, mats, st, pair);
     if (e != cudaSuccess) return cuda_fail(e, "group matrices");
     if (init) {
-        e = launch_init_states(c128, states, n, src, st);
+        e = launch_init_states(c128, states, n, src, st, pair);
         if (e != cudaSuccess) return cuda_fail(e, "state init");
     }
     // A pass that ends at a stored forward state writes its output there
@@ -741,7 +757,7 @@ sv_status tiles_forward(DeviceCtx *ctx, const PlanEntry *pe, int R, sv_dtype dt,
     const void *in = states;
     for (size_t i = 0; i < passes.size(); ++i) {
         const TilePass &tp = passes[i];
-        const int64_t tiles = (int64_t)src.n_slots << tp.n_tile_bits;
+        const int64_t tiles = (int64_t)n_states << tp.n_tile_bits;
         const uint32_t smem = tile_fwd_smem(c128, tp);
         if (smem > 220u * 1024u) return fail(SV_ERR_UNSUPPORTED, "tile pass needs too much shared memory");
         void *out = states;
@@ -754,8 +770,8 @@ sv_status tiles_forward(DeviceCtx *ctx, const PlanEntry *pe, int R, sv_dtype dt,
                                    err, in);
             if (e != cudaSuccess) return cuda_fail(e, "forward tile pass (tensor cores)");
         } else {
-            e = launch_tile_fwd(c128, tp, n, src.n_slots, mats, G, out, tile_blocks(ctx, tiles), st,
-                                in);
+            e = launch_tile_fwd(c128, tp, n, n_states, mats, G, out, tile_blocks(ctx, tiles), st, in,
+                                pair);
             if (e != cudaSuccess) return cuda_fail(e, "forward tile pass");
         }
         in = out;
@@ -785,18 +801,20 @@ sv_status tiles_energies(DeviceCtx *ctx, const sv_problem *p, const double *thet
     const size_t csz = c128 ? 16 : 8, sb = csz << n;
     const size_t mb = (size_t)pe->dev.n_groups * 4 * csz;
     const size_t per = sb + mb;
-    int64_t chunk = (int64_t)(big_budget(ctx, st) / (per + 512));
+    const bool pair = real_pairs(pe, obs, n_slots, cfg.tc);
+    const int per_state = pair ? 2 : 1;  // slots
+    int64_t chunk = (int64_t)(big_budget(ctx, st) / (per + 512));  // states
     if (chunk < 1) return fail(SV_ERR_OOM, "one state does not fit in free device memory");
-    if (chunk > n_slots) chunk = n_slots;
+    if (chunk > (n_slots + per_state - 1) / per_state) chunk = (n_slots + per_state - 1) / per_state;
     if (chunk > 65535) chunk = 65535;  // one grid row per state in the expectation
     void *big = nullptr;
     const size_t mats_off = ((size_t)chunk * sb + 255) & ~size_t(255);
     s = get_big_scratch(ctx, st, mats_off + (size_t)chunk * mb + 256, &big);
     if (s != SV_OK) return s;
-    for (int64_t c0 = 0; c0 < n_slots; c0 += chunk) {
+    for (int64_t c0 = 0; c0 < n_slots; c0 += chunk * per_state) {
         SlotSource src{};
         src.mode = mode;
-        src.n_slots = (int)std::min<int64_t>(chunk, n_slots - c0);
+        src.n_slots = (int)std::min<int64_t>(chunk * per_state, n_slots - c0);
         src.n_instances = I;
         src.refs = (const int64_t *)drefs;
         src.theta = theta;
@@ -804,9 +822,9 @@ sv_status tiles_energies(DeviceCtx *ctx, const sv_problem *p, const double *thet
         src.input_stride = p->input_stride;
         src.slot_base = slot_begin + (int)c0;
         s = tiles_forward(ctx, pe, cfg.R, dt, src, big, (char *)big + mats_off, true, nullptr, 0, st,
-                          cfg.tc);
+                          cfg.tc, pair);
         if (s != SV_OK) return s;
-        s = h_tiles(ctx, obs, n, dt, src.n_slots, big, nullptr, E + c0, st, &pe->host.layout);
+        s = h_tiles(ctx, obs, n, dt, src.n_slots, big, nullptr, E + c0, st, &pe->host.layout, pair);
         if (s != SV_OK) return s;
     }
     return SV_OK;
@@ -824,6 +842,7 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     ctx->phase_used = 0;
     ctx->last_every = 0;
     ctx->last_rev_bytes = 0;
+    ctx->last_states = 0;
     const sv_dtype dt = p->dtype;
     const int c128 = dt == SV_C128, n = p->circuit->n_qubits, I = p->n_instances;
     const int P = p->circuit->n_params, Pp = P > 0 ? P : 1;
@@ -872,9 +891,12 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     const int npass = (int)pe->tiles.size();
     const size_t csz = c128 ? 16 : 8, sb = csz << n;
     const size_t budget = big_budget(ctx, st);
-    auto per_instance = [&](int ev) {
+    const bool pair = real_pairs(pe, obs, I, cfg.tc);
+    const int per_state = pair ? 2 : 1;  // instances
+    const int n_states = (I + per_state - 1) / per_state;
+    auto bytes_per_state = [&](int ev) {
         const size_t ncp_ = npass > 1 ? (size_t)((npass - 1) / ev) : 0;
-        return (2 + ncp_) * sb + (size_t)G * 4 * csz + (size_t)G * 64;
+        return (2 + ncp_) * sb + (size_t)G * 4 * csz + (size_t)per_state * G * 64;
     };
     if (every <= 0) {
         // The most stored states that still let every instance run at once:
@@ -882,23 +904,23 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
         // writing psi, and un-computation rounding spans fewer passes.
         every = 4;
         for (int ev : {1, 2})
-            if (budget / (per_instance(ev) + 2048) >= (size_t)I) {
+            if (budget / (bytes_per_state(ev) + 2048) >= (size_t)n_states) {
                 every = ev;
                 break;
             }
     }
     const int ncp = npass > 1 ? (npass - 1) / every : 0;
     ctx->last_every = every;
-    const size_t per = per_instance(every);
-    int64_t chunk = (int64_t)(budget / (per + 2048));
+    const size_t per = bytes_per_state(every);
+    int64_t chunk = (int64_t)(budget / (per + 2048));  // states
     if (chunk < 1) return fail(SV_ERR_OOM, "psi, lambda and the stored states do not fit");
-    if (chunk > I) chunk = I;
+    if (chunk > n_states) chunk = n_states;
     if (chunk > 65535) chunk = 65535;
     auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
     const size_t o_lam = up((size_t)chunk * sb), o_ck = o_lam + up((size_t)chunk * sb);
     const size_t o_mats = o_ck + up((size_t)ncp * chunk * sb);
     const size_t o_rho = o_mats + up((size_t)chunk * G * 4 * csz);
-    const size_t total = o_rho + up((size_t)chunk * G * 64);
+    const size_t total = o_rho + up((size_t)chunk * per_state * G * 64);
     void *big = nullptr;
     s = get_big_scratch(ctx, st, total, &big);
     if (s != SV_OK) return s;
@@ -910,22 +932,24 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     SV_CUDA(cudaMemsetAsync(Gs, 0, sizeof(double) * (size_t)I * Pp, st));
     const CostSource cs = cost_of(p, weights);
     const auto &passes = pe->tiles;
-    for (int64_t c0 = 0; c0 < I; c0 += chunk) {
+    ctx->last_states = n_states;
+    for (int64_t c0 = 0; c0 < I; c0 += chunk * per_state) {
         SlotSource src{};
         src.mode = SLOTS_INSTANCES;
-        src.n_slots = (int)std::min<int64_t>(chunk, I - c0);
+        src.n_slots = (int)std::min<int64_t>(chunk * per_state, I - c0);
+        const int states = (src.n_slots + per_state - 1) / per_state;
         src.n_instances = I;
         src.refs = (const int64_t *)drefs;
         src.theta = theta;
         src.inputs = p->inputs;
         src.input_stride = p->input_stride;
         src.slot_base = (int)c0;
-        const size_t cb = (size_t)src.n_slots * sb;  // bytes of this group's states
+        const size_t cb = (size_t)states * sb;  // bytes of this group's states
         void *psi = bb, *lam = bb + o_lam, *ck = bb + o_ck, *mats = bb + o_mats;
         double *rho = (double *)(bb + o_rho);
         phase_mark(ctx, st);
         s = tiles_forward(ctx, pe, cfg.R, dt, src, psi, mats, true, ncp ? ck : nullptr, every, st,
-                          cfg.tc);
+                          cfg.tc, pair);
         if (s != SV_OK) return s;
         phase_mark(ctx, st);
         cudaError_t e = cudaSuccess;
@@ -933,11 +957,11 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
             e = launch_ddcl_lambda(c128, n, src.n_slots, psi, ddcl_target, lam, Es + c0, st);
             if (e != cudaSuccess) return cuda_fail(e, "JS divergence and its lambda");
         } else {
-            s = h_tiles(ctx, obs, n, dt, src.n_slots, psi, lam, Es + c0, st, &pe->host.layout);
+            s = h_tiles(ctx, obs, n, dt, src.n_slots, psi, lam, Es + c0, st, &pe->host.layout, pair);
             if (s != SV_OK) return s;
         }
         phase_mark(ctx, st);
-        SV_CUDA(cudaMemsetAsync(rho, 0, (size_t)src.n_slots * G * 64, st));
+        SV_CUDA(cudaMemsetAsync(rho, 0, (size_t)states * per_state * G * 64, st));
         for (int i = npass - 1; i >= 0; --i) {
             // restart psi from the stored forward state after pass i: the
             // reverse pass reads it there and writes psi (no copy)
@@ -945,17 +969,17 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
             if ((i + 1) % every == 0 && i + 1 < npass)
                 psi_in = (const char *)ck + (size_t)((i + 1) / every - 1) * cb;
             const TilePass &tp = passes[i];
-            const int64_t tiles = (int64_t)src.n_slots << tp.n_tile_bits;
+            const int64_t tiles = (int64_t)states << tp.n_tile_bits;
             const uint32_t smem = tile_rev_smem(c128, tp);
             if (smem > 220u * 1024u) return fail(SV_ERR_UNSUPPORTED, "reverse pass needs too much shared memory");
             // psi after this pass is needed only if the next reverse pass
             // un-computes from it (it restarts from a stored state otherwise)
             const bool write_psi = i > 0 && !(i % every == 0 && i < npass);
-            e = launch_tile_rev(c128, tp, n, src.n_slots, mats, G, psi, lam, rho,
-                                tile_blocks(ctx, tiles), st, psi_in, write_psi);
+            e = launch_tile_rev(c128, tp, n, states, mats, G, psi, lam, rho,
+                                tile_blocks(ctx, tiles), st, psi_in, write_psi, pair);
             if (e != cudaSuccess) return cuda_fail(e, "reverse tile pass");
             // psi (or its stored state) and lambda read, lambda (and psi) written
-            ctx->last_rev_bytes += (int64_t)cb * (write_psi ? 4 : 3);
+            ctx->last_rev_bytes += (int64_t)src.n_slots * (int64_t)sb * (write_psi ? 4 : 3);
         }
         phase_mark(ctx, st);
         e = launch_group_grads(c128, pe->dev, src, rho, cs, Es + c0, Gs + (size_t)c0 * Pp, st);
@@ -1777,6 +1801,7 @@ sv_status adjoint_locked(DeviceCtx *ctx, const sv_problem *p, const double *thet
     const int P = p->circuit->n_params, I = p->n_instances;
     ctx->last_every = 0;  // on chip unless the tile path records its own
     ctx->last_rev_bytes = 0;
+    ctx->last_states = 0;
     if (wants_tiles(p->circuit->n_qubits, p->dtype, p->opts))
         return tiles_adjoint(ctx, p, theta, weights, energy_out, loss_out, grad_out,
                              checkpoint_every, st);
@@ -2373,6 +2398,14 @@ sv_status sv_last_adjoint_info(int32_t *checkpoint_every, int64_t *reverse_bytes
     std::lock_guard<std::mutex> lk(ctx->mu);
     if (checkpoint_every) *checkpoint_every = ctx->last_every;
     if (reverse_bytes) *reverse_bytes = ctx->last_rev_bytes;
+    return SV_OK;
+}
+
+sv_status sv_last_adjoint_states(int32_t *states) {
+    DeviceCtx *ctx = context();
+    if (!ctx) return fail(SV_ERR_CUDA, "no CUDA device");
+    std::lock_guard<std::mutex> lk(ctx->mu);
+    if (states) *states = ctx->last_states;
     return SV_OK;
 }
 

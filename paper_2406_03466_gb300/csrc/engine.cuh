@@ -19,12 +19,8 @@ template <> struct CT<double> { using T = double2; };
 
 __device__ __forceinline__ float fmaR(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fmaR(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ void sincosR(float a, float *s, float *c) { sincosf(a, s, c); }
-__device__ __forceinline__ void sincosR(double a, double *s, double *c) { sincos(a, s, c); }
-__device__ __forceinline__ float asinR(float x) { return asinf(x); }
-__device__ __forceinline__ double asinR(double x) { return asin(x); }
-__device__ __forceinline__ float acosR(float x) { return acosf(x); }
-__device__ __forceinline__ double acosR(double x) { return acos(x); }
+__device__ __forceinline__ float sqrtR(float x) { return sqrtf(x); }
+__device__ __forceinline__ double sqrtR(double x) { return sqrt(x); }
 
 template <typename C> __device__ __forceinline__ C cmk(double re, double im) {
     C r;
@@ -131,11 +127,22 @@ __device__ SlotInfo resolve(const SlotSource &s, int b) {
 
 // ------------------------------------------------------- gate matrices
 
-// exp(-i a P / 2) for P = X (0), Y (1), Z (2), row-major [m00 m01 m10 m11].
+// sin and cos of a / 2.  FP32: the half angle's rounding to float is put back
+// to first order, so the pair carries the rounding of the function only.
+__device__ __forceinline__ void half_sincos(double a, float *s, float *c) {
+    const double h = 0.5 * a;
+    const float hi = (float)h, lo = (float)(h - (double)hi);
+    float s0, c0;
+    sincosf(hi, &s0, &c0);
+    *s = __fmaf_rn(lo, c0, s0);
+    *c = __fmaf_rn(-lo, s0, c0);
+}
+__device__ __forceinline__ void half_sincos(double a, double *s, double *c) { sincos(a * 0.5, s, c); }
+
+// exp(-i a P / 2) for P = X (0), Y (1), Z (2) from sin and cos of a / 2,
+// row-major [m00 m01 m10 m11].
 template <typename Real, typename C>
-__device__ __forceinline__ void rotation(int axis, Real a, C g[4]) {
-    Real s, c;
-    sincosR(a * Real(0.5), &s, &c);
+__device__ __forceinline__ void rotation(int axis, Real s, Real c, C g[4]) {
     if (axis == 0) {
         g[0] = cmk<C>(c, 0); g[1] = cmk<C>(0, -s); g[2] = cmk<C>(0, -s); g[3] = cmk<C>(c, 0);
     } else if (axis == 1) {
@@ -145,7 +152,14 @@ __device__ __forceinline__ void rotation(int axis, Real a, C g[4]) {
     }
 }
 
-template <typename Real, typename C>
+// An encoding's input: |x| <= 1, where a complex64 problem's x counts as
+// +-1 when it rounds to that in float (beyond it the matrix is NaN).
+template <typename In> __device__ __forceinline__ double enc_input(double x) {
+    return fabs(x) > 1.0 && fabs((double)(In)x) <= 1.0 ? copysign(1.0, x) : x;
+}
+
+// In: the precision of the problem (Real may be wider).
+template <typename Real, typename C, typename In = Real>
 __device__ void member_matrix(const Member &m, const SlotInfo &si, C g[4]) {
     switch (m.kind) {
     case M_RX:
@@ -153,7 +167,9 @@ __device__ void member_matrix(const Member &m, const SlotInfo &si, C g[4]) {
     case M_RZ: {
         double a = m.angle;
         if (m.param >= 0) a = si.theta[m.param] + (m.param == si.shift_param ? si.shift : 0.0);
-        rotation<Real, C>(m.kind - M_RX, (Real)a, g);
+        Real sn, cs;
+        half_sincos(a, &sn, &cs);
+        rotation<Real, C>(m.kind - M_RX, sn, cs, g);
         break;
     }
     case M_X:
@@ -164,14 +180,20 @@ __device__ void member_matrix(const Member &m, const SlotInfo &si, C g[4]) {
         g[0] = cmk<C>(h, 0); g[1] = cmk<C>(h, 0); g[2] = cmk<C>(h, 0); g[3] = cmk<C>(-h, 0);
         break;
     }
+    // The encodings' half angles without inverse functions: with a =
+    // arcsin x, cos a = sqrt(1 - x^2), cos(a/2) = sqrt((1 + cos a) / 2) and
+    // sin(a/2) = x / (2 cos(a/2)); with a = arccos u, cos(a/2) =
+    // sqrt((1 + u) / 2) and sin(a/2) = sqrt((1 - u) / 2).
     case M_ENC_RY_ASIN: {
-        const Real x = (Real)si.x[m.param];
-        rotation<Real, C>(1, asinR(x), g);
+        const double x = enc_input<In>(si.x[m.param]);
+        const Real ca = sqrtR((Real)((1.0 - x) * (1.0 + x)));
+        const Real cs = sqrtR((Real)0.5 * ((Real)1 + ca));
+        rotation<Real, C>(1, (Real)x / ((Real)2 * cs), cs, g);
         break;
     }
     default: {  // M_ENC_RZ_ACOS_SQ
-        const Real x = (Real)si.x[m.param];
-        rotation<Real, C>(2, acosR(x * x), g);
+        const double x = enc_input<In>(si.x[m.param]), u = x * x;
+        rotation<Real, C>(2, sqrtR((Real)(0.5 * (1.0 - u))), sqrtR((Real)(0.5 * (1.0 + u))), g);
         break;
     }
     }
@@ -185,13 +207,14 @@ template <typename C> __device__ __forceinline__ void matmul2(const C A[4], cons
 }
 
 // Fused matrix of group g for this slot: M = G_last ... G_first.
-template <typename Real, typename C>
+template <typename Real, typename C, typename In = Real>
 __device__ void group_matrix(const Program &p, int g, const SlotInfo &si, C *out) {
     const Group grp = p.groups[g];
-    C M[4] = {cmk<C>(1, 0), cmk<C>(0, 0), cmk<C>(0, 0), cmk<C>(1, 0)};
-    for (int m = grp.m_begin; m < grp.m_end; ++m) {
+    C M[4];
+    member_matrix<Real, C, In>(p.members[grp.m_begin], si, M);  // a group has a member
+    for (int m = grp.m_begin + 1; m < grp.m_end; ++m) {
         C G[4], T[4];
-        member_matrix<Real, C>(p.members[m], si, G);
+        member_matrix<Real, C, In>(p.members[m], si, G);
         matmul2(G, M, T);
         M[0] = T[0]; M[1] = T[1]; M[2] = T[2]; M[3] = T[3];
     }

@@ -28,28 +28,50 @@
 namespace svk {
 namespace {
 
-// Fused 2x2 matrices of every group for every slot: out[slot][group][4].
+// Real circuits in pairs: a circuit whose groups are all real, started from
+// a basis state, keeps real amplitudes, so one array of complex amplitudes
+// carries the states of two circuit slots, slot 2j in the real parts and slot
+// 2j + 1 in the imaginary parts (an odd last slot is paired with itself).
+// Every pass then moves and multiplies half as much per circuit; the matrices
+// stay per circuit (packed FMAs take one per component).
+
+// Fused 2x2 matrices of every group for every slot: out[slot][group][4], or
+// with pair out[slot pair][group][4], entry k = (first slot's, second slot's).
+// Formed in FP64 and rounded once, so that a pass's error is its own.  A
+// pair's real rotations come with c >= 0 (a state's sign is of no account
+// to its energy and its gradient), for the shear form.
 template <typename Real>
-__global__ void k_group_mats(Program p, SlotSource src, typename CT<Real>::T *out) {
+__global__ void k_group_mats(Program p, SlotSource src, int pair, typename CT<Real>::T *out) {
+    using C = typename CT<Real>::T;
     const int G = p.n_groups;
-    const int64_t total = (int64_t)src.n_slots * G;
+    const int64_t total = (int64_t)(pair ? (src.n_slots + 1) / 2 : src.n_slots) * G;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int b = (int)(i / G), g = (int)(i % G);
-        const SlotInfo si = resolve(src, b);
-        group_matrix<Real, typename CT<Real>::T>(p, g, si, out + (size_t)i * 4);
+        C m[4];
+        for (int c = 0; c < (pair ? 2 : 1); ++c) {
+            const SlotInfo si = resolve(src, pair ? min(2 * b + c, src.n_slots - 1) : b);
+            double2 d[4];
+            group_matrix<double, double2, Real>(p, g, si, d);
+            const double sg = d[0].x < 0.0 && d[0].x == d[3].x && d[1].x == -d[2].x ? -1.0 : 1.0;
+            for (int k = 0; k < 4; ++k) {
+                if (!pair) m[k] = cmk<C>(d[k].x, d[k].y);
+                else if (c == 0) m[k].x = (Real)(sg * d[k].x);
+                else m[k].y = (Real)(sg * d[k].x);
+            }
+        }
+        for (int k = 0; k < 4; ++k) out[(size_t)i * 4 + k] = m[k];
     }
 }
 
 // Sets amplitude |ref_b> of every (zeroed) slot state to 1.
 template <typename C>
-__global__ void k_set_ref(C *states, int n, SlotSource src) {
+__global__ void k_set_ref(C *states, int n, SlotSource src, int pair) {
     for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < src.n_slots; b += gridDim.x * blockDim.x) {
         const SlotInfo si = resolve(src, b);
-        C one;
-        one.x = 1;
-        one.y = 0;
-        states[((int64_t)b << n) + si.ref] = one;
+        C *s = states + ((int64_t)(pair ? b >> 1 : b) << n) + si.ref;
+        if (!pair || !(b & 1)) s->x = 1;
+        if (pair && ((b & 1) || b + 1 == src.n_slots)) s->y = 1;
     }
 }
 
@@ -57,19 +79,19 @@ __global__ void k_set_ref(C *states, int n, SlotSource src) {
 // One forward stage: a branch-free path when register bits 0..M-1 carry
 // real rotations in shear form or complex matrices (M from the stage
 // flags), tile_ops_fwd otherwise.
-template <typename C, int R, bool kReal>
+template <typename C, int R, int kMat>
 __device__ __forceinline__ void stage_ops_fwd(uint32_t ops, uint32_t flags, const C *sm,
                                               C (&a)[1 << R]) {
     const uint32_t m = flags & 15u;
     if constexpr (R >= 4) {
-        if (m == 4) return tile_ops_fwd_rot<C, R, 0, 4>(ops, sm, a);
+        if (m == 4) return tile_ops_fwd_rot<C, R, 0, 4, kMat>(ops, sm, a);
     }
     if constexpr (R >= 3) {
-        if (m == 3) return tile_ops_fwd_rot<C, R, 0, 3>(ops, sm, a);
+        if (m == 3) return tile_ops_fwd_rot<C, R, 0, 3, kMat>(ops, sm, a);
     }
-    if (m == 2) return tile_ops_fwd_rot<C, R, 0, 2>(ops, sm, a);
-    if (m == 1) return tile_ops_fwd_rot<C, R, 0, 1>(ops, sm, a);
-    if constexpr (!kReal) {
+    if (m == 2) return tile_ops_fwd_rot<C, R, 0, 2, kMat>(ops, sm, a);
+    if (m == 1) return tile_ops_fwd_rot<C, R, 0, 1, kMat>(ops, sm, a);
+    if constexpr (kMat == kAny) {
         const uint32_t mc = (flags >> 8) & 15u;
         if constexpr (R >= 4) {
             if (mc == 4) return tile_ops_fwd_cplx<C, R, 0, 4>(ops, sm, a);
@@ -80,10 +102,10 @@ __device__ __forceinline__ void stage_ops_fwd(uint32_t ops, uint32_t flags, cons
         if (mc == 2) return tile_ops_fwd_cplx<C, R, 0, 2>(ops, sm, a);
         if (mc == 1) return tile_ops_fwd_cplx<C, R, 0, 1>(ops, sm, a);
     }
-    tile_ops_fwd<C, R, 0, kReal>(ops, sm, a);
+    tile_ops_fwd<C, R, 0, kMat>(ops, sm, a);
 }
 
-template <typename Real, int R, bool kReal>
+template <typename Real, int R, int kMat>
 __device__ __forceinline__ void tile_fwd_body(const TilePass &P, int n, int n_slots,
                                               const typename CT<Real>::T *mats, int G,
                                               const typename CT<Real>::T *src_states,
@@ -131,11 +153,13 @@ __device__ __forceinline__ void tile_fwd_body(const TilePass &P, int n, int n_sl
             for (int x = tid; x < 4 * P.n_ops; x += T)
                 sm[x] = mats[((size_t)cur.slot * G + P.grp[x >> 2]) * 4 + (x & 3)];
             __syncthreads();
-            for (int u = tid; u < P.n_ops; u += T)
-                if ((P.real_mask >> u) & 1ull) stage_shears(sm + 4 * u);
+            for (int u = tid; u < P.n_ops; u += T) {
+                if constexpr (kMat == kPair) stage_shears_pair(sm + 4 * u);
+                else if ((P.real_mask >> u) & 1ull) stage_shears(sm + 4 * u);
+            }
             if constexpr (std::is_same<C, float2>::value) {
                 __syncthreads();  // the branch-free paths' stage flags
-                set_stage_flags(P, rec, sm);
+                set_stage_flags<C, kMat>(P, rec, sm);
             }
             mslot = cur.slot;
         }
@@ -152,9 +176,9 @@ __device__ __forceinline__ void tile_fwd_body(const TilePass &P, int n, int n_sl
             for (int r = 0; r < NA; ++r) a[r] = *reinterpret_cast<const C *>(tile + (bb.x ^ xsel<R>(r, lq)));
             // complex64: the branch-free paths where the stage allows
             if constexpr (std::is_same<C, float2>::value) {
-                stage_ops_fwd<C, R, kReal>(ops, rec[2 * s + 1].w, sm, a);
+                stage_ops_fwd<C, R, kMat>(ops, rec[2 * s + 1].w, sm, a);
             } else {
-                tile_ops_fwd<C, R, 0, kReal>(ops, sm, a);
+                tile_ops_fwd<C, R, 0, kMat>(ops, sm, a);
             }
             __syncthreads();
 #pragma unroll
@@ -173,7 +197,7 @@ __device__ __forceinline__ void tile_fwd_body(const TilePass &P, int n, int n_sl
 // src: the states the pass reads; states: where it writes them (the same
 // buffer, or another one when the pass's output is also kept as a stored
 // forward state).
-template <typename Real, int R, bool kReal>
+template <typename Real, int R, int kMat>
 __global__ void __launch_bounds__(256, R >= 4 ? 2 : 3)
 k_tile_fwd(const __grid_constant__ TilePass P, int n, int n_slots,
            const typename CT<Real>::T *mats, int G, const typename CT<Real>::T *src,
@@ -181,7 +205,7 @@ k_tile_fwd(const __grid_constant__ TilePass P, int n, int n_slots,
     extern __shared__ __align__(16) unsigned char smem[];
     int64_t t0, t_end;
     block_range((int64_t)n_slots << P.n_tile_bits, gridDim.x, blockIdx.x, t0, t_end);
-    tile_fwd_body<Real, R, kReal>(P, n, n_slots, mats, G, src, states, t0, t_end, smem);
+    tile_fwd_body<Real, R, kMat>(P, n, n_slots, mats, G, src, states, t0, t_end, smem);
 }
 
 // The derivative of a rotation exp(-i theta P / 2) inside a fused group is
@@ -283,38 +307,75 @@ __device__ __forceinline__ Real single_sum(const C (&a)[1 << R], const C (&l)[1 
     return v;
 }
 
+// k3 = sum x0 y1 - x1 y0 of each of a pair's two real states (component =
+// state) over the pairs of register bit I; k0..k2 vanish for real states.
+template <typename C, int R, int I>
+__device__ __forceinline__ C pair_sum(const C (&a)[1 << R], const C (&l)[1 << R]) {
+    if constexpr (std::is_same<C, float2>::value) {
+        // chains split as in single_sum
+        constexpr int NC = (1 << R) >= 8 ? 2 : 1;
+        uint64_t pa[NC], pb[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) pa[c] = pb[c] = 0;
+        int m = 0;
+#pragma unroll
+        for (int r = 0; r < (1 << R); ++r) {
+            if (r & (1 << I)) continue;
+            pa[m % NC] = f2fma(f2of(a[r]), f2of(l[r | (1 << I)]), pa[m % NC]);
+            pb[m % NC] = f2fma(f2of(a[r | (1 << I)]), f2of(l[r]), pb[m % NC]);
+            ++m;
+        }
+        float2 A = f2unpack(pa[0]), B = f2unpack(pb[0]);
+        if constexpr (NC > 1) {
+            const float2 A1 = f2unpack(pa[1]), B1 = f2unpack(pb[1]);
+            A.x += A1.x;
+            A.y += A1.y;
+            B.x += B1.x;
+            B.y += B1.y;
+        }
+        return make_float2(A.x - B.x, A.y - B.y);
+    } else {
+        C v;
+        v.x = v.y = 0;
+#pragma unroll
+        for (int r = 0; r < (1 << R); ++r) {
+            if (r & (1 << I)) continue;
+            const C x0 = a[r], x1 = a[r | (1 << I)], y0 = l[r], y1 = l[r | (1 << I)];
+            v.x = fmaR(x0.x, y1.x, fmaR(-x1.x, y0.x, v.x));
+            v.y = fmaR(x0.y, y1.y, fmaR(-x1.y, y0.y, v.y));
+        }
+        return v;
+    }
+}
+
 // Reverse of tile_ops_fwd, register bits I, I-1, ..., 0: per op, first its
 // sums (at the point after the group) into k — k0..k3 at k[4 I ..], or with
 // kSingle the one sum of its fmode at k[I] — then the inverse group (sm
 // holds the adjoint matrices) on psi and lambda.
-template <typename C, typename Real, int R, int I, int NV, bool kSingle, bool kReal>
+// kPair: the single Ry sum of each of the two states, at k[2 I] and k[2 I + 1].
+template <typename C, typename Real, int R, int I, int NV, bool kSingle, int kMat>
 __device__ __forceinline__ void tile_ops_rev(uint32_t ops, uint32_t modes, const C *sm,
                                              C (&a)[1 << R], C (&al)[1 << R], Real (&k)[NV]) {
     if constexpr (I >= 0) {
         const uint32_t ob = (ops >> (8 * I)) & 0xffu;
         if (ob) {
             if (ob & 128u) {
-                if constexpr (kSingle)
+                if constexpr (kMat == kPair) {
+                    const C v = pair_sum<C, R, I>(a, al);
+                    k[2 * I] = v.x;
+                    k[2 * I + 1] = v.y;
+                } else if constexpr (kSingle) {
                     k[I] = single_sum<C, Real, R, I>(a, al, (modes >> (8 * I)) & 3u);
-                else
+                } else {
                     kmat_bit<C, Real, R, I>(a, al, &k[4 * I]);
+                }
             }
             C m0, m1, m2, m3;
             load_mat(sm, (int)(ob & 63u) - 1, m0, m1, m2, m3);
-            if (kReal || (ob & 64u)) {
-                if (m2.y != 0) {
-                    rot3_bit<C, Real, R, I>(a, m0.y, m1.y);
-                    rot3_bit<C, Real, R, I>(al, m0.y, m1.y);
-                } else {
-                    u1r_bit<C, Real, R, I>(a, m0.x, m1.x, m2.x, m3.x);
-                    u1r_bit<C, Real, R, I>(al, m0.x, m1.x, m2.x, m3.x);
-                }
-            } else {
-                u1_bit<C, R, I>(a, m0, m1, m2, m3);
-                u1_bit<C, R, I>(al, m0, m1, m2, m3);
-            }
+            op_bit<C, R, I, kMat>((ob & 64u) != 0, m0, m1, m2, m3, a);
+            op_bit<C, R, I, kMat>((ob & 64u) != 0, m0, m1, m2, m3, al);
         }
-        tile_ops_rev<C, Real, R, I - 1, NV, kSingle, kReal>(ops, modes, sm, a, al, k);
+        tile_ops_rev<C, Real, R, I - 1, NV, kSingle, kMat>(ops, modes, sm, a, al, k);
     }
 }
 
@@ -322,35 +383,41 @@ __device__ __forceinline__ void tile_ops_rev(uint32_t ops, uint32_t modes, const
 // rotations in shear form with the single Ry sum (stage flags, bits 4-7):
 // the same arithmetic without its per-op branches, so the compiler can
 // overlap one op's dependent FMA chains with the next op's.
-template <typename C, typename Real, int R, int I, int NV>
+template <typename C, typename Real, int R, int I, int NV, int kMat>
 __device__ __forceinline__ void tile_ops_rev_rot(uint32_t ops, const C *sm, C (&a)[1 << R],
                                                  C (&al)[1 << R], Real (&k)[NV]) {
     if constexpr (I >= 0) {
-        k[I] = single_sum<C, Real, R, I>(a, al, 1u);
-        C m0, m1, m2, m3;
-        load_mat(sm, (int)((ops >> (8 * I)) & 63u) - 1, m0, m1, m2, m3);
-        rot3_bit<C, Real, R, I>(a, m0.y, m1.y);
-        rot3_bit<C, Real, R, I>(al, m0.y, m1.y);
-        tile_ops_rev_rot<C, Real, R, I - 1, NV>(ops, sm, a, al, k);
+        if constexpr (kMat == kPair) {
+            const C v = pair_sum<C, R, I>(a, al);
+            k[2 * I] = v.x;
+            k[2 * I + 1] = v.y;
+        } else {
+            k[I] = single_sum<C, Real, R, I>(a, al, 1u);
+        }
+        C alpha, beta;
+        load_shear<C, kMat>(sm, (int)((ops >> (8 * I)) & 63u) - 1, alpha, beta);
+        rot3_bit<C, R, I>(a, alpha, beta);
+        rot3_bit<C, R, I>(al, alpha, beta);
+        tile_ops_rev_rot<C, Real, R, I - 1, NV, kMat>(ops, sm, a, al, k);
     }
 }
 
 // One reverse stage of single-sum ops: the branch-free path when register
 // bits 0..M-1 carry parametrised real rotations (M from the stage flags),
 // tile_ops_rev otherwise.
-template <typename C, typename Real, int R, int NV, bool kReal>
+template <typename C, typename Real, int R, int NV, int kMat>
 __device__ __forceinline__ void stage_ops_rev(uint32_t ops, uint32_t modes, uint32_t m,
                                               const C *sm, C (&a)[1 << R], C (&al)[1 << R],
                                               Real (&k)[NV]) {
     if constexpr (R >= 4) {
-        if (m == 4) return tile_ops_rev_rot<C, Real, R, 3, NV>(ops, sm, a, al, k);
+        if (m == 4) return tile_ops_rev_rot<C, Real, R, 3, NV, kMat>(ops, sm, a, al, k);
     }
     if constexpr (R >= 3) {
-        if (m == 3) return tile_ops_rev_rot<C, Real, R, 2, NV>(ops, sm, a, al, k);
+        if (m == 3) return tile_ops_rev_rot<C, Real, R, 2, NV, kMat>(ops, sm, a, al, k);
     }
-    if (m == 2) return tile_ops_rev_rot<C, Real, R, 1, NV>(ops, sm, a, al, k);
-    if (m == 1) return tile_ops_rev_rot<C, Real, R, 0, NV>(ops, sm, a, al, k);
-    tile_ops_rev<C, Real, R, R - 1, NV, true, kReal>(ops, modes, sm, a, al, k);
+    if (m == 2) return tile_ops_rev_rot<C, Real, R, 1, NV, kMat>(ops, sm, a, al, k);
+    if (m == 1) return tile_ops_rev_rot<C, Real, R, 0, NV, kMat>(ops, sm, a, al, k);
+    tile_ops_rev<C, Real, R, R - 1, NV, true, kMat>(ops, modes, sm, a, al, k);
 }
 
 // tile_ops_rev's four-sum complex path when register bits 0..M-1 all carry
@@ -372,7 +439,7 @@ __device__ __forceinline__ void tile_ops_rev_cplx(uint32_t ops, const C *sm, C (
 // One reverse stage of four-sum ops: the branch-free complex path when
 // register bits 0..M-1 carry parametrised complex matrices, tile_ops_rev
 // otherwise.
-template <typename C, typename Real, int R, int NV, bool kReal>
+template <typename C, typename Real, int R, int NV>
 __device__ __forceinline__ void stage_ops_rev4(uint32_t ops, uint32_t modes, uint32_t m,
                                                const C *sm, C (&a)[1 << R], C (&al)[1 << R],
                                                Real (&k)[NV]) {
@@ -384,15 +451,36 @@ __device__ __forceinline__ void stage_ops_rev4(uint32_t ops, uint32_t modes, uin
     }
     if (m == 2) return tile_ops_rev_cplx<C, Real, R, 1, NV>(ops, sm, a, al, k);
     if (m == 1) return tile_ops_rev_cplx<C, Real, R, 0, NV>(ops, sm, a, al, k);
-    tile_ops_rev<C, Real, R, R - 1, NV, false, kReal>(ops, modes, sm, a, al, k);
+    tile_ops_rev<C, Real, R, R - 1, NV, false, kAny>(ops, modes, sm, a, al, k);
 }
 
 // Adds the block's sums of slot b (FP64 over warps and lane quads), as i K
 // in reduced-matrix form, to rho_g[b][group][8] and clears them.  Called by
 // every thread.
-template <typename Real, bool kSingle>
+// kPair: b is a slot pair; lanes of lane bit 0 = c hold the sums of slot 2b + c
+// (rho_g has a row for each, also past an odd last slot).
+template <typename Real, bool kSingle, int kMat>
 __device__ void flush_acc(const TilePass &P, Real *acc, int wps, double *rho_g, int b, int G) {
     __syncthreads();
+    if constexpr (kMat == kPair) {
+        for (int x = threadIdx.x; x < P.n_ops * 2; x += blockDim.x) {
+            const int u = x >> 1, c = x & 1;
+            if (!((P.param_mask >> u) & 1ull)) continue;
+            double k = 0.0;
+            for (int w = 0; w < wps; ++w)
+                for (int q = c; q < 32; q += 2) {
+                    Real &r = acc[(u * wps + w) * 32 + q];
+                    k += (double)r;
+                    r = 0;
+                }
+            if (k == 0.0) continue;
+            double *dst = rho_g + ((size_t)(2 * b + c) * G + P.grp[u]) * 8;
+            atomicAdd(dst + 2, 0.5 * k);
+            atomicAdd(dst + 4, -0.5 * k);
+        }
+        __syncthreads();
+        return;
+    }
     for (int x = threadIdx.x; x < P.n_ops * 4; x += blockDim.x) {
         const int u = x >> 2;
         if (!((P.param_mask >> u) & 1ull)) continue;
@@ -429,7 +517,7 @@ __device__ void flush_acc(const TilePass &P, Real *acc, int wps, double *rho_g, 
 // reduced matrices of its parametrised groups (as i K) into
 // rho_g[slot][group][8].  The sums run in the state's precision over one
 // warp and at most 64 tiles, then in FP64.
-template <typename Real, int R, bool kSingle, bool kReal, int NB = 2>
+template <typename Real, int R, bool kSingle, int kMat, int NB = 2>
 __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_slots,
                                               const typename CT<Real>::T *mats, int G,
                                               const typename CT<Real>::T *psi_src,
@@ -487,7 +575,7 @@ __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_sl
     for (int64_t tix = t0, i = 0; tix < t_end; ++tix, ++i) {
         const int buf = NB == 2 ? (int)(i & 1) : 0;
         if (cur.slot != mslot || since == kFlushTiles) {
-            if (mslot >= 0) flush_acc<Real, kSingle>(P, acc, wps, rho_g, mslot, G);
+            if (mslot >= 0) flush_acc<Real, kSingle, kMat>(P, acc, wps, rho_g, mslot, G);
             since = 0;
         }
         if (cur.slot != mslot) {  // adjoint matrices of this slot's groups
@@ -495,15 +583,17 @@ __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_sl
                 const C *m = mats + ((size_t)cur.slot * G + P.grp[x >> 2]) * 4;
                 const int e = x & 3, te = e == 1 ? 2 : (e == 2 ? 1 : e);
                 C d = m[te];
-                d.y = -d.y;
+                if constexpr (kMat != kPair) d.y = -d.y;
                 sm[x] = d;
             }
             __syncthreads();
-            for (int u = tid; u < P.n_ops; u += T)
-                if ((P.real_mask >> u) & 1ull) stage_shears(sm + 4 * u);
-            if constexpr (std::is_same<C, float2>::value && kSingle == kReal) {
+            for (int u = tid; u < P.n_ops; u += T) {
+                if constexpr (kMat == kPair) stage_shears_pair(sm + 4 * u);
+                else if ((P.real_mask >> u) & 1ull) stage_shears(sm + 4 * u);
+            }
+            if constexpr (std::is_same<C, float2>::value && kSingle == (kMat != kAny)) {
                 __syncthreads();  // the branch-free paths' stage flags
-                set_stage_flags(P, rec, sm);
+                set_stage_flags<C, kMat>(P, rec, sm);
             }
             mslot = cur.slot;
         }
@@ -525,21 +615,28 @@ __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_sl
             }
             // the stage's sums: over lane quads in registers, then per lane
             // into the warp's accumulators
-            constexpr int NV = kSingle ? 4 : (4 * R <= 8 ? 8 : 16);
+            constexpr int NV = kMat == kPair ? (R <= 2 ? 4 : 8) : kSingle ? 4 : (4 * R <= 8 ? 8 : 16);
             Real kk[NV];
 #pragma unroll
             for (int v = 0; v < NV; ++v) kk[v] = 0;
-            if constexpr (kSingle && kReal && std::is_same<C, float2>::value) {
-                stage_ops_rev<C, Real, R, NV, kReal>(ops, modes, (rec[2 * s + 1].w >> 4) & 15u, sm, a,
+            if constexpr (kSingle && kMat != kAny && std::is_same<C, float2>::value) {
+                stage_ops_rev<C, Real, R, NV, kMat>(ops, modes, (rec[2 * s + 1].w >> 4) & 15u, sm, a,
                                                      al, kk);
-            } else if constexpr (!kSingle && !kReal && std::is_same<C, float2>::value) {
-                stage_ops_rev4<C, Real, R, NV, kReal>(ops, modes, (rec[2 * s + 1].w >> 12) & 15u, sm,
+            } else if constexpr (!kSingle && kMat == kAny && std::is_same<C, float2>::value) {
+                stage_ops_rev4<C, Real, R, NV>(ops, modes, (rec[2 * s + 1].w >> 12) & 15u, sm,
                                                       a, al, kk);
             } else {
-                tile_ops_rev<C, Real, R, R - 1, NV, kSingle, kReal>(ops, modes, sm, a, al, kk);
+                tile_ops_rev<C, Real, R, R - 1, NV, kSingle, kMat>(ops, modes, sm, a, al, kk);
             }
             warp_reduce_quad<Real, NV>(kk, lane);
-            if constexpr (kSingle) {  // lane: the sum of register bit lane & 3
+            if constexpr (kMat == kPair) {  // lane: bit 2 m + (lane >> 1 & 1), state lane & 1
+#pragma unroll
+                for (int m = 0; m < NV / 4; ++m) {
+                    const int i = 2 * m + ((lane >> 1) & 1);
+                    const uint32_t ob = i < R ? (ops >> (8 * i)) & 0xffu : 0u;
+                    if (ob & 128u) accw[((int)(ob & 63u) - 1) * wps * 32] += kk[m];
+                }
+            } else if constexpr (kSingle) {  // lane: the sum of register bit lane & 3
                 const int m = lane & 3;
                 const uint32_t ob = m < R ? (ops >> (8 * m)) & 0xffu : 0u;
                 if (ob & 128u) accw[((int)(ob & 63u) - 1) * wps * 32] += kk[0];
@@ -583,11 +680,11 @@ __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_sl
         cur = nxt;
         nxt = tile_next(P, nxt);
     }
-    flush_acc<Real, kSingle>(P, acc, wps, rho_g, mslot, G);
+    flush_acc<Real, kSingle, kMat>(P, acc, wps, rho_g, mslot, G);
 }
 
 // NB = 1: launched with 64 threads only (at least five blocks per SM).
-template <typename Real, int R, bool kSingle, bool kReal, int NB = 2>
+template <typename Real, int R, bool kSingle, int kMat, int NB = 2>
 __global__ void __launch_bounds__(NB == 1 ? 64 : 256, NB == 1 ? 5 : (R >= 4 ? 1 : 2))
 k_tile_rev(const __grid_constant__ TilePass P, int n, int n_slots,
            const typename CT<Real>::T *mats, int G, const typename CT<Real>::T *psi_src,
@@ -595,7 +692,7 @@ k_tile_rev(const __grid_constant__ TilePass P, int n, int n_slots,
     extern __shared__ __align__(16) unsigned char smem[];
     int64_t t0, t_end;
     block_range((int64_t)n_slots << P.n_tile_bits, gridDim.x, blockIdx.x, t0, t_end);
-    tile_rev_body<Real, R, kSingle, kReal, NB>(P, n, n_slots, mats, G, psi_src, psi, lam, rho_g,
+    tile_rev_body<Real, R, kSingle, kMat, NB>(P, n, n_slots, mats, G, psi_src, psi, lam, rho_g,
                                                t0, t_end, smem, write_psi != 0);
 }
 
@@ -693,11 +790,11 @@ k_tile_sweep(const SweepTask *tasks, int n_tasks, long long n_tickets,
         const int64_t t0 = c * (int64_t)T.chunk_tiles;
         const int64_t t1 = min(T.tiles, t0 + (int64_t)T.chunk_tiles);
         if constexpr (kRev)
-            tile_rev_body<Real, R, false, false>(P, T.n, T.n_slots, (const C *)T.mats, T.G,
+            tile_rev_body<Real, R, false, kAny>(P, T.n, T.n_slots, (const C *)T.mats, T.G,
                                                  (const C *)T.psi, (C *)T.psi, (C *)T.lam, T.rho,
                                                  t0, t1, rest);
         else
-            tile_fwd_body<Real, R, false>(P, T.n, T.n_slots, (const C *)T.mats, T.G,
+            tile_fwd_body<Real, R, kAny>(P, T.n, T.n_slots, (const C *)T.mats, T.G,
                                           (const C *)T.psi, (C *)T.psi, t0, t1, rest);
         __syncthreads();  // every store of the chunk issued
         if (threadIdx.x == 0) {
@@ -752,11 +849,13 @@ template <typename Real> struct HCoef {
 // thread bits (the row's class coefficients times their register-bit signs,
 // built once per tile by the whole block), each row added with the sign of
 // its thread-bit mask.  Products in the state's precision, sums over the
-// block's amplitudes in FP64.  kLam = false: energies only.
-template <typename Real, int R, bool kLam, bool kRealH>
+// block's amplitudes in FP64.  kLam = false: energies only.  kPair (with
+// kRealH): each state holds the real states of slots 2 slot and 2 slot + 1,
+// whose energies are summed apart (those below e_rows are written).
+template <typename Real, int R, bool kLam, bool kRealH, bool kPairE>
 __global__ void __launch_bounds__(256)
 k_tile_h(const __grid_constant__ HPass P, int n, int n_slots, const typename CT<Real>::T *psi,
-         typename CT<Real>::T *lam, double *E) {
+         typename CT<Real>::T *lam, double *E, int e_rows) {
     using C = typename CT<Real>::T;
     constexpr int NA = 1 << R;
     static_assert(R <= kHRegBitsMax, "H kernel register bits");
@@ -799,14 +898,23 @@ k_tile_h(const __grid_constant__ HPass P, int n, int n_slots, const typename CT<
     TileCursor cur = h_cursor(P, t0);
     fetch(cur, 0);
     TileCursor nxt = h_next(P, cur);
-    double e_acc = 0.0;
+    double e_acc = 0.0, e_acc2 = 0.0;
     int eslot = cur.slot;
+    auto add_energy = [&]() {  // the slot's energy so far
+        const double s = block_sum(e_acc, red);
+        if constexpr (kPairE) {
+            const double s2 = block_sum(e_acc2, red);
+            if (tid == 0) atomicAdd(&E[2 * eslot], s);
+            if (tid == 0 && 2 * eslot + 1 < e_rows) atomicAdd(&E[2 * eslot + 1], s2);
+        } else {
+            if (tid == 0) atomicAdd(&E[eslot], s);
+        }
+        e_acc = e_acc2 = 0.0;
+    };
     for (int64_t tix = t0, i = 0; tix < t_end; ++tix, ++i) {
         const int buf = (int)(i & 1);
-        if (cur.slot != eslot) {  // the slot's energy so far
-            const double s = block_sum(e_acc, red);
-            if (tid == 0) atomicAdd(&E[eslot], s);
-            e_acc = 0.0;
+        if (cur.slot != eslot) {
+            add_energy();
             eslot = cur.slot;
         }
         for (int c = tid; c < P.n_classes; c += T) {  // this tile's class records
@@ -937,11 +1045,16 @@ k_tile_h(const __grid_constant__ HPass P, int n, int n_slots, const typename CT<
             }
         }
         if (add) cp_async_wait_prior();  // own copies of the lambda tile have landed
-        Real part = 0;
+        Real part = 0, part2 = 0;
 #pragma unroll
         for (int k = 0; k < NA; ++k) {
             const C pj = tile[tid + k * T];
-            part = fmaR(pj.x, acc[k].x, fmaR(pj.y, acc[k].y, part));
+            if constexpr (kPairE) {
+                part = fmaR(pj.x, acc[k].x, part);
+                part2 = fmaR(pj.y, acc[k].y, part2);
+            } else {
+                part = fmaR(pj.x, acc[k].x, fmaR(pj.y, acc[k].y, part));
+            }
             if constexpr (kLam) {
                 const uint32_t go = g0 ^ xsel<R>(k, gk);
                 C out = acc[k];
@@ -954,12 +1067,12 @@ k_tile_h(const __grid_constant__ HPass P, int n, int n_slots, const typename CT<
             }
         }
         e_acc += (double)part;
+        if constexpr (kPairE) e_acc2 += (double)part2;
         __syncthreads();  // coef and this buffer are rewritten next
         cur = nxt;
         nxt = h_next(P, nxt);
     }
-    const double s = block_sum(e_acc, red);
-    if (tid == 0) atomicAdd(&E[eslot], s);
+    add_energy();
 }
 
 // D_g(j) = sum_{t in g} c_t i^{phase_t} (-1)^{|j & z_t|} for one amplitude.
@@ -1180,21 +1293,22 @@ int grid_1d(int64_t work, int threads) {
     } while (0)
 
 cudaError_t launch_group_mats(int c128, const Program &p, const SlotSource &src, void *mats,
-                              cudaStream_t st) {
+                              cudaStream_t st, bool pair) {
     const int g = grid_1d((int64_t)src.n_slots * p.n_groups, 128);
-    if (c128) k_group_mats<double><<<g, 128, 0, st>>>(p, src, (double2 *)mats);
-    else k_group_mats<float><<<g, 128, 0, st>>>(p, src, (float2 *)mats);
+    if (c128) k_group_mats<double><<<g, 128, 0, st>>>(p, src, pair, (double2 *)mats);
+    else k_group_mats<float><<<g, 128, 0, st>>>(p, src, pair, (float2 *)mats);
     return cudaGetLastError();
 }
 
 cudaError_t launch_init_states(int c128, void *states, int n, const SlotSource &src,
-                               cudaStream_t st) {
-    const size_t bytes = ((size_t)src.n_slots << n) * (c128 ? 16 : 8);
+                               cudaStream_t st, bool pair) {
+    const size_t n_states = pair ? ((size_t)src.n_slots + 1) / 2 : (size_t)src.n_slots;
+    const size_t bytes = (n_states << n) * (c128 ? 16 : 8);
     cudaError_t e = cudaMemsetAsync(states, 0, bytes, st);
     if (e != cudaSuccess) return e;
     const int g = grid_1d(src.n_slots, 128);
-    if (c128) k_set_ref<double2><<<g, 128, 0, st>>>((double2 *)states, n, src);
-    else k_set_ref<float2><<<g, 128, 0, st>>>((float2 *)states, n, src);
+    if (c128) k_set_ref<double2><<<g, 128, 0, st>>>((double2 *)states, n, src, pair);
+    else k_set_ref<float2><<<g, 128, 0, st>>>((float2 *)states, n, src, pair);
     return cudaGetLastError();
 }
 
@@ -1214,13 +1328,14 @@ uint32_t tile_rev_smem(int c128, const TilePass &P, int bufs) {
 
 cudaError_t launch_tile_fwd(int c128, const TilePass &P, int n, int n_slots, const void *mats,
                             int G, void *states, int64_t max_blocks, cudaStream_t st,
-                            const void *src) {
+                            const void *src, bool pair) {
     const uint32_t smem = tile_fwd_smem(c128, P);
     const int threads = 1 << (P.t - P.R);
     if (!src) src = states;
     HBM_DISPATCH_R(c128, P.R, {
         using C = typename CT<Real>::T;
-        auto k = pass_all_real(P) ? k_tile_fwd<Real, RR, true> : k_tile_fwd<Real, RR, false>;
+        auto k = pair ? k_tile_fwd<Real, RR, kPair>
+                      : (pass_all_real(P) ? k_tile_fwd<Real, RR, kReal> : k_tile_fwd<Real, RR, kAny>);
         cudaError_t e = allow_smem(k, smem);
         if (e != cudaSuccess) return e;
         const int blocks = fill_blocks(k, threads, smem, max_blocks);
@@ -1232,22 +1347,24 @@ cudaError_t launch_tile_fwd(int c128, const TilePass &P, int n, int n_slots, con
 
 cudaError_t launch_tile_rev(int c128, const TilePass &P, int n, int n_slots, const void *mats,
                             int G, void *psi, void *lam, double *rho_g, int64_t max_blocks,
-                            cudaStream_t st, const void *psi_src, bool write_psi) {
+                            cudaStream_t st, const void *psi_src, bool write_psi, bool pair) {
     // passes of many stages are arithmetic-bound: one tile buffer, more
     // blocks per SM (complex64 real single-sum passes, tiles of 2^10 at 16
     // amplitudes per thread: 64 threads)
-    const bool one_buf = !c128 && P.R == 4 && P.t == 10 && P.all_single && pass_all_real(P) &&
+    const bool one_buf = !c128 && P.R == 4 && P.t == 10 &&
+                         (pair || (P.all_single && pass_all_real(P))) &&
                          P.n_stages >= kOneBufStages;
     const uint32_t smem = tile_rev_smem(c128, P, one_buf ? 1 : 2);
     const int threads = 1 << (P.t - P.R);
     HBM_DISPATCH_R(c128, P.R, {
         using C = typename CT<Real>::T;
-        auto k = P.all_single ? (pass_all_real(P) ? k_tile_rev<Real, RR, true, true>
-                                                  : k_tile_rev<Real, RR, true, false>)
-                              : (pass_all_real(P) ? k_tile_rev<Real, RR, false, true>
-                                                  : k_tile_rev<Real, RR, false, false>);
+        auto k = pair ? k_tile_rev<Real, RR, true, kPair>
+                 : P.all_single ? (pass_all_real(P) ? k_tile_rev<Real, RR, true, kReal>
+                                                    : k_tile_rev<Real, RR, true, kAny>)
+                                : (pass_all_real(P) ? k_tile_rev<Real, RR, false, kReal>
+                                                    : k_tile_rev<Real, RR, false, kAny>);
         if constexpr (std::is_same<Real, float>::value && RR == 4) {
-            if (one_buf) k = k_tile_rev<Real, RR, true, true, 1>;
+            if (one_buf) k = pair ? k_tile_rev<Real, RR, true, kPair, 1> : k_tile_rev<Real, RR, true, kReal, 1>;
         }
         cudaError_t e = allow_smem(k, smem);
         if (e != cudaSuccess) return e;
@@ -1269,7 +1386,7 @@ uint32_t tile_h_smem(int c128, const HPass &P) {
 }
 
 cudaError_t launch_tile_h(int c128, const HPass &P, int n, int n_slots, const void *psi, void *lam,
-                          double *E, int64_t max_blocks, cudaStream_t st) {
+                          double *E, int64_t max_blocks, cudaStream_t st, int pair_rows) {
     const uint32_t smem = tile_h_smem(c128, P);
     // 2^R amplitudes per thread (R = h_reg_bits(t), the planner's bucketing)
     const int R = h_reg_bits(P.t);
@@ -1279,22 +1396,26 @@ cudaError_t launch_tile_h(int c128, const HPass &P, int n, int n_slots, const vo
         cudaError_t e = allow_smem(k, smem);
         if (e != cudaSuccess) return e;
         const int blocks = fill_blocks(k, threads, smem, max_blocks);
-        k<<<blocks, threads, smem, st>>>(P, n, n_slots, psi_t, lam_t, E);
+        k<<<blocks, threads, smem, st>>>(P, n, n_slots, psi_t, lam_t, E, pair_rows);
         return cudaGetLastError();
     };
-    auto pick2 = [&](auto rr, auto re) -> cudaError_t {
+    auto pick2 = [&](auto rr, auto re, auto pr) -> cudaError_t {
         constexpr int RR = decltype(rr)::value;
-        constexpr bool RE = decltype(re)::value;
+        constexpr bool RE = decltype(re)::value, PR = decltype(pr)::value;
         if (c128) {
-            if (lam) return go(k_tile_h<double, RR, true, RE>, (const double2 *)psi, (double2 *)lam);
-            return go(k_tile_h<double, RR, false, RE>, (const double2 *)psi, (double2 *)nullptr);
+            if (lam) return go(k_tile_h<double, RR, true, RE, PR>, (const double2 *)psi, (double2 *)lam);
+            return go(k_tile_h<double, RR, false, RE, PR>, (const double2 *)psi, (double2 *)nullptr);
         }
-        if (lam) return go(k_tile_h<float, RR, true, RE>, (const float2 *)psi, (float2 *)lam);
-        return go(k_tile_h<float, RR, false, RE>, (const float2 *)psi, (float2 *)nullptr);
+        if (lam) return go(k_tile_h<float, RR, true, RE, PR>, (const float2 *)psi, (float2 *)lam);
+        return go(k_tile_h<float, RR, false, RE, PR>, (const float2 *)psi, (float2 *)nullptr);
     };
     auto pick = [&](auto rr) -> cudaError_t {
-        if (P.real) return pick2(rr, std::true_type());
-        return pick2(rr, std::false_type());
+        if (pair_rows > 0) {
+            if (!P.real) return cudaErrorInvalidValue;
+            return pick2(rr, std::true_type(), std::true_type());
+        }
+        if (P.real) return pick2(rr, std::true_type(), std::false_type());
+        return pick2(rr, std::false_type(), std::false_type());
     };
     if (R == 4) return pick(std::integral_constant<int, 4>());
     if (R == 3) return pick(std::integral_constant<int, 3>());

@@ -8,12 +8,15 @@
 
 namespace svk {
 
+// pair (here and below): two real circuits per state (slots 2j and 2j + 1 in
+// the components of state j); the launchers' slot counts are then pairs,
+// except in a SlotSource and in pair_rows.
 // mats: [slots][groups][4] complex of the state's precision.
 cudaError_t launch_group_mats(int c128, const Program &p, const SlotSource &src, void *mats,
-                              cudaStream_t st);
+                              cudaStream_t st, bool pair = false);
 // Zeroes the slot states and sets amplitude |ref> of each to 1.
 cudaError_t launch_init_states(int c128, void *states, int n, const SlotSource &src,
-                               cudaStream_t st);
+                               cudaStream_t st, bool pair = false);
 // Shared memory of one block of the forward / reverse kernels of pass P.
 uint32_t tile_fwd_smem(int c128, const TilePass &P);
 uint32_t tile_rev_smem(int c128, const TilePass &P, int bufs = 2);
@@ -21,16 +24,16 @@ uint32_t tile_rev_smem(int c128, const TilePass &P, int bufs = 2);
 // src (null: states) holds the pass's input; the output goes to states.
 cudaError_t launch_tile_fwd(int c128, const TilePass &P, int n, int n_slots, const void *mats,
                             int G, void *states, int64_t max_blocks, cudaStream_t st,
-                            const void *src = nullptr);
+                            const void *src = nullptr, bool pair = false);
 // Reverse pass P on psi and lambda; adds the reduced matrices of its
 // parametrised groups to rho_g[slot][G][8].  psi_src (null: psi) holds the
 // psi the pass reads (a stored forward state); its output psi goes to psi
 // unless write_psi is false (the next reverse pass restarts psi from a
-// stored state, or this is the last one).
+// stored state, or this is the last one).  pair: rho_g has two rows per state.
 cudaError_t launch_tile_rev(int c128, const TilePass &P, int n, int n_slots, const void *mats,
                             int G, void *psi, void *lam, double *rho_g, int64_t max_blocks,
                             cudaStream_t st, const void *psi_src = nullptr,
-                            bool write_psi = true);
+                            bool write_psi = true, bool pair = false);
 // Codes a kernel writes to the library's device error word when a bounded
 // device-side wait gives up (reported as SV_ERR_TIMEOUT by sv_sync_status).
 constexpr int SV_DEVERR_MMA_WAIT = 1;
@@ -63,9 +66,10 @@ cudaError_t launch_tile_sweep(int c128, int R, bool rev, const SweepTask *tasks,
                               int *err, int blocks, int threads, uint32_t smem, cudaStream_t st);
 // One tile pass of lambda = H psi (lam may be null: energies only); adds this
 // pass's part of <psi|H|psi> to E[slot] (zero E before the first pass).
+// pair_rows > 0: pairs of real states whose E has pair_rows entries.
 uint32_t tile_h_smem(int c128, const HPass &P);
 cudaError_t launch_tile_h(int c128, const HPass &P, int n, int n_slots, const void *psi, void *lam,
-                          double *E, int64_t max_blocks, cudaStream_t st);
+                          double *E, int64_t max_blocks, cudaStream_t st, int pair_rows = 0);
 // Data-driven circuit learning: js[r] = JS(target | |psi_r|^2) (zeroed here
 // first) and lam_r = dJS/d|psi_r|^2 * psi_r elementwise.
 cudaError_t launch_ddcl_lambda(int c128, int n, int n_rows, const void *psi, const double *target,

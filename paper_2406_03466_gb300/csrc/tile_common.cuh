@@ -148,10 +148,12 @@ __device__ __forceinline__ void load_mat(const double2 *sm, int u, double2 &m0, 
 // shears: x += alpha y; y += beta x; x += alpha y, with alpha = -s / (1 + c)
 // = -tan(angle / 2) and beta = s (both in [-1, 1]): three fused
 // multiply-adds per amplitude pair and component instead of four.
-template <typename C, typename Real, int R, int I>
-__device__ __forceinline__ void rot3_bit(C (&a)[1 << R], const Real alpha, const Real beta) {
+// alpha and beta are given per component: the same value twice for a complex
+// amplitude, two circuits' values for a pair of real states (kPair).
+template <typename C, int R, int I>
+__device__ __forceinline__ void rot3_bit(C (&a)[1 << R], const C alpha, const C beta) {
     if constexpr (std::is_same<C, float2>::value) {
-        const uint64_t pa = f2pack(alpha, alpha), pb = f2pack(beta, beta);
+        const uint64_t pa = f2of(alpha), pb = f2of(beta);
 #pragma unroll
         for (int r = 0; r < (1 << R); ++r) {
             if (r & (1 << I)) continue;
@@ -167,17 +169,49 @@ __device__ __forceinline__ void rot3_bit(C (&a)[1 << R], const Real alpha, const
         for (int r = 0; r < (1 << R); ++r) {
             if (r & (1 << I)) continue;
             C x = a[r], y = a[r | (1 << I)];
-            x.x = fmaR(alpha, y.x, x.x);
-            x.y = fmaR(alpha, y.y, x.y);
-            y.x = fmaR(beta, x.x, y.x);
-            y.y = fmaR(beta, x.y, y.y);
-            x.x = fmaR(alpha, y.x, x.x);
-            x.y = fmaR(alpha, y.y, x.y);
+            x.x = fmaR(alpha.x, y.x, x.x);
+            x.y = fmaR(alpha.y, y.y, x.y);
+            y.x = fmaR(beta.x, x.x, y.x);
+            y.y = fmaR(beta.y, x.y, y.y);
+            x.x = fmaR(alpha.x, y.x, x.x);
+            x.y = fmaR(alpha.y, y.y, x.y);
             a[r] = x;
             a[r | (1 << I)] = y;
         }
     }
 }
+template <typename C, typename Real> __device__ __forceinline__ C both(Real v) {
+    C c;
+    c.x = c.y = v;
+    return c;
+}
+
+// Real 2x2 matrices of a pair of real states (component = state) on register
+// bit I.
+template <typename C, int R, int I>
+__device__ __forceinline__ void u1p_bit(C (&a)[1 << R], const C m0, const C m1, const C m2,
+                                        const C m3) {
+#pragma unroll
+    for (int r = 0; r < (1 << R); ++r) {
+        if (r & (1 << I)) continue;
+        const C x = a[r], y = a[r | (1 << I)];
+        if constexpr (std::is_same<C, float2>::value) {
+            a[r] = f2unpack(f2fma(f2of(m0), f2of(x), f2mul(f2of(m1), f2of(y))));
+            a[r | (1 << I)] = f2unpack(f2fma(f2of(m2), f2of(x), f2mul(f2of(m3), f2of(y))));
+        } else {
+            a[r].x = fmaR(m0.x, x.x, m1.x * y.x);
+            a[r].y = fmaR(m0.y, x.y, m1.y * y.y);
+            a[r | (1 << I)].x = fmaR(m2.x, x.x, m3.x * y.x);
+            a[r | (1 << I)].y = fmaR(m2.y, x.y, m3.y * y.y);
+        }
+    }
+}
+
+// What a pass's staged matrices are.  kAny: complex or real per group.
+// kReal: every group real.  kPair: the amplitude's components are the real
+// amplitudes of two circuits and entry k of a matrix is (first circuit's,
+// second circuit's).
+enum MatKind { kAny = 0, kReal = 1, kPair = 2 };
 
 // The imaginary parts of a staged real matrix are unused: for a real
 // rotation with c > 0 they carry the shear form (m0.y = alpha, m1.y = beta,
@@ -193,25 +227,71 @@ __device__ __forceinline__ void stage_shears(C *m) {
     m[3].y = (Real)0;
 }
 
+// The same for a pair of real states: rotations of both circuits (c >= 0:
+// the matrices come with that sign) become m0 = alpha, m1 = beta, m2 = m3 =
+// 0, which no orthogonal matrix has.
+template <typename C> __device__ __forceinline__ void stage_shears_pair(C *m) {
+    using Real = decltype(m[0].x);
+    if (m[3].x != m[0].x || m[1].x != -m[2].x || m[0].x < (Real)0 || m[3].y != m[0].y ||
+        m[1].y != -m[2].y || m[0].y < (Real)0)
+        return;
+    const C s = m[2];
+    m[0].x = -s.x / ((Real)1 + m[0].x);
+    m[0].y = -s.y / ((Real)1 + m[0].y);
+    m[1] = s;
+    m[2].x = m[2].y = m[3].x = m[3].y = (Real)0;
+}
+template <typename C> __device__ __forceinline__ bool is_shear_pair(const C m2, const C m3) {
+    return m2.x == 0 && m3.x == 0;
+}
+
+// Matrix (m0..m3) of an op on register bit I, by what the pass stages; real:
+// the op's own flag (kAny).
+template <typename C, int R, int I, int kMat>
+__device__ __forceinline__ void op_bit(bool real, const C m0, const C m1, const C m2, const C m3,
+                                       C (&a)[1 << R]) {
+    if constexpr (kMat == kPair) {
+        if (is_shear_pair(m2, m3)) rot3_bit<C, R, I>(a, m0, m1);
+        else u1p_bit<C, R, I>(a, m0, m1, m2, m3);
+    } else if (kMat == kReal || real) {
+        if (m2.y != 0) rot3_bit<C, R, I>(a, both<C>(m0.y), both<C>(m1.y));
+        else u1r_bit<C, decltype(m0.x), R, I>(a, m0.x, m1.x, m2.x, m3.x);
+    } else {
+        u1_bit<C, R, I>(a, m0, m1, m2, m3);
+    }
+}
+
+// (alpha, beta) of op u's shear form.
+template <typename C, int kMat>
+__device__ __forceinline__ void load_shear(const C *sm, int u, C &alpha, C &beta) {
+    if constexpr (kMat == kPair) {
+        if constexpr (std::is_same<C, float2>::value) {
+            const float4 v = reinterpret_cast<const float4 *>(sm)[2 * u];
+            alpha = make_float2(v.x, v.y);
+            beta = make_float2(v.z, v.w);
+        } else {
+            alpha = sm[4 * u];
+            beta = sm[4 * u + 1];
+        }
+    } else {
+        C m0, m1, m2, m3;
+        load_mat(sm, u, m0, m1, m2, m3);
+        alpha = both<C>(m0.y);
+        beta = both<C>(m1.y);
+    }
+}
+
 // The group ops of one stage (op bytes `ops`), register bits I..R-1 in order.
-// kReal: every op of the pass has a real matrix (no complex path compiled).
-template <typename C, int R, int I, bool kReal>
+template <typename C, int R, int I, int kMat>
 __device__ __forceinline__ void tile_ops_fwd(uint32_t ops, const C *sm, C (&a)[1 << R]) {
     if constexpr (I < R) {
         const uint32_t ob = (ops >> (8 * I)) & 0xffu;
         if (ob) {
             C m0, m1, m2, m3;
             load_mat(sm, (int)(ob & 63u) - 1, m0, m1, m2, m3);
-            if (kReal || (ob & 64u)) {
-                if (m2.y != 0)
-                    rot3_bit<C, decltype(m0.x), R, I>(a, m0.y, m1.y);
-                else
-                    u1r_bit<C, decltype(m0.x), R, I>(a, m0.x, m1.x, m2.x, m3.x);
-            } else {
-                u1_bit<C, R, I>(a, m0, m1, m2, m3);
-            }
+            op_bit<C, R, I, kMat>((ob & 64u) != 0, m0, m1, m2, m3, a);
         }
-        tile_ops_fwd<C, R, I + 1, kReal>(ops, sm, a);
+        tile_ops_fwd<C, R, I + 1, kMat>(ops, sm, a);
     }
 }
 
@@ -219,13 +299,13 @@ __device__ __forceinline__ void tile_ops_fwd(uint32_t ops, const C *sm, C (&a)[1
 // shear form and the others carry no op (stage flags): the arithmetic of
 // tile_ops_fwd without its per-op branches, so the compiler can overlap one
 // op's dependent FMA chains with the next op's.
-template <typename C, int R, int I, int M>
+template <typename C, int R, int I, int M, int kMat>
 __device__ __forceinline__ void tile_ops_fwd_rot(uint32_t ops, const C *sm, C (&a)[1 << R]) {
     if constexpr (I < M) {
-        C m0, m1, m2, m3;
-        load_mat(sm, (int)((ops >> (8 * I)) & 63u) - 1, m0, m1, m2, m3);
-        rot3_bit<C, decltype(m0.x), R, I>(a, m0.y, m1.y);
-        tile_ops_fwd_rot<C, R, I + 1, M>(ops, sm, a);
+        C alpha, beta;
+        load_shear<C, kMat>(sm, (int)((ops >> (8 * I)) & 63u) - 1, alpha, beta);
+        rot3_bit<C, R, I>(a, alpha, beta);
+        tile_ops_fwd_rot<C, R, I + 1, M, kMat>(ops, sm, a);
     }
 }
 
@@ -252,7 +332,8 @@ __device__ __forceinline__ void tile_ops_fwd_cplx(uint32_t ops, const C *sm, C (
 // when those complex ops are moreover all parametrised (the reverse's
 // four-sum path); 0 otherwise.  Called by every thread once the slot's
 // shear forms are in shared memory; visible after the next barrier.
-template <typename C>
+// kPair: every op is real and its parameters all rotate about Y.
+template <typename C, int kMat>
 __device__ __forceinline__ void set_stage_flags(const TilePass &P, uint4 *rec, const C *sm) {
     for (int s = threadIdx.x; s < P.n_stages; s += blockDim.x) {
         const uint32_t ops = rec[2 * s].x, modes = rec[2 * s + 1].y;
@@ -261,10 +342,11 @@ __device__ __forceinline__ void set_stage_flags(const TilePass &P, uint4 *rec, c
         for (int i = 0; i < P.R; ++i) {
             const uint32_t ob = (ops >> (8 * i)) & 0xffu;
             if (!ob) break;
-            rot = rot && (ob & 64u) && sm[4 * ((int)(ob & 63u) - 1) + 2].y != 0;
+            const C *mt = sm + 4 * ((int)(ob & 63u) - 1);
+            rot = rot && (ob & 64u) && (kMat == kPair ? is_shear_pair(mt[2], mt[3]) : mt[2].y != 0);
             cplx = cplx && !(ob & 64u);
             if (rot) {
-                single = single && (ob & 128u) && ((modes >> (8 * i)) & 3u) == 1u;
+                single = single && (ob & 128u) && (kMat == kPair || ((modes >> (8 * i)) & 3u) == 1u);
                 m = i + 1;
             }
             if (cplx) {

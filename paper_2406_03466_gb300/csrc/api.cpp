@@ -799,7 +799,7 @@ sv_status tiles_energies(DeviceCtx *ctx, const sv_problem *p, const double *thet
     s = get_array(ctx, p->refs, sizeof(int64_t) * I, &drefs);
     if (s != SV_OK) return s;
     const size_t csz = c128 ? 16 : 8, sb = csz << n;
-    const size_t mb = (size_t)pe->dev.n_groups * 4 * csz;
+    const size_t mb = (size_t)pe->dev.n_groups * kMatVals * csz;
     const size_t per = sb + mb;
     const bool pair = real_pairs(pe, obs, n_slots, cfg.tc);
     const int per_state = pair ? 2 : 1;  // slots
@@ -896,7 +896,7 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     const int n_states = (I + per_state - 1) / per_state;
     auto bytes_per_state = [&](int ev) {
         const size_t ncp_ = npass > 1 ? (size_t)((npass - 1) / ev) : 0;
-        return (2 + ncp_) * sb + (size_t)G * 4 * csz + (size_t)per_state * G * 64;
+        return (2 + ncp_) * sb + (size_t)G * kMatVals * csz + (size_t)per_state * G * 64;
     };
     if (every <= 0) {
         // The most stored states that still let every instance run at once:
@@ -919,7 +919,7 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
     const size_t o_lam = up((size_t)chunk * sb), o_ck = o_lam + up((size_t)chunk * sb);
     const size_t o_mats = o_ck + up((size_t)ncp * chunk * sb);
-    const size_t o_rho = o_mats + up((size_t)chunk * G * 4 * csz);
+    const size_t o_rho = o_mats + up((size_t)chunk * G * kMatVals * csz);
     const size_t total = o_rho + up((size_t)chunk * per_state * G * 64);
     void *big = nullptr;
     s = get_big_scratch(ctx, st, total, &big);
@@ -1137,7 +1137,7 @@ sv_status multi_adjoint(DeviceCtx *ctx, const sv_problem *problems, int np,
         m.o_tp = take(sizeof(TilePass) * (size_t)m.npass);
         m.o_psi = take(((size_t)m.I << m.n) * csz);
         m.o_lam = take(((size_t)m.I << m.n) * csz);
-        m.o_mats = take((size_t)m.I * m.G * 4 * csz);
+        m.o_mats = take((size_t)m.I * m.G * kMatVals * csz);
         m.o_rho = take((size_t)m.I * m.G * 64);
         m.o_E = take(sizeof(double) * (size_t)m.I);
         m.o_G = take(sizeof(double) * (size_t)m.I * (m.P > 0 ? m.P : 1));
@@ -1380,7 +1380,7 @@ sv_status sv_apply_circuit_batch(sv_state state, const sv_circuit *circuits, int
             if (s != SV_OK) return s;
             const size_t csz = state->dtype == SV_C128 ? 16 : 8;
             void *mats = nullptr;
-            s = get_big_scratch(ctx, st, sub.size() * pe->dev.n_groups * 4 * csz + 256, &mats);
+            s = get_big_scratch(ctx, st, sub.size() * pe->dev.n_groups * kMatVals * csz + 256, &mats);
             if (s != SV_OK) return s;
             SlotSource src{};
             src.mode = SLOTS_EXPLICIT;
@@ -1974,7 +1974,7 @@ sv_status sv_grad_ddcl_param_shift(const sv_problem *p, const double *theta,
     if (s != SV_OK) return s;
     double *E = (double *)scr, *lp = E + B, *D = lp + 1;
     const size_t csz = c128 ? 16 : 8, sb = csz << n;
-    const size_t mb = (size_t)pe->dev.n_groups * 4 * csz;
+    const size_t mb = (size_t)pe->dev.n_groups * kMatVals * csz;
     int64_t chunk = (int64_t)(big_budget(ctx, st) / (sb + mb + 512));
     if (chunk < 1) return fail(SV_ERR_OOM, "one state does not fit in free device memory");
     if (chunk > B) chunk = B;

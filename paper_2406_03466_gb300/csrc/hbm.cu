@@ -37,6 +37,7 @@ namespace {
 
 // Fused 2x2 matrices of every group for every slot: out[slot][group][4], or
 // with pair out[slot pair][group][4], entry k = (first slot's, second slot's).
+// Without pair the groups' split forms follow, [slot][group][4].
 // Formed in FP64 and rounded once, so that a pass's error is its own.  A
 // pair's real rotations come with c >= 0 (a state's sign is of no account
 // to its energy and its gradient), for the shear form.
@@ -53,6 +54,7 @@ __global__ void k_group_mats(Program p, SlotSource src, int pair, typename CT<Re
             const SlotInfo si = resolve(src, pair ? min(2 * b + c, src.n_slots - 1) : b);
             double2 d[4];
             group_matrix<double, double2, Real>(p, g, si, d);
+            if (!pair) split_form(d, out + (size_t)(total + i) * 4);
             const double sg = d[0].x < 0.0 && d[0].x == d[3].x && d[1].x == -d[2].x ? -1.0 : 1.0;
             for (int k = 0; k < 4; ++k) {
                 if (!pair) m[k] = cmk<C>(d[k].x, d[k].y);
@@ -75,13 +77,12 @@ __global__ void k_set_ref(C *states, int n, SlotSource src, int pair) {
     }
 }
 
-// One forward pass over every tile of every slot.  mats: [slots][G][4].
 // One forward stage: a branch-free path when register bits 0..M-1 carry
-// real rotations in shear form or complex matrices (M from the stage
-// flags), tile_ops_fwd otherwise.
+// real rotations in shear form or the stage runs in split form (M from the
+// stage flags), tile_ops_fwd otherwise.
 template <typename C, int R, int kMat>
 __device__ __forceinline__ void stage_ops_fwd(uint32_t ops, uint32_t flags, const C *sm,
-                                              C (&a)[1 << R]) {
+                                              const C *tab, C (&a)[1 << R]) {
     const uint32_t m = flags & 15u;
     if constexpr (R >= 4) {
         if (m == 4) return tile_ops_fwd_rot<C, R, 0, 4, kMat>(ops, sm, a);
@@ -92,17 +93,60 @@ __device__ __forceinline__ void stage_ops_fwd(uint32_t ops, uint32_t flags, cons
     if (m == 2) return tile_ops_fwd_rot<C, R, 0, 2, kMat>(ops, sm, a);
     if (m == 1) return tile_ops_fwd_rot<C, R, 0, 1, kMat>(ops, sm, a);
     if constexpr (kMat == kAny) {
-        const uint32_t mc = (flags >> 8) & 15u;
+        const uint32_t ms = (flags >> 16) & 15u;
         if constexpr (R >= 4) {
-            if (mc == 4) return tile_ops_fwd_cplx<C, R, 0, 4>(ops, sm, a);
+            if (ms == 4) return split_fwd<C, R, 4>(ops, sm, tab, a);
         }
         if constexpr (R >= 3) {
-            if (mc == 3) return tile_ops_fwd_cplx<C, R, 0, 3>(ops, sm, a);
+            if (ms == 3) return split_fwd<C, R, 3>(ops, sm, tab, a);
         }
-        if (mc == 2) return tile_ops_fwd_cplx<C, R, 0, 2>(ops, sm, a);
-        if (mc == 1) return tile_ops_fwd_cplx<C, R, 0, 1>(ops, sm, a);
+        if (ms == 2) return split_fwd<C, R, 2>(ops, sm, tab, a);
     }
     tile_ops_fwd<C, R, 0, kMat>(ops, sm, a);
+}
+
+// Stages slot's matrices of the pass in shared memory (the reverse's
+// transposed and conjugated): split forms and phase tables for split stages,
+// shear forms for real rotations elsewhere, and the stage flags.  Called by
+// every thread at a slot's first tile, once the previous tile's stages are
+// past their last barrier; visible after the next barrier.
+template <typename C, int R, int kMat, bool kRev>
+__device__ __forceinline__ void stage_mats(const TilePass &P, uint4 *rec, int n_slots,
+                                           const C *mats, int G, int slot, C *sm, C *tab) {
+    const int tid = threadIdx.x, T = blockDim.x;
+    __syncthreads();  // the stage records (first slot)
+    for (int x = tid; x < P.n_stages * R * 4; x += T) {
+        const int s = x / (R * 4), i = (x >> 2) % R, e = x & 3;
+        const int u = (int)((rec[2 * s].x >> (8 * i)) & 63u) - 1;
+        if (u < 0) continue;
+        const C *m = mats + ((size_t)slot * G + P.grp[u]) * 4;
+        C d;
+        if (kMat == kAny && (rec[2 * s + 1].w >> 16)) {
+            d = m[(size_t)n_slots * G * 4 + e];
+            if (kRev && e == 0) {  // the inverse rotation
+                d.x = -d.x;
+                d.y = -d.y;
+            }
+        } else if (kRev) {
+            d = m[e == 1 ? 2 : (e == 2 ? 1 : e)];
+            if (kMat != kPair) d.y = -d.y;
+        } else {
+            d = m[e];
+        }
+        sm[4 * u + e] = d;
+    }
+    __syncthreads();
+    if constexpr (kMat == kAny) build_phase_tables<C, R, kRev>(P.n_stages, rec, sm, tab);
+    for (int x = tid; x < P.n_stages * R; x += T) {
+        const int s = x / R;
+        const uint32_t ob = (rec[2 * s].x >> (8 * (x % R))) & 0xffu;
+        C *m = sm + 4 * ((int)(ob & 63u) - 1);
+        if (!ob || (kMat == kAny && (rec[2 * s + 1].w >> 16))) continue;
+        if constexpr (kMat == kPair) stage_shears_pair(m);
+        else if (ob & 64u) stage_shears(m);
+    }
+    __syncthreads();
+    set_stage_flags<C, kMat>(P, rec, sm);
 }
 
 template <typename Real, int R, int kMat>
@@ -119,7 +163,8 @@ __device__ __forceinline__ void tile_fwd_body(const TilePass &P, int n, int n_sl
     uint2 *tb = reinterpret_cast<uint2 *>(smem + kBufs * tbytes);
     uint4 *rec = reinterpret_cast<uint4 *>(smem + kBufs * tbytes + (uint32_t)S * T * 8u);
     C *sm = reinterpret_cast<C *>(rec + 2 * S);
-    build_stage_recs(P, rec);
+    C *tab = sm + 4 * P.n_ops;  // kAny: phase tables [stage][2][NA]
+    build_stage_recs<kMat == kAny>(P, rec);
     for (int s = 0; s < S; ++s) {
         const TileStage &sg = P.st[s];
         uint32_t lb = 0, sb = 0;
@@ -150,17 +195,7 @@ __device__ __forceinline__ void tile_fwd_body(const TilePass &P, int n, int n_sl
     for (int64_t tix = t0, i = 0; tix < t_end; ++tix, ++i) {
         const int buf = (int)(i & 1);
         if (cur.slot != mslot) {  // the previous tile's stages are past their last barrier
-            for (int x = tid; x < 4 * P.n_ops; x += T)
-                sm[x] = mats[((size_t)cur.slot * G + P.grp[x >> 2]) * 4 + (x & 3)];
-            __syncthreads();
-            for (int u = tid; u < P.n_ops; u += T) {
-                if constexpr (kMat == kPair) stage_shears_pair(sm + 4 * u);
-                else if ((P.real_mask >> u) & 1ull) stage_shears(sm + 4 * u);
-            }
-            if constexpr (std::is_same<C, float2>::value) {
-                __syncthreads();  // the branch-free paths' stage flags
-                set_stage_flags<C, kMat>(P, rec, sm);
-            }
+            stage_mats<C, R, kMat, false>(P, rec, n_slots, mats, G, cur.slot, sm, tab);
             mslot = cur.slot;
         }
         cp_async_wait_all();
@@ -174,12 +209,7 @@ __device__ __forceinline__ void tile_fwd_body(const TilePass &P, int n, int n_sl
             C a[NA];
 #pragma unroll
             for (int r = 0; r < NA; ++r) a[r] = *reinterpret_cast<const C *>(tile + (bb.x ^ xsel<R>(r, lq)));
-            // complex64: the branch-free paths where the stage allows
-            if constexpr (std::is_same<C, float2>::value) {
-                stage_ops_fwd<C, R, kMat>(ops, rec[2 * s + 1].w, sm, a);
-            } else {
-                tile_ops_fwd<C, R, 0, kMat>(ops, sm, a);
-            }
+            stage_ops_fwd<C, R, kMat>(ops, rec[2 * s + 1].w, sm, tab + s * 2 * NA, a);
             __syncthreads();
 #pragma unroll
             for (int r = 0; r < NA; ++r) *reinterpret_cast<C *>(tile + (bb.y ^ xsel<R>(r, sq))) = a[r];
@@ -420,38 +450,119 @@ __device__ __forceinline__ void stage_ops_rev(uint32_t ops, uint32_t modes, uint
     tile_ops_rev<C, Real, R, R - 1, NV, true, kMat>(ops, modes, sm, a, al, k);
 }
 
-// tile_ops_rev's four-sum complex path when register bits 0..M-1 all carry
-// parametrised complex matrices (stage flags, bits 12-15), without its
-// per-op branches.
-template <typename C, typename Real, int R, int I, int NV>
-__device__ __forceinline__ void tile_ops_rev_cplx(uint32_t ops, const C *sm, C (&a)[1 << R],
-                                                  C (&al)[1 << R], Real (&k)[NV]) {
-    if constexpr (I >= 0) {
-        kmat_bit<C, Real, R, I>(a, al, &k[4 * I]);
-        C m0, m1, m2, m3;
-        load_mat(sm, (int)((ops >> (8 * I)) & 63u) - 1, m0, m1, m2, m3);
-        u1_bit<C, R, I>(a, m0, m1, m2, m3);
-        u1_bit<C, R, I>(al, m0, m1, m2, m3);
-        tile_ops_rev_cplx<C, Real, R, I - 1, NV>(ops, sm, a, al, k);
+// Sums of a split stage's group on register bit I at the point after its
+// rotation, before its phases p (a phase per group only turns K_01, and the
+// other groups' phases drop out), of psi = a and m = i lambda:
+//   k[0] = k0 - k1 = sum p0 . m0 - p1 . m1,  k[1] = k2 = sum p0 . m1 + p1 . m0,
+//   k[2] = k3 = sum Re(p0 conj l1) - Re(p1 conj l0)
+// (x . y as real 2-vectors; with i lambda in place of lambda the first two
+// are packed products).  k0 + k1 is of no account to a rotation's derivative.
+template <typename C, typename Real, int R, int I>
+__device__ __forceinline__ void split_sums(const C (&a)[1 << R], const C (&m)[1 << R], Real *k) {
+    if constexpr (std::is_same<C, float2>::value) {
+        uint64_t d0 = 0, d1 = 0, e0 = 0, e1 = 0;
+        float t0 = 0.f, t1 = 0.f;
+#pragma unroll
+        for (int r = 0; r < (1 << R); ++r) {
+            if (r & (1 << I)) continue;
+            const C p0 = a[r], p1 = a[r | (1 << I)], m0 = m[r], m1 = m[r | (1 << I)];
+            d0 = f2fma(f2of(p0), f2of(m0), d0);
+            d1 = f2fma(f2of(p1), f2of(m1), d1);
+            e0 = f2fma(f2of(p0), f2of(m1), e0);
+            e1 = f2fma(f2of(p1), f2of(m0), e1);
+            t0 = fmaR(p0.x, m1.y, fmaR(-p0.y, m1.x, t0));
+            t1 = fmaR(p1.y, m0.x, fmaR(-p1.x, m0.y, t1));
+        }
+        const float2 D0 = f2unpack(d0), D1 = f2unpack(d1), E0 = f2unpack(e0), E1 = f2unpack(e1);
+        k[0] = (D0.x + D0.y) - (D1.x + D1.y);
+        k[1] = (E0.x + E0.y) + (E1.x + E1.y);
+        k[2] = t0 + t1;
+    } else {
+        Real d = 0, e = 0, t = 0;
+#pragma unroll
+        for (int r = 0; r < (1 << R); ++r) {
+            if (r & (1 << I)) continue;
+            const C p0 = a[r], p1 = a[r | (1 << I)], m0 = m[r], m1 = m[r | (1 << I)];
+            d = fmaR(p0.x, m0.x, fmaR(p0.y, m0.y, fmaR(-p1.x, m1.x, fmaR(-p1.y, m1.y, d))));
+            e = fmaR(p0.x, m1.x, fmaR(p0.y, m1.y, fmaR(p1.x, m0.x, fmaR(p1.y, m0.y, e))));
+            t = fmaR(p0.x, m1.y, fmaR(-p0.y, m1.x, fmaR(p1.y, m0.x, fmaR(-p1.x, m0.y, t))));
+        }
+        k[0] = d;
+        k[1] = e;
+        k[2] = t;
     }
 }
 
-// One reverse stage of four-sum ops: the branch-free complex path when
-// register bits 0..M-1 carry parametrised complex matrices, tile_ops_rev
-// otherwise.
-template <typename C, typename Real, int R, int NV>
-__device__ __forceinline__ void stage_ops_rev4(uint32_t ops, uint32_t modes, uint32_t m,
-                                               const C *sm, C (&a)[1 << R], C (&al)[1 << R],
-                                               Real (&k)[NV]) {
-    if constexpr (R >= 4) {
-        if (m == 4) return tile_ops_rev_cplx<C, Real, R, 3, NV>(ops, sm, a, al, k);
+template <typename C, typename Real, int R, int I>
+__device__ __forceinline__ void split_unrots(uint32_t ops, const C *sm, C (&a)[1 << R],
+                                             C (&m)[1 << R], Real *k) {
+    if constexpr (I >= 0) {
+        split_sums<C, Real, R, I>(a, m, k + 3 * I);
+        C alpha, beta;
+        split_shears(sm, ops, I, alpha, beta);
+        rot3_bit<C, R, I>(a, alpha, beta);
+        rot3_bit<C, R, I>(m, alpha, beta);
+        split_unrots<C, Real, R, I - 1>(ops, sm, a, m, k);
     }
-    if constexpr (R >= 3) {
-        if (m == 3) return tile_ops_rev_cplx<C, Real, R, 2, NV>(ops, sm, a, al, k);
+}
+
+// A reverse stage in split form with groups on register bits 0..M-1 (tab:
+// conjugated): the phases p off, per group its sums and its rotation off,
+// the phases q off.  In between al holds i lambda (only names and signs).
+// k: three sums per register bit.
+template <typename C, typename Real, int R, int M>
+__device__ __forceinline__ void split_rev(uint32_t ops, const C *sm, const C *tab,
+                                          C (&a)[1 << R], C (&al)[1 << R], Real *k) {
+    constexpr int NA = 1 << R, NM = 1 << M;
+#pragma unroll
+    for (int q = 0; q < NM / 2; ++q) {
+        C p[2];
+        load_phases(tab + NA, q, p[0], p[1]);
+#pragma unroll
+        for (int r = 0; r < NA; r += NM)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int j = r + 2 * q + h;
+                a[j] = phase_mul(a[j], p[h]);
+                const C l = phase_mul(al[j], p[h]);
+                al[j].x = -l.y;
+                al[j].y = l.x;
+            }
     }
-    if (m == 2) return tile_ops_rev_cplx<C, Real, R, 1, NV>(ops, sm, a, al, k);
-    if (m == 1) return tile_ops_rev_cplx<C, Real, R, 0, NV>(ops, sm, a, al, k);
-    tile_ops_rev<C, Real, R, R - 1, NV, false, kAny>(ops, modes, sm, a, al, k);
+    split_unrots<C, Real, R, M - 1>(ops, sm, a, al, k);
+#pragma unroll
+    for (int q = 0; q < NM / 2; ++q) {
+        C p[2];
+        load_phases(tab, q, p[0], p[1]);
+#pragma unroll
+        for (int r = 0; r < NA; r += NM)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int j = r + 2 * q + h;
+                C l;
+                l.x = al[j].y;
+                l.y = -al[j].x;
+                const bool one = q == 0 && h == 0;  // that entry is 1
+                if (!one) a[j] = phase_mul(a[j], p[h]);
+                al[j] = one ? l : phase_mul(l, p[h]);
+            }
+    }
+}
+
+// x[m] (m < 3) = value 4 m + (lane & 3) of the twelve, summed over the four
+// lanes that differ in lane bits 0-1 (warp_reduce_quad of twelve values).
+template <typename Real>
+__device__ __forceinline__ void warp_reduce_quad12(Real (&x)[12], int lane) {
+    constexpr unsigned full = 0xffffffffu;
+#pragma unroll
+    for (int j = 0, M = 12; j < 2; ++j, M >>= 1) {
+        const bool b = (lane >> j) & 1;
+#pragma unroll
+        for (int m = 0; m < M / 2; ++m) {
+            const Real keep = b ? x[2 * m + 1] : x[2 * m], give = b ? x[2 * m] : x[2 * m + 1];
+            x[m] = keep + __shfl_xor_sync(full, give, 1 << j);
+        }
+    }
 }
 
 // Adds the block's sums of slot b (FP64 over warps and lane quads), as i K
@@ -459,9 +570,45 @@ __device__ __forceinline__ void stage_ops_rev4(uint32_t ops, uint32_t modes, uin
 // every thread.
 // kPair: b is a slot pair; lanes of lane bit 0 = c hold the sums of slot 2b + c
 // (rho_g has a row for each, also past an odd last slot).
-template <typename Real, bool kSingle, int kMat>
-__device__ void flush_acc(const TilePass &P, Real *acc, int wps, double *rho_g, int b, int G) {
+// A split stage (rec, sm: its staged records and forms): value 3 i + c of the
+// stage, i its register bit, lies in the lanes = 3 i + c mod 4; its phases
+// turn the sum k3 + i k2 by p0 conj(p1).
+template <typename Real, bool kSingle, int kMat, int R>
+__device__ void flush_acc(const TilePass &P, Real *acc, int wps, double *rho_g, int b, int G,
+                          const uint4 *rec, const typename CT<Real>::T *sm) {
     __syncthreads();
+    if constexpr (kMat == kAny && !kSingle) {
+        for (int x = threadIdx.x; x < P.n_stages * R; x += blockDim.x) {
+            const int s = x / R, i = x % R;
+            const uint32_t ob = (rec[2 * s].x >> (8 * i)) & 0xffu;
+            if (!(rec[2 * s + 1].w >> 16) || !(ob & 128u)) continue;
+            const int u = (int)(ob & 63u) - 1;
+            double k[3];
+            for (int c = 0; c < 3; ++c) {
+                k[c] = 0.0;
+                for (int w = 0; w < wps; ++w)
+                    for (int q = (3 * i + c) & 3; q < 32; q += 4) {
+                        Real &r = acc[(u * wps + w) * 32 + q];
+                        k[c] += (double)r;
+                        r = 0;
+                    }
+            }
+            if (k[0] == 0.0 && k[1] == 0.0 && k[2] == 0.0) continue;
+            const auto p0 = sm[4 * u + 1], p1 = sm[4 * u + 2];
+            const double fx = (double)p0.x * p1.x + (double)p0.y * p1.y;
+            const double fy = (double)p0.y * p1.x - (double)p0.x * p1.y;
+            const double re = 0.5 * (fx * k[2] - fy * k[1]), im = 0.5 * (fx * k[1] + fy * k[2]);
+            // i K = [[i (k0 - k1) / 2, z], [-conj(z), -i (k0 - k1) / 2]]
+            double *dst = rho_g + ((size_t)b * G + P.grp[u]) * 8;
+            atomicAdd(dst + 1, 0.5 * k[0]);
+            atomicAdd(dst + 7, -0.5 * k[0]);
+            atomicAdd(dst + 2, re);
+            atomicAdd(dst + 3, im);
+            atomicAdd(dst + 4, -re);
+            atomicAdd(dst + 5, im);
+        }
+        __syncthreads();
+    }
     if constexpr (kMat == kPair) {
         for (int x = threadIdx.x; x < P.n_ops * 2; x += blockDim.x) {
             const int u = x >> 1, c = x & 1;
@@ -535,8 +682,10 @@ __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_sl
     uint2 *tb = reinterpret_cast<uint2 *>(smem + 2 * NB * tbytes);
     uint4 *rec = reinterpret_cast<uint4 *>(smem + 2 * NB * tbytes + (uint32_t)S * T * 8u);
     C *sm = reinterpret_cast<C *>(rec + 2 * S);
-    Real *acc = reinterpret_cast<Real *>(sm + 4 * P.n_ops);
-    build_stage_recs(P, rec);
+    constexpr bool kSplit = kMat == kAny && !kSingle;
+    C *tab = sm + 4 * P.n_ops;  // kSplit: phase tables [stage][2][NA]
+    Real *acc = reinterpret_cast<Real *>(tab + (kSplit ? S * 2 * NA : 0));
+    build_stage_recs<kSplit>(P, rec);
     for (int s = 0; s < S; ++s) {
         const TileStage &sg = P.st[s];
         uint32_t lb = 0, sb = 0;
@@ -575,26 +724,12 @@ __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_sl
     for (int64_t tix = t0, i = 0; tix < t_end; ++tix, ++i) {
         const int buf = NB == 2 ? (int)(i & 1) : 0;
         if (cur.slot != mslot || since == kFlushTiles) {
-            if (mslot >= 0) flush_acc<Real, kSingle, kMat>(P, acc, wps, rho_g, mslot, G);
+            if (mslot >= 0) flush_acc<Real, kSingle, kMat, R>(P, acc, wps, rho_g, mslot, G, rec, sm);
             since = 0;
         }
         if (cur.slot != mslot) {  // adjoint matrices of this slot's groups
-            for (int x = tid; x < 4 * P.n_ops; x += T) {
-                const C *m = mats + ((size_t)cur.slot * G + P.grp[x >> 2]) * 4;
-                const int e = x & 3, te = e == 1 ? 2 : (e == 2 ? 1 : e);
-                C d = m[te];
-                if constexpr (kMat != kPair) d.y = -d.y;
-                sm[x] = d;
-            }
-            __syncthreads();
-            for (int u = tid; u < P.n_ops; u += T) {
-                if constexpr (kMat == kPair) stage_shears_pair(sm + 4 * u);
-                else if ((P.real_mask >> u) & 1ull) stage_shears(sm + 4 * u);
-            }
-            if constexpr (std::is_same<C, float2>::value && kSingle == (kMat != kAny)) {
-                __syncthreads();  // the branch-free paths' stage flags
-                set_stage_flags<C, kMat>(P, rec, sm);
-            }
+            stage_mats<C, R, kSplit || kMat != kAny ? kMat : kNoSplit, true>(P, rec, n_slots, mats, G,
+                                                                            cur.slot, sm, tab);
             mslot = cur.slot;
         }
         cp_async_wait_all();
@@ -619,32 +754,59 @@ __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_sl
             Real kk[NV];
 #pragma unroll
             for (int v = 0; v < NV; ++v) kk[v] = 0;
+            bool split = false;
             if constexpr (kSingle && kMat != kAny && std::is_same<C, float2>::value) {
                 stage_ops_rev<C, Real, R, NV, kMat>(ops, modes, (rec[2 * s + 1].w >> 4) & 15u, sm, a,
                                                      al, kk);
-            } else if constexpr (!kSingle && kMat == kAny && std::is_same<C, float2>::value) {
-                stage_ops_rev4<C, Real, R, NV>(ops, modes, (rec[2 * s + 1].w >> 12) & 15u, sm,
-                                                      a, al, kk);
             } else {
-                tile_ops_rev<C, Real, R, R - 1, NV, kSingle, kMat>(ops, modes, sm, a, al, kk);
-            }
-            warp_reduce_quad<Real, NV>(kk, lane);
-            if constexpr (kMat == kPair) {  // lane: bit 2 m + (lane >> 1 & 1), state lane & 1
+                if constexpr (kSplit) {
+                    const uint32_t ms = (rec[2 * s + 1].w >> 16) & 15u;
+                    if (ms) {
+                        Real k3[12];
 #pragma unroll
-                for (int m = 0; m < NV / 4; ++m) {
-                    const int i = 2 * m + ((lane >> 1) & 1);
-                    const uint32_t ob = i < R ? (ops >> (8 * i)) & 0xffu : 0u;
-                    if (ob & 128u) accw[((int)(ob & 63u) - 1) * wps * 32] += kk[m];
+                        for (int v = 0; v < 12; ++v) k3[v] = 0;
+                        const C *ts = tab + s * 2 * NA;
+                        if constexpr (R >= 4) {
+                            if (ms == 4) split_rev<C, Real, R, 4>(ops, sm, ts, a, al, k3);
+                        }
+                        if constexpr (R >= 3) {
+                            if (ms == 3) split_rev<C, Real, R, 3>(ops, sm, ts, a, al, k3);
+                        }
+                        if (ms == 2) split_rev<C, Real, R, 2>(ops, sm, ts, a, al, k3);
+                        warp_reduce_quad12<Real>(k3, lane);
+#pragma unroll
+                        for (int m = 0; m < 3; ++m) {
+                            const int i = (4 * m + (lane & 3)) / 3;
+                            const uint32_t ob = (ops >> (8 * i)) & 0xffu;
+                            if (ob & 128u) accw[((int)(ob & 63u) - 1) * wps * 32] += k3[m];
+                        }
+                    } else {
+                        tile_ops_rev<C, Real, R, R - 1, NV, kSingle, kMat>(ops, modes, sm, a, al, kk);
+                    }
+                    split = ms != 0;
+                } else {
+                    tile_ops_rev<C, Real, R, R - 1, NV, kSingle, kMat>(ops, modes, sm, a, al, kk);
                 }
-            } else if constexpr (kSingle) {  // lane: the sum of register bit lane & 3
-                const int m = lane & 3;
-                const uint32_t ob = m < R ? (ops >> (8 * m)) & 0xffu : 0u;
-                if (ob & 128u) accw[((int)(ob & 63u) - 1) * wps * 32] += kk[0];
-            } else {
+            }
+            if (!split) {
+                warp_reduce_quad<Real, NV>(kk, lane);
+                if constexpr (kMat == kPair) {  // lane: bit 2 m + (lane >> 1 & 1), state lane & 1
 #pragma unroll
-                for (int m = 0; m < R; ++m) {
-                    const uint32_t ob = (ops >> (8 * m)) & 0xffu;
-                    if (ob & 128u) accw[((int)(ob & 63u) - 1) * wps * 32] += kk[m];
+                    for (int m = 0; m < NV / 4; ++m) {
+                        const int i = 2 * m + ((lane >> 1) & 1);
+                        const uint32_t ob = i < R ? (ops >> (8 * i)) & 0xffu : 0u;
+                        if (ob & 128u) accw[((int)(ob & 63u) - 1) * wps * 32] += kk[m];
+                    }
+                } else if constexpr (kSingle) {  // lane: the sum of register bit lane & 3
+                    const int m = lane & 3;
+                    const uint32_t ob = m < R ? (ops >> (8 * m)) & 0xffu : 0u;
+                    if (ob & 128u) accw[((int)(ob & 63u) - 1) * wps * 32] += kk[0];
+                } else {
+#pragma unroll
+                    for (int m = 0; m < R; ++m) {
+                        const uint32_t ob = (ops >> (8 * m)) & 0xffu;
+                        if (ob & 128u) accw[((int)(ob & 63u) - 1) * wps * 32] += kk[m];
+                    }
                 }
             }
             __syncthreads();
@@ -680,7 +842,7 @@ __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_sl
         cur = nxt;
         nxt = tile_next(P, nxt);
     }
-    flush_acc<Real, kSingle, kMat>(P, acc, wps, rho_g, mslot, G);
+    flush_acc<Real, kSingle, kMat, R>(P, acc, wps, rho_g, mslot, G, rec, sm);
 }
 
 // NB = 1: launched with 64 threads only (at least five blocks per SM).
@@ -1312,18 +1474,25 @@ cudaError_t launch_init_states(int c128, void *states, int n, const SlotSource &
     return cudaGetLastError();
 }
 
-uint32_t tile_fwd_smem(int c128, const TilePass &P) {
+// Phase tables of the split stages (kernels of kind kAny).
+static uint32_t phase_table_bytes(int c128, const TilePass &P, bool any) {
+    return any ? (uint32_t)P.n_stages * ((c128 ? 32u : 16u) << P.R) : 0u;
+}
+
+uint32_t tile_fwd_smem(int c128, const TilePass &P, bool any) {
     const uint32_t csz = c128 ? 16u : 8u, T = 1u << (P.t - P.R);
-    return 2u * (csz << P.t) + (uint32_t)P.n_stages * (T * 8u + 32u) + (uint32_t)P.n_ops * 4u * csz;
+    const uint32_t tab = phase_table_bytes(c128, P, any || !pass_all_real(P));
+    return 2u * (csz << P.t) + (uint32_t)P.n_stages * (T * 8u + 32u) + (uint32_t)P.n_ops * 4u * csz + tab;
 }
 
 // Reverse passes with at least this many register stages run single-buffered.
 constexpr int kOneBufStages = 6;
 
-uint32_t tile_rev_smem(int c128, const TilePass &P, int bufs) {
+uint32_t tile_rev_smem(int c128, const TilePass &P, int bufs, bool any) {
     const uint32_t csz = c128 ? 16u : 8u, rsz = c128 ? 8u : 4u, T = 1u << (P.t - P.R);
+    const uint32_t tab = phase_table_bytes(c128, P, any || !pass_all_real(P));
     return 2u * (uint32_t)bufs * (csz << P.t) + (uint32_t)P.n_stages * (T * 8u + 32u) + (uint32_t)P.n_ops * 4u * csz +
-           (uint32_t)P.n_ops * T * rsz;
+           tab + (uint32_t)P.n_ops * T * rsz;
 }
 
 cudaError_t launch_tile_fwd(int c128, const TilePass &P, int n, int n_slots, const void *mats,
@@ -1426,7 +1595,7 @@ void set_capturing(bool on) { t_capturing = on; }
 
 uint32_t tile_sweep_smem(int c128, bool rev, const TilePass &P) {
     return (uint32_t)((sizeof(TilePass) + 255) & ~size_t(255)) +
-           (rev ? tile_rev_smem(c128, P) : tile_fwd_smem(c128, P));
+           (rev ? tile_rev_smem(c128, P, 2, true) : tile_fwd_smem(c128, P, true));
 }
 
 int tile_sweep_blocks_per_sm(int c128, int R, bool rev, uint32_t smem, int threads) {

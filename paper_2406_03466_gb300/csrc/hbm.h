@@ -11,15 +11,19 @@ namespace svk {
 // pair (here and below): two real circuits per state (slots 2j and 2j + 1 in
 // the components of state j); the launchers' slot counts are then pairs,
 // except in a SlotSource and in pair_rows.
-// mats: [slots][groups][4] complex of the state's precision.
+// mats: [slots][groups][4] complex of the state's precision, followed (not
+// with pair) by the groups' split form [slots][groups][4].  kMatVals complex
+// values per slot and group hold both.
+constexpr int kMatVals = 8;
 cudaError_t launch_group_mats(int c128, const Program &p, const SlotSource &src, void *mats,
                               cudaStream_t st, bool pair = false);
 // Zeroes the slot states and sets amplitude |ref> of each to 1.
 cudaError_t launch_init_states(int c128, void *states, int n, const SlotSource &src,
                                cudaStream_t st, bool pair = false);
 // Shared memory of one block of the forward / reverse kernels of pass P.
-uint32_t tile_fwd_smem(int c128, const TilePass &P);
-uint32_t tile_rev_smem(int c128, const TilePass &P, int bufs = 2);
+// (any: of a kernel that takes complex and real passes alike).
+uint32_t tile_fwd_smem(int c128, const TilePass &P, bool any = false);
+uint32_t tile_rev_smem(int c128, const TilePass &P, int bufs = 2, bool any = false);
 // Forward pass P over n_slots states of n qubits (mats: [slots][G][4]).
 // src (null: states) holds the pass's input; the output goes to states.
 cudaError_t launch_tile_fwd(int c128, const TilePass &P, int n, int n_slots, const void *mats,

@@ -203,7 +203,7 @@ k_tile_fwd_tc(const __grid_constant__ TilePass P, int n, int n_slots, const floa
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + 1);
     const uint32_t bar_a = smem_addr(bar);
 
-    build_stage_recs(P, rec);
+    build_stage_recs<false>(P, rec);
     for (int s = 0; s < S; ++s) {
         const TileStage &sg = P.st[s];
         uint32_t lb = 0, sbv = 0;

@@ -91,7 +91,9 @@ __device__ __forceinline__ TileCursor tile_next(const TilePass &P, TileCursor c)
 // addresses): word 0 holds one op byte per register bit, (u + 1) | real << 6
 // | parametrised << 7 for pass-local op u (0: no op); word 1 + i holds
 // ldq[i] | stq[i] << 16 (byte offsets, < 2^16 for every supported tile);
-// word 5 holds the ops' fmode bytes.
+// word 5 holds the ops' fmode bytes; word 7 bits 16-19: M when the stage runs
+// in split form (below), with ops on register bits 0..M-1.
+template <bool kSplit>
 __device__ __forceinline__ void build_stage_recs(const TilePass &P, uint4 *rec) {
     for (int s = threadIdx.x; s < P.n_stages; s += blockDim.x) {
         const TileStage &sg = P.st[s];
@@ -106,6 +108,12 @@ __device__ __forceinline__ void build_stage_recs(const TilePass &P, uint4 *rec) 
             w[1 + i] = sg.ldq[i] | (sg.stq[i] << 16);
             if (u >= 0) w[5] |= (uint32_t)(P.fmode[u] & 3) << (8 * i);
         }
+        int m = 0;
+        bool all_real = true;
+        for (; m < P.R && m < 4 && sg.op[m] >= 0; ++m)
+            all_real = all_real && ((P.real_mask >> sg.op[m]) & 1ull);
+        if (kSplit && m >= 2 && !all_real && (m == 4 || (w[0] >> (8 * m)) == 0u))
+            w[7] = (uint32_t)m << 16;
         rec[2 * s] = make_uint4(w[0], w[1], w[2], w[3]);
         rec[2 * s + 1] = make_uint4(w[4], w[5], w[6], w[7]);
     }
@@ -210,8 +218,8 @@ __device__ __forceinline__ void u1p_bit(C (&a)[1 << R], const C m0, const C m1, 
 // What a pass's staged matrices are.  kAny: complex or real per group.
 // kReal: every group real.  kPair: the amplitude's components are the real
 // amplitudes of two circuits and entry k of a matrix is (first circuit's,
-// second circuit's).
-enum MatKind { kAny = 0, kReal = 1, kPair = 2 };
+// second circuit's).  kNoSplit: kAny whose stages all keep matrices.
+enum MatKind { kAny = 0, kReal = 1, kPair = 2, kNoSplit = 3 };
 
 // The imaginary parts of a staged real matrix are unused: for a real
 // rotation with c > 0 they carry the shear form (m0.y = alpha, m1.y = beta,
@@ -309,17 +317,115 @@ __device__ __forceinline__ void tile_ops_fwd_rot(uint32_t ops, const C *sm, C (&
     }
 }
 
-// The forward stage ops when register bits 0..M-1 carry complex matrices
-// and the others carry no op (stage flags, bits 8-11): tile_ops_fwd's
-// complex arithmetic without its per-op branches.
-template <typename C, int R, int I, int M>
-__device__ __forceinline__ void tile_ops_fwd_cplx(uint32_t ops, const C *sm, C (&a)[1 << R]) {
-    if constexpr (I < M) {
-        C m0, m1, m2, m3;
-        load_mat(sm, (int)((ops >> (8 * I)) & 63u) - 1, m0, m1, m2, m3);
-        u1_bit<C, R, I>(a, m0, m1, m2, m3);
-        tile_ops_fwd_cplx<C, R, I + 1, M>(ops, sm, a);
+// ------------------------------------------------------------ split form
+//
+// Every 2x2 unitary is diag(p0, p1) R diag(1, q) with a real rotation R of
+// c, s >= 0 and unit phases p0, p1, q.  A stage with complex groups on M >= 2
+// register bits multiplies its amplitudes once by the product of the groups'
+// q (a table over the M register bits), applies the M rotations as shears,
+// and multiplies once by the product of the p: per amplitude 4 + 1.5 M + 4
+// instructions instead of 8 M for M complex 2x2 products.  With M = 1 the
+// products cost less.
+
+// The split form of a group's matrix u (FP64): out = (alpha, beta), p0, p1, q
+// with the rotation's shears alpha = -s / (1 + c), beta = s.  The larger of
+// c and s fixes q, so nothing is divided by a small number.
+template <typename C> __device__ __forceinline__ void split_form(const double2 (&u)[4], C *out) {
+    const double c = sqrt(u[0].x * u[0].x + u[0].y * u[0].y);
+    const double s = sqrt(u[2].x * u[2].x + u[2].y * u[2].y);
+    double2 p0 = make_double2(1.0, 0.0), p1 = p0, q;
+    if (c > 1e-30) p0 = make_double2(u[0].x / c, u[0].y / c);
+    if (s > 1e-30) p1 = make_double2(u[2].x / s, u[2].y / s);
+    if (c >= s) q = cmul(u[3], cconj(p1));                          // u11 = p1 c q
+    else q = cmul(make_double2(-u[1].x, -u[1].y), cconj(p0));       // u01 = -p0 s q
+    const double l = sqrt(q.x * q.x + q.y * q.y);
+    out[0] = cmk<C>(-s / (1.0 + c), s);
+    out[1] = cmk<C>(p0.x, p0.y);
+    out[2] = cmk<C>(p1.x, p1.y);
+    out[3] = cmk<C>(q.x / l, q.y / l);
+}
+
+// Phase tables of the split stages, tab[s][0][r] = product of the q and
+// tab[s][1][r] = product of the p over the stage's register bits, from the
+// staged split forms (conjugated for the reverse sweep).
+template <typename C, int R, bool kConj>
+__device__ __forceinline__ void build_phase_tables(int n_stages, const uint4 *rec, const C *sm,
+                                                   C *tab) {
+    constexpr int NA = 1 << R;
+    for (int x = threadIdx.x; x < n_stages * 2 * NA; x += blockDim.x) {
+        const int s = x / (2 * NA), post = (x / NA) & 1, r = x & (NA - 1);
+        const int m = (int)((rec[2 * s + 1].w >> 16) & 15u);
+        const uint32_t ops = rec[2 * s].x;
+        C f = cmk<C>(1, 0);
+        for (int i = 0; i < m; ++i) {
+            const C *e = sm + 4 * ((int)((ops >> (8 * i)) & 63u) - 1);
+            const int b = (r >> i) & 1;
+            if (post) f = cmul(f, e[1 + b]);
+            else if (b) f = cmul(f, e[3]);
+        }
+        if (m) tab[x] = kConj ? cconj(f) : f;
     }
+}
+
+// a * p in two products and two fused multiply-adds.
+template <typename C> __device__ __forceinline__ C phase_mul(const C a, const C p) {
+    C r;
+    r.x = fmaR(a.x, p.x, -(a.y * p.y));
+    r.y = fmaR(a.x, p.y, a.y * p.x);
+    return r;
+}
+
+// Table entries 2q and 2q + 1 (a table starts on 16 bytes).
+__device__ __forceinline__ void load_phases(const float2 *tab, int q, float2 &p, float2 &n) {
+    const float4 v = reinterpret_cast<const float4 *>(tab)[q];
+    p = make_float2(v.x, v.y);
+    n = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void load_phases(const double2 *tab, int q, double2 &p, double2 &n) {
+    p = tab[2 * q];
+    n = tab[2 * q + 1];
+}
+
+// a[r] *= tab[r mod 2^M]; kFirst: entry 0 is 1.
+template <typename C, int R, int M, bool kFirst>
+__device__ __forceinline__ void apply_phases(const C *tab, C (&a)[1 << R]) {
+#pragma unroll
+    for (int q = 0; q < (1 << M) / 2; ++q) {
+        C p, n;
+        load_phases(tab, q, p, n);
+#pragma unroll
+        for (int r = 0; r < (1 << R); r += 1 << M) {
+            if (!kFirst || q) a[r + 2 * q] = phase_mul(a[r + 2 * q], p);
+            a[r + 2 * q + 1] = phase_mul(a[r + 2 * q + 1], n);
+        }
+    }
+}
+
+// (alpha, beta) of a staged split form.
+template <typename C>
+__device__ __forceinline__ void split_shears(const C *sm, uint32_t ops, int i, C &alpha, C &beta) {
+    const C v = sm[4 * ((int)((ops >> (8 * i)) & 63u) - 1)];
+    alpha = both<C>(v.x);
+    beta = both<C>(v.y);
+}
+
+template <typename C, int R, int I, int M>
+__device__ __forceinline__ void split_rots(uint32_t ops, const C *sm, C (&a)[1 << R]) {
+    if constexpr (I < M) {
+        C alpha, beta;
+        split_shears(sm, ops, I, alpha, beta);
+        rot3_bit<C, R, I>(a, alpha, beta);
+        split_rots<C, R, I + 1, M>(ops, sm, a);
+    }
+}
+
+// A forward stage in split form with groups on register bits 0..M-1.
+template <typename C, int R, int M>
+__device__ __forceinline__ void split_fwd(uint32_t ops, const C *sm, const C *tab,
+                                          C (&a)[1 << R]) {
+    apply_phases<C, R, M, true>(tab, a);
+    split_rots<C, R, 0, M>(ops, sm, a);
+    apply_phases<C, R, M, false>(tab + (1 << R), a);
 }
 
 // Stage flags, the w word of a stage's second record, set for the staged
@@ -327,38 +433,29 @@ __device__ __forceinline__ void tile_ops_fwd_cplx(uint32_t ops, const C *sm, C (
 // 0..M-1 carry ops with real matrices in shear form (rotations with c > 0)
 // and the other bits none (the forward's branch-free path); bits 4-7: the
 // same M when those ops are moreover parametrised with the single Ry sum
-// (fmode 1; the reverse's); bits 8-11: M when register bits 0..M-1 carry
-// ops with complex matrices and the other bits none; bits 12-15: that M
-// when those complex ops are moreover all parametrised (the reverse's
-// four-sum path); 0 otherwise.  Called by every thread once the slot's
-// shear forms are in shared memory; visible after the next barrier.
+// (fmode 1; the reverse's); 0 otherwise.  Called by every thread once the
+// slot's shear forms are in shared memory; visible after the next barrier.
 // kPair: every op is real and its parameters all rotate about Y.
 template <typename C, int kMat>
 __device__ __forceinline__ void set_stage_flags(const TilePass &P, uint4 *rec, const C *sm) {
     for (int s = threadIdx.x; s < P.n_stages; s += blockDim.x) {
         const uint32_t ops = rec[2 * s].x, modes = rec[2 * s + 1].y;
-        int m = 0, mc = 0;
-        bool single = true, rot = true, cplx = true, cpar = true;
+        int m = 0;
+        bool single = true, rot = !(rec[2 * s + 1].w >> 16);  // no shears in split form
         for (int i = 0; i < P.R; ++i) {
             const uint32_t ob = (ops >> (8 * i)) & 0xffu;
             if (!ob) break;
             const C *mt = sm + 4 * ((int)(ob & 63u) - 1);
             rot = rot && (ob & 64u) && (kMat == kPair ? is_shear_pair(mt[2], mt[3]) : mt[2].y != 0);
-            cplx = cplx && !(ob & 64u);
             if (rot) {
                 single = single && (ob & 128u) && (kMat == kPair || ((modes >> (8 * i)) & 3u) == 1u);
                 m = i + 1;
             }
-            if (cplx) {
-                cpar = cpar && (ob & 128u);
-                mc = i + 1;
-            }
         }
         // the bits above M must carry no op
         if (m > 0 && m < 4 && (ops >> (8 * m)) != 0u) m = 0;
-        if (mc > 0 && mc < 4 && (ops >> (8 * mc)) != 0u) mc = 0;
-        rec[2 * s + 1].w = (uint32_t)m | (single ? (uint32_t)m << 4 : 0u) | ((uint32_t)mc << 8) |
-                           (cpar ? (uint32_t)mc << 12 : 0u);
+        rec[2 * s + 1].w =
+            (rec[2 * s + 1].w & 0xf0000u) | (uint32_t)m | (single ? (uint32_t)m << 4 : 0u);
     }
 }
 

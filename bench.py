@@ -255,8 +255,9 @@ def measured_hbm_gbs():
 
 def forward_passes_roofline(sv, w, dev, flush, stream, reps=5, opts=None):
     """Times the forward simulation of workload `w` (all instances, states in
-    device memory) and reports it against the HBM roofline: each tile pass
-    reads and writes every state once, the |ref> initialisation writes them."""
+    device memory) and reports it against the HBM roofline: the bytes its
+    tile passes read and write (every state once each way, but for the first
+    passes' known zeros)."""
     import torch
     d = 0 if w.inputs is None else 1
     circ = sv.Circuit(w.n_qubits, w.gates, w.n_params, d)
@@ -274,7 +275,7 @@ def forward_passes_roofline(sv, w, dev, flush, stream, reps=5, opts=None):
     fn = lambda: sv.sv_apply_circuit_batch(st, [circ], slots, theta, xin, opts)  # noqa: E731
     fn()
     t = timed_loop(fn, reps, flush, stream) / reps
-    nbytes = (2 * info["n_passes"] + 1) * I * (8 << n)
+    nbytes = sv.sv_last_moved()["forward_bytes"]
     peak, src = measured_hbm_gbs()
     achieved = nbytes / t / 1e9
     st.free()
@@ -308,17 +309,17 @@ def adjoint_phases(sv, w, prob, theta, out, info, flush, stream, reps, step=None
     sv.sv_phase_timing(False)
     torch.cuda.synchronize()
     n, I = w.n_qubits, w.n_instances
-    # states the passes moved: two instances of a real problem share one
-    states = sv.sv_last_adjoint_states()
-    state = states * (8 << n)
+    # what the passes moved: two instances of a real problem share a state, and
+    # the first passes leave out amplitudes that are still zero
+    moved = sv.sv_last_moved()
+    states = moved["states"]
     last = sv.sv_last_adjoint_info()
-    nbytes = last["reverse_bytes"] // I * states
+    nbytes = moved["reverse_bytes"]
     peak, src = measured_hbm_gbs()
     achieved = nbytes / (ph["reverse_ms"] * 1e-3) / 1e9
-    # the gradient's own forward passes (the same relabeling plan), 16 B per
-    # amplitude per pass; the phase also holds |ref>, the group matrices and
-    # the stored checkpoint copies
-    fwd_bytes = 2 * info["n_passes"] * state
+    # the gradient's own forward passes (the same relabeling plan); the phase
+    # also holds the group matrices
+    fwd_bytes = moved["forward_bytes"]
     traffic = reverse_traffic(w, info["tile_bits"], reg_bits, last["checkpoint_every"])
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "traffic": traffic,

@@ -429,13 +429,17 @@ sv_status sv_last_phase_ms(float *forward_ms, float *h_ms, float *reverse_ms);
  * out-pointer may be NULL. */
 sv_status sv_last_adjoint_info(int32_t *checkpoint_every, int64_t *reverse_bytes);
 
-/* How many states in device memory that adjoint swept: one per instance, or
- * half as many (rounded up) when the instances' amplitudes are all real (Ry,
- * X, H, CNOT and CZ gates, Ry encodings, an observable without odd Y counts)
- * and two instances share one complex state.  The passes then move that share
- * of reverse_bytes, which counts a state per instance.  0 after an adjoint
- * that ran on chip. */
-sv_status sv_last_adjoint_states(int32_t *states);
+/* What the tile passes of that adjoint moved: `states`, the states in device
+ * memory it swept -- one per instance, or half as many (rounded up) when the
+ * instances' amplitudes are all real (Ry, X, H, CNOT and CZ gates, Ry
+ * encodings, an observable without odd Y counts) and two instances share one
+ * complex state; 0 after an adjoint that ran on chip -- and the bytes its
+ * forward and reverse passes read and wrote.  These are less than the passes'
+ * share of whole states (reverse_bytes above): the first passes leave out
+ * the amplitudes that are still zero because the state starts as one basis
+ * state.  forward_bytes also follows the forward passes of
+ * sv_apply_circuit_batch.  Any out-pointer may be NULL. */
+sv_status sv_last_adjoint_states(int32_t *states, int64_t *forward_bytes, int64_t *reverse_bytes);
 
 /* ------------------------------------------------------------- autotune */
 

@@ -126,7 +126,7 @@ def _load():
     lib.sv_phase_timing.argtypes = [I32]
     lib.sv_last_phase_ms.argtypes = [P(ctypes.c_float)] * 3
     lib.sv_last_adjoint_info.argtypes = [P(ctypes.c_int32), P(ctypes.c_int64)]
-    lib.sv_last_adjoint_states.argtypes = [P(I32)]
+    lib.sv_last_adjoint_states.argtypes = [P(I32), P(ctypes.c_int64), P(ctypes.c_int64)]
     lib.sv_status_string.argtypes = [I32]
     lib.sv_status_string.restype = ctypes.c_char_p
     lib.sv_last_error.restype = ctypes.c_char_p
@@ -598,9 +598,16 @@ def sv_last_adjoint_info() -> dict:
 def sv_last_adjoint_states() -> int:
     """States in device memory the last adjoint swept (two instances of a real
     problem share one; 0 after an on-chip adjoint)."""
-    n = ctypes.c_int32()
-    _check(_lib.sv_last_adjoint_states(ctypes.byref(n)), "sv_last_adjoint_states")
-    return n.value
+    return sv_last_moved()["states"]
+
+
+def sv_last_moved() -> dict:
+    """States swept by the last device-memory adjoint, and the bytes the last
+    forward and reverse tile passes read and wrote."""
+    n, f, r = ctypes.c_int32(), ctypes.c_int64(), ctypes.c_int64()
+    _check(_lib.sv_last_adjoint_states(ctypes.byref(n), ctypes.byref(f), ctypes.byref(r)),
+           "sv_last_adjoint_states")
+    return {"states": n.value, "forward_bytes": f.value, "reverse_bytes": r.value}
 
 
 def sv_status_string(status: int) -> str:

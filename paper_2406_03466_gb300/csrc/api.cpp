@@ -124,7 +124,10 @@ struct DeviceCtx {
     // the algorithmic bytes of its reverse tile passes.
     int last_every = 0;
     int64_t last_rev_bytes = 0;
-    int last_states = 0;  // states it swept (two real circuits share one)
+    // What the last calls' tile passes moved: states of the last adjoint (two
+    // real circuits share one), bytes of the last forward and reverse passes.
+    int last_states = 0;
+    int64_t moved_fwd = 0, moved_rev = 0;
     // Uneven batches: one instantiated graph per configuration, and the
     // stream the captures run on.
     std::unordered_map<uint64_t, std::unique_ptr<struct MultiGraph>> graphs;
@@ -659,7 +662,7 @@ sv_status h_tiles(DeviceCtx *ctx, ObsEntry *obs, int n, sv_dtype dt, int n_rows,
 // costs what one complex state costs.  One slot alone gains nothing; the
 // tensor-core blocks are complex.
 bool real_pairs(const PlanEntry *pe, const ObsEntry *obs, int n_slots, bool tc) {
-    return n_slots >= 2 && !tc && pe->real && obs && obs->dev.real;
+    return n_slots >= 2 && !tc && pe->real && !pe->tiles.empty() && obs && obs->dev.real;
 }
 
 bool wants_tiles(int n, sv_dtype dt, const sv_plan_opts *o) {
@@ -734,27 +737,72 @@ int64_t tile_blocks(const DeviceCtx *ctx, int64_t tiles) {
     return b < tiles ? b : tiles;
 }
 
-// Forward tile passes of `pe` over src.n_slots states (|ref> first when init).
-// After pass i with (i + 1) % every == 0 (and not the last pass) the states
-// are copied to checkpoint (i + 1) / every - 1 of `ck`.  pair: real slots
-// two to a state.
+// The index bits in which the references of a state's two slots differ, over
+// every pair that src can form (pairs of real circuits; slot s is instance
+// s mod I).  They count as spread from the start.
+uint32_t pair_support(const SlotSource &src, const int64_t *refs) {
+    const int64_t I = src.n_instances;
+    uint32_t m = 0;
+    for (int64_t j = 0; 2 * j + 1 < src.n_slots && j < I; ++j) {
+        const int64_t s = (int64_t)src.slot_base + 2 * j;
+        m |= (uint32_t)(refs[s % I] ^ refs[(s + 1) % I]);
+    }
+    return m;
+}
+
+// The sparse form of every pass (see Sparse in hbm.h) for states that start
+// from basis states: passes with their tile counts, and the mask of index
+// bits that the last pass leaves spread (all n bits: the states are dense).
+uint32_t sparse_plan(const PlanEntry *pe, uint32_t support, const int64_t *drefs,
+                     std::vector<TilePass> *tp, std::vector<Sparse> *sp) {
+    for (size_t i = 0; i < pe->tiles.size(); ++i) {
+        tp->push_back(pe->tiles[i]);
+        sp->push_back(sparse_pass(&tp->back(), support, drefs, i == 0));
+        for (int b = 0; b < tp->back().t; ++b) support |= tp->back().gl[b];
+    }
+    return support;
+}
+
+// Where a slot source's reference indices lie behind the group matrices.
+int64_t *refs_of(void *mats, size_t n_states, int G, size_t csz) {
+    return (int64_t *)((char *)mats + n_states * G * kMatVals * csz);
+}
+size_t mats_bytes(size_t n_states, int G, size_t csz) {
+    return n_states * (G * kMatVals * csz + 2 * sizeof(int64_t));
+}
+
+// Forward tile passes of `pe` over src.n_slots states from |ref>.  After pass
+// i with (i + 1) % every == 0 (and not the last pass) the states are written
+// to checkpoint (i + 1) / every - 1 of `ck`; outside the amplitudes that can
+// be nonzero a checkpoint holds anything.  The last pass's output in `states`
+// is whole.  refs: the instances' reference indices (pair: real slots two to
+// a state).  mats: mats_bytes().
 sv_status tiles_forward(DeviceCtx *ctx, const PlanEntry *pe, int R, sv_dtype dt,
-                        const SlotSource &src, void *states, void *mats, bool init, void *ck,
-                        int every, cudaStream_t st, bool tc = false, bool pair = false) {
+                        const SlotSource &src, const int64_t *refs, void *states, void *mats,
+                        void *ck, int every, cudaStream_t st, bool tc = false, bool pair = false) {
     const int c128 = dt == SV_C128, n = pe->n, G = pe->dev.n_groups;
     const int n_states = pair ? (src.n_slots + 1) / 2 : src.n_slots;
-    const size_t sbytes = ((size_t)n_states << n) * (c128 ? 16 : 8);
-    cudaError_t e = launch_group_mats(c128, pe->dev, src, mats, st, pair);
+    const size_t csz = c128 ? 16 : 8, sbytes = ((size_t)n_states << n) * csz;
+    int64_t *drefs = refs_of(mats, n_states, G, csz);
+    cudaError_t e = launch_group_mats(c128, pe->dev, src, mats, drefs, st, pair);
     if (e != cudaSuccess) return cuda_fail(e, "group matrices");
-    if (init) {
-        e = launch_init_states(c128, states, n, src, st, pair);
-        if (e != cudaSuccess) return cuda_fail(e, "state init");
+    std::vector<TilePass> passes;
+    std::vector<Sparse> sp;
+    const uint32_t all = n >= 32 ? ~0u : (1u << n) - 1u;
+    uint32_t spread = sparse_plan(pe, pair ? pair_support(src, refs) : 0u, drefs, &passes, &sp);
+    if (tc || passes.empty()) {  // the tensor-core passes are dense
+        passes = pe->tiles;
+        sp.assign(passes.size(), Sparse{});
+        e = launch_init_states(c128, states, n, src, st);
+    } else if (spread != all) {
+        e = cudaMemsetAsync(states, 0, sbytes, st);
     }
+    if (e != cudaSuccess) return cuda_fail(e, "state init");
     // A pass that ends at a stored forward state writes its output there
     // (out of place) and the next pass reads it from there: no copies.  The
     // last pass always writes `states`.
-    const auto &passes = pe->tiles;
     const void *in = states;
+    ctx->moved_fwd = 0;
     for (size_t i = 0; i < passes.size(); ++i) {
         const TilePass &tp = passes[i];
         const int64_t tiles = (int64_t)n_states << tp.n_tile_bits;
@@ -766,14 +814,15 @@ sv_status tiles_forward(DeviceCtx *ctx, const PlanEntry *pe, int R, sv_dtype dt,
         if (tc && tile_fwd_tc_supported(c128, tp)) {
             int *err = device_err(ctx);
             if (!err) return fail(SV_ERR_CUDA, "device error word");
-            e = launch_tile_fwd_tc(tp, n, src.n_slots, mats, G, out, tile_blocks(ctx, tiles), st,
-                                   err, in);
+            e = launch_tile_fwd_tc(tp, n, n_states, mats, G, out, tile_blocks(ctx, tiles), st, err, in);
             if (e != cudaSuccess) return cuda_fail(e, "forward tile pass (tensor cores)");
         } else {
             e = launch_tile_fwd(c128, tp, n, n_states, mats, G, out, tile_blocks(ctx, tiles), st, in,
-                                pair);
+                                pair, sp[i]);
             if (e != cudaSuccess) return cuda_fail(e, "forward tile pass");
         }
+        const int64_t moved = (tiles << tp.t) * (int64_t)csz;
+        ctx->moved_fwd += moved + (sp[i].init ? 0 : moved >> __builtin_popcount(sp[i].zero));
         in = out;
     }
     return SV_OK;
@@ -799,7 +848,7 @@ sv_status tiles_energies(DeviceCtx *ctx, const sv_problem *p, const double *thet
     s = get_array(ctx, p->refs, sizeof(int64_t) * I, &drefs);
     if (s != SV_OK) return s;
     const size_t csz = c128 ? 16 : 8, sb = csz << n;
-    const size_t mb = (size_t)pe->dev.n_groups * kMatVals * csz;
+    const size_t mb = mats_bytes(1, pe->dev.n_groups, csz);
     const size_t per = sb + mb;
     const bool pair = real_pairs(pe, obs, n_slots, cfg.tc);
     const int per_state = pair ? 2 : 1;  // slots
@@ -821,7 +870,7 @@ sv_status tiles_energies(DeviceCtx *ctx, const sv_problem *p, const double *thet
         src.inputs = p->inputs;
         src.input_stride = p->input_stride;
         src.slot_base = slot_begin + (int)c0;
-        s = tiles_forward(ctx, pe, cfg.R, dt, src, big, (char *)big + mats_off, true, nullptr, 0, st,
+        s = tiles_forward(ctx, pe, cfg.R, dt, src, p->refs, big, (char *)big + mats_off, nullptr, 0, st,
                           cfg.tc, pair);
         if (s != SV_OK) return s;
         s = h_tiles(ctx, obs, n, dt, src.n_slots, big, nullptr, E + c0, st, &pe->host.layout, pair);
@@ -896,7 +945,7 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     const int n_states = (I + per_state - 1) / per_state;
     auto bytes_per_state = [&](int ev) {
         const size_t ncp_ = npass > 1 ? (size_t)((npass - 1) / ev) : 0;
-        return (2 + ncp_) * sb + (size_t)G * kMatVals * csz + (size_t)per_state * G * 64;
+        return (2 + ncp_) * sb + mats_bytes(1, G, csz) + (size_t)per_state * G * 64;
     };
     if (every <= 0) {
         // The most stored states that still let every instance run at once:
@@ -919,7 +968,7 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
     const size_t o_lam = up((size_t)chunk * sb), o_ck = o_lam + up((size_t)chunk * sb);
     const size_t o_mats = o_ck + up((size_t)ncp * chunk * sb);
-    const size_t o_rho = o_mats + up((size_t)chunk * G * kMatVals * csz);
+    const size_t o_rho = o_mats + up(mats_bytes((size_t)chunk, G, csz));
     const size_t total = o_rho + up((size_t)chunk * per_state * G * 64);
     void *big = nullptr;
     s = get_big_scratch(ctx, st, total, &big);
@@ -931,8 +980,9 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     double *Gs = (double *)scr, *Es = Gs + (size_t)I * Pp;
     SV_CUDA(cudaMemsetAsync(Gs, 0, sizeof(double) * (size_t)I * Pp, st));
     const CostSource cs = cost_of(p, weights);
-    const auto &passes = pe->tiles;
     ctx->last_states = n_states;
+    int64_t moved_fwd = 0;
+    ctx->moved_rev = 0;
     for (int64_t c0 = 0; c0 < I; c0 += chunk * per_state) {
         SlotSource src{};
         src.mode = SLOTS_INSTANCES;
@@ -948,9 +998,14 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
         void *psi = bb, *lam = bb + o_lam, *ck = bb + o_ck, *mats = bb + o_mats;
         double *rho = (double *)(bb + o_rho);
         phase_mark(ctx, st);
-        s = tiles_forward(ctx, pe, cfg.R, dt, src, psi, mats, true, ncp ? ck : nullptr, every, st,
+        s = tiles_forward(ctx, pe, cfg.R, dt, src, p->refs, psi, mats, ncp ? ck : nullptr, every, st,
                           cfg.tc, pair);
         if (s != SV_OK) return s;
+        moved_fwd += ctx->moved_fwd;
+        std::vector<TilePass> passes;
+        std::vector<Sparse> sp;
+        sparse_plan(pe, pair ? pair_support(src, p->refs) : 0u,
+                    refs_of(mats, (size_t)states, G, csz), &passes, &sp);
         phase_mark(ctx, st);
         cudaError_t e = cudaSuccess;
         if (ddcl_target) {
@@ -976,8 +1031,9 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
             // un-computes from it (it restarts from a stored state otherwise)
             const bool write_psi = i > 0 && !(i % every == 0 && i < npass);
             e = launch_tile_rev(c128, tp, n, states, mats, G, psi, lam, rho,
-                                tile_blocks(ctx, tiles), st, psi_in, write_psi, pair);
+                                tile_blocks(ctx, tiles), st, psi_in, write_psi, pair, sp[i]);
             if (e != cudaSuccess) return cuda_fail(e, "reverse tile pass");
+            ctx->moved_rev += (tiles << tp.t) * (int64_t)csz * (write_psi ? 4 : 3);
             // psi (or its stored state) and lambda read, lambda (and psi) written
             ctx->last_rev_bytes += (int64_t)src.n_slots * (int64_t)sb * (write_psi ? 4 : 3);
         }
@@ -985,6 +1041,7 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
         e = launch_group_grads(c128, pe->dev, src, rho, cs, Es + c0, Gs + (size_t)c0 * Pp, st);
         if (e != cudaSuccess) return cuda_fail(e, "per-slot gradients");
     }
+    ctx->moved_fwd = moved_fwd;
     cudaError_t e = launch_adjoint_combine(Gs, Es, I, P, cs, energy_out, loss_out, grad_out, st);
     if (e != cudaSuccess) return cuda_fail(e, "adjoint combine");
     return SV_OK;
@@ -999,6 +1056,8 @@ struct MultiProblem {
     ObsEntry *obs = nullptr;
     const void *drefs = nullptr;
     int n = 0, I = 0, P = 0, G = 0, npass = 0;
+    std::vector<TilePass> tiles;  // the passes' sparse forms
+    std::vector<Sparse> sparse;
     size_t o_tp = 0, o_psi = 0, o_lam = 0, o_mats = 0, o_rho = 0, o_E = 0, o_G = 0;
     SlotSource src{};
 };
@@ -1023,7 +1082,8 @@ sv_status multi_sequence(DeviceCtx *ctx, std::vector<MultiProblem> &mp, sv_dtype
     if (!err) return fail(SV_ERR_CUDA, "device error word");
     for (MultiProblem &m : mp) {
         m.src.theta = theta[&m - &mp[0]];
-        cudaError_t e = launch_group_mats(c128, m.pe->dev, m.src, base + m.o_mats, st);
+        cudaError_t e = launch_group_mats(c128, m.pe->dev, m.src, base + m.o_mats,
+                                          refs_of(base + m.o_mats, m.I, m.G, c128 ? 16 : 8), st);
         if (e == cudaSuccess) e = launch_init_states(c128, base + m.o_psi, m.n, m.src, st);
         if (e != cudaSuccess) return cuda_fail(e, "uneven batch: group matrices / init");
     }
@@ -1127,6 +1187,7 @@ sv_status multi_adjoint(DeviceCtx *ctx, const sv_problem *problems, int np,
         if (s != SV_OK) return s;
         m.G = m.pe->dev.n_groups;
         m.npass = (int)m.pe->tiles.size();
+        sparse_plan(m.pe, 0u, nullptr, &m.tiles, &m.sparse);
         max_pass = std::max(max_pass, m.npass);
         m.src.mode = SLOTS_INSTANCES;
         m.src.n_slots = m.I;
@@ -1137,7 +1198,7 @@ sv_status multi_adjoint(DeviceCtx *ctx, const sv_problem *problems, int np,
         m.o_tp = take(sizeof(TilePass) * (size_t)m.npass);
         m.o_psi = take(((size_t)m.I << m.n) * csz);
         m.o_lam = take(((size_t)m.I << m.n) * csz);
-        m.o_mats = take((size_t)m.I * m.G * kMatVals * csz);
+        m.o_mats = take(mats_bytes(m.I, m.G, csz));
         m.o_rho = take((size_t)m.I * m.G * 64);
         m.o_E = take(sizeof(double) * (size_t)m.I);
         m.o_G = take(sizeof(double) * (size_t)m.I * (m.P > 0 ? m.P : 1));
@@ -1158,7 +1219,7 @@ sv_status multi_adjoint(DeviceCtx *ctx, const sv_problem *problems, int np,
                 const MultiProblem &m = mp[j];
                 if (k >= m.npass) continue;
                 const int pi = rev ? m.npass - 1 - k : k;
-                const TilePass &tp = m.pe->tiles[pi];
+                const TilePass &tp = m.tiles[pi];
                 sw[rev].smem = std::max(sw[rev].smem, tile_sweep_smem(c128, rev != 0, tp));
                 SweepTask T{};
                 T.n = m.n;
@@ -1199,13 +1260,15 @@ sv_status multi_adjoint(DeviceCtx *ctx, const sv_problem *problems, int np,
     ng->buf.bytes = off;
     unsigned char *base = (unsigned char *)ng->buf.ptr;
     for (MultiProblem &m : mp)
-        SV_CUDA(cudaMemcpy(base + m.o_tp, m.pe->tiles.data(), sizeof(TilePass) * (size_t)m.npass,
+        SV_CUDA(cudaMemcpy(base + m.o_tp, m.tiles.data(), sizeof(TilePass) * (size_t)m.npass,
                            cudaMemcpyHostToDevice));
     for (int rev = 0; rev < 2; ++rev) {
         for (size_t i = 0; i < tasks[rev].size(); ++i) {
             const MultiProblem &m = mp[who[rev][i].first];
             SweepTask &T = tasks[rev][i];
             T.P = (const TilePass *)(base + m.o_tp) + who[rev][i].second;
+            T.refs = refs_of(base + m.o_mats, m.I, m.G, csz);
+            T.fixed = m.sparse[who[rev][i].second].fixed;
             T.mats = base + m.o_mats;
             T.psi = base + m.o_psi;
             T.lam = base + m.o_lam;
@@ -1380,7 +1443,7 @@ sv_status sv_apply_circuit_batch(sv_state state, const sv_circuit *circuits, int
             if (s != SV_OK) return s;
             const size_t csz = state->dtype == SV_C128 ? 16 : 8;
             void *mats = nullptr;
-            s = get_big_scratch(ctx, st, sub.size() * pe->dev.n_groups * kMatVals * csz + 256, &mats);
+            s = get_big_scratch(ctx, st, mats_bytes(sub.size(), pe->dev.n_groups, csz) + 256, &mats);
             if (s != SV_OK) return s;
             SlotSource src{};
             src.mode = SLOTS_EXPLICIT;
@@ -1391,7 +1454,7 @@ sv_status sv_apply_circuit_batch(sv_state state, const sv_circuit *circuits, int
             src.input_stride = input_stride;
             src.slots = (const sv_slot *)dslots;
             char *rows0 = (char *)state->ptr + (size_t)rows[0] * (csz << state->n);
-            s = tiles_forward(ctx, pe, cfg.R, state->dtype, src, rows0, mats, true, nullptr, 0, st,
+            s = tiles_forward(ctx, pe, cfg.R, state->dtype, src, nullptr, rows0, mats, nullptr, 0, st,
                               cfg.tc);
             if (s != SV_OK) return s;
             continue;
@@ -1974,7 +2037,7 @@ sv_status sv_grad_ddcl_param_shift(const sv_problem *p, const double *theta,
     if (s != SV_OK) return s;
     double *E = (double *)scr, *lp = E + B, *D = lp + 1;
     const size_t csz = c128 ? 16 : 8, sb = csz << n;
-    const size_t mb = (size_t)pe->dev.n_groups * kMatVals * csz;
+    const size_t mb = mats_bytes(1, pe->dev.n_groups, csz);
     int64_t chunk = (int64_t)(big_budget(ctx, st) / (sb + mb + 512));
     if (chunk < 1) return fail(SV_ERR_OOM, "one state does not fit in free device memory");
     if (chunk > B) chunk = B;
@@ -1993,7 +2056,7 @@ sv_status sv_grad_ddcl_param_shift(const sv_problem *p, const double *theta,
     // the unshifted circuit (slot 0): JS and the table dJS/dP_theta
     src.n_slots = 1;
     src.slot_base = 0;
-    s = tiles_forward(ctx, pe, cfg.R, dt, src, big, (char *)big + mats_off, true, nullptr, 0, st,
+    s = tiles_forward(ctx, pe, cfg.R, dt, src, p->refs, big, (char *)big + mats_off, nullptr, 0, st,
                       cfg.tc);
     if (s != SV_OK) return s;
     cudaError_t e = launch_ddcl_diag(c128, n, big, target, D, js_out, st);
@@ -2002,7 +2065,7 @@ sv_status sv_grad_ddcl_param_shift(const sv_problem *p, const double *theta,
     for (int64_t c0 = 0; c0 < B; c0 += chunk) {
         src.n_slots = (int)std::min<int64_t>(chunk, B - c0);
         src.slot_base = (int)c0;
-        s = tiles_forward(ctx, pe, cfg.R, dt, src, big, (char *)big + mats_off, true, nullptr, 0, st,
+        s = tiles_forward(ctx, pe, cfg.R, dt, src, p->refs, big, (char *)big + mats_off, nullptr, 0, st,
                           cfg.tc);
         if (s != SV_OK) return s;
         e = launch_diag_expect(c128, n, src.n_slots, big, D, E + c0, st);
@@ -2401,11 +2464,13 @@ sv_status sv_last_adjoint_info(int32_t *checkpoint_every, int64_t *reverse_bytes
     return SV_OK;
 }
 
-sv_status sv_last_adjoint_states(int32_t *states) {
+sv_status sv_last_adjoint_states(int32_t *states, int64_t *forward_bytes, int64_t *reverse_bytes) {
     DeviceCtx *ctx = context();
     if (!ctx) return fail(SV_ERR_CUDA, "no CUDA device");
     std::lock_guard<std::mutex> lk(ctx->mu);
     if (states) *states = ctx->last_states;
+    if (forward_bytes) *forward_bytes = ctx->moved_fwd;
+    if (reverse_bytes) *reverse_bytes = ctx->moved_rev;
     return SV_OK;
 }
 

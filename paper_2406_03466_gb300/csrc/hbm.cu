@@ -42,10 +42,13 @@ namespace {
 // pair's real rotations come with c >= 0 (a state's sign is of no account
 // to its energy and its gradient), for the shear form.
 template <typename Real>
-__global__ void k_group_mats(Program p, SlotSource src, int pair, typename CT<Real>::T *out) {
+__global__ void k_group_mats(Program p, SlotSource src, int pair, typename CT<Real>::T *out,
+                             int64_t *refs) {
     using C = typename CT<Real>::T;
-    const int G = p.n_groups;
-    const int64_t total = (int64_t)(pair ? (src.n_slots + 1) / 2 : src.n_slots) * G;
+    const int G = p.n_groups, n_states = pair ? (src.n_slots + 1) / 2 : src.n_slots;
+    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < 2 * n_states; b += gridDim.x * blockDim.x)
+        refs[b] = resolve(src, pair ? min(b, src.n_slots - 1) : b >> 1).ref;
+    const int64_t total = (int64_t)n_states * G;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int b = (int)(i / G), g = (int)(i % G);
@@ -68,12 +71,13 @@ __global__ void k_group_mats(Program p, SlotSource src, int pair, typename CT<Re
 
 // Sets amplitude |ref_b> of every (zeroed) slot state to 1.
 template <typename C>
-__global__ void k_set_ref(C *states, int n, SlotSource src, int pair) {
+__global__ void k_set_ref(C *states, int n, SlotSource src) {
     for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < src.n_slots; b += gridDim.x * blockDim.x) {
         const SlotInfo si = resolve(src, b);
-        C *s = states + ((int64_t)(pair ? b >> 1 : b) << n) + si.ref;
-        if (!pair || !(b & 1)) s->x = 1;
-        if (pair && ((b & 1) || b + 1 == src.n_slots)) s->y = 1;
+        C one;
+        one.x = 1;
+        one.y = 0;
+        states[((int64_t)b << n) + si.ref] = one;
     }
 }
 
@@ -154,7 +158,8 @@ __device__ __forceinline__ void tile_fwd_body(const TilePass &P, int n, int n_sl
                                               const typename CT<Real>::T *mats, int G,
                                               const typename CT<Real>::T *src_states,
                                               typename CT<Real>::T *states, int64_t t0,
-                                              int64_t t_end, unsigned char *smem) {
+                                              int64_t t_end, unsigned char *smem,
+                                              const Sparse &sp) {
     using C = typename CT<Real>::T;
     constexpr int NA = 1 << R;
     constexpr uint32_t kBufs = 2u;
@@ -184,13 +189,32 @@ __device__ __forceinline__ void tile_fwd_body(const TilePass &P, int n, int n_sl
     auto fetch = [&](const TileCursor &c, int buf) {
         const C *src = src_states + ((int64_t)c.slot << n) + c.base;
         const uint32_t d = sh + (uint32_t)buf * tbytes;
+        if (sp.zero | (uint32_t)sp.init) {  // known zeros are not read
+            const int64_t *rf = sp.refs + 2 * (int64_t)c.slot;
+            const uint32_t ra = (uint32_t)rf[0], rb = (uint32_t)rf[1];
 #pragma unroll
-        for (int k = 0; k < NA; ++k) cp_async_amp(d + (p0 ^ xsel<R>(k, pk)), src + (g0 ^ xsel<R>(k, gk)));
+            for (int k = 0; k < NA; ++k) {
+                const uint32_t so = p0 ^ xsel<R>(k, pk), go = g0 ^ xsel<R>(k, gk);
+                C v;
+                v.x = v.y = 0;
+                if (sp.init) {
+                    if (kMat == kPair) v.y = (c.base ^ go) == rb ? 1 : 0;
+                    v.x = (c.base ^ go) == ra ? 1 : 0;
+                } else if (((go ^ ra) & sp.zero) == 0u) {
+                    cp_async_amp(d + so, src + go);
+                    continue;
+                }
+                *reinterpret_cast<C *>(smem + (uint32_t)buf * tbytes + so) = v;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < NA; ++k) cp_async_amp(d + (p0 ^ xsel<R>(k, pk)), src + (g0 ^ xsel<R>(k, gk)));
+        }
         cp_async_commit();
     };
-    TileCursor cur = tile_cursor(P, t0);
+    TileCursor cur = tile_cursor(P, t0, sp.refs, sp.fixed);
     fetch(cur, 0);
-    TileCursor nxt = tile_next(P, cur);
+    TileCursor nxt = tile_next(P, cur, sp.refs, sp.fixed, n_slots);
     int mslot = -1;
     for (int64_t tix = t0, i = 0; tix < t_end; ++tix, ++i) {
         const int buf = (int)(i & 1);
@@ -220,7 +244,7 @@ __device__ __forceinline__ void tile_fwd_body(const TilePass &P, int n, int n_sl
         for (int k = 0; k < NA; ++k)
             dst[g0 ^ xsel<R>(k, gk)] = *reinterpret_cast<const C *>(tile + (n0 ^ xsel<R>(k, nk)));
         cur = nxt;
-        nxt = tile_next(P, nxt);
+        nxt = tile_next(P, nxt, sp.refs, sp.fixed, n_slots);
     }
 }
 
@@ -231,11 +255,11 @@ template <typename Real, int R, int kMat>
 __global__ void __launch_bounds__(256, R >= 4 ? 2 : 3)
 k_tile_fwd(const __grid_constant__ TilePass P, int n, int n_slots,
            const typename CT<Real>::T *mats, int G, const typename CT<Real>::T *src,
-           typename CT<Real>::T *states) {
+           typename CT<Real>::T *states, Sparse sp) {
     extern __shared__ __align__(16) unsigned char smem[];
     int64_t t0, t_end;
     block_range((int64_t)n_slots << P.n_tile_bits, gridDim.x, blockIdx.x, t0, t_end);
-    tile_fwd_body<Real, R, kMat>(P, n, n_slots, mats, G, src, states, t0, t_end, smem);
+    tile_fwd_body<Real, R, kMat>(P, n, n_slots, mats, G, src, states, t0, t_end, smem, sp);
 }
 
 // The derivative of a rotation exp(-i theta P / 2) inside a fused group is
@@ -670,7 +694,8 @@ __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_sl
                                               const typename CT<Real>::T *psi_src,
                                               typename CT<Real>::T *psi, typename CT<Real>::T *lam,
                                               double *rho_g, int64_t t0, int64_t t_end,
-                                              unsigned char *smem, bool write_psi = true) {
+                                              unsigned char *smem, const int64_t *refs,
+                                              uint32_t fixed, bool write_psi = true) {
     using C = typename CT<Real>::T;
     constexpr int NA = 1 << R;
     constexpr int kFlushTiles = 64;
@@ -717,9 +742,9 @@ __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_sl
         }
         cp_async_commit();
     };
-    TileCursor cur = tile_cursor(P, t0);
+    TileCursor cur = tile_cursor(P, t0, refs, fixed);
     fetch(cur, 0);
-    TileCursor nxt = tile_next(P, cur);
+    TileCursor nxt = tile_next(P, cur, refs, fixed, n_slots);
     int mslot = -1, since = 0;
     for (int64_t tix = t0, i = 0; tix < t_end; ++tix, ++i) {
         const int buf = NB == 2 ? (int)(i & 1) : 0;
@@ -840,7 +865,7 @@ __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_sl
             fetch(nxt, 0);
         }
         cur = nxt;
-        nxt = tile_next(P, nxt);
+        nxt = tile_next(P, nxt, refs, fixed, n_slots);
     }
     flush_acc<Real, kSingle, kMat, R>(P, acc, wps, rho_g, mslot, G, rec, sm);
 }
@@ -850,12 +875,13 @@ template <typename Real, int R, bool kSingle, int kMat, int NB = 2>
 __global__ void __launch_bounds__(NB == 1 ? 64 : 256, NB == 1 ? 5 : (R >= 4 ? 1 : 2))
 k_tile_rev(const __grid_constant__ TilePass P, int n, int n_slots,
            const typename CT<Real>::T *mats, int G, const typename CT<Real>::T *psi_src,
-           typename CT<Real>::T *psi, typename CT<Real>::T *lam, double *rho_g, int write_psi) {
+           typename CT<Real>::T *psi, typename CT<Real>::T *lam, double *rho_g, Sparse sp,
+           int write_psi) {
     extern __shared__ __align__(16) unsigned char smem[];
     int64_t t0, t_end;
     block_range((int64_t)n_slots << P.n_tile_bits, gridDim.x, blockIdx.x, t0, t_end);
     tile_rev_body<Real, R, kSingle, kMat, NB>(P, n, n_slots, mats, G, psi_src, psi, lam, rho_g,
-                                               t0, t_end, smem, write_psi != 0);
+                                               t0, t_end, smem, sp.refs, sp.fixed, write_psi != 0);
 }
 
 // Sum of v over the block (every thread gets it); red: one double per warp.
@@ -954,10 +980,11 @@ k_tile_sweep(const SweepTask *tasks, int n_tasks, long long n_tickets,
         if constexpr (kRev)
             tile_rev_body<Real, R, false, kAny>(P, T.n, T.n_slots, (const C *)T.mats, T.G,
                                                  (const C *)T.psi, (C *)T.psi, (C *)T.lam, T.rho,
-                                                 t0, t1, rest);
+                                                 t0, t1, rest, T.refs, T.fixed);
         else
             tile_fwd_body<Real, R, kAny>(P, T.n, T.n_slots, (const C *)T.mats, T.G,
-                                          (const C *)T.psi, (C *)T.psi, t0, t1, rest);
+                                         (const C *)T.psi, (C *)T.psi, t0, t1, rest,
+                                         Sparse{T.refs, T.fixed, 0u, 0, 0});
         __syncthreads();  // every store of the chunk issued
         if (threadIdx.x == 0) {
             __threadfence();
@@ -1455,23 +1482,46 @@ int grid_1d(int64_t work, int threads) {
     } while (0)
 
 cudaError_t launch_group_mats(int c128, const Program &p, const SlotSource &src, void *mats,
-                              cudaStream_t st, bool pair) {
-    const int g = grid_1d((int64_t)src.n_slots * p.n_groups, 128);
-    if (c128) k_group_mats<double><<<g, 128, 0, st>>>(p, src, pair, (double2 *)mats);
-    else k_group_mats<float><<<g, 128, 0, st>>>(p, src, pair, (float2 *)mats);
+                              int64_t *refs, cudaStream_t st, bool pair) {
+    // one warp a block: the FP64 sines of a few thousand groups spread over
+    // every SM (32 slots x 190 groups: 22 us in blocks of 128 threads)
+    const int g = grid_1d((int64_t)src.n_slots * std::max(1, p.n_groups), 32);
+    if (c128) k_group_mats<double><<<g, 32, 0, st>>>(p, src, pair, (double2 *)mats, refs);
+    else k_group_mats<float><<<g, 32, 0, st>>>(p, src, pair, (float2 *)mats, refs);
     return cudaGetLastError();
 }
 
 cudaError_t launch_init_states(int c128, void *states, int n, const SlotSource &src,
-                               cudaStream_t st, bool pair) {
-    const size_t n_states = pair ? ((size_t)src.n_slots + 1) / 2 : (size_t)src.n_slots;
-    const size_t bytes = (n_states << n) * (c128 ? 16 : 8);
+                               cudaStream_t st) {
+    const size_t bytes = ((size_t)src.n_slots << n) * (c128 ? 16 : 8);
     cudaError_t e = cudaMemsetAsync(states, 0, bytes, st);
     if (e != cudaSuccess) return e;
     const int g = grid_1d(src.n_slots, 128);
-    if (c128) k_set_ref<double2><<<g, 128, 0, st>>>((double2 *)states, n, src, pair);
-    else k_set_ref<float2><<<g, 128, 0, st>>>((float2 *)states, n, src, pair);
+    if (c128) k_set_ref<double2><<<g, 128, 0, st>>>((double2 *)states, n, src);
+    else k_set_ref<float2><<<g, 128, 0, st>>>((float2 *)states, n, src);
     return cudaGetLastError();
+}
+
+Sparse sparse_pass(TilePass *P, uint32_t support, const int64_t *refs, bool init) {
+    Sparse sp{};
+    sp.refs = refs;
+    sp.init = init;
+    uint32_t prev = 0, acc = 0;
+    int nt = 0;
+    const int n_tile_bits = P->n_tile_bits;
+    for (int k = 0; k < n_tile_bits; ++k) {
+        const uint32_t bit = P->gpre[k] ^ prev;
+        prev = P->gpre[k];
+        if (bit & support) {
+            acc ^= bit;
+            P->gpre[nt++] = acc;
+        } else {
+            sp.fixed |= bit;
+        }
+    }
+    P->n_tile_bits = nt;
+    for (int b = 0; b < P->t; ++b) sp.zero |= P->gl[b] & ~support;
+    return sp;
 }
 
 // Phase tables of the split stages (kernels of kind kAny).
@@ -1497,7 +1547,7 @@ uint32_t tile_rev_smem(int c128, const TilePass &P, int bufs, bool any) {
 
 cudaError_t launch_tile_fwd(int c128, const TilePass &P, int n, int n_slots, const void *mats,
                             int G, void *states, int64_t max_blocks, cudaStream_t st,
-                            const void *src, bool pair) {
+                            const void *src, bool pair, const Sparse &sp) {
     const uint32_t smem = tile_fwd_smem(c128, P);
     const int threads = 1 << (P.t - P.R);
     if (!src) src = states;
@@ -1509,14 +1559,15 @@ cudaError_t launch_tile_fwd(int c128, const TilePass &P, int n, int n_slots, con
         if (e != cudaSuccess) return e;
         const int blocks = fill_blocks(k, threads, smem, max_blocks);
         k<<<blocks, threads, smem, st>>>(P, n, n_slots, (const C *)mats, G, (const C *)src,
-                                         (C *)states);
+                                         (C *)states, sp);
     });
     return cudaGetLastError();
 }
 
 cudaError_t launch_tile_rev(int c128, const TilePass &P, int n, int n_slots, const void *mats,
                             int G, void *psi, void *lam, double *rho_g, int64_t max_blocks,
-                            cudaStream_t st, const void *psi_src, bool write_psi, bool pair) {
+                            cudaStream_t st, const void *psi_src, bool write_psi, bool pair,
+                            const Sparse &sp) {
     // passes of many stages are arithmetic-bound: one tile buffer, more
     // blocks per SM (complex64 real single-sum passes, tiles of 2^10 at 16
     // amplitudes per thread: 64 threads)
@@ -1540,7 +1591,7 @@ cudaError_t launch_tile_rev(int c128, const TilePass &P, int n, int n_slots, con
         const int blocks = fill_blocks(k, threads, smem, max_blocks);
         k<<<blocks, threads, smem, st>>>(P, n, n_slots, (const C *)mats, G,
                                          (const C *)(psi_src ? psi_src : psi), (C *)psi, (C *)lam,
-                                         rho_g, write_psi ? 1 : 0);
+                                         rho_g, sp, write_psi ? 1 : 0);
     });
     return cudaGetLastError();
 }

@@ -15,11 +15,30 @@ namespace svk {
 // with pair) by the groups' split form [slots][groups][4].  kMatVals complex
 // values per slot and group hold both.
 constexpr int kMatVals = 8;
+// refs: [states][2], the states' reference indices (pair: of the two slots;
+// otherwise the slot's twice).
 cudaError_t launch_group_mats(int c128, const Program &p, const SlotSource &src, void *mats,
-                              cudaStream_t st, bool pair = false);
+                              int64_t *refs, cudaStream_t st, bool pair = false);
 // Zeroes the slot states and sets amplitude |ref> of each to 1.
 cudaError_t launch_init_states(int c128, void *states, int n, const SlotSource &src,
-                               cudaStream_t st, bool pair = false);
+                               cudaStream_t st);
+// Where a pass's states are known to be zero.  A state starts as |ref>, and a
+// pass spreads it over the index bits local to it only, so before pass i
+// every amplitude is zero whose bits outside the union of the earlier passes'
+// local bits differ from ref's.  A sparse pass walks the tiles that can hold
+// a nonzero amplitude (its TilePass counts the tile-number bits inside the
+// union; `fixed` are the others, taken from ref), and reads only amplitudes
+// whose local bits in `zero` equal ref's (the others are zero and need not be
+// in memory).  init: the state before the pass is |ref> itself, not read.
+// All zero: a dense pass.
+struct Sparse {
+    const int64_t *refs;  // [states][2]
+    uint32_t fixed, zero;
+    int32_t init, pad;
+};
+// The sparse form of pass P when the amplitudes' bits in `support` (an index
+// mask) are the ones that may differ from ref; sets P's tile count.
+Sparse sparse_pass(TilePass *P, uint32_t support, const int64_t *refs, bool init);
 // Shared memory of one block of the forward / reverse kernels of pass P.
 // (any: of a kernel that takes complex and real passes alike).
 uint32_t tile_fwd_smem(int c128, const TilePass &P, bool any = false);
@@ -28,7 +47,8 @@ uint32_t tile_rev_smem(int c128, const TilePass &P, int bufs = 2, bool any = fal
 // src (null: states) holds the pass's input; the output goes to states.
 cudaError_t launch_tile_fwd(int c128, const TilePass &P, int n, int n_slots, const void *mats,
                             int G, void *states, int64_t max_blocks, cudaStream_t st,
-                            const void *src = nullptr, bool pair = false);
+                            const void *src = nullptr, bool pair = false,
+                            const Sparse &sp = Sparse{});
 // Reverse pass P on psi and lambda; adds the reduced matrices of its
 // parametrised groups to rho_g[slot][G][8].  psi_src (null: psi) holds the
 // psi the pass reads (a stored forward state); its output psi goes to psi
@@ -37,7 +57,8 @@ cudaError_t launch_tile_fwd(int c128, const TilePass &P, int n, int n_slots, con
 cudaError_t launch_tile_rev(int c128, const TilePass &P, int n, int n_slots, const void *mats,
                             int G, void *psi, void *lam, double *rho_g, int64_t max_blocks,
                             cudaStream_t st, const void *psi_src = nullptr,
-                            bool write_psi = true, bool pair = false);
+                            bool write_psi = true, bool pair = false,
+                            const Sparse &sp = Sparse{});
 // Codes a kernel writes to the library's device error word when a bounded
 // device-side wait gives up (reported as SV_ERR_TIMEOUT by sv_sync_status).
 constexpr int SV_DEVERR_MMA_WAIT = 1;

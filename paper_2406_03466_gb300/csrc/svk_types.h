@@ -160,6 +160,8 @@ struct Observable {
 struct SweepTask {
     const TilePass *P;  // device descriptor
     int32_t n, n_slots, G, dep;
+    const int64_t *refs;  // [slots][2]: sparse passes' reference indices
+    uint32_t fixed, pad2; // tile-number bits taken from the reference (hbm.h: Sparse)
     int64_t tiles, chunk_begin, n_chunks;
     int32_t chunk_tiles, pad;
     const void *mats;   // [slots][G][4]

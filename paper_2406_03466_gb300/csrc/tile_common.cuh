@@ -59,28 +59,40 @@ __device__ __forceinline__ void block_range(int64_t tiles, int nblk, int blk, in
 
 // Position of one tile in the walk over (slot, tile): global offset of the
 // tile's first amplitude within its state.
+// fix: the fixed tile-number bits of the slot's reference (sparse passes).
 struct TileCursor {
     int slot;
-    uint32_t local, base;
+    uint32_t local, base, fix;
 };
+__device__ __forceinline__ uint32_t fixed_bits(const int64_t *refs, uint32_t fixed, int slot) {
+    return fixed ? (uint32_t)refs[2 * (int64_t)slot] & fixed : 0u;
+}
 
-__device__ __forceinline__ TileCursor tile_cursor(const TilePass &P, int64_t tix) {
+__device__ __forceinline__ TileCursor tile_cursor(const TilePass &P, int64_t tix,
+                                                  const int64_t *refs = nullptr,
+                                                  uint32_t fixed = 0) {
     TileCursor c;
     c.slot = (int)(tix >> P.n_tile_bits);
     c.local = (uint32_t)(tix & ((int64_t(1) << P.n_tile_bits) - 1));
     c.base = 0;
     for (int k = 0; k < P.n_tile_bits; ++k)
         if ((c.local >> k) & 1u) c.base ^= P.gpre[k] ^ (k ? P.gpre[k - 1] : 0u);
+    c.fix = fixed_bits(refs, fixed, c.slot);
+    c.base ^= c.fix;
     return c;
 }
 
-// Next tile: counting up flips tile-number bits 0..ctz(local + 1).
-__device__ __forceinline__ TileCursor tile_next(const TilePass &P, TileCursor c) {
+// Next tile: counting up flips tile-number bits 0..ctz(local + 1) (past the
+// last slot: not used).
+__device__ __forceinline__ TileCursor tile_next(const TilePass &P, TileCursor c,
+                                                const int64_t *refs = nullptr,
+                                                uint32_t fixed = 0, int n_slots = 0) {
     ++c.local;
     if ((c.local >> P.n_tile_bits) != 0u) {
         c.local = 0;
-        c.base = 0;
         ++c.slot;
+        if (fixed && c.slot < n_slots) c.fix = fixed_bits(refs, fixed, c.slot);
+        c.base = c.fix;
     } else {
         c.base ^= P.gpre[__ffs((int)c.local) - 1];
     }

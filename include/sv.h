@@ -394,7 +394,9 @@ sv_status sv_grad_adjoint_multi(const sv_problem *problems, int32_t n_problems,
  * the whole state stays in one block's shared memory, else the number of tile
  * passes over device memory and their tile size (2^tile_bits amplitudes), as
  * the energy and gradient entry points plan them (relabeling passes unless
- * opts->no_relabel; sv_apply_circuit_batch plans with no_relabel set);
+ * opts->no_relabel; sv_apply_circuit_batch plans with no_relabel set; with
+ * opts->tile_bits at zero they may take the circuit's trailing CNOTs into the
+ * observable and run fewer, see sv_last_adjoint_states);
  * n_stages: register stages of the program; n_groups: fused single-qubit
  * groups.  Host-only (plans the circuit, launches nothing).  Any out-pointer
  * may be NULL. */
@@ -433,13 +435,14 @@ sv_status sv_last_adjoint_info(int32_t *checkpoint_every, int64_t *reverse_bytes
  * memory it swept -- one per instance, or half as many (rounded up) when the
  * instances' amplitudes are all real (Ry, X, H, CNOT and CZ gates, Ry
  * encodings, an observable without odd Y counts) and two instances share one
- * complex state; 0 after an adjoint that ran on chip -- and the bytes its
- * forward and reverse passes read and wrote.  These are less than the passes'
+ * complex state; 0 after an adjoint that ran on chip -- its passes each way,
+ * and the bytes the forward and the reverse passes read and wrote.  These are less than the passes'
  * share of whole states (reverse_bytes above): the first passes leave out
  * the amplitudes that are still zero because the state starts as one basis
  * state.  forward_bytes also follows the forward passes of
  * sv_apply_circuit_batch.  Any out-pointer may be NULL. */
-sv_status sv_last_adjoint_states(int32_t *states, int64_t *forward_bytes, int64_t *reverse_bytes);
+sv_status sv_last_adjoint_states(int32_t *states, int32_t *passes, int64_t *forward_bytes,
+                                 int64_t *reverse_bytes);
 
 /* ------------------------------------------------------------- autotune */
 

@@ -55,6 +55,17 @@ sv_status sv_debug_h_passes(const sv_pauli_sum *h, int32_t tile_bits, int32_t co
  * SV_ERR_TIMEOUT).  limit: 1..2^20. */
 sv_status sv_debug_wait_expiry(int32_t limit, sv_stream_t stream);
 
+/* The relabeling tile plan without the circuit's trailing CNOTs: passes kept,
+ * the CNOTs left out (control, target pairs in time order; tail holds
+ * 2 n_gates entries) and the layout, as sv_debug_tile_passes gives it. */
+sv_status sv_debug_drop_tail(const sv_circuit *c, int32_t tile_bits, int32_t reg_bits,
+                             int32_t dtype, int32_t *n_passes, int32_t *n_tail, int32_t *tail,
+                             int32_t *layout);
+/* Pauli strings (x, z masks) conjugated by CNOTs (pairs in time order): the
+ * masks are replaced, sign[i] is +1 or -1. */
+sv_status sv_debug_conjugate(const int32_t *tail, int32_t n_tail, int32_t n_terms, uint64_t *x,
+                             uint64_t *z, int32_t *sign);
+
 #ifdef __cplusplus
 }
 #endif

@@ -126,7 +126,7 @@ def _load():
     lib.sv_phase_timing.argtypes = [I32]
     lib.sv_last_phase_ms.argtypes = [P(ctypes.c_float)] * 3
     lib.sv_last_adjoint_info.argtypes = [P(ctypes.c_int32), P(ctypes.c_int64)]
-    lib.sv_last_adjoint_states.argtypes = [P(I32), P(ctypes.c_int64), P(ctypes.c_int64)]
+    lib.sv_last_adjoint_states.argtypes = [P(I32), P(I32), P(ctypes.c_int64), P(ctypes.c_int64)]
     lib.sv_status_string.argtypes = [I32]
     lib.sv_status_string.restype = ctypes.c_char_p
     lib.sv_last_error.restype = ctypes.c_char_p
@@ -602,12 +602,13 @@ def sv_last_adjoint_states() -> int:
 
 
 def sv_last_moved() -> dict:
-    """States swept by the last device-memory adjoint, and the bytes the last
-    forward and reverse tile passes read and wrote."""
-    n, f, r = ctypes.c_int32(), ctypes.c_int64(), ctypes.c_int64()
-    _check(_lib.sv_last_adjoint_states(ctypes.byref(n), ctypes.byref(f), ctypes.byref(r)),
-           "sv_last_adjoint_states")
-    return {"states": n.value, "forward_bytes": f.value, "reverse_bytes": r.value}
+    """States swept by the last device-memory adjoint, its passes each way, and
+    the bytes the last forward and reverse tile passes read and wrote."""
+    n, k, f, r = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int64(), ctypes.c_int64()
+    _check(_lib.sv_last_adjoint_states(ctypes.byref(n), ctypes.byref(k), ctypes.byref(f),
+                                       ctypes.byref(r)), "sv_last_adjoint_states")
+    return {"states": n.value, "passes": k.value, "forward_bytes": f.value,
+            "reverse_bytes": r.value}
 
 
 def sv_status_string(status: int) -> str:

@@ -90,7 +90,8 @@ struct ObsEntry {
     DeviceBuf buf;
     Observable dev{};
     DeviceBuf dtab;  // diagonal tables D_g(j) for on-chip sizes, or empty
-    // by tile bits and the qubits' bit layout of the states they run on
+    // by tile bits and what the states they run on leave to the observable:
+    // the qubits' bit layout and the trailing CNOTs (get_hplan)
     std::map<std::pair<int, std::vector<int>>, std::unique_ptr<HPlanEntry>> hplans;
 };
 
@@ -126,7 +127,7 @@ struct DeviceCtx {
     int64_t last_rev_bytes = 0;
     // What the last calls' tile passes moved: states of the last adjoint (two
     // real circuits share one), bytes of the last forward and reverse passes.
-    int last_states = 0;
+    int last_states = 0, last_passes = 0;
     int64_t moved_fwd = 0, moved_rev = 0;
     // Uneven batches: one instantiated graph per configuration, and the
     // stream the captures run on.
@@ -216,7 +217,8 @@ int swz_bits(sv_dtype d) { return d == SV_C128 ? 3 : 4; }
 // tile_bits > 0: the circuit cut into tile passes of 2^tile_bits amplitudes
 // (states in device memory) instead of one on-chip program.
 sv_status get_plan(DeviceCtx *ctx, const sv_circuit &c, int R, bool fuse, sv_dtype dt,
-                   PlanEntry **out, int tile_bits = 0, int coalesce = 0, bool relabel = false) {
+                   PlanEntry **out, int tile_bits = 0, int coalesce = 0, bool relabel = false,
+                   bool drop_tail = false) {
     if (coalesce <= 0) coalesce = dt == SV_C128 ? 3 : 4;
     if (tile_bits <= 0) relabel = false;
     uint64_t key = hash_circuit(c);
@@ -225,7 +227,7 @@ sv_status get_plan(DeviceCtx *ctx, const sv_circuit &c, int R, bool fuse, sv_dty
     key = mix64(key, (uint64_t)swz_bits(dt));
     key = mix64(key, (uint64_t)(1000 + tile_bits));
     key = mix64(key, (uint64_t)(2000 + coalesce));
-    key = mix64(key, relabel ? 0x7e1abe1ull : 0ull);
+    key = mix64(key, (relabel ? 0x7e1abe1ull : 0ull) + (drop_tail ? 0x1000000000ull : 0ull));
     auto it = ctx->plans.find(key);
     if (it != ctx->plans.end()) {
         PlanEntry *e = it->second.get();
@@ -239,7 +241,7 @@ sv_status get_plan(DeviceCtx *ctx, const sv_circuit &c, int R, bool fuse, sv_dty
     std::unique_ptr<PlanEntry> e(new PlanEntry());
     std::string err;
     if (tile_bits > 0) {
-        err = plan_passes(c, tile_bits, coalesce, R, fuse, swz_bits(dt), &e->host, relabel);
+        err = plan_passes(c, tile_bits, coalesce, R, fuse, swz_bits(dt), &e->host, relabel, drop_tail);
         if (err.empty()) err = build_tile_passes(e->host, dt == SV_C128 ? 16 : 8, &e->tiles);
     } else {
         err = plan_circuit(c, R, fuse, swz_bits(dt), &e->host);
@@ -569,42 +571,53 @@ int h_tile_bits(int n, sv_dtype dt) {
     return n < t ? n : t;
 }
 
-// layout: qubit q in bit layout[q] of the amplitude index (states left
-// relabeled by tile passes), or null / empty for the identity; the terms'
-// masks are moved to those bits.
+// left (null: states in qubit order): the plan that left the states; its
+// trailing CNOTs are taken into the observable, whose terms' masks are then
+// moved to the index bits that hold the qubits.
 sv_status get_hplan(ObsEntry *obs, int n, sv_dtype dt, HPlanEntry **out,
-                    const std::vector<int> *layout = nullptr) {
+                    const HostProgram *left = nullptr) {
     const int t = h_tile_bits(n, dt);
-    std::vector<int> lay;
-    if (layout)
-        for (int q = 0; q < (int)layout->size(); ++q)
-            if ((*layout)[q] != q) {
-                lay = *layout;
+    std::vector<int> lay, key;
+    if (left)
+        for (int q = 0; q < (int)left->layout.size(); ++q)
+            if (left->layout[q] != q) {
+                lay = left->layout;
                 break;
             }
-    std::unique_ptr<HPlanEntry> &slot = obs->hplans[{t, lay}];
+    key = lay;
+    if (left && !left->tail.empty()) {
+        key.push_back(-1);
+        for (const auto &g : left->tail) {
+            key.push_back(g.first);
+            key.push_back(g.second);
+        }
+    }
+    std::unique_ptr<HPlanEntry> &slot = obs->hplans[{t, key}];
     if (!slot) {
         std::unique_ptr<HPlanEntry> e(new HPlanEntry());
         const HostObservable *ho = &obs->host;
         HostObservable moved;
-        if (!lay.empty()) {
+        if (!key.empty()) {
             auto move = [&](uint64_t m) {
+                if (lay.empty()) return m;
                 uint64_t r = 0;
                 for (int q = 0; q < n; ++q)
                     if ((m >> q) & 1ull) r |= 1ull << lay[q];
                 return r;
             };
-            std::vector<uint64_t> xm(obs->xm.size()), zm(obs->zm.size());
+            std::vector<uint64_t> xm(obs->xm), zm(obs->zm);
+            std::vector<double> cf(obs->c);
             for (size_t i = 0; i < xm.size(); ++i) {
-                xm[i] = move(obs->xm[i]);
-                zm[i] = move(obs->zm[i]);
+                cf[i] *= conjugate_by_cnots(left->tail, &xm[i], &zm[i]);
+                xm[i] = move(xm[i]);
+                zm[i] = move(zm[i]);
             }
             sv_pauli_sum h{};
             h.n_qubits = n;
             h.n_terms = (int32_t)xm.size();
             h.x_mask = xm.data();
             h.z_mask = zm.data();
-            h.coeff = obs->c.data();
+            h.coeff = cf.data();
             std::string err = plan_observable(h, n, swz_bits(dt), &moved);
             if (!err.empty()) return fail(SV_ERR_ARG, "observable: " + err);
             ho = &moved;
@@ -639,14 +652,14 @@ sv_status get_hplan(ObsEntry *obs, int n, sv_dtype dt, HPlanEntry **out,
 int64_t tile_blocks(const DeviceCtx *ctx, int64_t tiles);
 
 // E[r] = <psi_r|H|psi_r> for n_rows states (and lam = H psi unless lam is
-// null) by tile passes.  pair: the rows lie two to a state.
+// null) by tile passes.  pair: the rows lie two to a state.  zeroed: E is 0.
 sv_status h_tiles(DeviceCtx *ctx, ObsEntry *obs, int n, sv_dtype dt, int n_rows, const void *psi,
-                  void *lam, double *E, cudaStream_t st, const std::vector<int> *layout = nullptr,
-                  bool pair = false) {
+                  void *lam, double *E, cudaStream_t st, const HostProgram *left = nullptr,
+                  bool pair = false, bool zeroed = false) {
     HPlanEntry *hp = nullptr;
-    sv_status s = get_hplan(obs, n, dt, &hp, layout);
+    sv_status s = get_hplan(obs, n, dt, &hp, left);
     if (s != SV_OK) return s;
-    SV_CUDA(cudaMemsetAsync(E, 0, sizeof(double) * (size_t)n_rows, st));
+    if (!zeroed) SV_CUDA(cudaMemsetAsync(E, 0, sizeof(double) * (size_t)n_rows, st));
     const int n_states = pair ? (n_rows + 1) / 2 : n_rows;
     for (const HPass &P : hp->passes) {
         const int64_t tiles = (int64_t)n_states << P.n_tile_bits;
@@ -730,6 +743,40 @@ sv_status tile_cfg(int n, sv_dtype dt, const sv_plan_opts *o, TileCfg *cfg,
     return SV_OK;
 }
 
+// The tile plan of an energy or gradient problem.  A layered circuit ends in
+// CNOTs, which as passes only permute the states; they go into the
+// observable instead (a Pauli sum again, of wider strings) when that saves
+// more traffic than the H passes then add.  A plan whose tile_bits the caller
+// fixes (opts) keeps every gate in its passes.
+sv_status problem_plan(DeviceCtx *ctx, const sv_problem *p, const TileCfg &cfg, ObsEntry *obs,
+                       PlanEntry **out) {
+    const bool fuse = use_fusion(p->opts), relabel = use_relabel(p->opts);
+    sv_status s = get_plan(ctx, *p->circuit, cfg.R, fuse, p->dtype, out, cfg.t, cfg.c, relabel);
+    if (s != SV_OK || !relabel || (p->opts && p->opts->tile_bits > 0)) return s;
+    PlanEntry *cut = nullptr;
+    s = get_plan(ctx, *p->circuit, cfg.R, fuse, p->dtype, &cut, cfg.t, cfg.c, relabel, true);
+    if (s != SV_OK) return s;
+    const size_t np = (*out)->tiles.size(), nc = cut->tiles.size();
+    if (nc >= np || nc == 0) return SV_OK;
+    HPlanEntry *hw = nullptr, *hc = nullptr;
+    const int n = p->circuit->n_qubits;
+    s = get_hplan(obs, n, p->dtype, &hw, &(*out)->host);
+    if (s == SV_OK) s = get_hplan(obs, n, p->dtype, &hc, &cut->host);
+    if (s != SV_OK) return s;
+    // In bytes moved an amplitude (complex64): a pass 16 forward and 24 in
+    // reverse, an H pass 24, a group whose partners come from global memory 8.
+    // A row of Z masks is one multiply-add an amplitude: half a byte's time
+    // in FP32, that of 5 (of complex128's doubled bytes) in FP64.
+    auto cost = [&](const HPlanEntry *h, size_t passes) {
+        size_t far = 0;
+        for (const HGroup &g : h->host.groups) far += g.xfar != 0;
+        return 40.0 * passes + 24.0 * h->passes.size() + 8.0 * far +
+               (p->dtype == SV_C128 ? 5.0 : 0.5) * h->host.rows.size();
+    };
+    if (cost(hc, nc) < cost(hw, np)) *out = cut;
+    return SV_OK;
+}
+
 // Upper bound on the blocks of a tile-pass launch (the launcher caps it by
 // the kernel's occupancy): at most one block per tile.
 int64_t tile_blocks(const DeviceCtx *ctx, int64_t tiles) {
@@ -763,28 +810,27 @@ uint32_t sparse_plan(const PlanEntry *pe, uint32_t support, const int64_t *drefs
     return support;
 }
 
-// Where a slot source's reference indices lie behind the group matrices.
-int64_t *refs_of(void *mats, size_t n_states, int G, size_t csz) {
-    return (int64_t *)((char *)mats + n_states * G * kMatVals * csz);
-}
-size_t mats_bytes(size_t n_states, int G, size_t csz) {
-    return n_states * (G * kMatVals * csz + 2 * sizeof(int64_t));
+// Bytes of the group buffer (GroupBuf) of n_states states.
+size_t mats_bytes(const PlanEntry *pe, size_t n_states, size_t csz, bool pair) {
+    return group_buf(csz == 16, pe->dev, n_states, pair).bytes;
 }
 
 // Forward tile passes of `pe` over src.n_slots states from |ref>.  After pass
 // i with (i + 1) % every == 0 (and not the last pass) the states are written
 // to checkpoint (i + 1) / every - 1 of `ck`; outside the amplitudes that can
 // be nonzero a checkpoint holds anything.  The last pass's output in `states`
-// is whole.  refs: the instances' reference indices (pair: real slots two to
+// is whole.  clear: arrays zeroed before the first pass.  refs: the instances' reference indices (pair: real slots two to
 // a state).  mats: mats_bytes().
 sv_status tiles_forward(DeviceCtx *ctx, const PlanEntry *pe, int R, sv_dtype dt,
                         const SlotSource &src, const int64_t *refs, void *states, void *mats,
-                        void *ck, int every, cudaStream_t st, bool tc = false, bool pair = false) {
+                        void *ck, int every, cudaStream_t st, bool tc = false, bool pair = false,
+                        const ClearList &clear = ClearList{}) {
     const int c128 = dt == SV_C128, n = pe->n, G = pe->dev.n_groups;
     const int n_states = pair ? (src.n_slots + 1) / 2 : src.n_slots;
     const size_t csz = c128 ? 16 : 8, sbytes = ((size_t)n_states << n) * csz;
-    int64_t *drefs = refs_of(mats, n_states, G, csz);
-    cudaError_t e = launch_group_mats(c128, pe->dev, src, mats, drefs, st, pair);
+    const GroupBuf gb = group_buf(c128, pe->dev, (size_t)n_states, pair);
+    const int64_t *drefs = (const int64_t *)((char *)mats + gb.refs);
+    cudaError_t e = launch_group_mats(c128, pe->dev, src, mats, st, pair, clear);
     if (e != cudaSuccess) return cuda_fail(e, "group matrices");
     std::vector<TilePass> passes;
     std::vector<Sparse> sp;
@@ -802,6 +848,7 @@ sv_status tiles_forward(DeviceCtx *ctx, const PlanEntry *pe, int R, sv_dtype dt,
     // (out of place) and the next pass reads it from there: no copies.  The
     // last pass always writes `states`.
     const void *in = states;
+    int stage0 = 0;
     ctx->moved_fwd = 0;
     for (size_t i = 0; i < passes.size(); ++i) {
         const TilePass &tp = passes[i];
@@ -817,11 +864,12 @@ sv_status tiles_forward(DeviceCtx *ctx, const PlanEntry *pe, int R, sv_dtype dt,
             e = launch_tile_fwd_tc(tp, n, n_states, mats, G, out, tile_blocks(ctx, tiles), st, err, in);
             if (e != cudaSuccess) return cuda_fail(e, "forward tile pass (tensor cores)");
         } else {
-            e = launch_tile_fwd(c128, tp, n, n_states, mats, G, out, tile_blocks(ctx, tiles), st, in,
-                                pair, sp[i]);
+            e = launch_tile_fwd(c128, tp, n, n_states, group_mats_of(gb, mats, stage0), out,
+                                tile_blocks(ctx, tiles), st, in, pair, sp[i]);
             if (e != cudaSuccess) return cuda_fail(e, "forward tile pass");
         }
         const int64_t moved = (tiles << tp.t) * (int64_t)csz;
+        stage0 += tp.n_stages;
         ctx->moved_fwd += moved + (sp[i].init ? 0 : moved >> __builtin_popcount(sp[i].zero));
         in = out;
     }
@@ -837,20 +885,19 @@ sv_status tiles_energies(DeviceCtx *ctx, const sv_problem *p, const double *thet
     TileCfg cfg{};
     sv_status s = tile_cfg(n, dt, p->opts, &cfg, find_tuned(ctx, p, kTileEnergyKey, p->n_instances));
     if (s != SV_OK) return s;
-    PlanEntry *pe = nullptr;
-    s = get_plan(ctx, *p->circuit, cfg.R, use_fusion(p->opts), dt, &pe, cfg.t, cfg.c,
-                 use_relabel(p->opts));
-    if (s != SV_OK) return s;
     ObsEntry *obs = nullptr;
     s = get_obs(ctx, *p->observable, n, dt, &obs, st);
+    if (s != SV_OK) return s;
+    PlanEntry *pe = nullptr;
+    s = problem_plan(ctx, p, cfg, obs, &pe);
     if (s != SV_OK) return s;
     const void *drefs = nullptr;
     s = get_array(ctx, p->refs, sizeof(int64_t) * I, &drefs);
     if (s != SV_OK) return s;
     const size_t csz = c128 ? 16 : 8, sb = csz << n;
-    const size_t mb = mats_bytes(1, pe->dev.n_groups, csz);
-    const size_t per = sb + mb;
     const bool pair = real_pairs(pe, obs, n_slots, cfg.tc);
+    const size_t mb = mats_bytes(pe, 1, csz, pair);
+    const size_t per = sb + mb;
     const int per_state = pair ? 2 : 1;  // slots
     int64_t chunk = (int64_t)(big_budget(ctx, st) / (per + 512));  // states
     if (chunk < 1) return fail(SV_ERR_OOM, "one state does not fit in free device memory");
@@ -871,9 +918,9 @@ sv_status tiles_energies(DeviceCtx *ctx, const sv_problem *p, const double *thet
         src.input_stride = p->input_stride;
         src.slot_base = slot_begin + (int)c0;
         s = tiles_forward(ctx, pe, cfg.R, dt, src, p->refs, big, (char *)big + mats_off, nullptr, 0, st,
-                          cfg.tc, pair);
+                          cfg.tc, pair, ClearList{{E + c0}, {src.n_slots}});
         if (s != SV_OK) return s;
-        s = h_tiles(ctx, obs, n, dt, src.n_slots, big, nullptr, E + c0, st, &pe->host.layout, pair);
+        s = h_tiles(ctx, obs, n, dt, src.n_slots, big, nullptr, E + c0, st, &pe->host, pair, true);
         if (s != SV_OK) return s;
     }
     return SV_OK;
@@ -891,7 +938,7 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     ctx->phase_used = 0;
     ctx->last_every = 0;
     ctx->last_rev_bytes = 0;
-    ctx->last_states = 0;
+    ctx->last_states = ctx->last_passes = 0;
     const sv_dtype dt = p->dtype;
     const int c128 = dt == SV_C128, n = p->circuit->n_qubits, I = p->n_instances;
     const int P = p->circuit->n_params, Pp = P > 0 ? P : 1;
@@ -900,8 +947,14 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     if (s != SV_OK) return s;
     if (forced) cfg = *forced;
     PlanEntry *pe = nullptr;
-    s = get_plan(ctx, *p->circuit, cfg.R, use_fusion(p->opts), dt, &pe, cfg.t, cfg.c,
-                 use_relabel(p->opts));
+    ObsEntry *obs = nullptr;
+    if (ddcl_target) {
+        s = get_plan(ctx, *p->circuit, cfg.R, use_fusion(p->opts), dt, &pe, cfg.t, cfg.c,
+                     use_relabel(p->opts));
+    } else {
+        s = get_obs(ctx, *p->observable, n, dt, &obs, st);
+        if (s == SV_OK) s = problem_plan(ctx, p, cfg, obs, &pe);
+    }
     if (s != SV_OK) return s;
     if (ddcl_target) {
         // The passes leave qubit q in index bit layout[q]: rewrite the target
@@ -928,11 +981,6 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
             ddcl_target = (const double *)buf->ptr;
         }
     }
-    ObsEntry *obs = nullptr;
-    if (!ddcl_target) {
-        s = get_obs(ctx, *p->observable, n, dt, &obs, st);
-        if (s != SV_OK) return s;
-    }
     const void *drefs = nullptr;
     s = get_array(ctx, p->refs, sizeof(int64_t) * I, &drefs);
     if (s != SV_OK) return s;
@@ -945,7 +993,7 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     const int n_states = (I + per_state - 1) / per_state;
     auto bytes_per_state = [&](int ev) {
         const size_t ncp_ = npass > 1 ? (size_t)((npass - 1) / ev) : 0;
-        return (2 + ncp_) * sb + mats_bytes(1, G, csz) + (size_t)per_state * G * 64;
+        return (2 + ncp_) * sb + mats_bytes(pe, 1, csz, pair) + (size_t)per_state * G * 64;
     };
     if (every <= 0) {
         // The most stored states that still let every instance run at once:
@@ -968,7 +1016,7 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
     const size_t o_lam = up((size_t)chunk * sb), o_ck = o_lam + up((size_t)chunk * sb);
     const size_t o_mats = o_ck + up((size_t)ncp * chunk * sb);
-    const size_t o_rho = o_mats + up(mats_bytes((size_t)chunk, G, csz));
+    const size_t o_rho = o_mats + up(mats_bytes(pe, (size_t)chunk, csz, pair));
     const size_t total = o_rho + up((size_t)chunk * per_state * G * 64);
     void *big = nullptr;
     s = get_big_scratch(ctx, st, total, &big);
@@ -978,9 +1026,9 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     s = get_scratch(ctx, st, sizeof(double) * ((size_t)I * Pp + I), &scr);
     if (s != SV_OK) return s;
     double *Gs = (double *)scr, *Es = Gs + (size_t)I * Pp;
-    SV_CUDA(cudaMemsetAsync(Gs, 0, sizeof(double) * (size_t)I * Pp, st));
     const CostSource cs = cost_of(p, weights);
     ctx->last_states = n_states;
+    ctx->last_passes = npass;
     int64_t moved_fwd = 0;
     ctx->moved_rev = 0;
     for (int64_t c0 = 0; c0 < I; c0 += chunk * per_state) {
@@ -998,25 +1046,29 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
         void *psi = bb, *lam = bb + o_lam, *ck = bb + o_ck, *mats = bb + o_mats;
         double *rho = (double *)(bb + o_rho);
         phase_mark(ctx, st);
+        // this group's energies, per-slot gradients and reduced matrices
+        const ClearList clear{{Es + c0, Gs + (size_t)c0 * Pp, rho},
+                              {src.n_slots, (int64_t)src.n_slots * Pp, (int64_t)states * per_state * G * 8}};
         s = tiles_forward(ctx, pe, cfg.R, dt, src, p->refs, psi, mats, ncp ? ck : nullptr, every, st,
-                          cfg.tc, pair);
+                          cfg.tc, pair, clear);
         if (s != SV_OK) return s;
         moved_fwd += ctx->moved_fwd;
         std::vector<TilePass> passes;
         std::vector<Sparse> sp;
+        const GroupBuf gb = group_buf(c128, pe->dev, (size_t)states, pair);
         sparse_plan(pe, pair ? pair_support(src, p->refs) : 0u,
-                    refs_of(mats, (size_t)states, G, csz), &passes, &sp);
+                    (const int64_t *)((char *)mats + gb.refs), &passes, &sp);
+        int stage0 = pe->dev.n_stages;
         phase_mark(ctx, st);
         cudaError_t e = cudaSuccess;
         if (ddcl_target) {
             e = launch_ddcl_lambda(c128, n, src.n_slots, psi, ddcl_target, lam, Es + c0, st);
             if (e != cudaSuccess) return cuda_fail(e, "JS divergence and its lambda");
         } else {
-            s = h_tiles(ctx, obs, n, dt, src.n_slots, psi, lam, Es + c0, st, &pe->host.layout, pair);
+            s = h_tiles(ctx, obs, n, dt, src.n_slots, psi, lam, Es + c0, st, &pe->host, pair, true);
             if (s != SV_OK) return s;
         }
         phase_mark(ctx, st);
-        SV_CUDA(cudaMemsetAsync(rho, 0, (size_t)states * per_state * G * 64, st));
         for (int i = npass - 1; i >= 0; --i) {
             // restart psi from the stored forward state after pass i: the
             // reverse pass reads it there and writes psi (no copy)
@@ -1030,7 +1082,8 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
             // psi after this pass is needed only if the next reverse pass
             // un-computes from it (it restarts from a stored state otherwise)
             const bool write_psi = i > 0 && !(i % every == 0 && i < npass);
-            e = launch_tile_rev(c128, tp, n, states, mats, G, psi, lam, rho,
+            stage0 -= tp.n_stages;
+            e = launch_tile_rev(c128, tp, n, states, group_mats_of(gb, mats, stage0), psi, lam, rho,
                                 tile_blocks(ctx, tiles), st, psi_in, write_psi, pair, sp[i]);
             if (e != cudaSuccess) return cuda_fail(e, "reverse tile pass");
             ctx->moved_rev += (tiles << tp.t) * (int64_t)csz * (write_psi ? 4 : 3);
@@ -1082,8 +1135,7 @@ sv_status multi_sequence(DeviceCtx *ctx, std::vector<MultiProblem> &mp, sv_dtype
     if (!err) return fail(SV_ERR_CUDA, "device error word");
     for (MultiProblem &m : mp) {
         m.src.theta = theta[&m - &mp[0]];
-        cudaError_t e = launch_group_mats(c128, m.pe->dev, m.src, base + m.o_mats,
-                                          refs_of(base + m.o_mats, m.I, m.G, c128 ? 16 : 8), st);
+        cudaError_t e = launch_group_mats(c128, m.pe->dev, m.src, base + m.o_mats, st);
         if (e == cudaSuccess) e = launch_init_states(c128, base + m.o_psi, m.n, m.src, st);
         if (e != cudaSuccess) return cuda_fail(e, "uneven batch: group matrices / init");
     }
@@ -1092,7 +1144,7 @@ sv_status multi_sequence(DeviceCtx *ctx, std::vector<MultiProblem> &mp, sv_dtype
         if (rev) {  // between the sweeps: lambda = H psi, cleared sums
             for (MultiProblem &m : mp) {
                 sv_status s = h_tiles(ctx, m.obs, m.n, dt, m.I, base + m.o_psi, base + m.o_lam,
-                                      (double *)(base + m.o_E), st, &m.pe->host.layout);
+                                      (double *)(base + m.o_E), st, &m.pe->host);
                 if (s != SV_OK) return s;
                 SV_CUDA(cudaMemsetAsync(base + m.o_rho, 0, (size_t)m.I * m.G * 64, st));
                 SV_CUDA(cudaMemsetAsync(base + m.o_G, 0, sizeof(double) * (size_t)m.I * (m.P > 0 ? m.P : 1), st));
@@ -1178,12 +1230,11 @@ sv_status multi_adjoint(DeviceCtx *ctx, const sv_problem *problems, int np,
         m.n = m.p->circuit->n_qubits;
         m.I = m.p->n_instances;
         m.P = m.p->circuit->n_params;
-        sv_status s = get_plan(ctx, *m.p->circuit, cfg.R, use_fusion(m.p->opts), dt, &m.pe, cfg.t,
-                               cfg.c, use_relabel(m.p->opts));
-        if (s == SV_OK) s = get_obs(ctx, *m.p->observable, m.n, dt, &m.obs, st);
+        sv_status s = get_obs(ctx, *m.p->observable, m.n, dt, &m.obs, st);
+        if (s == SV_OK) s = problem_plan(ctx, m.p, cfg, m.obs, &m.pe);
         if (s == SV_OK) s = get_array(ctx, m.p->refs, sizeof(int64_t) * m.I, &m.drefs);
         HPlanEntry *hp = nullptr;
-        if (s == SV_OK) s = get_hplan(m.obs, m.n, dt, &hp, &m.pe->host.layout);
+        if (s == SV_OK) s = get_hplan(m.obs, m.n, dt, &hp, &m.pe->host);
         if (s != SV_OK) return s;
         m.G = m.pe->dev.n_groups;
         m.npass = (int)m.pe->tiles.size();
@@ -1198,7 +1249,7 @@ sv_status multi_adjoint(DeviceCtx *ctx, const sv_problem *problems, int np,
         m.o_tp = take(sizeof(TilePass) * (size_t)m.npass);
         m.o_psi = take(((size_t)m.I << m.n) * csz);
         m.o_lam = take(((size_t)m.I << m.n) * csz);
-        m.o_mats = take(mats_bytes(m.I, m.G, csz));
+        m.o_mats = take(mats_bytes(m.pe, m.I, csz, false));
         m.o_rho = take((size_t)m.I * m.G * 64);
         m.o_E = take(sizeof(double) * (size_t)m.I);
         m.o_G = take(sizeof(double) * (size_t)m.I * (m.P > 0 ? m.P : 1));
@@ -1267,9 +1318,16 @@ sv_status multi_adjoint(DeviceCtx *ctx, const sv_problem *problems, int np,
             const MultiProblem &m = mp[who[rev][i].first];
             SweepTask &T = tasks[rev][i];
             T.P = (const TilePass *)(base + m.o_tp) + who[rev][i].second;
-            T.refs = refs_of(base + m.o_mats, m.I, m.G, csz);
-            T.fixed = m.sparse[who[rev][i].second].fixed;
-            T.mats = base + m.o_mats;
+            const GroupBuf gb = group_buf(c128, m.pe->dev, m.I, false);
+            const int pi = who[rev][i].second;
+            T.refs = (const int64_t *)(base + m.o_mats + gb.refs);
+            T.fixed = m.sparse[pi].fixed;
+            for (int k = 0; k < pi; ++k) T.stage0 += m.tiles[k].n_stages;
+            const GroupMats gm = group_mats_of(gb, base + m.o_mats, T.stage0);
+            T.mats = gm.mats;
+            T.tabs = gm.tabs;
+            T.split = gm.split;
+            T.n_stages = gm.n_stages;
             T.psi = base + m.o_psi;
             T.lam = base + m.o_lam;
             T.rho = (double *)(base + m.o_rho);
@@ -1443,7 +1501,7 @@ sv_status sv_apply_circuit_batch(sv_state state, const sv_circuit *circuits, int
             if (s != SV_OK) return s;
             const size_t csz = state->dtype == SV_C128 ? 16 : 8;
             void *mats = nullptr;
-            s = get_big_scratch(ctx, st, mats_bytes(sub.size(), pe->dev.n_groups, csz) + 256, &mats);
+            s = get_big_scratch(ctx, st, mats_bytes(pe, sub.size(), csz, false) + 256, &mats);
             if (s != SV_OK) return s;
             SlotSource src{};
             src.mode = SLOTS_EXPLICIT;
@@ -1864,7 +1922,7 @@ sv_status adjoint_locked(DeviceCtx *ctx, const sv_problem *p, const double *thet
     const int P = p->circuit->n_params, I = p->n_instances;
     ctx->last_every = 0;  // on chip unless the tile path records its own
     ctx->last_rev_bytes = 0;
-    ctx->last_states = 0;
+    ctx->last_states = ctx->last_passes = 0;
     if (wants_tiles(p->circuit->n_qubits, p->dtype, p->opts))
         return tiles_adjoint(ctx, p, theta, weights, energy_out, loss_out, grad_out,
                              checkpoint_every, st);
@@ -2037,7 +2095,7 @@ sv_status sv_grad_ddcl_param_shift(const sv_problem *p, const double *theta,
     if (s != SV_OK) return s;
     double *E = (double *)scr, *lp = E + B, *D = lp + 1;
     const size_t csz = c128 ? 16 : 8, sb = csz << n;
-    const size_t mb = mats_bytes(1, pe->dev.n_groups, csz);
+    const size_t mb = mats_bytes(pe, 1, csz, false);
     int64_t chunk = (int64_t)(big_budget(ctx, st) / (sb + mb + 512));
     if (chunk < 1) return fail(SV_ERR_OOM, "one state does not fit in free device memory");
     if (chunk > B) chunk = B;
@@ -2464,11 +2522,13 @@ sv_status sv_last_adjoint_info(int32_t *checkpoint_every, int64_t *reverse_bytes
     return SV_OK;
 }
 
-sv_status sv_last_adjoint_states(int32_t *states, int64_t *forward_bytes, int64_t *reverse_bytes) {
+sv_status sv_last_adjoint_states(int32_t *states, int32_t *passes, int64_t *forward_bytes,
+                                 int64_t *reverse_bytes) {
     DeviceCtx *ctx = context();
     if (!ctx) return fail(SV_ERR_CUDA, "no CUDA device");
     std::lock_guard<std::mutex> lk(ctx->mu);
     if (states) *states = ctx->last_states;
+    if (passes) *passes = ctx->last_passes;
     if (forward_bytes) *forward_bytes = ctx->moved_fwd;
     if (reverse_bytes) *reverse_bytes = ctx->moved_rev;
     return SV_OK;

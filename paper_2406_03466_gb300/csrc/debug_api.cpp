@@ -82,6 +82,33 @@ sv_status sv_debug_tile_passes(const sv_circuit *c, int32_t tile_bits, int32_t r
     return SV_OK;
 }
 
+sv_status sv_debug_drop_tail(const sv_circuit *c, int32_t tile_bits, int32_t reg_bits,
+                             int32_t dtype, int32_t *n_passes, int32_t *n_tail, int32_t *tail,
+                             int32_t *layout) {
+    if (!c || !n_passes || !n_tail || !tail) return SV_ERR_ARG;
+    const int w = dtype == SV_C128 ? 3 : 4;
+    HostProgram h;
+    if (!plan_passes(*c, tile_bits, w, reg_bits, true, w, &h, true, true).empty()) return SV_ERR_ARG;
+    *n_passes = (int32_t)h.passes.size();
+    *n_tail = (int32_t)h.tail.size();
+    for (size_t i = 0; i < h.tail.size(); ++i) {
+        tail[2 * i] = h.tail[i].first;
+        tail[2 * i + 1] = h.tail[i].second;
+    }
+    if (layout)
+        for (size_t q = 0; q < h.layout.size(); ++q) layout[q] = h.layout[q];
+    return SV_OK;
+}
+
+sv_status sv_debug_conjugate(const int32_t *tail, int32_t n_tail, int32_t n_terms, uint64_t *x,
+                             uint64_t *z, int32_t *sign) {
+    if (!tail || !x || !z || !sign) return SV_ERR_ARG;
+    std::vector<std::pair<int, int>> t;
+    for (int i = 0; i < n_tail; ++i) t.push_back({tail[2 * i], tail[2 * i + 1]});
+    for (int i = 0; i < n_terms; ++i) sign[i] = conjugate_by_cnots(t, &x[i], &z[i]);
+    return SV_OK;
+}
+
 sv_status sv_debug_h_passes(const sv_pauli_sum *h, int32_t tile_bits, int32_t coalesce_bits,
                             int32_t *counts, void *passes, void *groups, void *classes,
                             void *terms, void *rows) {

@@ -82,6 +82,37 @@ __device__ __forceinline__ C mad2(const C m, const C x, const C k, const C y) {
     return r;
 }
 
+// Programmatic dependent launch: a kernel launched behind another one
+// (launch_dep) may be scheduled once every block of that one has called
+// pdl_trigger or ended; pdl_wait returns when that grid is complete and its
+// writes are visible.  Every kernel launched so calls pdl_wait in every
+// thread before its first access to memory the stream's earlier work touches.
+__device__ __forceinline__ void pdl_trigger() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_dep_if(bool dep, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                          cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = dep ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_dep(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                       cudaStream_t st, Args... args) {
+    return launch_dep_if(true, kernel, grid, block, smem, st, args...);
+}
+
 // ------------------------------------------------------------------ slots
 
 struct SlotInfo {

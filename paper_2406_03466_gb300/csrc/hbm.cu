@@ -20,6 +20,7 @@
 #include <mutex>
 #include <type_traits>
 #include <utility>
+#include <vector>
 
 #include "engine.cuh"
 #include "hbm.h"
@@ -35,37 +36,240 @@ namespace {
 // Every pass then moves and multiplies half as much per circuit; the matrices
 // stay per circuit (packed FMAs take one per component).
 
-// Fused 2x2 matrices of every group for every slot: out[slot][group][4], or
-// with pair out[slot pair][group][4], entry k = (first slot's, second slot's).
-// Without pair the groups' split forms follow, [slot][group][4].
-// Formed in FP64 and rounded once, so that a pass's error is its own.  A
-// pair's real rotations come with c >= 0 (a state's sign is of no account
-// to its energy and its gradient), for the shear form.
-template <typename Real>
-__global__ void k_group_mats(Program p, SlotSource src, int pair, typename CT<Real>::T *out,
-                             int64_t *refs) {
-    using C = typename CT<Real>::T;
-    const int G = p.n_groups, n_states = pair ? (src.n_slots + 1) / 2 : src.n_slots;
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < 2 * n_states; b += gridDim.x * blockDim.x)
-        refs[b] = resolve(src, pair ? min(b, src.n_slots - 1) : b >> 1).ref;
-    const int64_t total = (int64_t)n_states * G;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int b = (int)(i / G), g = (int)(i % G);
-        C m[4];
-        for (int c = 0; c < (pair ? 2 : 1); ++c) {
-            const SlotInfo si = resolve(src, pair ? min(2 * b + c, src.n_slots - 1) : b);
-            double2 d[4];
-            group_matrix<double, double2, Real>(p, g, si, d);
-            if (!pair) split_form(d, out + (size_t)(total + i) * 4);
-            const double sg = d[0].x < 0.0 && d[0].x == d[3].x && d[1].x == -d[2].x ? -1.0 : 1.0;
-            for (int k = 0; k < 4; ++k) {
-                if (!pair) m[k] = cmk<C>(d[k].x, d[k].y);
-                else if (c == 0) m[k].x = (Real)(sg * d[k].x);
-                else m[k].y = (Real)(sg * d[k].x);
+// Group matrices of complex64 problems need more than FP32 (a matrix entry's
+// rounding acts on a whole state) but not FP64 to the last bit, and GB300 does
+// 2 FP64 multiply-adds a clock and SM: sines by argument reduction to a table
+// of step pi / 64 and a short Taylor polynomial in the remainder (Tang's
+// table-driven method, ACM TOMS 15(2), 1989), inverse roots by one Newton
+// step from the FP32 ones.  Errors below 1e-10; with the library's
+// FP64 functions the kernel took 15-20 us where this takes 4.
+__device__ const double kSinTab[33] = {  // sin(j pi / 64)
+    0.0, 0.049067674327418015, 0.0980171403295606, 0.14673047445536175,
+    0.19509032201612828, 0.2429801799032639, 0.2902846772544624, 0.33688985339222005,
+    0.3826834323650898, 0.4275550934302821, 0.47139673682599764, 0.5141027441932218,
+    0.5555702330196022, 0.5956993044924334, 0.6343932841636455, 0.6715589548470184,
+    0.7071067811865476, 0.7409511253549591, 0.773010453362737, 0.8032075314806449,
+    0.8314696123025452, 0.8577286100002721, 0.881921264348355, 0.9039892931234433,
+    0.9238795325112867, 0.9415440651830208, 0.9569403357322088, 0.970031253194544,
+    0.9807852804032304, 0.989176509964781, 0.9951847266721969, 0.9987954562051724,
+    1.0};
+
+__device__ __forceinline__ void quick_sincos(double h, double *s, double *c) {
+    if (!(fabs(h) < 1e6)) {
+        sincos(h, s, c);
+        return;
+    }
+    const double kf = rint(h * 20.371832715762604);
+    const double r = fma(kf, -1.9135106236677394e-18, fma(kf, -0.04908738521234052, h));
+    const int k = (int)kf & 127, j = k & 31;
+    const double sj = __ldg(kSinTab + j), cj = __ldg(kSinTab + 32 - j);
+    const double S = (k & 32) ? cj : sj, C = (k & 32) ? -sj : cj;
+    const float rf = (float)r, z = rf * rf;
+    const double sr = r + (double)(rf * z * (-1.f / 6.f + z * (1.f / 120.f)));  // sin r
+    const double cr = (double)(z * (-0.5f + z * (1.f / 24.f)));                 // cos r - 1
+    const double sn = S + fma(S, cr, C * sr), cs = C + fma(C, cr, -S * sr);
+    *s = (k & 64) ? -sn : sn;
+    *c = (k & 64) ? -cs : cs;
+}
+
+__device__ __forceinline__ double quick_rsqrt(double x) {
+    const double y = (double)rsqrtf((float)x);
+    return y * fma(-0.5 * x * y, y, 1.5);
+}
+// sqrt of x >= 0 (NaN below).
+__device__ __forceinline__ double quick_sqrt(double x) {
+    return x < 1e-30 && x >= 0.0 ? 0.0 : x * quick_rsqrt(x);
+}
+
+// Axis (M_RX, M_RY, M_RZ) and half-angle sine and cosine of one member; -1
+// when it is neither a rotation nor an encoding.
+__device__ int quick_member(const Member &mb, const SlotInfo &si, double &s, double &c) {
+    if (mb.kind <= M_RZ) {
+        double t = mb.angle;
+        if (mb.param >= 0)
+            t = si.theta[mb.param] + (mb.param == si.shift_param ? si.shift : 0.0);
+        quick_sincos(0.5 * t, &s, &c);
+        return mb.kind;
+    }
+    if (mb.kind == M_ENC_RY_ASIN) {  // the half angles of member_matrix
+        const double x = enc_input<float>(si.x[mb.param]);
+        const double h = 0.5 * (1.0 + quick_sqrt((1.0 - x) * (1.0 + x))), rh = quick_rsqrt(h);
+        c = h * rh;
+        s = 0.5 * x * rh;
+        return M_RY;
+    }
+    if (mb.kind == M_ENC_RZ_ACOS_SQ) {
+        const double x = enc_input<float>(si.x[mb.param]), u = x * x;
+        c = quick_sqrt(0.5 * (1.0 + u));
+        s = quick_sqrt(0.5 * (1.0 - u));
+        return M_RZ;
+    }
+    return -1;
+}
+
+// The first column (a, b) of group g's matrix [[a, -conj(b)], [b, conj(a)]]
+// when its members are rotations and encodings only; false otherwise.  L
+// lanes (consecutive, all with the same g) share a group: each forms every
+// L-th member, so a group's loads and sines are in flight together; all
+// multiply them.  Called by whole warps.
+template <int L>
+__device__ bool quick_group(const Program &p, int g, const SlotInfo &si, double2 &a, double2 &b) {
+    const Group grp = p.groups[g];
+    const int lane = threadIdx.x & (L - 1);
+    a = make_double2(1.0, 0.0);
+    b = make_double2(0.0, 0.0);
+    int last = grp.m_end - grp.m_begin;  // the longest group of the warp
+    for (int off = 16; off; off >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, off));
+    bool ok = true;
+    for (int m0 = 0; m0 < last; m0 += L) {
+        double ms = 0.0, mc = 1.0;
+        int ax = M_RZ;  // past the end: the identity
+        if (grp.m_begin + m0 + lane < grp.m_end)
+            ax = quick_member(p.members[grp.m_begin + m0 + lane], si, ms, mc);
+#pragma unroll
+        for (int l = 0; l < L; ++l) {
+            const int axis = L > 1 ? __shfl_sync(0xffffffffu, ax, l, L) : ax;
+            const double s = L > 1 ? __shfl_sync(0xffffffffu, ms, l, L) : ms;
+            const double c = L > 1 ? __shfl_sync(0xffffffffu, mc, l, L) : mc;
+            ok = ok && axis >= 0;
+            double2 na, nb;
+            if (axis == M_RX) {  // (c a - i s b, c b - i s a)
+                na = make_double2(fma(s, b.y, c * a.x), fma(-s, b.x, c * a.y));
+                nb = make_double2(fma(s, a.y, c * b.x), fma(-s, a.x, c * b.y));
+            } else if (axis == M_RY) {  // (c a - s b, c b + s a)
+                na = make_double2(fma(-s, b.x, c * a.x), fma(-s, b.y, c * a.y));
+                nb = make_double2(fma(s, a.x, c * b.x), fma(s, a.y, c * b.y));
+            } else {  // ((c - i s) a, (c + i s) b)
+                na = make_double2(fma(s, a.y, c * a.x), fma(-s, a.x, c * a.y));
+                nb = make_double2(fma(-s, b.y, c * b.x), fma(s, b.x, c * b.y));
             }
+            a = na;
+            b = nb;
         }
-        for (int k = 0; k < 4; ++k) out[(size_t)i * 4 + k] = m[k];
+    }
+    return ok;
+}
+
+// split_form of [[a, -conj(b)], [b, conj(a)]]: there q = conj(p0 p1).
+__device__ __forceinline__ void quick_split(double2 a, double2 b, double2 *out) {
+    const double c2 = fma(a.x, a.x, a.y * a.y), s2 = fma(b.x, b.x, b.y * b.y);
+    double2 p0 = make_double2(1.0, 0.0), p1 = p0;
+    double c = 0.0, s = 0.0;
+    if (!(c2 < 1e-30)) {
+        const double r = quick_rsqrt(c2);
+        c = c2 * r;
+        p0 = make_double2(a.x * r, a.y * r);
+    }
+    if (!(s2 < 1e-30)) {
+        const double r = quick_rsqrt(s2);
+        s = s2 * r;
+        p1 = make_double2(b.x * r, b.y * r);
+    }
+    const double d = 1.0 + c, y = (double)(1.f / (float)d);  // 1 / d by one Newton step
+    out[0] = make_double2(-s * (y * fma(-d, y, 2.0)), s);
+    out[1] = p0;
+    out[2] = p1;
+    out[3] = cconj(cmul(p0, p1));
+}
+
+// What the passes read of every state's groups (hbm.h: GroupBuf): the fused
+// 2x2 matrices and, without pair, their split forms; with pair entry k is
+// (first slot's, second slot's), and where both matrices are rotations their
+// shears alpha, beta stand in entries 0 and 1 (zeros in 2 and 3).  Formed in
+// FP64 and rounded once, so that a pass's error is its own.  A pair's real
+// rotations are taken with c >= 0 (a state's sign is of no account to its
+// energy and its gradient).
+// L lanes per group (complex64).
+template <typename Real, int L>
+__global__ void __launch_bounds__(32)
+k_group_mats(Program p, SlotSource src, int pair, typename CT<Real>::T *out, double2 *split,
+             int64_t *refs, ClearList clear) {
+    using C = typename CT<Real>::T;
+    constexpr bool kQuick = std::is_same<Real, float>::value;
+    pdl_trigger();
+    pdl_wait();
+    const int G = p.n_groups, n_states = pair ? (src.n_slots + 1) / 2 : src.n_slots;
+    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t b = tid; b < 2 * n_states; b += step)
+        refs[b] = resolve(src, pair ? min((int)b, src.n_slots - 1) : (int)b >> 1).ref;
+    for (int k = 0; k < 3; ++k)
+        for (int64_t x = tid; x < clear.n[k]; x += step) clear.p[k][x] = 0.0;
+    const int64_t total = (int64_t)n_states * G;
+    // whole warps: the quick groups shuffle
+    for (int64_t x = tid; (x & ~31ll) < total * L; x += step) {
+        const int64_t i = min(x / L, total - 1);
+        const int b = (int)(i / G), g = (int)(i % G);
+        double2 d[4], u, v;
+        C m[4];
+        if (!pair) {
+            const SlotInfo si = resolve(src, b);
+            if (kQuick && quick_group<L>(p, g, si, u, v)) {
+                d[0] = u;
+                d[1] = make_double2(-v.x, v.y);
+                d[2] = v;
+                d[3] = cconj(u);
+                quick_split(u, v, split + i * 4);
+            } else {
+                group_matrix<double, double2, Real>(p, g, si, d);
+                split_form(d, split + i * 4);
+            }
+            for (int k = 0; k < 4; ++k) m[k] = cmk<C>(d[k].x, d[k].y);
+        } else {
+            double r[2][4];
+            bool rot = true;
+            for (int c = 0; c < 2; ++c) {
+                const SlotInfo si = resolve(src, min(2 * b + c, src.n_slots - 1));
+                if (kQuick && quick_group<L>(p, g, si, u, v)) {
+                    r[c][0] = r[c][3] = u.x;
+                    r[c][1] = -v.x;
+                    r[c][2] = v.x;
+                } else {
+                    group_matrix<double, double2, Real>(p, g, si, d);
+                    for (int k = 0; k < 4; ++k) r[c][k] = d[k].x;
+                }
+                rot = rot && r[c][0] == r[c][3] && r[c][1] == -r[c][2];
+            }
+            for (int c = 0; c < 2 && rot; ++c) {
+                const double sg = r[c][0] < 0.0 ? -1.0 : 1.0, s = sg * r[c][2];
+                r[c][0] = -s / (1.0 + sg * r[c][0]);
+                r[c][1] = s;
+                r[c][2] = r[c][3] = 0.0;
+            }
+            for (int k = 0; k < 4; ++k) m[k] = cmk<C>(r[0][k], r[1][k]);
+        }
+        if (x == i * L)  // one lane of the group writes
+            for (int k = 0; k < 4; ++k) out[i * 4 + k] = m[k];
+    }
+}
+
+// Phase tables of the split stages, tabs[state][stage][0][r] = product of
+// the groups' q and tabs[state][stage][1][r] = product of their p over the
+// stage's register bits.  Products in FP64: a table entry multiplies whole
+// slices of a state, so its rounding does not average out.
+template <typename Real>
+__global__ void k_phase_tables(Program p, int n_states, const double2 *split,
+                               typename CT<Real>::T *tabs) {
+    pdl_trigger();
+    pdl_wait();
+    const int NA = 1 << p.R;
+    const int64_t total = (int64_t)n_states * p.n_stages * 2 * NA;
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < total;
+         x += (int64_t)gridDim.x * blockDim.x) {
+        const int r = (int)(x & (NA - 1)), post = (int)(x >> p.R) & 1;
+        const int64_t ss = x >> (p.R + 1);
+        const Stage *sg = p.stages + ss % p.n_stages;
+        const double2 *e = split + ss / p.n_stages * p.n_groups * 4;
+        double2 f = make_double2(1.0, 0.0);
+        bool real = true;
+        for (int o = sg->op_begin; o < sg->op_end; ++o) {
+            const Op op = p.ops[o];
+            real = real && p.groups[op.group].real;
+            const int b = (r >> op.a) & 1;
+            if (post) f = cmul(f, e[op.group * 4 + 1 + b]);
+            else if (b) f = cmul(f, e[op.group * 4 + 3]);
+        }
+        if (!real && sg->op_end - sg->op_begin >= 2) tabs[x] = cmk<typename CT<Real>::T>(f.x, f.y);
     }
 }
 
@@ -110,52 +314,67 @@ __device__ __forceinline__ void stage_ops_fwd(uint32_t ops, uint32_t flags, cons
 }
 
 // Stages slot's matrices of the pass in shared memory (the reverse's
-// transposed and conjugated): split forms and phase tables for split stages,
-// shear forms for real rotations elsewhere, and the stage flags.  Called by
-// every thread at a slot's first tile, once the previous tile's stages are
-// past their last barrier; visible after the next barrier.
+// transposed and conjugated): (alpha, beta) and p0 conj(p1) of a split
+// stage's groups and its phase tables, shear forms for real rotations
+// elsewhere, and the stage flags.  Called by every thread at a slot's first
+// tile, once the previous tile's stages are past their last barrier; visible
+// after the next barrier.
 template <typename C, int R, int kMat, bool kRev>
-__device__ __forceinline__ void stage_mats(const TilePass &P, uint4 *rec, int n_slots,
-                                           const C *mats, int G, int slot, C *sm, C *tab) {
+__device__ __forceinline__ void stage_mats(const TilePass &P, uint4 *rec, const GroupMats &gm,
+                                           int slot, C *sm, C *tab) {
+    constexpr int NA = 1 << R;
     const int tid = threadIdx.x, T = blockDim.x;
+    const C *mats = (const C *)gm.mats + (size_t)slot * gm.G * 4;
     __syncthreads();  // the stage records (first slot)
     for (int x = tid; x < P.n_stages * R * 4; x += T) {
         const int s = x / (R * 4), i = (x >> 2) % R, e = x & 3;
         const int u = (int)((rec[2 * s].x >> (8 * i)) & 63u) - 1;
         if (u < 0) continue;
-        const C *m = mats + ((size_t)slot * G + P.grp[u]) * 4;
+        const int g = P.grp[u];
         C d;
         if (kMat == kAny && (rec[2 * s + 1].w >> 16)) {
-            d = m[(size_t)n_slots * G * 4 + e];
-            if (kRev && e == 0) {  // the inverse rotation
+            if (e > 1) continue;
+            const double2 *f = gm.split + ((size_t)slot * gm.G + g) * 4;
+            double2 v = f[0];
+            if (e == 1) v = cmul(f[1], cconj(f[2]));
+            else if (kRev) v = make_double2(-v.x, -v.y);  // the inverse rotation
+            d = cmk<C>(v.x, v.y);
+        } else if (kRev) {
+            const C *m = mats + g * 4;
+            if (kMat == kPair && is_shear_pair(m[2], m[3])) {
+                d = m[e];
                 d.x = -d.x;
                 d.y = -d.y;
+            } else {
+                d = m[e == 1 ? 2 : (e == 2 ? 1 : e)];
+                if (kMat != kPair) d.y = -d.y;
             }
-        } else if (kRev) {
-            d = m[e == 1 ? 2 : (e == 2 ? 1 : e)];
-            if (kMat != kPair) d.y = -d.y;
         } else {
-            d = m[e];
+            d = mats[g * 4 + e];
         }
         sm[4 * u + e] = d;
     }
-    __syncthreads();
-    if constexpr (kMat == kAny) build_phase_tables<C, R, kRev>(P.n_stages, rec, sm, tab);
-    for (int x = tid; x < P.n_stages * R; x += T) {
-        const int s = x / R;
-        const uint32_t ob = (rec[2 * s].x >> (8 * (x % R))) & 0xffu;
-        C *m = sm + 4 * ((int)(ob & 63u) - 1);
-        if (!ob || (kMat == kAny && (rec[2 * s + 1].w >> 16))) continue;
-        if constexpr (kMat == kPair) stage_shears_pair(m);
-        else if (ob & 64u) stage_shears(m);
+    if constexpr (kMat == kAny) {
+        const C *tabs = (const C *)gm.tabs + ((size_t)slot * gm.n_stages + gm.stage0) * 2 * NA;
+        for (int x = tid; x < P.n_stages * 2 * NA; x += T)
+            if (rec[2 * (x / (2 * NA)) + 1].w >> 16) tab[x] = kRev ? cconj(tabs[x]) : tabs[x];
     }
     __syncthreads();
+    if constexpr (kMat != kPair) {
+        for (int x = tid; x < P.n_stages * R; x += T) {
+            const int s = x / R;
+            const uint32_t ob = (rec[2 * s].x >> (8 * (x % R))) & 0xffu;
+            if ((ob & 64u) && !(kMat == kAny && (rec[2 * s + 1].w >> 16)))
+                stage_shears(sm + 4 * ((int)(ob & 63u) - 1));
+        }
+        __syncthreads();
+    }
     set_stage_flags<C, kMat>(P, rec, sm);
 }
 
-template <typename Real, int R, int kMat>
+template <typename Real, int R, int kMat, bool kDep = false>
 __device__ __forceinline__ void tile_fwd_body(const TilePass &P, int n, int n_slots,
-                                              const typename CT<Real>::T *mats, int G,
+                                              const GroupMats &gm,
                                               const typename CT<Real>::T *src_states,
                                               typename CT<Real>::T *states, int64_t t0,
                                               int64_t t_end, unsigned char *smem,
@@ -185,6 +404,7 @@ __device__ __forceinline__ void tile_fwd_body(const TilePass &P, int n, int n_sl
     const uint32_t p0 = bit_vectors<R>(P.ldperm, t, tid, pk);
     const uint32_t n0 = bit_vectors<R>(P.nat, t, tid, nk);
     const uint32_t sh = (uint32_t)__cvta_generic_to_shared(smem);
+    if constexpr (kDep) pdl_wait();  // the pass's descriptor work needs no memory
     if (t0 >= t_end) return;
     auto fetch = [&](const TileCursor &c, int buf) {
         const C *src = src_states + ((int64_t)c.slot << n) + c.base;
@@ -219,7 +439,7 @@ __device__ __forceinline__ void tile_fwd_body(const TilePass &P, int n, int n_sl
     for (int64_t tix = t0, i = 0; tix < t_end; ++tix, ++i) {
         const int buf = (int)(i & 1);
         if (cur.slot != mslot) {  // the previous tile's stages are past their last barrier
-            stage_mats<C, R, kMat, false>(P, rec, n_slots, mats, G, cur.slot, sm, tab);
+            stage_mats<C, R, kMat, false>(P, rec, gm, cur.slot, sm, tab);
             mslot = cur.slot;
         }
         cp_async_wait_all();
@@ -253,13 +473,13 @@ __device__ __forceinline__ void tile_fwd_body(const TilePass &P, int n, int n_sl
 // forward state).
 template <typename Real, int R, int kMat>
 __global__ void __launch_bounds__(256, R >= 4 ? 2 : 3)
-k_tile_fwd(const __grid_constant__ TilePass P, int n, int n_slots,
-           const typename CT<Real>::T *mats, int G, const typename CT<Real>::T *src,
-           typename CT<Real>::T *states, Sparse sp) {
+k_tile_fwd(const __grid_constant__ TilePass P, int n, int n_slots, GroupMats gm,
+           const typename CT<Real>::T *src, typename CT<Real>::T *states, Sparse sp) {
     extern __shared__ __align__(16) unsigned char smem[];
+    pdl_trigger();
     int64_t t0, t_end;
     block_range((int64_t)n_slots << P.n_tile_bits, gridDim.x, blockIdx.x, t0, t_end);
-    tile_fwd_body<Real, R, kMat>(P, n, n_slots, mats, G, src, states, t0, t_end, smem, sp);
+    tile_fwd_body<Real, R, kMat, true>(P, n, n_slots, gm, src, states, t0, t_end, smem, sp);
 }
 
 // The derivative of a rotation exp(-i theta P / 2) inside a fused group is
@@ -618,9 +838,7 @@ __device__ void flush_acc(const TilePass &P, Real *acc, int wps, double *rho_g, 
                     }
             }
             if (k[0] == 0.0 && k[1] == 0.0 && k[2] == 0.0) continue;
-            const auto p0 = sm[4 * u + 1], p1 = sm[4 * u + 2];
-            const double fx = (double)p0.x * p1.x + (double)p0.y * p1.y;
-            const double fy = (double)p0.y * p1.x - (double)p0.x * p1.y;
+            const double fx = sm[4 * u + 1].x, fy = sm[4 * u + 1].y;  // p0 conj(p1)
             const double re = 0.5 * (fx * k[2] - fy * k[1]), im = 0.5 * (fx * k[1] + fy * k[2]);
             // i K = [[i (k0 - k1) / 2, z], [-conj(z), -i (k0 - k1) / 2]]
             double *dst = rho_g + ((size_t)b * G + P.grp[u]) * 8;
@@ -688,9 +906,9 @@ __device__ void flush_acc(const TilePass &P, Real *acc, int wps, double *rho_g, 
 // reduced matrices of its parametrised groups (as i K) into
 // rho_g[slot][group][8].  The sums run in the state's precision over one
 // warp and at most 64 tiles, then in FP64.
-template <typename Real, int R, bool kSingle, int kMat, int NB = 2>
+template <typename Real, int R, bool kSingle, int kMat, int NB = 2, bool kDep = false>
 __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_slots,
-                                              const typename CT<Real>::T *mats, int G,
+                                              const GroupMats &gm,
                                               const typename CT<Real>::T *psi_src,
                                               typename CT<Real>::T *psi, typename CT<Real>::T *lam,
                                               double *rho_g, int64_t t0, int64_t t_end,
@@ -699,6 +917,7 @@ __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_sl
     using C = typename CT<Real>::T;
     constexpr int NA = 1 << R;
     constexpr int kFlushTiles = 64;
+    const int G = gm.G;
     const int tid = threadIdx.x, T = blockDim.x, t = P.t, S = P.n_stages;
     const int lane = tid & 31, wps = T >> 5;
     const uint32_t tbytes = (uint32_t)sizeof(C) << t;
@@ -728,6 +947,7 @@ __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_sl
     const uint32_t p0 = bit_vectors<R>(P.ldperm, t, tid, pk);
     const uint32_t n0 = bit_vectors<R>(P.nat, t, tid, nk);
     const uint32_t sh = (uint32_t)__cvta_generic_to_shared(smem);
+    if constexpr (kDep) pdl_wait();
     if (t0 >= t_end) return;
     // psi tile of buffer j at [j tbytes], lambda tile at [(NB + j) tbytes]
     auto fetch = [&](const TileCursor &c, int buf) {
@@ -753,8 +973,8 @@ __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_sl
             since = 0;
         }
         if (cur.slot != mslot) {  // adjoint matrices of this slot's groups
-            stage_mats<C, R, kSplit || kMat != kAny ? kMat : kNoSplit, true>(P, rec, n_slots, mats, G,
-                                                                            cur.slot, sm, tab);
+            stage_mats<C, R, kSplit || kMat != kAny ? kMat : kNoSplit, true>(P, rec, gm, cur.slot, sm,
+                                                                            tab);
             mslot = cur.slot;
         }
         cp_async_wait_all();
@@ -873,14 +1093,15 @@ __device__ __forceinline__ void tile_rev_body(const TilePass &P, int n, int n_sl
 // NB = 1: launched with 64 threads only (at least five blocks per SM).
 template <typename Real, int R, bool kSingle, int kMat, int NB = 2>
 __global__ void __launch_bounds__(NB == 1 ? 64 : 256, NB == 1 ? 5 : (R >= 4 ? 1 : 2))
-k_tile_rev(const __grid_constant__ TilePass P, int n, int n_slots,
-           const typename CT<Real>::T *mats, int G, const typename CT<Real>::T *psi_src,
+k_tile_rev(const __grid_constant__ TilePass P, int n, int n_slots, GroupMats gm,
+           const typename CT<Real>::T *psi_src,
            typename CT<Real>::T *psi, typename CT<Real>::T *lam, double *rho_g, Sparse sp,
            int write_psi) {
     extern __shared__ __align__(16) unsigned char smem[];
+    pdl_trigger();
     int64_t t0, t_end;
     block_range((int64_t)n_slots << P.n_tile_bits, gridDim.x, blockIdx.x, t0, t_end);
-    tile_rev_body<Real, R, kSingle, kMat, NB>(P, n, n_slots, mats, G, psi_src, psi, lam, rho_g,
+    tile_rev_body<Real, R, kSingle, kMat, NB, true>(P, n, n_slots, gm, psi_src, psi, lam, rho_g,
                                                t0, t_end, smem, sp.refs, sp.fixed, write_psi != 0);
 }
 
@@ -977,12 +1198,13 @@ k_tile_sweep(const SweepTask *tasks, int n_tasks, long long n_tickets,
         const long long c = tk - T.chunk_begin;
         const int64_t t0 = c * (int64_t)T.chunk_tiles;
         const int64_t t1 = min(T.tiles, t0 + (int64_t)T.chunk_tiles);
+        const GroupMats gm{T.mats, T.tabs, (const double2 *)T.split, T.G, T.n_stages, T.stage0, 0};
         if constexpr (kRev)
-            tile_rev_body<Real, R, false, kAny>(P, T.n, T.n_slots, (const C *)T.mats, T.G,
+            tile_rev_body<Real, R, false, kAny>(P, T.n, T.n_slots, gm,
                                                  (const C *)T.psi, (C *)T.psi, (C *)T.lam, T.rho,
                                                  t0, t1, rest, T.refs, T.fixed);
         else
-            tile_fwd_body<Real, R, kAny>(P, T.n, T.n_slots, (const C *)T.mats, T.G,
+            tile_fwd_body<Real, R, kAny>(P, T.n, T.n_slots, gm,
                                          (const C *)T.psi, (C *)T.psi, t0, t1, rest,
                                          Sparse{T.refs, T.fixed, 0u, 0, 0});
         __syncthreads();  // every store of the chunk issued
@@ -1050,6 +1272,7 @@ k_tile_h(const __grid_constant__ HPass P, int n, int n_slots, const typename CT<
     static_assert(R <= kHRegBitsMax, "H kernel register bits");
     extern __shared__ __align__(16) unsigned char smem[];
     // 256 threads whenever R >= 3 (tiles of 2^11 and 2^12 amplitudes)
+    pdl_trigger();
     const int tid = threadIdx.x, T = R >= 3 ? 256 : (int)blockDim.x, t = P.t;
     const uint32_t tbytes = (uint32_t)sizeof(C) << t;
     // psi tiles at [0, 2 tbytes), the lambda tile being added to at [2 tbytes,
@@ -1075,6 +1298,7 @@ k_tile_h(const __grid_constant__ HPass P, int n, int n_slots, const typename CT<
     const int64_t tiles = (int64_t)n_slots << P.n_tile_bits;
     const int64_t per = (tiles + gridDim.x - 1) / gridDim.x;
     const int64_t t0 = per * blockIdx.x, t_end = min(tiles, t0 + per);
+    pdl_wait();  // the plan's arrays are older than the stream's work
     if (t0 >= t_end) return;
     auto fetch = [&](const TileCursor &c, int buf) {
         const C *src = psi + ((int64_t)c.slot << n) + c.base;
@@ -1395,6 +1619,8 @@ __global__ void k_ddcl_lambda(int n, const typename CT<Real>::T *psi, const doub
 template <typename Real>
 __global__ void k_group_grads(Program p, SlotSource src, const double *rho_g, CostSource cs,
                               const double *E, double *slot_grads) {
+    pdl_trigger();
+    pdl_wait();
     const int G = p.n_groups, P = p.n_params;
     const int64_t total = (int64_t)src.n_slots * G;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
@@ -1438,17 +1664,46 @@ template <typename K> cudaError_t allow_smem(K kernel, uint32_t bytes) {
     return e;
 }
 
-// Resident blocks of kernel k on the whole GPU, at most max_blocks.
+// Resident blocks of kernel k on the whole GPU, at most max_blocks.  The
+// occupancy of a launch shape is a constant of the device: kept per thread,
+// since a call of a small state is launch after launch.
 template <typename K> int fill_blocks(K kernel, int threads, uint32_t smem, int64_t max_blocks) {
-    int dev = 0, sms = 0, per = 0;
+    struct Seen {
+        const void *kernel;
+        int dev, threads, blocks;
+        uint32_t smem;
+    };
+    static thread_local std::vector<Seen> seen;
+    int dev = 0;
     cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem) != cudaSuccess ||
-        per < 1)
-        per = 1;
-    int64_t b = (int64_t)sms * per;
+    int64_t b = 0;
+    for (const Seen &s : seen)
+        if (s.kernel == (const void *)kernel && s.dev == dev && s.threads == threads && s.smem == smem) {
+            b = s.blocks;
+            break;
+        }
+    if (!b) {
+        int sms = 0, per = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem) != cudaSuccess ||
+            per < 1)
+            per = 1;
+        b = (int64_t)sms * per;
+        if (seen.size() >= 256) seen.clear();
+        seen.push_back({(const void *)kernel, dev, threads, (int)b, smem});
+    }
     if (b > max_blocks) b = max_blocks;
     return b < 1 ? 1 : (int)b;
+}
+
+// Whether a pass over n_tiles tiles of 2^t amplitudes is launched as a
+// dependent of the one before: passes over at most 64 MiB, whose launch gaps
+// and descriptor work show.  Longer ones lose more than they gain: their
+// blocks then start wherever blocks of the pass before ended, on the other
+// die from the L2 that holds their tiles (20-qubit states, 512 MiB passes of
+// 200 us: 5833 against 5482 us).
+bool pass_dep(int c128, int t, int64_t n_tiles) {
+    return ((n_tiles << t) * (c128 ? 16 : 8)) <= (int64_t(64) << 20);
 }
 
 int grid_1d(int64_t work, int threads) {
@@ -1481,14 +1736,30 @@ int grid_1d(int64_t work, int threads) {
         }                                                                   \
     } while (0)
 
-cudaError_t launch_group_mats(int c128, const Program &p, const SlotSource &src, void *mats,
-                              int64_t *refs, cudaStream_t st, bool pair) {
-    // one warp a block: the FP64 sines of a few thousand groups spread over
-    // every SM (32 slots x 190 groups: 22 us in blocks of 128 threads)
-    const int g = grid_1d((int64_t)src.n_slots * std::max(1, p.n_groups), 32);
-    if (c128) k_group_mats<double><<<g, 32, 0, st>>>(p, src, pair, (double2 *)mats, refs);
-    else k_group_mats<float><<<g, 32, 0, st>>>(p, src, pair, (float2 *)mats, refs);
-    return cudaGetLastError();
+cudaError_t launch_group_mats(int c128, const Program &p, const SlotSource &src, void *base,
+                              cudaStream_t st, bool pair, const ClearList &clear) {
+    const int n_states = pair ? (src.n_slots + 1) / 2 : src.n_slots;
+    const GroupBuf b = group_buf(c128, p, (size_t)n_states, pair);
+    double2 *split = (double2 *)((char *)base + b.split);
+    int64_t *refs = (int64_t *)((char *)base + b.refs);
+    void *tabs = (char *)base + b.tabs;
+    // One warp a block: the FP64 work of a few thousand groups spreads over
+    // every SM (32 slots x 190 groups: 22 us in blocks of 128 threads).  Four
+    // lanes a group while that fits the SMs' schedulers in one wave: the
+    // latency of a group's loads and sines counts then, not their number.
+    const int64_t groups = (int64_t)n_states * std::max(1, p.n_groups);
+    const bool wide = !c128 && groups * 4 <= 152 * 4 * 32;
+    const int g = grid_1d(wide ? groups * 4 : groups, 32);
+    cudaError_t e =
+        c128   ? launch_dep(k_group_mats<double, 1>, g, 32, 0, st, p, src, (int)pair, (double2 *)base, split, refs, clear)
+        : wide ? launch_dep(k_group_mats<float, 4>, g, 32, 0, st, p, src, (int)pair, (float2 *)base, split, refs, clear)
+               : launch_dep(k_group_mats<float, 1>, g, 32, 0, st, p, src, (int)pair, (float2 *)base, split, refs, clear);
+    if (e == cudaSuccess && !pair && p.n_stages > 0) {
+        const int gt = grid_1d(((int64_t)n_states * p.n_stages * 2) << p.R, 64);
+        e = c128 ? launch_dep(k_phase_tables<double>, gt, 64, 0, st, p, n_states, split, (double2 *)tabs)
+                 : launch_dep(k_phase_tables<float>, gt, 64, 0, st, p, n_states, split, (float2 *)tabs);
+    }
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 cudaError_t launch_init_states(int c128, void *states, int n, const SlotSource &src,
@@ -1545,8 +1816,8 @@ uint32_t tile_rev_smem(int c128, const TilePass &P, int bufs, bool any) {
            tab + (uint32_t)P.n_ops * T * rsz;
 }
 
-cudaError_t launch_tile_fwd(int c128, const TilePass &P, int n, int n_slots, const void *mats,
-                            int G, void *states, int64_t max_blocks, cudaStream_t st,
+cudaError_t launch_tile_fwd(int c128, const TilePass &P, int n, int n_slots,
+                            const GroupMats &gm, void *states, int64_t max_blocks, cudaStream_t st,
                             const void *src, bool pair, const Sparse &sp) {
     const uint32_t smem = tile_fwd_smem(c128, P);
     const int threads = 1 << (P.t - P.R);
@@ -1558,14 +1829,15 @@ cudaError_t launch_tile_fwd(int c128, const TilePass &P, int n, int n_slots, con
         cudaError_t e = allow_smem(k, smem);
         if (e != cudaSuccess) return e;
         const int blocks = fill_blocks(k, threads, smem, max_blocks);
-        k<<<blocks, threads, smem, st>>>(P, n, n_slots, (const C *)mats, G, (const C *)src,
-                                         (C *)states, sp);
+        e = launch_dep_if(pass_dep(c128, P.t, (int64_t)n_slots << P.n_tile_bits), k, blocks, threads,
+                          smem, st, P, n, n_slots, gm, (const C *)src, (C *)states, sp);
+        if (e != cudaSuccess) return e;
     });
     return cudaGetLastError();
 }
 
-cudaError_t launch_tile_rev(int c128, const TilePass &P, int n, int n_slots, const void *mats,
-                            int G, void *psi, void *lam, double *rho_g, int64_t max_blocks,
+cudaError_t launch_tile_rev(int c128, const TilePass &P, int n, int n_slots,
+                            const GroupMats &gm, void *psi, void *lam, double *rho_g, int64_t max_blocks,
                             cudaStream_t st, const void *psi_src, bool write_psi, bool pair,
                             const Sparse &sp) {
     // passes of many stages are arithmetic-bound: one tile buffer, more
@@ -1589,9 +1861,10 @@ cudaError_t launch_tile_rev(int c128, const TilePass &P, int n, int n_slots, con
         cudaError_t e = allow_smem(k, smem);
         if (e != cudaSuccess) return e;
         const int blocks = fill_blocks(k, threads, smem, max_blocks);
-        k<<<blocks, threads, smem, st>>>(P, n, n_slots, (const C *)mats, G,
-                                         (const C *)(psi_src ? psi_src : psi), (C *)psi, (C *)lam,
-                                         rho_g, sp, write_psi ? 1 : 0);
+        e = launch_dep_if(pass_dep(c128, P.t, (int64_t)n_slots << P.n_tile_bits), k, blocks, threads,
+                       smem, st, P, n, n_slots, gm, (const C *)(psi_src ? psi_src : psi), (C *)psi, (C *)lam, rho_g, sp,
+                       write_psi ? 1 : 0);
+        if (e != cudaSuccess) return e;
     });
     return cudaGetLastError();
 }
@@ -1616,8 +1889,8 @@ cudaError_t launch_tile_h(int c128, const HPass &P, int n, int n_slots, const vo
         cudaError_t e = allow_smem(k, smem);
         if (e != cudaSuccess) return e;
         const int blocks = fill_blocks(k, threads, smem, max_blocks);
-        k<<<blocks, threads, smem, st>>>(P, n, n_slots, psi_t, lam_t, E, pair_rows);
-        return cudaGetLastError();
+        return launch_dep_if(pass_dep(c128, P.t, (int64_t)n_slots << P.n_tile_bits), k, blocks,
+                             threads, smem, st, P, n, n_slots, psi_t, lam_t, E, pair_rows);
     };
     auto pick2 = [&](auto rr, auto re, auto pr) -> cudaError_t {
         constexpr int RR = decltype(rr)::value;
@@ -1831,9 +2104,8 @@ cudaError_t launch_group_grads(int c128, const Program &p, const SlotSource &src
                                const double *rho_g, const CostSource &cs, const double *E,
                                double *slot_grads, cudaStream_t st) {
     const int g = grid_1d((int64_t)src.n_slots * p.n_groups, 128);
-    if (c128) k_group_grads<double><<<g, 128, 0, st>>>(p, src, rho_g, cs, E, slot_grads);
-    else k_group_grads<float><<<g, 128, 0, st>>>(p, src, rho_g, cs, E, slot_grads);
-    return cudaGetLastError();
+    return c128 ? launch_dep(k_group_grads<double>, g, 128, 0, st, p, src, rho_g, cs, E, slot_grads)
+                : launch_dep(k_group_grads<float>, g, 128, 0, st, p, src, rho_g, cs, E, slot_grads);
 }
 
 }  // namespace svk

@@ -11,14 +11,48 @@ namespace svk {
 // pair (here and below): two real circuits per state (slots 2j and 2j + 1 in
 // the components of state j); the launchers' slot counts are then pairs,
 // except in a SlotSource and in pair_rows.
-// mats: [slots][groups][4] complex of the state's precision, followed (not
-// with pair) by the groups' split form [slots][groups][4].  kMatVals complex
-// values per slot and group hold both.
-constexpr int kMatVals = 8;
-// refs: [states][2], the states' reference indices (pair: of the two slots;
+// What the passes read of every state's groups, in one buffer (offsets in
+// bytes): mats [states][groups][4] complex of the state's precision; without
+// pair also split [states][groups][4] double2, the groups' split forms, and
+// tabs [states][stages][2][2^R] complex, the split stages' phase tables; refs
+// [states][2], the states' reference indices (pair: of its two slots;
 // otherwise the slot's twice).
-cudaError_t launch_group_mats(int c128, const Program &p, const SlotSource &src, void *mats,
-                              int64_t *refs, cudaStream_t st, bool pair = false);
+struct GroupBuf {
+    size_t split = 0, tabs = 0, refs = 0, bytes = 0;
+    int G = 0, n_stages = 0;
+};
+inline GroupBuf group_buf(int c128, const Program &p, size_t n_states, bool pair) {
+    const size_t csz = c128 ? 16 : 8;
+    GroupBuf b;
+    b.G = p.n_groups;
+    b.n_stages = p.n_stages;
+    size_t off = n_states * b.G * 4 * csz;
+    b.split = off;
+    if (!pair) off += n_states * b.G * 64;
+    b.tabs = off;
+    if (!pair) off += (n_states * b.n_stages * 2 * csz) << p.R;
+    b.refs = off;
+    b.bytes = off + n_states * 16;
+    return b;
+}
+// The part of a pass whose first stage is stage0 of the plan.
+struct GroupMats {
+    const void *mats, *tabs;
+    const double2 *split;
+    int32_t G, n_stages, stage0, pad;
+};
+inline GroupMats group_mats_of(const GroupBuf &b, const void *base, int stage0) {
+    const char *p = (const char *)base;
+    return GroupMats{p, p + b.tabs, (const double2 *)(p + b.split), b.G, b.n_stages, stage0, 0};
+}
+// Arrays of doubles set to zero on the way (sums that later kernels add to).
+struct ClearList {
+    double *p[3];
+    int64_t n[3];
+};
+cudaError_t launch_group_mats(int c128, const Program &p, const SlotSource &src, void *base,
+                              cudaStream_t st, bool pair = false,
+                              const ClearList &clear = ClearList{});
 // Zeroes the slot states and sets amplitude |ref> of each to 1.
 cudaError_t launch_init_states(int c128, void *states, int n, const SlotSource &src,
                                cudaStream_t st);
@@ -43,10 +77,10 @@ Sparse sparse_pass(TilePass *P, uint32_t support, const int64_t *refs, bool init
 // (any: of a kernel that takes complex and real passes alike).
 uint32_t tile_fwd_smem(int c128, const TilePass &P, bool any = false);
 uint32_t tile_rev_smem(int c128, const TilePass &P, int bufs = 2, bool any = false);
-// Forward pass P over n_slots states of n qubits (mats: [slots][G][4]).
+// Forward pass P over n_slots states of n qubits.
 // src (null: states) holds the pass's input; the output goes to states.
-cudaError_t launch_tile_fwd(int c128, const TilePass &P, int n, int n_slots, const void *mats,
-                            int G, void *states, int64_t max_blocks, cudaStream_t st,
+cudaError_t launch_tile_fwd(int c128, const TilePass &P, int n, int n_slots,
+                            const GroupMats &gm, void *states, int64_t max_blocks, cudaStream_t st,
                             const void *src = nullptr, bool pair = false,
                             const Sparse &sp = Sparse{});
 // Reverse pass P on psi and lambda; adds the reduced matrices of its
@@ -54,8 +88,8 @@ cudaError_t launch_tile_fwd(int c128, const TilePass &P, int n, int n_slots, con
 // psi the pass reads (a stored forward state); its output psi goes to psi
 // unless write_psi is false (the next reverse pass restarts psi from a
 // stored state, or this is the last one).  pair: rho_g has two rows per state.
-cudaError_t launch_tile_rev(int c128, const TilePass &P, int n, int n_slots, const void *mats,
-                            int G, void *psi, void *lam, double *rho_g, int64_t max_blocks,
+cudaError_t launch_tile_rev(int c128, const TilePass &P, int n, int n_slots,
+                            const GroupMats &gm, void *psi, void *lam, double *rho_g, int64_t max_blocks,
                             cudaStream_t st, const void *psi_src = nullptr,
                             bool write_psi = true, bool pair = false,
                             const Sparse &sp = Sparse{});

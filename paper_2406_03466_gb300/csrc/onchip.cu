@@ -165,6 +165,7 @@ __global__ void __launch_bounds__(512) k_adjoint(Program p, Observable o, SlotSo
 __global__ void k_ps_combine(const double *E, int I, int P, CostSource c, double *lp,
                              double *energy_out, double *loss_out, double *grad_out) {
     __shared__ double red[32];
+    pdl_wait();
     ps_combine_block(E, I, P, c, lp, energy_out, loss_out, grad_out, red);
 }
 
@@ -185,6 +186,7 @@ __global__ void k_ps_combine_dep(const double *E, int I, int P, CostSource c, do
 // Adjoint combination: dL/dtheta = sum_i (weighted per-instance gradients).
 __global__ void k_adjoint_combine(const double *Gs, const double *E, int I, int P, CostSource c,
                                   double *energy_out, double *loss_out, double *grad_out) {
+    pdl_wait();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < P) {
         double g = 0.0;
@@ -507,8 +509,7 @@ cudaError_t launch_onchip_adjoint(int c128, const OnchipShape &sh, const Program
 cudaError_t launch_ps_combine(const double *E, int I, int P, const CostSource &c, double *lp,
                               double *energy_out, double *loss_out, double *grad_out,
                               cudaStream_t st) {
-    k_ps_combine<<<1, 256, 0, st>>>(E, I, P, c, lp, energy_out, loss_out, grad_out);
-    return cudaGetLastError();
+    return launch_dep(k_ps_combine, 1, 256, 0, st, E, I, P, c, lp, energy_out, loss_out, grad_out);
 }
 
 cudaError_t launch_adjoint_combine(const double *G, const double *E, int I, int P,
@@ -517,8 +518,8 @@ cudaError_t launch_adjoint_combine(const double *G, const double *E, int I, int 
     const int threads = 256;
     int blocks = (P + threads - 1) / threads;
     if (blocks < 1) blocks = 1;
-    k_adjoint_combine<<<blocks, threads, 0, st>>>(G, E, I, P, c, energy_out, loss_out, grad_out);
-    return cudaGetLastError();
+    return launch_dep(k_adjoint_combine, blocks, threads, 0, st, G, E, I, P, c, energy_out, loss_out,
+                      grad_out);
 }
 
 }  // namespace svk

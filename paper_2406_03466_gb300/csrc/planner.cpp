@@ -301,7 +301,8 @@ std::string plan_circuit(const sv_circuit &c, int reg_bits, bool fuse, int swz_b
 }
 
 std::string plan_passes(const sv_circuit &c0, int tile_bits, int coalesce_bits, int reg_bits,
-                        bool fuse, int swz_bits, HostProgram *P, bool relabel) {
+                        bool fuse, int swz_bits, HostProgram *P, bool relabel,
+                        bool drop_tail) {
     // CZ(a, b) = H_b CNOT(a -> b) H_b: tile passes run fused single-qubit
     // groups and CNOT permutations only.
     std::vector<sv_gate> gates;
@@ -345,6 +346,23 @@ std::string plan_passes(const sv_circuit &c0, int tile_bits, int coalesce_bits, 
     P->swz_bits = swz_bits;
     P->members = F.members;
     P->groups = F.groups;
+    if (drop_tail) {
+        std::vector<LOp> keep;
+        uint32_t busy = 0;
+        for (size_t i = F.lops.size(); i-- > 0;) {
+            const LOp &o = F.lops[i];
+            const uint32_t q = lop_qubits(o);
+            if (o.kind == 1 && !(q & busy)) {
+                P->tail.push_back({o.a, o.b});
+            } else {
+                busy |= q;
+                keep.push_back(o);
+            }
+        }
+        std::reverse(P->tail.begin(), P->tail.end());
+        std::reverse(keep.begin(), keep.end());
+        F.lops.swap(keep);
+    }
     // phys[q]: the bit of the amplitude index that holds qubit q; who[b]: the
     // qubit held by bit b.
     std::vector<int> phys(n), who(n);
@@ -542,6 +560,21 @@ std::string plan_passes(const sv_circuit &c0, int tile_bits, int coalesce_bits, 
     return "";
 }
 
+int conjugate_by_cnots(const std::vector<std::pair<int, int>> &tail, uint64_t *x, uint64_t *z) {
+    int sign = 1;
+    for (size_t i = tail.size(); i-- > 0;) {
+        // X_c -> X_c X_t, Z_t -> Z_c Z_t (Y on both counted in), with a minus
+        // sign on X_c Z_t and Y_c Y_t
+        const int c = tail[i].first, t = tail[i].second;
+        const uint64_t xc = (*x >> c) & 1, xt = (*x >> t) & 1, zc = (*z >> c) & 1,
+                       zt = (*z >> t) & 1;
+        if (xc && zt && xt == zc) sign = -sign;
+        *x ^= xc << t;
+        *z ^= zt << c;
+    }
+    return sign;
+}
+
 // Kernel descriptors of every pass of a tile plan (amplitudes of csz bytes).
 std::string build_tile_passes(const HostProgram &P, int csz, std::vector<TilePass> *out) {
     out->clear();
@@ -623,23 +656,54 @@ std::string plan_h_passes(const HostObservable &h, int tile_bits, int coalesce_b
     const uint32_t forced = (1u << coalesce_bits) - 1u;
     std::vector<int> pending(h.tgroups.size());
     for (size_t i = 0; i < pending.size(); ++i) pending[i] = (int)i;
+    // The groups of each pass: those whose flip masks fit its tile, and those
+    // whose partners it reads from global memory (far, first pass only).
+    struct Taken {
+        uint32_t L;
+        std::vector<int> near, far;
+    };
+    std::vector<Taken> plan;
     while (!pending.empty()) {
-        uint32_t L = forced;
-        std::vector<int> taken, rest;
-        std::vector<int> far;  // flip masks that fit no tile: partners from global memory
+        Taken tk;
+        tk.L = forced;
+        std::vector<int> rest;
         for (int gi : pending) {
             const uint32_t x = h.tgroups[gi].x;
             if (__builtin_popcount(forced | x) > t) {
-                far.push_back(gi);
-            } else if (__builtin_popcount(L | x) <= t) {
-                L |= x;
-                taken.push_back(gi);
+                tk.far.push_back(gi);  // fits no tile
+            } else if (__builtin_popcount(tk.L | x) <= t) {
+                tk.L |= x;
+                tk.near.push_back(gi);
             } else {
                 rest.push_back(gi);
             }
         }
-        if (taken.empty() && far.empty()) return "internal: H pass planner made no progress";
-        for (int gi : far) taken.push_back(gi);
+        if (tk.near.empty() && tk.far.empty()) return "internal: H pass planner made no progress";
+        plan.push_back(tk);
+        pending.swap(rest);
+    }
+    // A later pass of one or two groups costs more than they do as far groups
+    // of the first: reading partners moves 8 bytes an amplitude and group
+    // (whole 128-byte runs), a pass reads psi, reads lambda and writes it (24
+    // bytes) and is a launch of its own.  At most kFarTerms terms' worth, so
+    // that the first pass's records stay small beside its tiles.
+    constexpr int kFarTerms = 96;
+    int moved = 0;
+    for (size_t i = 1; i < plan.size();) {
+        int terms = 0;
+        for (int gi : plan[i].near) terms += h.tgroups[gi].t_end - h.tgroups[gi].t_begin;
+        if (plan[i].near.size() > 2 || !plan[i].far.empty() || moved + terms > kFarTerms) {
+            ++i;
+            continue;
+        }
+        moved += terms;
+        plan[0].far.insert(plan[0].far.end(), plan[i].near.begin(), plan[i].near.end());
+        plan.erase(plan.begin() + i);
+    }
+    for (const Taken &tk : plan) {
+        uint32_t L = tk.L;
+        std::vector<int> taken = tk.near;
+        taken.insert(taken.end(), tk.far.begin(), tk.far.end());
         for (int q = 0; __builtin_popcount(L) < t && q < n; ++q) L |= 1u << q;
         HPass P{};
         P.t = t;
@@ -731,7 +795,6 @@ std::string plan_h_passes(const HostObservable &h, int tile_bits, int coalesce_b
         P.n_terms = (int)out->terms.size() - t0;
         P.n_rows = (int)out->rows.size() - r0;
         out->passes.push_back(P);
-        pending.swap(rest);
     }
     out->g_begin.push_back((int)out->groups.size());
     out->c_begin.push_back((int)out->classes.size());

@@ -2,6 +2,7 @@
 // the on-chip kernels, and a Pauli sum into X-mask term groups.
 #pragma once
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "sv.h"
@@ -24,6 +25,9 @@ struct HostProgram {
     // Layout after the last tile pass: qubit q lives in bit layout[q] of the
     // amplitude index (the identity unless the passes relabel).
     std::vector<int> layout;
+    // Trailing CNOTs (control, target), in time order, that the passes leave
+    // to the observable (plan_passes with drop_tail).
+    std::vector<std::pair<int, int>> tail;
     std::vector<ThreadBase> tbase;                 // [stages][2^(t-R)] thread bases
 };
 
@@ -53,8 +57,17 @@ void stage_lops(const std::vector<LOp> &lops, const std::vector<int> &pos, int t
 // may store its tile with its qubits in other bits of the same tile, moving
 // into the low bits qubits that the next pass needs (P->layout gives the
 // final bit of every qubit); otherwise every qubit keeps its own bit.
+// drop_tail: the CNOTs that no other gate follows on their qubits stay out of
+// the passes (P->tail); expectation values then take the observable
+// conjugated by them (conjugate_by_cnots).
 std::string plan_passes(const sv_circuit &c, int tile_bits, int coalesce_bits, int reg_bits,
-                        bool fuse, int swz_bits, HostProgram *P, bool relabel = false);
+                        bool fuse, int swz_bits, HostProgram *P, bool relabel = false,
+                        bool drop_tail = false);
+
+// U^dag P U for the Pauli string with masks (*x, *z), U the CNOTs of `tail` in
+// time order: again a Pauli string, whose masks replace *x and *z; returns
+// its sign (+1 or -1).
+int conjugate_by_cnots(const std::vector<std::pair<int, int>> &tail, uint64_t *x, uint64_t *z);
 
 // Kernel descriptors of every pass of a tile plan (amplitudes of csz bytes).
 std::string build_tile_passes(const HostProgram &P, int csz, std::vector<TilePass> *out);

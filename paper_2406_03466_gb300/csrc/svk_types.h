@@ -164,7 +164,9 @@ struct SweepTask {
     uint32_t fixed, pad2; // tile-number bits taken from the reference (hbm.h: Sparse)
     int64_t tiles, chunk_begin, n_chunks;
     int32_t chunk_tiles, pad;
-    const void *mats;   // [slots][G][4]
+    const void *mats, *tabs;  // the groups' matrices, tables and split forms (hbm.h: GroupMats)
+    const void *split;
+    int32_t n_stages, stage0;
     void *psi, *lam;    // the problem's states
     double *rho;        // reverse: [slots][G][8]
 };

@@ -247,20 +247,8 @@ __device__ __forceinline__ void stage_shears(C *m) {
     m[3].y = (Real)0;
 }
 
-// The same for a pair of real states: rotations of both circuits (c >= 0:
-// the matrices come with that sign) become m0 = alpha, m1 = beta, m2 = m3 =
-// 0, which no orthogonal matrix has.
-template <typename C> __device__ __forceinline__ void stage_shears_pair(C *m) {
-    using Real = decltype(m[0].x);
-    if (m[3].x != m[0].x || m[1].x != -m[2].x || m[0].x < (Real)0 || m[3].y != m[0].y ||
-        m[1].y != -m[2].y || m[0].y < (Real)0)
-        return;
-    const C s = m[2];
-    m[0].x = -s.x / ((Real)1 + m[0].x);
-    m[0].y = -s.y / ((Real)1 + m[0].y);
-    m[1] = s;
-    m[2].x = m[2].y = m[3].x = m[3].y = (Real)0;
-}
+// A pair of real states' rotations come as m0 = alpha, m1 = beta, m2 = m3 =
+// 0 (k_group_mats), which no orthogonal matrix has.
 template <typename C> __device__ __forceinline__ bool is_shear_pair(const C m2, const C m3) {
     return m2.x == 0 && m3.x == 0;
 }
@@ -342,7 +330,7 @@ __device__ __forceinline__ void tile_ops_fwd_rot(uint32_t ops, const C *sm, C (&
 // The split form of a group's matrix u (FP64): out = (alpha, beta), p0, p1, q
 // with the rotation's shears alpha = -s / (1 + c), beta = s.  The larger of
 // c and s fixes q, so nothing is divided by a small number.
-template <typename C> __device__ __forceinline__ void split_form(const double2 (&u)[4], C *out) {
+__device__ __forceinline__ void split_form(const double2 (&u)[4], double2 *out) {
     const double c = sqrt(u[0].x * u[0].x + u[0].y * u[0].y);
     const double s = sqrt(u[2].x * u[2].x + u[2].y * u[2].y);
     double2 p0 = make_double2(1.0, 0.0), p1 = p0, q;
@@ -351,32 +339,10 @@ template <typename C> __device__ __forceinline__ void split_form(const double2 (
     if (c >= s) q = cmul(u[3], cconj(p1));                          // u11 = p1 c q
     else q = cmul(make_double2(-u[1].x, -u[1].y), cconj(p0));       // u01 = -p0 s q
     const double l = sqrt(q.x * q.x + q.y * q.y);
-    out[0] = cmk<C>(-s / (1.0 + c), s);
-    out[1] = cmk<C>(p0.x, p0.y);
-    out[2] = cmk<C>(p1.x, p1.y);
-    out[3] = cmk<C>(q.x / l, q.y / l);
-}
-
-// Phase tables of the split stages, tab[s][0][r] = product of the q and
-// tab[s][1][r] = product of the p over the stage's register bits, from the
-// staged split forms (conjugated for the reverse sweep).
-template <typename C, int R, bool kConj>
-__device__ __forceinline__ void build_phase_tables(int n_stages, const uint4 *rec, const C *sm,
-                                                   C *tab) {
-    constexpr int NA = 1 << R;
-    for (int x = threadIdx.x; x < n_stages * 2 * NA; x += blockDim.x) {
-        const int s = x / (2 * NA), post = (x / NA) & 1, r = x & (NA - 1);
-        const int m = (int)((rec[2 * s + 1].w >> 16) & 15u);
-        const uint32_t ops = rec[2 * s].x;
-        C f = cmk<C>(1, 0);
-        for (int i = 0; i < m; ++i) {
-            const C *e = sm + 4 * ((int)((ops >> (8 * i)) & 63u) - 1);
-            const int b = (r >> i) & 1;
-            if (post) f = cmul(f, e[1 + b]);
-            else if (b) f = cmul(f, e[3]);
-        }
-        if (m) tab[x] = kConj ? cconj(f) : f;
-    }
+    out[0] = make_double2(-s / (1.0 + c), s);
+    out[1] = p0;
+    out[2] = p1;
+    out[3] = make_double2(q.x / l, q.y / l);
 }
 
 // a * p in two products and two fused multiply-adds.

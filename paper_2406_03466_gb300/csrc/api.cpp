@@ -70,6 +70,8 @@ struct PlanEntry {
     std::vector<sv_gate> gates;  // exact key check against hash collisions
     int n = 0, n_params = 0, input_dim = 0;
     bool real = false;  // every group's matrix is real
+    bool y_only = false;  // every group is Y rotations and Ry encodings
+    bool one_per_bit = false;  // stages: sorted, at most one group a register bit
     HostProgram host;
     std::vector<TilePass> tiles;  // tile plans: one kernel descriptor per pass
     DeviceBuf buf;
@@ -254,6 +256,14 @@ sv_status get_plan(DeviceCtx *ctx, const sv_circuit &c, int R, bool fuse, sv_dty
     const HostProgram &h = e->host;
     e->real = true;
     for (const Group &g : h.groups) e->real = e->real && g.real;
+    e->y_only = e->one_per_bit = true;
+    for (const Member &m : h.members)
+        e->y_only = e->y_only && (m.kind == M_RY || m.kind == M_ENC_RY_ASIN);
+    for (const Stage &sg : h.stages) {
+        e->one_per_bit = e->one_per_bit && sg.sorted != 0;
+        for (int i = 0; i < kRMax; ++i)
+            e->one_per_bit = e->one_per_bit && sg.bit_begin[i + 1] - sg.bit_begin[i] <= 1;
+    }
     Packer pk;
     size_t o_st = pk.add(h.stages.data(), h.stages.size() * sizeof(Stage));
     size_t o_op = pk.add(h.ops.data(), h.ops.size() * sizeof(Op));
@@ -719,13 +729,17 @@ sv_status tile_cfg(int n, sv_dtype dt, const sv_plan_opts *o, TileCfg *cfg,
     const int c = (o && o->coalesce_bits > 0) ? o->coalesce_bits : (dt == SV_C128 ? 3 : 4);
     const int rmax = dt == SV_C128 ? 3 : 4;
     // Default: 2^11 (complex64) / 2^10 (complex128) amplitudes per tile with
-    // 4 / 2 register bits: 128 / 256 threads per block.
+    // 4 / 2-3 register bits: 128 / 256-128 threads per block.
     int t = (o && o->tile_bits > 0) ? o->tile_bits : (dt == SV_C128 ? 10 : 11);
     if (t > n) t = n;
     if (t < c + 2 || t > 12)
         return fail(SV_ERR_UNSUPPORTED, "tile passes need 2^tile_bits amplitudes with tile_bits in "
                                         "[coalesced bits + 2, 12] and at most n_qubits");
-    int R = (o && o->reg_bits > 0) ? o->reg_bits : std::min(dt == SV_C128 ? 2 : 4, t - 5);
+    // 8 amplitudes per thread for larger complex128 states: fewer stages, and
+    // the FP64 unit, not the warps in flight, is the limit (19-qubit MC-VQE
+    // adjoint 2206 against 2580 us, 16-qubit circuit learning 5474 against 6134)
+    const int r_def = dt == SV_C128 ? (n >= 16 && t >= 10 ? 3 : 2) : 4;
+    int R = (o && o->reg_bits > 0) ? o->reg_bits : std::min(r_def, t - 5);
     if (R < 2 || R > rmax) return fail(SV_ERR_ARG, "reg_bits for tile passes must be 2..4 (2..3 complex128)");
     if (t - R > 8) R = t - 8;
     if (R > rmax) return fail(SV_ERR_UNSUPPORTED, "tile too large for the register width");
@@ -1187,13 +1201,15 @@ sv_status multi_adjoint(DeviceCtx *ctx, const sv_problem *problems, int np,
     const size_t csz = c128 ? 16 : 8;
     TileCfg cfg{};
     uint64_t key = mix64(0x5e17ull, (uint64_t)np);
+    int n_min = problems[0].circuit->n_qubits;  // one default shape: the smallest circuit's
+    for (int j = 1; j < np; ++j) n_min = std::min(n_min, problems[j].circuit->n_qubits);
     for (int j = 0; j < np; ++j) {
         const sv_problem *p = &problems[j];
         if (p->dtype != dt) return fail(SV_ERR_ARG, "uneven batch: problems differ in dtype");
         if (!wants_tiles(p->circuit->n_qubits, dt, p->opts))
             return fail(SV_ERR_UNSUPPORTED, "uneven batch: every problem must take the tile path");
         TileCfg c{};
-        sv_status s = tile_cfg(p->circuit->n_qubits, dt, p->opts, &c);
+        sv_status s = tile_cfg(n_min, dt, p->opts, &c);
         if (s != SV_OK) return s;
         if (j == 0) cfg = c;
         else if (c.t != cfg.t || c.R != cfg.R || c.c != cfg.c)
@@ -1914,6 +1930,85 @@ sv_status sv_energies(const sv_problem *p, const double *theta, double *energy_o
 
 namespace {
 
+// The on-chip adjoint of chip.cu where it applies: the default shape, stages
+// of at most one fused group a register bit (no CZ, fusion on), diagonal
+// tables at hand, a whole warp per state.  *done: whether it ran.  Register
+// bits: the fewest (most threads per state: the sweep is a chain of stages)
+// that keep the whole batch at 512 threads an SM.
+sv_status chip_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta,
+                       const double *weights, ObsEntry *obs, double *energy_out, double *loss_out,
+                       double *grad_out, int every, cudaStream_t st, bool *done) {
+    *done = false;
+    const sv_plan_opts *o = p->opts;
+    if ((o && (o->reg_bits > 0 || o->threads_per_block > 0 || o->epilogue == 1)) || !obs->dtab.ptr)
+        return SV_OK;
+    const int c128 = p->dtype == SV_C128, n = p->circuit->n_qubits, I = p->n_instances;
+    const int P = p->circuit->n_params, Pp = P > 0 ? P : 1;
+    const int rmax = c128 ? 3 : 4;
+    // below, the engine that forms its matrices in the same kernel is as fast
+    // (complex64, 8 and 9 qubits: 50-52 against 53-54 us) or a state is less
+    // than a warp
+    if (n < (c128 ? 7 : 10)) return SV_OK;
+    int R = std::max(2, n - 9);
+    while (R < rmax && R < n - 5 && ((int64_t)I << (n - R)) > (int64_t)ctx->sms * 512) ++R;
+    if (R > rmax) return SV_OK;
+    PlanEntry *pe = nullptr;
+    sv_status s = get_plan(ctx, *p->circuit, R, use_fusion(o), p->dtype, &pe);
+    if (s != SV_OK) return s;
+    if (!pe->one_per_bit || pe->host.stages.empty() || pe->dev.n_groups > 65535) return SV_OK;
+    // pairs of real states once single ones would share SMs
+    const bool real = pe->y_only && obs->dev.real;
+    const int kind = !real ? 0 : (I > ctx->sms ? 1 : 2);
+    const int n_states = kind == 1 ? (I + 1) / 2 : I;
+    if (c128 && n >= 11 && n_states < ctx->sms) {
+        // complex128 runs at 2 multiply-adds a clock and SM: few large states
+        // leave most SMs idle, as tile passes they use all of them.  Per group
+        // and amplitude about 23 multiply-adds (real: 5.5), per set of flipped
+        // qubits 4 (2); tile passes spread that with a third lost and about
+        // 250 us of launches.  12 qubits, 32 circuit-learning instances: 703
+        // us as tile passes, 1855 us on chip; 11 qubits, 12 MC-VQE references:
+        // 281 against 235 us.
+        const double w = (double)(int64_t(1) << n) *
+                         (pe->dev.n_groups * (real ? 5.5 : 23.0) + obs->dev.n_tgroups * (real ? 2.0 : 4.0));
+        const double us = w / (2.0 * 2000.0);  // one state on its SM
+        if (us * n_states / ctx->sms * 1.33 + 250.0 < us) {
+            TileCfg cfg{8, 2, 3, false};
+            while (cfg.t < 10 && ((int64_t)n_states << (n - cfg.t)) > 2 * ctx->sms) ++cfg.t;
+            *done = true;
+            return tiles_adjoint(ctx, p, theta, weights, energy_out, loss_out, grad_out, every, st,
+                                 nullptr, &cfg);
+        }
+    }
+    ChipShape sh{};
+    if (chip_shape(kind, n, R, c128, pe->dev.n_groups, P, pe->dev.n_stages, n_states, ctx->sms, &sh))
+        return SV_OK;
+    const void *drefs = nullptr;
+    s = get_array(ctx, p->refs, sizeof(int64_t) * I, &drefs);
+    if (s != SV_OK) return s;
+    void *scr = nullptr, *big = nullptr;
+    s = get_scratch(ctx, st, sizeof(double) * ((size_t)I * Pp + I), &scr);
+    if (s != SV_OK) return s;
+    s = get_big_scratch(ctx, st, group_buf(c128, pe->dev, (size_t)n_states, kind != 0).bytes, &big);
+    if (s != SV_OK) return s;
+    double *G = (double *)scr, *E = G + (size_t)I * Pp;
+    SlotSource src{};
+    src.mode = SLOTS_INSTANCES;
+    src.n_slots = I;
+    src.n_instances = I;
+    src.refs = (const int64_t *)drefs;
+    src.theta = theta;
+    src.inputs = p->inputs;
+    src.input_stride = p->input_stride;
+    const CostSource cs = cost_of(p, weights);
+    cudaError_t e = launch_chip_adjoint(c128, kind, sh, pe->dev, obs->dev, src, cs, big,
+                                        obs->dtab.ptr, G, E, st);
+    if (e != cudaSuccess) return cuda_fail(e, "on-chip adjoint launch");
+    e = launch_adjoint_combine(G, E, I, P, cs, energy_out, loss_out, grad_out, st);
+    if (e != cudaSuccess) return cuda_fail(e, "adjoint combine launch");
+    *done = true;
+    return SV_OK;
+}
+
 // The adjoint gradient with ctx->mu held (arguments checked by the caller).
 sv_status adjoint_locked(DeviceCtx *ctx, const sv_problem *p, const double *theta,
                          const double *weights, double *energy_out, double *loss_out,
@@ -1931,6 +2026,10 @@ sv_status adjoint_locked(DeviceCtx *ctx, const sv_problem *p, const double *thet
     ObsEntry *obs = nullptr;
     s = get_obs(ctx, *p->observable, p->circuit->n_qubits, p->dtype, &obs, st);
     if (s != SV_OK) return s;
+    bool done = false;
+    s = chip_adjoint(ctx, p, theta, weights, obs, energy_out, loss_out, grad_out, checkpoint_every,
+                     st, &done);
+    if (s != SV_OK || done) return s;
     BlockConst bc{};
     s = plan_and_shape(ctx, ONCHIP_ADJOINT, *p->circuit, p->dtype, I, p->opts, &plan, &sh,
                        find_tuned(ctx, p, ONCHIP_ADJOINT, I), obs, nullptr, &bc);

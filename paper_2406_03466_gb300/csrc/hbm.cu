@@ -172,6 +172,22 @@ __device__ __forceinline__ void quick_split(double2 a, double2 b, double2 *out) 
     out[3] = cconj(cmul(p0, p1));
 }
 
+// (c, s) of a group of Y rotations and Ry encodings, exactly (complex128);
+// false for any other member.
+__device__ bool y_group(const Program &p, int g, const SlotInfo &si, double2 &cs) {
+    const Group grp = p.groups[g];
+    cs = make_double2(1.0, 0.0);
+    for (int m = grp.m_begin; m < grp.m_end; ++m) {
+        const int kind = p.members[m].kind;
+        if (kind != M_RY && kind != M_ENC_RY_ASIN) return false;
+        double2 r[4];
+        member_matrix<double, double2>(p.members[m], si, r);
+        const double c = r[0].x, s = r[2].x;
+        cs = make_double2(fma(cs.x, c, -cs.y * s), fma(cs.x, s, cs.y * c));
+    }
+    return true;
+}
+
 // What the passes read of every state's groups (hbm.h: GroupBuf): the fused
 // 2x2 matrices and, without pair, their split forms; with pair entry k is
 // (first slot's, second slot's), and where both matrices are rotations their
@@ -179,15 +195,17 @@ __device__ __forceinline__ void quick_split(double2 a, double2 b, double2 *out) 
 // FP64 and rounded once, so that a pass's error is its own.  A pair's real
 // rotations are taken with c >= 0 (a state's sign is of no account to its
 // energy and its gradient).
-// L lanes per group (complex64).
+// kind: 0 complex, 1 pair, 2 one real slot per state (both components the
+// slot's).  L lanes per group (complex64).
 template <typename Real, int L>
 __global__ void __launch_bounds__(32)
-k_group_mats(Program p, SlotSource src, int pair, typename CT<Real>::T *out, double2 *split,
+k_group_mats(Program p, SlotSource src, int kind, typename CT<Real>::T *out, double2 *split,
              int64_t *refs, ClearList clear) {
     using C = typename CT<Real>::T;
     constexpr bool kQuick = std::is_same<Real, float>::value;
     pdl_trigger();
     pdl_wait();
+    const bool pair = kind == 1;
     const int G = p.n_groups, n_states = pair ? (src.n_slots + 1) / 2 : src.n_slots;
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t step = (int64_t)gridDim.x * blockDim.x;
@@ -202,7 +220,7 @@ k_group_mats(Program p, SlotSource src, int pair, typename CT<Real>::T *out, dou
         const int b = (int)(i / G), g = (int)(i % G);
         double2 d[4], u, v;
         C m[4];
-        if (!pair) {
+        if (kind == 0) {
             const SlotInfo si = resolve(src, b);
             if (kQuick && quick_group<L>(p, g, si, u, v)) {
                 d[0] = u;
@@ -218,9 +236,13 @@ k_group_mats(Program p, SlotSource src, int pair, typename CT<Real>::T *out, dou
         } else {
             double r[2][4];
             bool rot = true;
-            for (int c = 0; c < 2; ++c) {
-                const SlotInfo si = resolve(src, min(2 * b + c, src.n_slots - 1));
-                if (kQuick && quick_group<L>(p, g, si, u, v)) {
+            for (int c = 0; c < (pair ? 2 : 1); ++c) {
+                const SlotInfo si = resolve(src, pair ? min(2 * b + c, src.n_slots - 1) : b);
+                if (!kQuick && y_group(p, g, si, u)) {
+                    r[c][0] = r[c][3] = u.x;
+                    r[c][1] = -u.y;
+                    r[c][2] = u.y;
+                } else if (kQuick && quick_group<L>(p, g, si, u, v)) {
                     r[c][0] = r[c][3] = u.x;
                     r[c][1] = -v.x;
                     r[c][2] = v.x;
@@ -230,6 +252,8 @@ k_group_mats(Program p, SlotSource src, int pair, typename CT<Real>::T *out, dou
                 }
                 rot = rot && r[c][0] == r[c][3] && r[c][1] == -r[c][2];
             }
+            if (!pair)
+                for (int k = 0; k < 4; ++k) r[1][k] = r[0][k];
             for (int c = 0; c < 2 && rot; ++c) {
                 const double sg = r[c][0] < 0.0 ? -1.0 : 1.0, s = sg * r[c][2];
                 r[c][0] = -s / (1.0 + sg * r[c][0]);
@@ -245,10 +269,10 @@ k_group_mats(Program p, SlotSource src, int pair, typename CT<Real>::T *out, dou
 
 // Phase tables of the split stages, tabs[state][stage][0][r] = product of
 // the groups' q and tabs[state][stage][1][r] = product of their p over the
-// stage's register bits.  Products in FP64: a table entry multiplies whole
+// stage's register bits (every: of all stages).  Products in FP64: a table entry multiplies whole
 // slices of a state, so its rounding does not average out.
 template <typename Real>
-__global__ void k_phase_tables(Program p, int n_states, const double2 *split,
+__global__ void k_phase_tables(Program p, int n_states, const double2 *split, int every,
                                typename CT<Real>::T *tabs) {
     pdl_trigger();
     pdl_wait();
@@ -269,7 +293,7 @@ __global__ void k_phase_tables(Program p, int n_states, const double2 *split,
             if (post) f = cmul(f, e[op.group * 4 + 1 + b]);
             else if (b) f = cmul(f, e[op.group * 4 + 3]);
         }
-        if (!real && sg->op_end - sg->op_begin >= 2) tabs[x] = cmk<typename CT<Real>::T>(f.x, f.y);
+        if (every || (!real && sg->op_end - sg->op_begin >= 2)) tabs[x] = cmk<typename CT<Real>::T>(f.x, f.y);
     }
 }
 
@@ -504,24 +528,6 @@ __device__ __forceinline__ void kmat_bit(const C (&a)[1 << R], const C (&l)[1 <<
     }
 }
 
-// Partial sum over the lanes of NV values x[0..NV-1] (NV = 8 or 16):
-// afterwards x[m] (m < NV / 4) holds value 4 m + (lane & 3) summed over the
-// four lanes that differ in lane bits 0-1 (a reduce-scatter of two levels;
-// the kept half follows the lane bit).
-template <typename Real, int NV>
-__device__ __forceinline__ void warp_reduce_quad(Real (&x)[NV], int lane) {
-    constexpr unsigned full = 0xffffffffu;
-#pragma unroll
-    for (int j = 0, M = NV; j < 2; ++j, M >>= 1) {
-        const bool b = (lane >> j) & 1;
-#pragma unroll
-        for (int m = 0; m < M / 2; ++m) {
-            const Real keep = b ? x[2 * m + 1] : x[2 * m], give = b ? x[2 * m] : x[2 * m + 1];
-            x[m] = keep + __shfl_xor_sync(full, give, 1 << j);
-        }
-    }
-}
-
 // The one sum a group needs when its only rotation is its last member
 // (fmode md): 1: k3 (RY), 2: k2 (RX), 3: k0 - k1 (RZ), over the pairs of
 // register bit I.
@@ -694,49 +700,6 @@ __device__ __forceinline__ void stage_ops_rev(uint32_t ops, uint32_t modes, uint
     tile_ops_rev<C, Real, R, R - 1, NV, true, kMat>(ops, modes, sm, a, al, k);
 }
 
-// Sums of a split stage's group on register bit I at the point after its
-// rotation, before its phases p (a phase per group only turns K_01, and the
-// other groups' phases drop out), of psi = a and m = i lambda:
-//   k[0] = k0 - k1 = sum p0 . m0 - p1 . m1,  k[1] = k2 = sum p0 . m1 + p1 . m0,
-//   k[2] = k3 = sum Re(p0 conj l1) - Re(p1 conj l0)
-// (x . y as real 2-vectors; with i lambda in place of lambda the first two
-// are packed products).  k0 + k1 is of no account to a rotation's derivative.
-template <typename C, typename Real, int R, int I>
-__device__ __forceinline__ void split_sums(const C (&a)[1 << R], const C (&m)[1 << R], Real *k) {
-    if constexpr (std::is_same<C, float2>::value) {
-        uint64_t d0 = 0, d1 = 0, e0 = 0, e1 = 0;
-        float t0 = 0.f, t1 = 0.f;
-#pragma unroll
-        for (int r = 0; r < (1 << R); ++r) {
-            if (r & (1 << I)) continue;
-            const C p0 = a[r], p1 = a[r | (1 << I)], m0 = m[r], m1 = m[r | (1 << I)];
-            d0 = f2fma(f2of(p0), f2of(m0), d0);
-            d1 = f2fma(f2of(p1), f2of(m1), d1);
-            e0 = f2fma(f2of(p0), f2of(m1), e0);
-            e1 = f2fma(f2of(p1), f2of(m0), e1);
-            t0 = fmaR(p0.x, m1.y, fmaR(-p0.y, m1.x, t0));
-            t1 = fmaR(p1.y, m0.x, fmaR(-p1.x, m0.y, t1));
-        }
-        const float2 D0 = f2unpack(d0), D1 = f2unpack(d1), E0 = f2unpack(e0), E1 = f2unpack(e1);
-        k[0] = (D0.x + D0.y) - (D1.x + D1.y);
-        k[1] = (E0.x + E0.y) + (E1.x + E1.y);
-        k[2] = t0 + t1;
-    } else {
-        Real d = 0, e = 0, t = 0;
-#pragma unroll
-        for (int r = 0; r < (1 << R); ++r) {
-            if (r & (1 << I)) continue;
-            const C p0 = a[r], p1 = a[r | (1 << I)], m0 = m[r], m1 = m[r | (1 << I)];
-            d = fmaR(p0.x, m0.x, fmaR(p0.y, m0.y, fmaR(-p1.x, m1.x, fmaR(-p1.y, m1.y, d))));
-            e = fmaR(p0.x, m1.x, fmaR(p0.y, m1.y, fmaR(p1.x, m0.x, fmaR(p1.y, m0.y, e))));
-            t = fmaR(p0.x, m1.y, fmaR(-p0.y, m1.x, fmaR(p1.y, m0.x, fmaR(-p1.x, m0.y, t))));
-        }
-        k[0] = d;
-        k[1] = e;
-        k[2] = t;
-    }
-}
-
 template <typename C, typename Real, int R, int I>
 __device__ __forceinline__ void split_unrots(uint32_t ops, const C *sm, C (&a)[1 << R],
                                              C (&m)[1 << R], Real *k) {
@@ -790,22 +753,6 @@ __device__ __forceinline__ void split_rev(uint32_t ops, const C *sm, const C *ta
                 if (!one) a[j] = phase_mul(a[j], p[h]);
                 al[j] = one ? l : phase_mul(l, p[h]);
             }
-    }
-}
-
-// x[m] (m < 3) = value 4 m + (lane & 3) of the twelve, summed over the four
-// lanes that differ in lane bits 0-1 (warp_reduce_quad of twelve values).
-template <typename Real>
-__device__ __forceinline__ void warp_reduce_quad12(Real (&x)[12], int lane) {
-    constexpr unsigned full = 0xffffffffu;
-#pragma unroll
-    for (int j = 0, M = 12; j < 2; ++j, M >>= 1) {
-        const bool b = (lane >> j) & 1;
-#pragma unroll
-        for (int m = 0; m < M / 2; ++m) {
-            const Real keep = b ? x[2 * m + 1] : x[2 * m], give = b ? x[2 * m] : x[2 * m + 1];
-            x[m] = keep + __shfl_xor_sync(full, give, 1 << j);
-        }
     }
 }
 
@@ -1664,10 +1611,11 @@ template <typename K> cudaError_t allow_smem(K kernel, uint32_t bytes) {
     return e;
 }
 
-// Resident blocks of kernel k on the whole GPU, at most max_blocks.  The
+// Resident blocks of kernel k on the whole GPU (*full), at most max_blocks.  The
 // occupancy of a launch shape is a constant of the device: kept per thread,
 // since a call of a small state is launch after launch.
-template <typename K> int fill_blocks(K kernel, int threads, uint32_t smem, int64_t max_blocks) {
+template <typename K>
+int fill_blocks(K kernel, int threads, uint32_t smem, int64_t max_blocks, int *full = nullptr) {
     struct Seen {
         const void *kernel;
         int dev, threads, blocks;
@@ -1692,18 +1640,21 @@ template <typename K> int fill_blocks(K kernel, int threads, uint32_t smem, int6
         if (seen.size() >= 256) seen.clear();
         seen.push_back({(const void *)kernel, dev, threads, (int)b, smem});
     }
+    if (full) *full = (int)b;
     if (b > max_blocks) b = max_blocks;
     return b < 1 ? 1 : (int)b;
 }
 
-// Whether a pass over n_tiles tiles of 2^t amplitudes is launched as a
-// dependent of the one before: passes over at most 64 MiB, whose launch gaps
-// and descriptor work show.  Longer ones lose more than they gain: their
-// blocks then start wherever blocks of the pass before ended, on the other
-// die from the L2 that holds their tiles (20-qubit states, 512 MiB passes of
-// 200 us: 5833 against 5482 us).
-bool pass_dep(int c128, int t, int64_t n_tiles) {
-    return ((n_tiles << t) * (c128 ? 16 : 8)) <= (int64_t(64) << 20);
+// Whether a pass is launched as a dependent of the one before, which hides
+// its launch and its descriptor work.  Such blocks start wherever blocks of
+// the pass before end, packed onto few SMs when they do not fill the GPU: no
+// harm to a handful of FP32 blocks, but complex128 passes share one SM's FP64
+// unit then (12 qubits, 32 instances: 1200 against 800 us), and a half-filled
+// grid idles the other half.  Full grids over more than 64 MiB lose as well:
+// their tiles' L2 lines are on the other die (20-qubit states, 512 MiB a
+// pass: 5833 against 5482 us).
+bool pass_dep(int c128, int t, int64_t n_tiles, int blocks, int full) {
+    return !c128 && ((n_tiles << t) * 8) <= (int64_t(64) << 20) && (blocks <= 64 || blocks >= full);
 }
 
 int grid_1d(int64_t work, int threads) {
@@ -1737,13 +1688,13 @@ int grid_1d(int64_t work, int threads) {
     } while (0)
 
 cudaError_t launch_group_mats(int c128, const Program &p, const SlotSource &src, void *base,
-                              cudaStream_t st, bool pair, const ClearList &clear) {
-    const int n_states = pair ? (src.n_slots + 1) / 2 : src.n_slots;
-    const GroupBuf b = group_buf(c128, p, (size_t)n_states, pair);
+                              cudaStream_t st, int kind, const ClearList &clear, bool every) {
+    const int n_states = kind == 1 ? (src.n_slots + 1) / 2 : src.n_slots;
+    const GroupBuf b = group_buf(c128, p, (size_t)n_states, kind != 0);
     double2 *split = (double2 *)((char *)base + b.split);
     int64_t *refs = (int64_t *)((char *)base + b.refs);
     void *tabs = (char *)base + b.tabs;
-    // One warp a block: the FP64 work of a few thousand groups spreads over
+    // Not dependent launches (pass_dep).  One warp a block: the FP64 work of a few thousand groups spreads over
     // every SM (32 slots x 190 groups: 22 us in blocks of 128 threads).  Four
     // lanes a group while that fits the SMs' schedulers in one wave: the
     // latency of a group's loads and sines counts then, not their number.
@@ -1751,13 +1702,13 @@ cudaError_t launch_group_mats(int c128, const Program &p, const SlotSource &src,
     const bool wide = !c128 && groups * 4 <= 152 * 4 * 32;
     const int g = grid_1d(wide ? groups * 4 : groups, 32);
     cudaError_t e =
-        c128   ? launch_dep(k_group_mats<double, 1>, g, 32, 0, st, p, src, (int)pair, (double2 *)base, split, refs, clear)
-        : wide ? launch_dep(k_group_mats<float, 4>, g, 32, 0, st, p, src, (int)pair, (float2 *)base, split, refs, clear)
-               : launch_dep(k_group_mats<float, 1>, g, 32, 0, st, p, src, (int)pair, (float2 *)base, split, refs, clear);
-    if (e == cudaSuccess && !pair && p.n_stages > 0) {
+        c128   ? launch_dep_if(false, k_group_mats<double, 1>, g, 32, 0, st, p, src, kind, (double2 *)base, split, refs, clear)
+        : wide ? launch_dep_if(false, k_group_mats<float, 4>, g, 32, 0, st, p, src, kind, (float2 *)base, split, refs, clear)
+               : launch_dep_if(false, k_group_mats<float, 1>, g, 32, 0, st, p, src, kind, (float2 *)base, split, refs, clear);
+    if (e == cudaSuccess && kind == 0 && p.n_stages > 0) {
         const int gt = grid_1d(((int64_t)n_states * p.n_stages * 2) << p.R, 64);
-        e = c128 ? launch_dep(k_phase_tables<double>, gt, 64, 0, st, p, n_states, split, (double2 *)tabs)
-                 : launch_dep(k_phase_tables<float>, gt, 64, 0, st, p, n_states, split, (float2 *)tabs);
+        e = c128 ? launch_dep_if(false, k_phase_tables<double>, gt, 64, 0, st, p, n_states, split, (int)every, (double2 *)tabs)
+                 : launch_dep_if(false, k_phase_tables<float>, gt, 64, 0, st, p, n_states, split, (int)every, (float2 *)tabs);
     }
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
@@ -1828,8 +1779,9 @@ cudaError_t launch_tile_fwd(int c128, const TilePass &P, int n, int n_slots,
                       : (pass_all_real(P) ? k_tile_fwd<Real, RR, kReal> : k_tile_fwd<Real, RR, kAny>);
         cudaError_t e = allow_smem(k, smem);
         if (e != cudaSuccess) return e;
-        const int blocks = fill_blocks(k, threads, smem, max_blocks);
-        e = launch_dep_if(pass_dep(c128, P.t, (int64_t)n_slots << P.n_tile_bits), k, blocks, threads,
+        int full = 0;
+        const int blocks = fill_blocks(k, threads, smem, max_blocks, &full);
+        e = launch_dep_if(pass_dep(c128, P.t, (int64_t)n_slots << P.n_tile_bits, blocks, full), k, blocks, threads,
                           smem, st, P, n, n_slots, gm, (const C *)src, (C *)states, sp);
         if (e != cudaSuccess) return e;
     });
@@ -1860,8 +1812,9 @@ cudaError_t launch_tile_rev(int c128, const TilePass &P, int n, int n_slots,
         }
         cudaError_t e = allow_smem(k, smem);
         if (e != cudaSuccess) return e;
-        const int blocks = fill_blocks(k, threads, smem, max_blocks);
-        e = launch_dep_if(pass_dep(c128, P.t, (int64_t)n_slots << P.n_tile_bits), k, blocks, threads,
+        int full = 0;
+        const int blocks = fill_blocks(k, threads, smem, max_blocks, &full);
+        e = launch_dep_if(pass_dep(c128, P.t, (int64_t)n_slots << P.n_tile_bits, blocks, full), k, blocks, threads,
                        smem, st, P, n, n_slots, gm, (const C *)(psi_src ? psi_src : psi), (C *)psi, (C *)lam, rho_g, sp,
                        write_psi ? 1 : 0);
         if (e != cudaSuccess) return e;
@@ -1888,8 +1841,9 @@ cudaError_t launch_tile_h(int c128, const HPass &P, int n, int n_slots, const vo
     auto go = [&](auto k, auto *psi_t, auto *lam_t) -> cudaError_t {
         cudaError_t e = allow_smem(k, smem);
         if (e != cudaSuccess) return e;
-        const int blocks = fill_blocks(k, threads, smem, max_blocks);
-        return launch_dep_if(pass_dep(c128, P.t, (int64_t)n_slots << P.n_tile_bits), k, blocks,
+        int full = 0;
+        const int blocks = fill_blocks(k, threads, smem, max_blocks, &full);
+        return launch_dep_if(pass_dep(c128, P.t, (int64_t)n_slots << P.n_tile_bits, blocks, full), k, blocks,
                              threads, smem, st, P, n, n_slots, psi_t, lam_t, E, pair_rows);
     };
     auto pick2 = [&](auto rr, auto re, auto pr) -> cudaError_t {

@@ -45,14 +45,17 @@ inline GroupMats group_mats_of(const GroupBuf &b, const void *base, int stage0) 
     const char *p = (const char *)base;
     return GroupMats{p, p + b.tabs, (const double2 *)(p + b.split), b.G, b.n_stages, stage0, 0};
 }
+// kind: 0 complex states, 1 pairs, 2 one real state per slot (coefficients as
+// of a pair of the slot with itself).  every: phase tables of every stage (the
+// on-chip engine), not only of the passes' split stages.
 // Arrays of doubles set to zero on the way (sums that later kernels add to).
 struct ClearList {
     double *p[3];
     int64_t n[3];
 };
 cudaError_t launch_group_mats(int c128, const Program &p, const SlotSource &src, void *base,
-                              cudaStream_t st, bool pair = false,
-                              const ClearList &clear = ClearList{});
+                              cudaStream_t st, int kind = 0,
+                              const ClearList &clear = ClearList{}, bool every = false);
 // Zeroes the slot states and sets amplitude |ref> of each to 1.
 cudaError_t launch_init_states(int c128, void *states, int n, const SlotSource &src,
                                cudaStream_t st);
@@ -154,5 +157,21 @@ cudaError_t launch_apply_h_big(int c128, const Observable &o, int n, int n_rows,
 cudaError_t launch_group_grads(int c128, const Program &p, const SlotSource &src,
                                const double *rho_g, const CostSource &cs, const double *E,
                                double *slot_grads, cudaStream_t st);
+
+// On-chip adjoint of chip.cu.  kind: 0 complex, 1 pairs of real states, 2
+// single real states (circuits of Y rotations and CNOTs, real observable).
+// The plan has R register bits, sorted stages of at most one group a bit.
+struct ChipShape {
+    int32_t R, S, blocks;  // S states per block
+    uint32_t smem, off_rec, off_tb, off_slot, off_red, slot_bytes;
+    uint32_t o_coef, o_tabs, o_rw, o_grad;
+};
+const char *chip_shape(int kind, int n, int R, int c128, int G, int P, int n_stages, int n_states,
+                       int sms, ChipShape *out);
+// group_base: group_buf(...) bytes; dtab: the observable's diagonal tables.
+cudaError_t launch_chip_adjoint(int c128, int kind, const ChipShape &sh, const Program &p,
+                                const Observable &o, const SlotSource &src, const CostSource &cs,
+                                void *group_base, const void *dtab, double *slot_grads,
+                                double *slot_E, cudaStream_t st);
 
 }  // namespace svk

@@ -184,13 +184,24 @@ __global__ void k_ps_combine_dep(const double *E, int I, int P, CostSource c, do
 }
 
 // Adjoint combination: dL/dtheta = sum_i (weighted per-instance gradients).
-__global__ void k_adjoint_combine(const double *Gs, const double *E, int I, int P, CostSource c,
-                                  double *energy_out, double *loss_out, double *grad_out) {
+// A block sums 32 parameters, 8 instances of each in flight per step (one
+// thread per parameter waited for the loads of every instance in turn: 29 us
+// for 256 instances).
+__global__ void __launch_bounds__(256)
+k_adjoint_combine(const double *Gs, const double *E, int I, int P, CostSource c,
+                  double *energy_out, double *loss_out, double *grad_out) {
+    __shared__ double part_g[8][33];
     pdl_wait();
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    const int col = threadIdx.x & 31, row = threadIdx.x >> 5, k = blockIdx.x * 32 + col;
+    double g = 0.0;
     if (k < P) {
-        double g = 0.0;
-        for (int i = 0; i < I; ++i) g += Gs[(int64_t)i * P + k];
+#pragma unroll 4
+        for (int i = row; i < I; i += 8) g += Gs[(int64_t)i * P + k];
+    }
+    part_g[row][col] = g;
+    __syncthreads();
+    if (row == 0 && k < P) {
+        for (int r = 1; r < 8; ++r) g += part_g[r][col];
         grad_out[k] = g;
     }
     if (blockIdx.x == 0) {
@@ -244,6 +255,12 @@ const char *onchip_shape(int kind, int n, int n_groups, int n_params, int c128, 
         R = kind == ONCHIP_ADJOINT ? 3 : rmax;
         const int64_t want = (int64_t)num_sms * 4 * 32 * 2;
         while (R > 2 && (int64_t)n_slots * (int64_t(1) << (n > R ? n - R : 0)) < want) --R;
+        // complex128 issues one FP64 instruction of a warp in 16 clocks: a
+        // batch that leaves most SMs without a warp halves them once more (33
+        // circuits of 4 qubits: 30.2 -> 18.4 us)
+        if (c128 && R == 2 && kind == ONCHIP_ENERGY &&
+            ((int64_t)n_slots << (n > 2 ? n - 2 : 0)) < (int64_t)num_sms * 32)
+            R = 1;
     }
     if (R < 1 || R > rmax) return "reg_bits out of range for this kernel";
     if (R > n) R = n;
@@ -515,9 +532,7 @@ cudaError_t launch_ps_combine(const double *E, int I, int P, const CostSource &c
 cudaError_t launch_adjoint_combine(const double *G, const double *E, int I, int P,
                                    const CostSource &c, double *energy_out, double *loss_out,
                                    double *grad_out, cudaStream_t st) {
-    const int threads = 256;
-    int blocks = (P + threads - 1) / threads;
-    if (blocks < 1) blocks = 1;
+    const int threads = 256, blocks = P > 32 ? (P + 31) / 32 : 1;
     return launch_dep(k_adjoint_combine, blocks, threads, 0, st, G, E, I, P, c, energy_out, loss_out,
                       grad_out);
 }

@@ -437,6 +437,83 @@ __device__ __forceinline__ void set_stage_flags(const TilePass &P, uint4 *rec, c
     }
 }
 
+// Partial sum over the lanes of NV values x[0..NV-1] (NV = 8 or 16):
+// afterwards x[m] (m < NV / 4) holds value 4 m + (lane & 3) summed over the
+// four lanes that differ in lane bits 0-1 (a reduce-scatter of two levels;
+// the kept half follows the lane bit).
+template <typename Real, int NV>
+__device__ __forceinline__ void warp_reduce_quad(Real (&x)[NV], int lane) {
+    constexpr unsigned full = 0xffffffffu;
+#pragma unroll
+    for (int j = 0, M = NV; j < 2; ++j, M >>= 1) {
+        const bool b = (lane >> j) & 1;
+#pragma unroll
+        for (int m = 0; m < M / 2; ++m) {
+            const Real keep = b ? x[2 * m + 1] : x[2 * m], give = b ? x[2 * m] : x[2 * m + 1];
+            x[m] = keep + __shfl_xor_sync(full, give, 1 << j);
+        }
+    }
+}
+
+// Sums of a split stage's group on register bit I at the point after its
+// rotation, before its phases p (a phase per group only turns K_01, and the
+// other groups' phases drop out), of psi = a and m = i lambda:
+//   k[0] = k0 - k1 = sum p0 . m0 - p1 . m1,  k[1] = k2 = sum p0 . m1 + p1 . m0,
+//   k[2] = k3 = sum Re(p0 conj l1) - Re(p1 conj l0)
+// (x . y as real 2-vectors; with i lambda in place of lambda the first two
+// are packed products).  k0 + k1 is of no account to a rotation's derivative.
+template <typename C, typename Real, int R, int I>
+__device__ __forceinline__ void split_sums(const C (&a)[1 << R], const C (&m)[1 << R], Real *k) {
+    if constexpr (std::is_same<C, float2>::value) {
+        uint64_t d0 = 0, d1 = 0, e0 = 0, e1 = 0;
+        float t0 = 0.f, t1 = 0.f;
+#pragma unroll
+        for (int r = 0; r < (1 << R); ++r) {
+            if (r & (1 << I)) continue;
+            const C p0 = a[r], p1 = a[r | (1 << I)], m0 = m[r], m1 = m[r | (1 << I)];
+            d0 = f2fma(f2of(p0), f2of(m0), d0);
+            d1 = f2fma(f2of(p1), f2of(m1), d1);
+            e0 = f2fma(f2of(p0), f2of(m1), e0);
+            e1 = f2fma(f2of(p1), f2of(m0), e1);
+            t0 = fmaR(p0.x, m1.y, fmaR(-p0.y, m1.x, t0));
+            t1 = fmaR(p1.y, m0.x, fmaR(-p1.x, m0.y, t1));
+        }
+        const float2 D0 = f2unpack(d0), D1 = f2unpack(d1), E0 = f2unpack(e0), E1 = f2unpack(e1);
+        k[0] = (D0.x + D0.y) - (D1.x + D1.y);
+        k[1] = (E0.x + E0.y) + (E1.x + E1.y);
+        k[2] = t0 + t1;
+    } else {
+        Real d = 0, e = 0, t = 0;
+#pragma unroll
+        for (int r = 0; r < (1 << R); ++r) {
+            if (r & (1 << I)) continue;
+            const C p0 = a[r], p1 = a[r | (1 << I)], m0 = m[r], m1 = m[r | (1 << I)];
+            d = fmaR(p0.x, m0.x, fmaR(p0.y, m0.y, fmaR(-p1.x, m1.x, fmaR(-p1.y, m1.y, d))));
+            e = fmaR(p0.x, m1.x, fmaR(p0.y, m1.y, fmaR(p1.x, m0.x, fmaR(p1.y, m0.y, e))));
+            t = fmaR(p0.x, m1.y, fmaR(-p0.y, m1.x, fmaR(p1.y, m0.x, fmaR(-p1.x, m0.y, t))));
+        }
+        k[0] = d;
+        k[1] = e;
+        k[2] = t;
+    }
+}
+
+// x[m] (m < 3) = value 4 m + (lane & 3) of the twelve, summed over the four
+// lanes that differ in lane bits 0-1 (warp_reduce_quad of twelve values).
+template <typename Real>
+__device__ __forceinline__ void warp_reduce_quad12(Real (&x)[12], int lane) {
+    constexpr unsigned full = 0xffffffffu;
+#pragma unroll
+    for (int j = 0, M = 12; j < 2; ++j, M >>= 1) {
+        const bool b = (lane >> j) & 1;
+#pragma unroll
+        for (int m = 0; m < M / 2; ++m) {
+            const Real keep = b ? x[2 * m + 1] : x[2 * m], give = b ? x[2 * m] : x[2 * m + 1];
+            x[m] = keep + __shfl_xor_sync(full, give, 1 << j);
+        }
+    }
+}
+
 // Every op of pass P has a real matrix.
 __host__ __device__ inline bool pass_all_real(const TilePass &P) {
     const uint64_t all = P.n_ops >= 64 ? ~0ull : ((1ull << P.n_ops) - 1ull);

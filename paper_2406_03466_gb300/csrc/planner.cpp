@@ -575,6 +575,76 @@ int conjugate_by_cnots(const std::vector<std::pair<int, int>> &tail, uint64_t *x
     return sign;
 }
 
+namespace {
+
+// GF(2) rank of the low w bits of the vectors v.
+int low_rank(const std::vector<uint32_t> &v, int w) {
+    uint32_t bas[32] = {};
+    int r = 0;
+    for (uint32_t x : v) {
+        x &= (1u << w) - 1u;
+        for (int h = w - 1; h >= 0 && x; --h)
+            if ((x >> h) & 1u) {
+                if (!bas[h]) {
+                    bas[h] = x;
+                    ++r;
+                    break;
+                }
+                x ^= bas[h];
+            }
+    }
+    return r;
+}
+
+// A shared-memory address map of one exchange between stages: index bit b >= w
+// also flips the low address bits low[b] (invertible for any low).
+struct BankMap {
+    int w;
+    uint32_t low[32];
+    uint32_t operator()(uint32_t idx) const {
+        uint32_t a = idx;
+        for (int b = w; idx >> b; ++b)
+            if ((idx >> b) & 1u) a ^= low[b];
+        return a;
+    }
+};
+
+// The map of an exchange whose writing lanes differ by the index vectors wr
+// and whose reading lanes by rd (w each): both sets of 2^w lanes should hit
+// distinct banks.  Starts from the swizzle's fold, then draws maps; every
+// exchange rewrites its whole tile, so each can have a map of its own (with
+// one fold for all, up to a third of a pass's shared-memory wavefronts were
+// conflicts: the images of CNOT ladders are long runs, which it folds to
+// dependent vectors).
+BankMap pick_bank_map(int t, int w, const std::vector<uint32_t> &wr,
+                      const std::vector<uint32_t> &rd) {
+    BankMap best{}, m{};
+    int best_rank = -1;
+    uint64_t seed = 0x9e3779b97f4a7c15ull;
+    for (int attempt = 0; attempt < 256 && best_rank < 2 * w; ++attempt) {
+        m.w = w;
+        for (int b = w; b < t; ++b) {
+            if (attempt == 0) {
+                m.low[b] = 1u << (b % w);
+            } else {
+                seed = seed * 6364136223846793005ull + 1442695040888963407ull;
+                m.low[b] = (uint32_t)(seed >> 40) & ((1u << w) - 1u);
+            }
+        }
+        std::vector<uint32_t> a, c;
+        for (uint32_t v : wr) a.push_back(m(v));
+        for (uint32_t v : rd) c.push_back(m(v));
+        const int r = low_rank(a, w) + low_rank(c, w);
+        if (r > best_rank) {
+            best_rank = r;
+            best = m;
+        }
+    }
+    return best;
+}
+
+}  // namespace
+
 // Kernel descriptors of every pass of a tile plan (amplitudes of csz bytes).
 std::string build_tile_passes(const HostProgram &P, int csz, std::vector<TilePass> *out) {
     out->clear();
@@ -638,6 +708,30 @@ std::string build_tile_passes(const HostProgram &P, int csz, std::vector<TilePas
                 }
                 ++u;
             }
+        }
+        // Bank maps: exchange 0 is written by the tile load and read by the
+        // first stage, exchange k written by stage k - 1 and read by stage k,
+        // the last one read by the tile store (the reverse pass runs the same
+        // exchanges the other way).  The plan's vectors carry the swizzle,
+        // which undoes itself.
+        for (int e = 0; e <= tp.n_stages; ++e) {
+            const int lanes = std::min(w, pd.t - R);
+            uint32_t *wr = e == 0 ? tp.ldperm : tp.st[e - 1].stt;
+            uint32_t *rd = e == tp.n_stages ? tp.nat : tp.st[e].ldt;
+            auto plain = [&](uint32_t a) { return swizzle(a / (uint32_t)csz, w); };
+            std::vector<uint32_t> wl, rl;
+            for (int k = 0; k < lanes; ++k) {
+                wl.push_back(plain(wr[k]));
+                rl.push_back(plain(rd[k]));
+            }
+            const BankMap m = pick_bank_map(pd.t, w, wl, rl);
+            auto move = [&](uint32_t *v, int count) {
+                for (int k = 0; k < count; ++k) v[k] = m(plain(v[k])) * (uint32_t)csz;
+            };
+            move(wr, e == 0 ? pd.t : pd.t - R);
+            move(rd, e == tp.n_stages ? pd.t : pd.t - R);
+            if (e > 0) move(tp.st[e - 1].stq, R);
+            if (e < tp.n_stages) move(tp.st[e].ldq, R);
         }
         tp.n_ops = u;
         tp.all_single = 1;

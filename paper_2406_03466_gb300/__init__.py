@@ -149,8 +149,8 @@ def _check(status, where):
 
 def _stream(stream):
     import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:  # the raw handle: a Stream object costs 3 us of a 25 us call
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
     return ctypes.c_void_p(stream.cuda_stream)
 
 

@@ -1795,9 +1795,13 @@ sv_status sv_grad_param_shift_host(const sv_problem *p, const double *theta_host
     fc.P = P;
     fc.cost = cost_of(p, nullptr);
     fc.lp = E + B;
-    fc.loss_out = d + nP;
-    fc.grad_out = d + nP + 1;
-    fc.energy_out = d + 2 * nP + 1;
+    // on chip the assembly writes its results straight to the pinned buffer (a
+    // few hundred stores instead of a copy node behind it)
+    const bool chip = !wants_tiles(p->circuit->n_qubits, p->dtype, p->opts);
+    double *res = chip ? h : d;
+    fc.loss_out = res + nP;
+    fc.grad_out = res + nP + 1;
+    fc.energy_out = res + 2 * nP + 1;
     if (P > 0) std::memcpy(h, theta_host, sizeof(double) * P);
     auto copy_in = [&](cudaStream_t q) {
         return P > 0 ? cudaMemcpyAsync(d, h, sizeof(double) * P, cudaMemcpyHostToDevice, q)
@@ -1808,7 +1812,7 @@ sv_status sv_grad_param_shift_host(const sv_problem *p, const double *theta_host
     };
     EnergyLaunch L;
     L.valid = 0;
-    if (!wants_tiles(p->circuit->n_qubits, p->dtype, p->opts)) {
+    if (chip) {
         s = ps_energies_locked(ctx, p, d, E, B, st, &fc, 0, &L);
         if (s != SV_OK) return s;
     }
@@ -1837,8 +1841,7 @@ sv_status sv_grad_param_shift_host(const sv_problem *p, const double *theta_host
             cudaError_t e = launch_onchip_energy(L.c128, L.sh, L.prog, L.obs, L.src, L.E, st, L.dtab,
                                                  &fc, &L.bc);
             if (e != cudaSuccess) return cuda_fail(e, "param-shift energy launch");
-            SV_CUDA(copy_out(st));
-            if (!g) {  // record the same three steps once for later calls
+            if (!g) {  // record the same steps once for later calls
                 g.reset(new HostGraph());
                 if (!ctx->capture_stream)
                     SV_CUDA(cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking));
@@ -1848,8 +1851,7 @@ sv_status sv_grad_param_shift_host(const sv_problem *p, const double *theta_host
                 if (ok) {
                     ok = copy_in(cap) == cudaSuccess &&
                          launch_onchip_energy(L.c128, L.sh, L.prog, L.obs, L.src, L.E, cap, L.dtab,
-                                              &fc, &L.bc) == cudaSuccess &&
-                         copy_out(cap) == cudaSuccess;
+                                              &fc, &L.bc) == cudaSuccess;
                     ok = cudaStreamEndCapture(cap, &graph) == cudaSuccess && ok && graph;
                 }
                 if (ok) ok = cudaGraphInstantiate(&g->exec, graph, 0) == cudaSuccess;
@@ -2708,7 +2710,8 @@ sv_status sv_debug_wait_expiry(int32_t limit, sv_stream_t stream) {
 }
 
 sv_status sv_shutdown(void) {
-    svk::noalloc_forget();
+    svk::forget_smem_limits();
+    noalloc_forget();
     std::lock_guard<std::mutex> lk(g_mu);
     for (auto &kv : g_ctx) {
         int cur = 0;

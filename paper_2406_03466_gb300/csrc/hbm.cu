@@ -1596,6 +1596,11 @@ template <typename K> cudaError_t allow_smem(K kernel, uint32_t bytes);
 
 cudaError_t allow_smem_attr(const void *kernel, uint32_t bytes) { return allow_smem(kernel, bytes); }
 
+void forget_smem_limits() {
+    std::lock_guard<std::mutex> lk(g_smem_mu);
+    g_smem_limit.clear();
+}
+
 namespace {
 
 template <typename K> cudaError_t allow_smem(K kernel, uint32_t bytes) {

@@ -103,6 +103,8 @@ constexpr int SV_DEVERR_SWEEP_WAIT = 2;
 // Raises kernel's dynamic shared-memory limit to `bytes` (limits only grow;
 // no attribute change while a graph capture runs: fails instead).
 cudaError_t allow_smem_attr(const void *kernel, uint32_t bytes);
+// Forgets the limits set so far (a device reset drops them).
+void forget_smem_limits();
 // Forward pass P with every register stage applied as one dense 16 x 16
 // complex block on the tensor cores (tc.cu; complex64, R = 4, t = 11 or 12).
 // err: the device error word (bounded waits), or null.

@@ -16,6 +16,7 @@
 #include <algorithm>
 
 #include "engine.cuh"
+#include "hbm.h"
 #include "kernels.h"
 
 namespace svk {
@@ -232,8 +233,9 @@ template <typename T> T *kptr(void *p) { return reinterpret_cast<T *>(p); }
 
 uint32_t up16(size_t x) { return (uint32_t)((x + 15) & ~size_t(15)); }
 
+// (the limit only grows: no call once a launch of this size has run)
 template <typename K> cudaError_t prep(K kernel, uint32_t smem) {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return allow_smem_attr((const void *)kernel, smem);
 }
 
 }  // namespace

@@ -81,8 +81,8 @@ __device__ __forceinline__ double quick_sqrt(double x) {
     return x < 1e-30 && x >= 0.0 ? 0.0 : x * quick_rsqrt(x);
 }
 
-// Axis (M_RX, M_RY, M_RZ) and half-angle sine and cosine of one member; -1
-// when it is neither a rotation nor an encoding.
+// Axis (M_RX, M_RY, M_RZ) and half-angle sine and cosine of one member, or
+// M_X, M_H.
 __device__ int quick_member(const Member &mb, const SlotInfo &si, double &s, double &c) {
     if (mb.kind <= M_RZ) {
         double t = mb.angle;
@@ -104,23 +104,23 @@ __device__ int quick_member(const Member &mb, const SlotInfo &si, double &s, dou
         s = quick_sqrt(0.5 * (1.0 - u));
         return M_RZ;
     }
-    return -1;
+    s = c = mb.kind == M_H ? 0.70710678118654752440 : 1.0;
+    return mb.kind;
 }
 
-// The first column (a, b) of group g's matrix [[a, -conj(b)], [b, conj(a)]]
-// when its members are rotations and encodings only; false otherwise.  L
-// lanes (consecutive, all with the same g) share a group: each forms every
+// Group g's matrix as i^k [[a, -conj(b)], [b, conj(a)]]: returns k, the number
+// of its X and H members (-i X and -i H have determinant 1).  L lanes (consecutive, all with the same g) share a group: each forms every
 // L-th member, so a group's loads and sines are in flight together; all
 // multiply them.  Called by whole warps.
 template <int L>
-__device__ bool quick_group(const Program &p, int g, const SlotInfo &si, double2 &a, double2 &b) {
+__device__ int quick_group(const Program &p, int g, const SlotInfo &si, double2 &a, double2 &b) {
     const Group grp = p.groups[g];
     const int lane = threadIdx.x & (L - 1);
     a = make_double2(1.0, 0.0);
     b = make_double2(0.0, 0.0);
     int last = grp.m_end - grp.m_begin;  // the longest group of the warp
     for (int off = 16; off; off >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, off));
-    bool ok = true;
+    int turns = 0;
     for (int m0 = 0; m0 < last; m0 += L) {
         double ms = 0.0, mc = 1.0;
         int ax = M_RZ;  // past the end: the identity
@@ -131,7 +131,6 @@ __device__ bool quick_group(const Program &p, int g, const SlotInfo &si, double2
             const int axis = L > 1 ? __shfl_sync(0xffffffffu, ax, l, L) : ax;
             const double s = L > 1 ? __shfl_sync(0xffffffffu, ms, l, L) : ms;
             const double c = L > 1 ? __shfl_sync(0xffffffffu, mc, l, L) : mc;
-            ok = ok && axis >= 0;
             double2 na, nb;
             if (axis == M_RX) {  // (c a - i s b, c b - i s a)
                 na = make_double2(fma(s, b.y, c * a.x), fma(-s, b.x, c * a.y));
@@ -139,6 +138,14 @@ __device__ bool quick_group(const Program &p, int g, const SlotInfo &si, double2
             } else if (axis == M_RY) {  // (c a - s b, c b + s a)
                 na = make_double2(fma(-s, b.x, c * a.x), fma(-s, b.y, c * a.y));
                 nb = make_double2(fma(s, a.x, c * b.x), fma(s, a.y, c * b.y));
+            } else if (axis == M_X) {  // -i (b, a)
+                na = make_double2(b.y, -b.x);
+                nb = make_double2(a.y, -a.x);
+                ++turns;
+            } else if (axis == M_H) {  // -i s (a + b, a - b)
+                na = make_double2(s * (a.y + b.y), -s * (a.x + b.x));
+                nb = make_double2(s * (a.y - b.y), -s * (a.x - b.x));
+                ++turns;
             } else {  // ((c - i s) a, (c + i s) b)
                 na = make_double2(fma(s, a.y, c * a.x), fma(-s, a.x, c * a.y));
                 nb = make_double2(fma(-s, b.y, c * b.x), fma(s, b.x, c * b.y));
@@ -147,29 +154,36 @@ __device__ bool quick_group(const Program &p, int g, const SlotInfo &si, double2
             b = nb;
         }
     }
-    return ok;
+    return turns;
 }
 
-// split_form of [[a, -conj(b)], [b, conj(a)]]: there q = conj(p0 p1).
-__device__ __forceinline__ void quick_split(double2 a, double2 b, double2 *out) {
+// i^k v.
+__device__ __forceinline__ double2 turn(double2 v, int k) {
+    if (k & 2) v = make_double2(-v.x, -v.y);
+    return (k & 1) ? make_double2(-v.y, v.x) : v;
+}
+
+// split_form of i^k [[a, -conj(b)], [b, conj(a)]]: with a = c pa and b = s pb
+// there p0 = i^k pa, p1 = i^k pb and q = conj(pa pb).
+__device__ __forceinline__ void quick_split(double2 a, double2 b, int k, double2 *out) {
     const double c2 = fma(a.x, a.x, a.y * a.y), s2 = fma(b.x, b.x, b.y * b.y);
-    double2 p0 = make_double2(1.0, 0.0), p1 = p0;
+    double2 pa = make_double2(1.0, 0.0), pb = pa;
     double c = 0.0, s = 0.0;
     if (!(c2 < 1e-30)) {
         const double r = quick_rsqrt(c2);
         c = c2 * r;
-        p0 = make_double2(a.x * r, a.y * r);
+        pa = make_double2(a.x * r, a.y * r);
     }
     if (!(s2 < 1e-30)) {
         const double r = quick_rsqrt(s2);
         s = s2 * r;
-        p1 = make_double2(b.x * r, b.y * r);
+        pb = make_double2(b.x * r, b.y * r);
     }
     const double d = 1.0 + c, y = (double)(1.f / (float)d);  // 1 / d by one Newton step
     out[0] = make_double2(-s * (y * fma(-d, y, 2.0)), s);
-    out[1] = p0;
-    out[2] = p1;
-    out[3] = cconj(cmul(p0, p1));
+    out[1] = turn(pa, k);
+    out[2] = turn(pb, k);
+    out[3] = cconj(cmul(pa, pb));
 }
 
 // (c, s) of a group of Y rotations and Ry encodings, exactly (complex128);
@@ -222,12 +236,13 @@ k_group_mats(Program p, SlotSource src, int kind, typename CT<Real>::T *out, dou
         C m[4];
         if (kind == 0) {
             const SlotInfo si = resolve(src, b);
-            if (kQuick && quick_group<L>(p, g, si, u, v)) {
-                d[0] = u;
-                d[1] = make_double2(-v.x, v.y);
-                d[2] = v;
-                d[3] = cconj(u);
-                quick_split(u, v, split + i * 4);
+            if (kQuick) {
+                const int k = quick_group<L>(p, g, si, u, v);
+                d[0] = turn(u, k);
+                d[1] = turn(make_double2(-v.x, v.y), k);
+                d[2] = turn(v, k);
+                d[3] = turn(cconj(u), k);
+                quick_split(u, v, k, split + i * 4);
             } else {
                 group_matrix<double, double2, Real>(p, g, si, d);
                 split_form(d, split + i * 4);
@@ -242,7 +257,7 @@ k_group_mats(Program p, SlotSource src, int kind, typename CT<Real>::T *out, dou
                     r[c][0] = r[c][3] = u.x;
                     r[c][1] = -u.y;
                     r[c][2] = u.y;
-                } else if (kQuick && quick_group<L>(p, g, si, u, v)) {
+                } else if (kQuick && quick_group<L>(p, g, si, u, v) == 0) {
                     r[c][0] = r[c][3] = u.x;
                     r[c][1] = -v.x;
                     r[c][2] = v.x;
@@ -383,6 +398,8 @@ __device__ __forceinline__ void stage_mats(const TilePass &P, uint4 *rec, const 
         for (int x = tid; x < P.n_stages * 2 * NA; x += T)
             if (rec[2 * (x / (2 * NA)) + 1].w >> 16) tab[x] = kRev ? cconj(tabs[x]) : tabs[x];
     }
+    if constexpr (kMat == kAny)  // no shears, no flags
+        if (!has_plain_stage(P.n_stages, rec)) return;
     __syncthreads();
     if constexpr (kMat != kPair) {
         for (int x = tid; x < P.n_stages * R; x += T) {
@@ -769,46 +786,63 @@ __device__ void flush_acc(const TilePass &P, Real *acc, int wps, double *rho_g, 
                           const uint4 *rec, const typename CT<Real>::T *sm) {
     __syncthreads();
     if constexpr (kMat == kAny && !kSingle) {
-        for (int x = threadIdx.x; x < P.n_stages * R; x += blockDim.x) {
-            const int s = x / R, i = x % R;
+        // four threads a group, one per sum (whole warps: they exchange them)
+        const int items = P.n_stages * R * 4;
+        for (int x = threadIdx.x; (x & ~31) < items; x += blockDim.x) {
+            const int y = min(x, items - 1), s = y / (4 * R), i = (y >> 2) % R, c = y & 3;
             const uint32_t ob = (rec[2 * s].x >> (8 * i)) & 0xffu;
-            if (!(rec[2 * s + 1].w >> 16) || !(ob & 128u)) continue;
-            const int u = (int)(ob & 63u) - 1;
-            double k[3];
-            for (int c = 0; c < 3; ++c) {
-                k[c] = 0.0;
-                for (int w = 0; w < wps; ++w)
-                    for (int q = (3 * i + c) & 3; q < 32; q += 4) {
-                        Real &r = acc[(u * wps + w) * 32 + q];
-                        k[c] += (double)r;
-                        r = 0;
+            const bool on = x < items && (rec[2 * s + 1].w >> 16) && (ob & 128u);
+            const int u = max(0, (int)(ob & 63u) - 1);
+            double k = 0.0;
+            if (on && c < 3)
+                for (int w = 0; w < wps; ++w) {
+                    Real *r = acc + (u * wps + w) * 32 + ((3 * i + c) & 3);
+                    double ka = 0.0, kb = 0.0;
+#pragma unroll
+                    for (int q = 0; q < 32; q += 8) {
+                        ka += (double)r[q];
+                        kb += (double)r[q + 4];
+                        r[q] = r[q + 4] = 0;
                     }
-            }
-            if (k[0] == 0.0 && k[1] == 0.0 && k[2] == 0.0) continue;
+                    k += ka + kb;
+                }
+            const double k1 = __shfl_sync(0xffffffffu, k, 1, 4), k2 = __shfl_sync(0xffffffffu, k, 2, 4);
+            if (!on || c > 2) continue;
             const double fx = sm[4 * u + 1].x, fy = sm[4 * u + 1].y;  // p0 conj(p1)
-            const double re = 0.5 * (fx * k[2] - fy * k[1]), im = 0.5 * (fx * k[1] + fy * k[2]);
             // i K = [[i (k0 - k1) / 2, z], [-conj(z), -i (k0 - k1) / 2]]
             double *dst = rho_g + ((size_t)b * G + P.grp[u]) * 8;
-            atomicAdd(dst + 1, 0.5 * k[0]);
-            atomicAdd(dst + 7, -0.5 * k[0]);
-            atomicAdd(dst + 2, re);
-            atomicAdd(dst + 3, im);
-            atomicAdd(dst + 4, -re);
-            atomicAdd(dst + 5, im);
+            if (c == 0) {
+                atomicAdd(dst + 1, 0.5 * k);
+                atomicAdd(dst + 7, -0.5 * k);
+            } else if (c == 1) {
+                const double re = 0.5 * (fx * k2 - fy * k1);
+                atomicAdd(dst + 2, re);
+                atomicAdd(dst + 4, -re);
+            } else {
+                const double im = 0.5 * (fx * k1 + fy * k2);
+                atomicAdd(dst + 3, im);
+                atomicAdd(dst + 5, im);
+            }
         }
         __syncthreads();
+        if (!has_plain_stage(P.n_stages, rec)) return;
     }
     if constexpr (kMat == kPair) {
         for (int x = threadIdx.x; x < P.n_ops * 2; x += blockDim.x) {
             const int u = x >> 1, c = x & 1;
             if (!((P.param_mask >> u) & 1ull)) continue;
             double k = 0.0;
-            for (int w = 0; w < wps; ++w)
-                for (int q = c; q < 32; q += 2) {
-                    Real &r = acc[(u * wps + w) * 32 + q];
-                    k += (double)r;
-                    r = 0;
+            for (int w = 0; w < wps; ++w) {
+                Real *r = acc + (u * wps + w) * 32 + c;
+                double ka = 0.0, kb = 0.0;
+#pragma unroll
+                for (int q = 0; q < 32; q += 4) {
+                    ka += (double)r[q];
+                    kb += (double)r[q + 2];
+                    r[q] = r[q + 2] = 0;
                 }
+                k += ka + kb;
+            }
             if (k == 0.0) continue;
             double *dst = rho_g + ((size_t)(2 * b + c) * G + P.grp[u]) * 8;
             atomicAdd(dst + 2, 0.5 * k);

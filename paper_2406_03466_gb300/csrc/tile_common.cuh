@@ -146,6 +146,13 @@ __device__ __forceinline__ uint32_t read_stage_rec(const uint4 *rec, int s, uint
     return a.x;
 }
 
+// Whether some stage has ops and does not run in split form.
+__device__ __forceinline__ bool has_plain_stage(int n_stages, const uint4 *rec) {
+    bool plain = false;
+    for (int s = 0; s < n_stages; ++s) plain = plain || (rec[2 * s].x && !(rec[2 * s + 1].w >> 16));
+    return plain;
+}
+
 // The four entries of matrix u (32-byte aligned records) as two 16-byte loads.
 __device__ __forceinline__ void load_mat(const float2 *sm, int u, float2 &m0, float2 &m1,
                                          float2 &m2, float2 &m3) {

@@ -1947,10 +1947,7 @@ sv_status chip_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta,
     const int c128 = p->dtype == SV_C128, n = p->circuit->n_qubits, I = p->n_instances;
     const int P = p->circuit->n_params, Pp = P > 0 ? P : 1;
     const int rmax = c128 ? 3 : 4;
-    // below, the engine that forms its matrices in the same kernel is as fast
-    // (complex64, 8 and 9 qubits: 50-52 against 53-54 us) or a state is less
-    // than a warp
-    if (n < (c128 ? 7 : 10)) return SV_OK;
+    if (n < 7) return SV_OK;  // a state is less than a warp
     int R = std::max(2, n - 9);
     while (R < rmax && R < n - 5 && ((int64_t)I << (n - R)) > (int64_t)ctx->sms * 512) ++R;
     if (R > rmax) return SV_OK;
@@ -1958,9 +1955,28 @@ sv_status chip_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta,
     sv_status s = get_plan(ctx, *p->circuit, R, use_fusion(o), p->dtype, &pe);
     if (s != SV_OK) return s;
     if (!pe->one_per_bit || pe->host.stages.empty() || pe->dev.n_groups > 65535) return SV_OK;
-    // pairs of real states once single ones would share SMs
     const bool real = pe->y_only && obs->dev.real;
-    const int kind = !real ? 0 : (I > ctx->sms ? 1 : 2);
+    // Small circuits stay with the engine that forms its matrices in the same
+    // kernel: one or two launches less are worth more than cheaper stages.
+    // Measured, chip.cu against that engine (us):
+    //   real complex64, groups x amplitudes: 10 qubits, 40 groups (41 k) 41.3 /
+    //   41.3; 11 qubits, 22 (45 k) 41.3 / 39.5; 10, 50 (51 k) 45.4 / 47.8
+    //   complex complex64: 12 qubits, 36 groups 80 / 78, 13 qubits, 39 groups
+    //   115 / 128, 11 qubits, 44 groups 75 / 84; 10 qubits, 60 groups (61 k)
+    //   66.7 / 65.9, 80 groups (82 k) 79 / 95
+    //   the same with 256 states: 10 qubits, 30 groups 68 / 58, 40 groups 74 /
+    //   96; 12 qubits, 24 groups 82 / 115 (66 / 58 with 4 states)
+    //   complex complex128: 7 qubits, 7 groups 71 / 62, 14 groups 104 / 101, 28
+    //   groups 152 / 168; 8 qubits, 16 groups 107 / 111
+    const int64_t groups = pe->dev.n_groups, work = groups << n;
+    const bool many = I > ctx->sms;  // more than one state per SM
+    const bool gain = c128   ? real || work >= 2048
+                      : real ? work >= 48 * 1024
+                             : (groups >= 38 && (work >= 64 * 1024 || (n >= 10 && many))) ||
+                                   (n >= 12 && many);
+    if (!gain) return SV_OK;
+    // pairs of real states once single ones would share SMs
+    const int kind = !real ? 0 : (many ? 1 : 2);
     const int n_states = kind == 1 ? (I + 1) / 2 : I;
     if (c128 && n >= 11 && n_states < ctx->sms) {
         // complex128 runs at 2 multiply-adds a clock and SM: few large states

@@ -105,3 +105,32 @@ def test_chip_adjoint_many_instances(sv, dtype, real, n, instances):
     q = sv.Problem.from_spec(wl.Workload(**{**w.__dict__, "weights": wt.cpu().numpy()}), dtype)
     _, _, g2 = sv.sv_grad_adjoint(q, theta)
     close(g1.cpu(), g2.cpu(), 1e-12)
+
+
+@pytest.mark.parametrize("dtype,real,n,layers,instances", [
+    ("c64", True, 10, 4, 3), ("c64", True, 10, 5, 3), ("c64", True, 11, 2, 2), ("c64", True, 11, 3, 2),
+    ("c64", False, 12, 3, 2), ("c64", False, 11, 4, 2), ("c64", False, 10, 4, 152),
+    ("c64", False, 10, 4, 153), ("c64", False, 12, 2, 152), ("c64", False, 12, 2, 153),
+    ("c64", False, 13, 3, 3), ("c128", False, 7, 2, 3), ("c128", False, 7, 3, 3)])
+def test_default_route_matches_fixed_shape(sv, dtype, real, n, layers, instances):
+    """Both sides of the lines between the two on-chip engines: the default
+    route against the engine a fixed shape selects."""
+    import torch
+    rng = np.random.default_rng(100 * n + layers)
+    gates, p = [], 0
+    for _ in range(layers):
+        for q in range(n):
+            for op in (["RY"] if real else ["RX", "RZ"]):
+                gates.append(wl.Gate(op, target=q, param=p))
+                p += 1
+        gates += wl.cnot_ladder(n)
+    letters = rng.choice([0, 1, 3], size=(6, n)).astype(np.int8)
+    w = wl.Workload("route", n, gates, p, rng.uniform(-3, 3, p), letters, rng.normal(size=6),
+                    rng.integers(0, 1 << n, instances).astype(np.int64),
+                    weights=rng.uniform(0.2, 1, instances))
+    theta = torch.as_tensor(w.theta, dtype=torch.float64, device="cuda")
+    a = sv.sv_grad_adjoint(sv.Problem.from_spec(w, dtype), theta)
+    b = sv.sv_grad_adjoint(sv.Problem.from_spec(w, dtype, opts=sv.plan_opts(reg_bits=max(2, n - 9))), theta)
+    close(a[0].cpu(), b[0].cpu(), TOL[dtype]["E"])
+    close(a[1].cpu(), b[1].cpu(), TOL[dtype]["E"])
+    close(a[2].cpu(), b[2].cpu(), TOL[dtype]["G"])

@@ -260,7 +260,10 @@ sv_status sv_grad_param_shift_host(const sv_problem *problem, const double *thet
  * followed by such a restart writes only lambda).  0 = every pass, else
  * every 2nd, if that many stored states still let all instances run at
  * once in free device memory, else every 4th.
- * Uses library scratch of I * P doubles, plus for device-memory states
+ * Uses library scratch of I * P doubles, on chip also of the fused groups'
+ * matrices (without memory for these it runs the form that keeps them on
+ * chip; a call recorded into a graph keeps its buffer until sv_shutdown), plus
+ * for device-memory states
  * (2 + checkpoints) states per instance processed at once (instances are
  * processed in groups that fit in free device memory). */
 sv_status sv_grad_adjoint(const sv_problem *problem, const double *theta, const double *weights,

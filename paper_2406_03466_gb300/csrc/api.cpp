@@ -118,6 +118,8 @@ struct DeviceCtx {
     std::unordered_map<uint64_t, std::unique_ptr<ArrayEntry>> arrays;
     std::unordered_map<cudaStream_t, std::unique_ptr<DeviceBuf>> scratch;
     std::unordered_map<cudaStream_t, std::unique_ptr<DeviceBuf>> scratch_big;  // device-memory states
+    // what adjoints of on-chip sizes work in, the newest last
+    std::unordered_map<cudaStream_t, std::vector<std::unique_ptr<DeviceBuf>>> scratch_chip;
     // Phase timing of tile adjoints: per chunk, events before the forward,
     // H and reverse phases and after the reverse.
     bool timing = false;
@@ -561,6 +563,32 @@ sv_status get_big_scratch(DeviceCtx *ctx, cudaStream_t st, size_t bytes, void **
         s->bytes = bytes;
     }
     *out = s->ptr;
+    return SV_OK;
+}
+
+// Per-stream scratch of adjoints of on-chip sizes.  They may have been recorded
+// into a caller's graph, so an outgrown buffer is kept: each is at least twice
+// the one before, all together less than twice the newest.  *out stays null,
+// without an error, when the buffer would have to grow during stream capture or
+// memory is short: the caller then takes the engine that needs none.
+sv_status get_chip_scratch(DeviceCtx *ctx, cudaStream_t st, size_t bytes, void **out) {
+    auto &v = ctx->scratch_chip[st];
+    *out = nullptr;
+    if (v.empty() || v.back()->bytes < bytes) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        SV_CUDA(cudaStreamIsCapturing(st, &cap));
+        if (cap != cudaStreamCaptureStatusNone) return SV_OK;
+        std::unique_ptr<DeviceBuf> b(new DeviceBuf());
+        const size_t want = std::max(bytes, v.empty() ? (size_t)65536 : 2 * v.back()->bytes);
+        if (cudaMalloc(&b->ptr, want) != cudaSuccess) {
+            cudaGetLastError();
+            b->ptr = nullptr;
+            return SV_OK;
+        }
+        b->bytes = want;
+        v.push_back(std::move(b));
+    }
+    *out = v.back()->ptr;
     return SV_OK;
 }
 
@@ -1032,13 +1060,18 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     const size_t o_mats = o_ck + up((size_t)ncp * chunk * sb);
     const size_t o_rho = o_mats + up(mats_bytes(pe, (size_t)chunk, csz, pair));
     const size_t total = o_rho + up((size_t)chunk * per_state * G * 64);
-    void *big = nullptr;
-    s = get_big_scratch(ctx, st, total, &big);
+    void *big = nullptr, *scr = nullptr;
+    const size_t sums = sizeof(double) * ((size_t)I * Pp + I);
+    if (forced) {
+        s = get_chip_scratch(ctx, st, up(total) + sums, &big);
+        scr = (char *)big + up(total);
+    } else {
+        s = get_big_scratch(ctx, st, total, &big);
+        if (s == SV_OK) s = get_scratch(ctx, st, sums, &scr);
+    }
     if (s != SV_OK) return s;
+    if (!big) return fail(SV_ERR_OOM, "no scratch for the states");
     char *bb = (char *)big;
-    void *scr = nullptr;
-    s = get_scratch(ctx, st, sizeof(double) * ((size_t)I * Pp + I), &scr);
-    if (s != SV_OK) return s;
     double *Gs = (double *)scr, *Es = Gs + (size_t)I * Pp;
     const CostSource cs = cost_of(p, weights);
     ctx->last_states = n_states;
@@ -1992,9 +2025,12 @@ sv_status chip_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta,
         if (us * n_states / ctx->sms * 1.33 + 250.0 < us) {
             TileCfg cfg{8, 2, 3, false};
             while (cfg.t < 10 && ((int64_t)n_states << (n - cfg.t)) > 2 * ctx->sms) ++cfg.t;
-            *done = true;
-            return tiles_adjoint(ctx, p, theta, weights, energy_out, loss_out, grad_out, every, st,
-                                 nullptr, &cfg);
+            s = tiles_adjoint(ctx, p, theta, weights, energy_out, loss_out, grad_out, every, st,
+                              nullptr, &cfg);
+            *done = s != SV_ERR_OOM;
+            if (*done) return s;
+            ctx->last_every = 0;  // no memory for it: on chip after all
+            ctx->last_rev_bytes = 0;
         }
     }
     ChipShape sh{};
@@ -2003,12 +2039,11 @@ sv_status chip_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta,
     const void *drefs = nullptr;
     s = get_array(ctx, p->refs, sizeof(int64_t) * I, &drefs);
     if (s != SV_OK) return s;
-    void *scr = nullptr, *big = nullptr;
-    s = get_scratch(ctx, st, sizeof(double) * ((size_t)I * Pp + I), &scr);
-    if (s != SV_OK) return s;
-    s = get_big_scratch(ctx, st, group_buf(c128, pe->dev, (size_t)n_states, kind != 0).bytes, &big);
-    if (s != SV_OK) return s;
-    double *G = (double *)scr, *E = G + (size_t)I * Pp;
+    void *big = nullptr;
+    const size_t sums = (group_buf(c128, pe->dev, (size_t)n_states, kind != 0).bytes + 255) & ~size_t(255);
+    s = get_chip_scratch(ctx, st, sums + sizeof(double) * ((size_t)I * Pp + I), &big);
+    if (s != SV_OK || !big) return s;
+    double *G = (double *)((char *)big + sums), *E = G + (size_t)I * Pp;
     SlotSource src{};
     src.mode = SLOTS_INSTANCES;
     src.n_slots = I;

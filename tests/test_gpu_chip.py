@@ -134,3 +134,31 @@ def test_default_route_matches_fixed_shape(sv, dtype, real, n, layers, instances
     close(a[0].cpu(), b[0].cpu(), TOL[dtype]["E"])
     close(a[1].cpu(), b[1].cpu(), TOL[dtype]["E"])
     close(a[2].cpu(), b[2].cpu(), TOL[dtype]["G"])
+
+
+@pytest.mark.parametrize("dtype,n,instances", [("c64", 12, 160), ("c128", 8, 3), ("c128", 12, 3)])
+def test_recorded_adjoint_outlives_scratch_growth(sv, dtype, n, instances):
+    """A recorded call keeps its scratch when larger calls follow on the stream."""
+    import torch
+    w = workload(n, instances, False, 7 * n, False)
+    prob = sv.Problem.from_spec(w, dtype)
+    big = [sv.Problem.from_spec(workload(m, k, False, m, False), dtype) for m, k in ((n, 4 * instances), (14, 4))]
+    other = [torch.as_tensor(workload(m, 1, False, m, False).theta, dtype=torch.float64, device="cuda")
+             for m in (n, 14)]
+    theta = torch.as_tensor(w.theta, dtype=torch.float64, device="cuda")
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        sv.sv_grad_adjoint(prob, theta)
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            out = sv.sv_grad_adjoint(prob, theta)
+        for p, t in zip(big, other):
+            sv.sv_grad_adjoint(p, t)
+        theta.mul_(0.75)
+        g.replay()
+        want = sv.sv_grad_adjoint(prob, theta)
+        s.synchronize()
+        for a, b in zip(out, want):
+            close(a.cpu(), b.cpu(), TOL[dtype]["G"])

@@ -323,7 +323,7 @@ def adjoint_phases(sv, w, prob, theta, out, info, flush, stream, reps, step=None
     traffic = reverse_traffic(w, info["tile_bits"], reg_bits, last["checkpoint_every"])
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "traffic": traffic,
-            "kernel": f"k_tile_rev x {info['n_passes']} reverse tile passes of "
+            "kernel": f"k_tile_rev x {moved['passes']} reverse tile passes of "
                       f"2^{info['tile_bits']} amplitudes ({w.name}: {states} states of {n} "
                       f"qubits for {I} instances; "
                       "psi and lambda read and lambda written per pass, psi written "
@@ -423,20 +423,23 @@ def run_device_memory(args, sv, dev, stream, dist, world, rank):
     gps, t_dev = job_throughput(t_dev, args.steps, dist, dev)
     d = 0 if w.inputs is None else 1
     info = sv.sv_plan_info(sv.Circuit(w.n_qubits, w.gates, w.n_params, d), "c64", opts)
+    moved = sv.sv_last_moved()
     hinfo = sv.sv_h_plan_info(sv.PauliSum(w.n_qubits, w.pauli_letters, w.pauli_coeffs), "c64")
     result = {"metric": METRIC, "value": gps, "unit": "gradients/s", "n_gpus": world,
               "steps": args.steps, "warmup": args.warmup,
               "ms_per_step": 1e3 * t_dev / args.steps, "higher_is_better": True,
               "scaling": "weak", "vs_baseline": None, "dtype": "c64", "data": "synthetic",
-              "config": {"workload": device_workload_name(w), "tile_passes": info["n_passes"],
+              "config": {"workload": device_workload_name(w), "tile_passes": moved["passes"],
                          "tuned_tile": {"tile_bits": tile_bits, "reg_bits": R,
                                         "tensor_blocks": tc},
                          "h_passes": hinfo["n_passes"],
                          "l2": "states larger than L2; 256 MiB flush before each step",
                          "parallelism": f"replicas x{world}"},
-              # per adjoint: group matrices, |ref>, forward and reverse passes, the
-              # passes of lambda = H psi, per-slot gradients, combination
-              "gpu_launches": args.steps * (2 * info["n_passes"] + hinfo["n_passes"] + 4),
+              # per adjoint: group matrices (and phase tables of complex circuits),
+              # forward and reverse passes, the passes of lambda = H psi, per-slot
+              # gradients, combination
+              "gpu_launches": args.steps * (2 * moved["passes"] + hinfo["n_passes"] + 3
+                                            + (moved["states"] == w.n_instances)),
               "clocks": clk, "wall_s_timed_region": t_wall}
     if rank == 0:
         result["roofline"] = adjoint_phases(sv, w, prob, theta, out, info, flush, stream,
@@ -649,20 +652,21 @@ def run_uneven(args, sv, dev, stream, dist, world, rank):
     t_wall = time.perf_counter() - t_wall
     clk = clocks.stop()
     gps, t_dev = job_throughput(t_dev, args.steps * len(ws), dist, dev)
-    # algorithmic HBM bytes of one step: |ref> writes, forward passes (read +
-    # write), lambda = H psi passes, reverse passes (psi and lambda, read + write)
+    # HBM bytes of one step were every pass dense: forward passes (read + write),
+    # lambda = H psi passes, reverse passes (psi and lambda, read + write).  The
+    # sweeps leave out amplitudes that are still zero, so no fraction is given
     nbytes, launches, max_pass = 0, 0, 0
     for w in ws:
         circ = sv.Circuit(w.n_qubits, w.gates, w.n_params, 1)
         npass = sv.sv_plan_info(circ, "c64")["n_passes"]
         nh = sv.sv_h_plan_info(sv.PauliSum(w.n_qubits, w.pauli_letters, w.pauli_coeffs))["n_passes"]
         state = w.n_instances * (8 << w.n_qubits)
-        nbytes += state * (1 + 2 * npass + 2 + 3 * (nh - 1) + 4 * npass)
+        nbytes += state * (2 * npass + 2 + 3 * (nh - 1) + 4 * npass)
+        # group matrices, phase tables, per-slot gradients, combination
         launches += 4 + nh
         max_pass = max(max_pass, npass)
     launches += 2  # the two persistent sweeps (forward, reverse) of all circuits
     peak, src = measured_hbm_gbs()
-    achieved = nbytes * args.steps / t_dev / 1e9 / world
     result = {"metric": METRIC, "value": gps, "unit": "gradients/s", "n_gpus": world,
               "steps": args.steps, "warmup": args.warmup,
               "ms_per_step": 1e3 * t_dev / args.steps, "higher_is_better": True,
@@ -672,11 +676,11 @@ def run_uneven(args, sv, dev, stream, dist, world, rank):
                          "parallelism": f"replicas x{world}"},
               "gpu_launches": args.steps * launches,
               "clocks": clk, "wall_s_timed_region": t_wall,
-              "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                           "frac": achieved / peak, "traffic": None,
+              "roofline": {"bound": "hbm", "achieved": None, "peak": peak, "unit": "GB/s",
+                           "frac": None, "traffic": None,
                            "kernel": "whole step: persistent forward sweep (k_tile_sweep) + k_tile_h "
                                      "+ persistent reverse sweep of all circuits, one graph",
-                           "bytes_per_step": nbytes, "peak_source": src}}
+                           "dense_bytes_per_step": nbytes, "peak_source": src}}
     if rank == 0:
         th_host = [torch.as_tensor(w.theta, dtype=torch.float64).pin_memory() for w in ws]
         g_host = [torch.empty(w.n_params, dtype=torch.float64).pin_memory() for w in ws]

@@ -8,7 +8,8 @@
 //   k_adjoint  - forward pass, lambda = H psi, reverse sweep with the
 //                derivative of every rotation (paper's method evaluates
 //                gradients by parameter shift, Sec. 4.1; the adjoint sweep
-//                gives the same numbers from 2 states per circuit).
+//                gives the same numbers from 2 states per circuit);
+//                small circuits and fixed shapes, the others run chip.cu.
 // Products run in the state's precision (FP32 for complex64); every
 // reduction across amplitudes, threads or terms is accumulated in FP64.
 #include <cuda_runtime.h>

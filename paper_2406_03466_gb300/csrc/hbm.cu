@@ -210,11 +210,14 @@ __device__ bool y_group(const Program &p, int g, const SlotInfo &si, double2 &cs
 // rotations are taken with c >= 0 (a state's sign is of no account to its
 // energy and its gradient).
 // kind: 0 complex, 1 pair, 2 one real slot per state (both components the
-// slot's).  L lanes per group (complex64).
+// slot's).  y_only: every group is Y rotations and encodings, whose shears are
+// formed whatever their values are: the on-chip engine reads no other form,
+// and a slot whose matrix is NaN (an encoded input outside [-1, 1]) must leave
+// the other slot of its pair alone.  L lanes per group (complex64).
 template <typename Real, int L>
 __global__ void __launch_bounds__(32)
-k_group_mats(Program p, SlotSource src, int kind, typename CT<Real>::T *out, double2 *split,
-             int64_t *refs, ClearList clear) {
+k_group_mats(Program p, SlotSource src, int kind, bool y_only, typename CT<Real>::T *out,
+             double2 *split, int64_t *refs, ClearList clear) {
     using C = typename CT<Real>::T;
     constexpr bool kQuick = std::is_same<Real, float>::value;
     pdl_trigger();
@@ -265,7 +268,7 @@ k_group_mats(Program p, SlotSource src, int kind, typename CT<Real>::T *out, dou
                     group_matrix<double, double2, Real>(p, g, si, d);
                     for (int k = 0; k < 4; ++k) r[c][k] = d[k].x;
                 }
-                rot = rot && r[c][0] == r[c][3] && r[c][1] == -r[c][2];
+                rot = y_only || (rot && r[c][0] == r[c][3] && r[c][1] == -r[c][2]);
             }
             if (!pair)
                 for (int k = 0; k < 4; ++k) r[1][k] = r[0][k];
@@ -1740,10 +1743,11 @@ cudaError_t launch_group_mats(int c128, const Program &p, const SlotSource &src,
     const int64_t groups = (int64_t)n_states * std::max(1, p.n_groups);
     const bool wide = !c128 && groups * 4 <= 152 * 4 * 32;
     const int g = grid_1d(wide ? groups * 4 : groups, 32);
+    const bool y_only = every && kind != 0;  // (the on-chip engine's real kinds)
     cudaError_t e =
-        c128   ? launch_dep_if(false, k_group_mats<double, 1>, g, 32, 0, st, p, src, kind, (double2 *)base, split, refs, clear)
-        : wide ? launch_dep_if(false, k_group_mats<float, 4>, g, 32, 0, st, p, src, kind, (float2 *)base, split, refs, clear)
-               : launch_dep_if(false, k_group_mats<float, 1>, g, 32, 0, st, p, src, kind, (float2 *)base, split, refs, clear);
+        c128   ? launch_dep_if(false, k_group_mats<double, 1>, g, 32, 0, st, p, src, kind, y_only, (double2 *)base, split, refs, clear)
+        : wide ? launch_dep_if(false, k_group_mats<float, 4>, g, 32, 0, st, p, src, kind, y_only, (float2 *)base, split, refs, clear)
+               : launch_dep_if(false, k_group_mats<float, 1>, g, 32, 0, st, p, src, kind, y_only, (float2 *)base, split, refs, clear);
     if (e == cudaSuccess && kind == 0 && p.n_stages > 0) {
         const int gt = grid_1d(((int64_t)n_states * p.n_stages * 2) << p.R, 64);
         e = c128 ? launch_dep_if(false, k_phase_tables<double>, gt, 64, 0, st, p, n_states, split, (int)every, (double2 *)tabs)

@@ -159,10 +159,17 @@ __device__ SlotInfo resolve(const SlotSource &s, int b) {
 // ------------------------------------------------------- gate matrices
 
 // sin and cos of a / 2.  FP32: the half angle's rounding to float is put back
-// to first order, so the pair carries the rounding of the function only.
+// to first order, so the pair carries the rounding of the function only.  That
+// rounding grows with the angle, and with it the pair's distance from the unit
+// circle (its square / 2): beyond 512 (3e-5) whole turns come off first, 2 pi
+// as a sum of two doubles; what is still beyond (past 1e18) goes without.
 __device__ __forceinline__ void half_sincos(double a, float *s, float *c) {
-    const double h = 0.5 * a;
-    const float hi = (float)h, lo = (float)(h - (double)hi);
+    double h = 0.5 * a;
+    if (fabs(h) > 512.0) {
+        const double k = rint(h * 0.15915494309189535);
+        h = fma(k, -2.4492935982947064e-16, fma(k, -6.283185307179586, h));
+    }
+    const float hi = (float)h, lo = fabs(h) > 512.0 ? 0.f : (float)(h - (double)hi);
     float s0, c0;
     sincosf(hi, &s0, &c0);
     *s = __fmaf_rn(lo, c0, s0);

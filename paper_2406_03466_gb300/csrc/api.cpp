@@ -593,10 +593,15 @@ sv_status get_chip_scratch(DeviceCtx *ctx, cudaStream_t st, size_t bytes, void *
 }
 
 // Bytes a tile-pass call may claim: 80 % of what is free plus what its own
-// big scratch already holds.
-size_t big_budget(DeviceCtx *ctx, cudaStream_t st) {
+// big scratch already holds; of an on-chip size (chip), whose outgrown buffers
+// stay, 80 % of what is free or its newest buffer.
+size_t big_budget(DeviceCtx *ctx, cudaStream_t st, bool chip = false) {
     size_t fr = 0, tot = 0;
     cudaMemGetInfo(&fr, &tot);
+    if (chip) {
+        const auto &v = ctx->scratch_chip[st];
+        return std::max((size_t)(0.8 * (double)fr), v.empty() ? (size_t)0 : v.back()->bytes);
+    }
     auto it = ctx->scratch_big.find(st);
     const size_t have = (it != ctx->scratch_big.end() && it->second) ? it->second->bytes : 0;
     return (size_t)(0.8 * (double)fr) + have;
@@ -973,10 +978,13 @@ sv_status tiles_energies(DeviceCtx *ctx, const sv_problem *p, const double *thet
 // reduced matrices, per-slot gradients, then the sum over instances.
 // ddcl_target (device [2^n]) replaces lambda = H psi by the JS divergence's
 // lambda (data-driven circuit learning); the slot energies are then JS.
+// forced: the tile shape.  chip: an adjoint of an on-chip size, which works in
+// the scratch of those (get_chip_scratch).
 sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta,
                         const double *weights, double *energy_out, double *loss_out,
                         double *grad_out, int every, cudaStream_t st,
-                        const double *ddcl_target = nullptr, const TileCfg *forced = nullptr) {
+                        const double *ddcl_target = nullptr, const TileCfg *forced = nullptr,
+                        bool chip = false) {
     ctx->phase_used = 0;
     ctx->last_every = 0;
     ctx->last_rev_bytes = 0;
@@ -1029,7 +1037,7 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     const int G = pe->dev.n_groups;
     const int npass = (int)pe->tiles.size();
     const size_t csz = c128 ? 16 : 8, sb = csz << n;
-    const size_t budget = big_budget(ctx, st);
+    const size_t budget = big_budget(ctx, st, chip);
     const bool pair = real_pairs(pe, obs, I, cfg.tc);
     const int per_state = pair ? 2 : 1;  // instances
     const int n_states = (I + per_state - 1) / per_state;
@@ -1062,7 +1070,7 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     const size_t total = o_rho + up((size_t)chunk * per_state * G * 64);
     void *big = nullptr, *scr = nullptr;
     const size_t sums = sizeof(double) * ((size_t)I * Pp + I);
-    if (forced) {
+    if (chip) {
         s = get_chip_scratch(ctx, st, up(total) + sums, &big);
         scr = (char *)big + up(total);
     } else {
@@ -2026,7 +2034,7 @@ sv_status chip_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta,
             TileCfg cfg{8, 2, 3, false};
             while (cfg.t < 10 && ((int64_t)n_states << (n - cfg.t)) > 2 * ctx->sms) ++cfg.t;
             s = tiles_adjoint(ctx, p, theta, weights, energy_out, loss_out, grad_out, every, st,
-                              nullptr, &cfg);
+                              nullptr, &cfg, true);
             *done = s != SV_ERR_OOM;
             if (*done) return s;
             ctx->last_every = 0;  // no memory for it: on chip after all

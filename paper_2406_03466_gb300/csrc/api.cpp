@@ -82,7 +82,8 @@ struct PlanEntry {
 struct HPlanEntry {
     HostHPlan host;
     DeviceBuf buf;
-    std::vector<HPass> passes;  // with device pointers
+    std::vector<HPass> passes;
+    uint32_t smem = 0;  // the largest pass's (tile_h_smem)  // with device pointers
 };
 
 struct ObsEntry {
@@ -665,7 +666,8 @@ sv_status get_hplan(ObsEntry *obs, int n, sv_dtype dt, HPlanEntry **out,
             if (!err.empty()) return fail(SV_ERR_ARG, "observable: " + err);
             ho = &moved;
         }
-        std::string err = plan_h_passes(*ho, t, dt == SV_C128 ? 3 : 4, &e->host);
+        std::string err = plan_h_passes(*ho, t, dt == SV_C128 ? 3 : 4, dt == SV_C128 ? 16 : 8,
+                                        &e->host);
         if (!err.empty()) return fail(SV_ERR_ARG, "observable: " + err);
         const HostHPlan &h = e->host;
         Packer pk;
@@ -684,6 +686,7 @@ sv_status get_hplan(ObsEntry *obs, int n, sv_dtype dt, HPlanEntry **out,
             P.classes = (const HClass *)(base + oc) + h.c_begin[i];
             P.terms = (const HTerm *)(base + ot) + h.t_begin[i];
             P.rows = (const HRow *)(base + orw) + h.r_begin[i];
+            e->smem = std::max(e->smem, tile_h_smem(dt == SV_C128, P));
             e->passes.push_back(P);
         }
         slot = std::move(e);
@@ -810,6 +813,7 @@ sv_status problem_plan(DeviceCtx *ctx, const sv_problem *p, const TileCfg &cfg, 
     s = get_hplan(obs, n, p->dtype, &hw, &(*out)->host);
     if (s == SV_OK) s = get_hplan(obs, n, p->dtype, &hc, &cut->host);
     if (s != SV_OK) return s;
+    if (hc->smem > kHSmemBlock) return SV_OK;  // the wider strings would not run
     // In bytes moved an amplitude (complex64): a pass 16 forward and 24 in
     // reverse, an H pass 24, a group whose partners come from global memory 8.
     // A row of Z masks is one multiply-add an amplitude: half a byte's time
@@ -1004,6 +1008,12 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     } else {
         s = get_obs(ctx, *p->observable, n, dt, &obs, st);
         if (s == SV_OK) s = problem_plan(ctx, p, cfg, obs, &pe);
+        if (s == SV_OK && chip) {  // the on-chip engines take any number of terms
+            HPlanEntry *hp = nullptr;
+            s = get_hplan(obs, n, dt, &hp, &pe->host);
+            if (s == SV_OK && hp->smem > kHSmemBlock)
+                s = fail(SV_ERR_UNSUPPORTED, "observable too large for an H pass");
+        }
     }
     if (s != SV_OK) return s;
     if (ddcl_target) {
@@ -2035,9 +2045,9 @@ sv_status chip_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta,
             while (cfg.t < 10 && ((int64_t)n_states << (n - cfg.t)) > 2 * ctx->sms) ++cfg.t;
             s = tiles_adjoint(ctx, p, theta, weights, energy_out, loss_out, grad_out, every, st,
                               nullptr, &cfg, true);
-            *done = s != SV_ERR_OOM;
+            *done = s != SV_ERR_OOM && s != SV_ERR_UNSUPPORTED;
             if (*done) return s;
-            ctx->last_every = 0;  // no memory for it: on chip after all
+            ctx->last_every = 0;  // no memory for it, or an H pass too large: on chip after all
             ctx->last_rev_bytes = 0;
         }
     }
@@ -2637,7 +2647,7 @@ sv_status sv_h_plan_info(const sv_pauli_sum *h, sv_dtype dt, int32_t *n_passes,
     std::string err = plan_observable(*h, h->n_qubits, swz_bits(dt), &ho);
     const int t = h_tile_bits(h->n_qubits, dt);
     HostHPlan hp;
-    if (err.empty()) err = plan_h_passes(ho, t, dt == SV_C128 ? 3 : 4, &hp);
+    if (err.empty()) err = plan_h_passes(ho, t, dt == SV_C128 ? 3 : 4, dt == SV_C128 ? 16 : 8, &hp);
     if (!err.empty()) return fail(SV_ERR_ARG, "observable: " + err);
     if (n_passes) *n_passes = (int32_t)hp.passes.size();
     if (tile_bits) *tile_bits = t;

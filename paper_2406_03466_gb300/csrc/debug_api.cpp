@@ -116,7 +116,7 @@ sv_status sv_debug_h_passes(const sv_pauli_sum *h, int32_t tile_bits, int32_t co
     HostObservable ho;
     std::string err = plan_observable(*h, h->n_qubits, 4, &ho);
     HostHPlan hp;
-    if (err.empty()) err = plan_h_passes(ho, tile_bits, coalesce_bits, &hp);
+    if (err.empty()) err = plan_h_passes(ho, tile_bits, coalesce_bits, coalesce_bits <= 3 ? 16 : 8, &hp);
     if (!err.empty()) return SV_ERR_ARG;
     counts[0] = (int32_t)hp.passes.size();
     counts[1] = (int32_t)hp.groups.size();

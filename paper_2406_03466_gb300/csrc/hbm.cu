@@ -1865,15 +1865,6 @@ cudaError_t launch_tile_rev(int c128, const TilePass &P, int n, int n_slots,
     return cudaGetLastError();
 }
 
-uint32_t tile_h_smem(int c128, const HPass &P) {
-    const uint32_t csz = c128 ? 16u : 8u;
-    const uint32_t row_vals = (1u << h_reg_bits(P.t)) * (P.real ? 1u : 2u);
-    return 3u * (csz << P.t) + (uint32_t)P.n_rows * (row_vals * (csz / 2u) + (uint32_t)sizeof(HRow)) +
-           (uint32_t)P.n_groups * (uint32_t)sizeof(HGroup) +
-           (uint32_t)P.n_classes * (csz + 8u + (uint32_t)sizeof(HClass)) +
-           (uint32_t)P.n_terms * (uint32_t)sizeof(HTerm) + 32u * 8u + 16u;
-}
-
 cudaError_t launch_tile_h(int c128, const HPass &P, int n, int n_slots, const void *psi, void *lam,
                           double *E, int64_t max_blocks, cudaStream_t st, int pair_rows) {
     const uint32_t smem = tile_h_smem(c128, P);

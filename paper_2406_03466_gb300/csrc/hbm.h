@@ -131,7 +131,6 @@ cudaError_t launch_tile_sweep(int c128, int R, bool rev, const SweepTask *tasks,
 // One tile pass of lambda = H psi (lam may be null: energies only); adds this
 // pass's part of <psi|H|psi> to E[slot] (zero E before the first pass).
 // pair_rows > 0: pairs of real states whose E has pair_rows entries.
-uint32_t tile_h_smem(int c128, const HPass &P);
 cudaError_t launch_tile_h(int c128, const HPass &P, int n, int n_slots, const void *psi, void *lam,
                           double *E, int64_t max_blocks, cudaStream_t st, int pair_rows = 0);
 // Data-driven circuit learning: js[r] = JS(target | |psi_r|^2) (zeroed here

@@ -742,7 +742,7 @@ std::string build_tile_passes(const HostProgram &P, int csz, std::vector<TilePas
     return "";
 }
 
-std::string plan_h_passes(const HostObservable &h, int tile_bits, int coalesce_bits,
+std::string plan_h_passes(const HostObservable &h, int tile_bits, int coalesce_bits, int csz,
                           HostHPlan *out) {
     const int n = h.n, t = tile_bits;
     if (t < coalesce_bits + 1 || t > n || t > kTileBitsMax) return "bad tile_bits for H passes";
@@ -776,25 +776,8 @@ std::string plan_h_passes(const HostObservable &h, int tile_bits, int coalesce_b
         plan.push_back(tk);
         pending.swap(rest);
     }
-    // A later pass of one or two groups costs more than they do as far groups
-    // of the first: reading partners moves 8 bytes an amplitude and group
-    // (whole 128-byte runs), a pass reads psi, reads lambda and writes it (24
-    // bytes) and is a launch of its own.  At most kFarTerms terms' worth, so
-    // that the first pass's records stay small beside its tiles.
-    constexpr int kFarTerms = 96;
-    int moved = 0;
-    for (size_t i = 1; i < plan.size();) {
-        int terms = 0;
-        for (int gi : plan[i].near) terms += h.tgroups[gi].t_end - h.tgroups[gi].t_begin;
-        if (plan[i].near.size() > 2 || !plan[i].far.empty() || moved + terms > kFarTerms) {
-            ++i;
-            continue;
-        }
-        moved += terms;
-        plan[0].far.insert(plan[0].far.end(), plan[i].near.begin(), plan[i].near.end());
-        plan.erase(plan.begin() + i);
-    }
-    for (const Taken &tk : plan) {
+    // Appends one pass's descriptor, groups, classes, rows and terms.
+    auto build = [&](const Taken &tk, HostHPlan *out) {
         uint32_t L = tk.L;
         std::vector<int> taken = tk.near;
         taken.insert(taken.end(), tk.far.begin(), tk.far.end());
@@ -889,7 +872,41 @@ std::string plan_h_passes(const HostObservable &h, int tile_bits, int coalesce_b
         P.n_terms = (int)out->terms.size() - t0;
         P.n_rows = (int)out->rows.size() - r0;
         out->passes.push_back(P);
+    };
+    auto first_smem = [&](const Taken &tk) {
+        HostHPlan one;
+        build(tk, &one);
+        return tile_h_smem(csz == 16, one.passes[0]);
+    };
+    // A later pass of one or two groups costs more than they do as far groups
+    // of the first: reading partners moves 8 bytes an amplitude and group
+    // (whole 128-byte runs), a pass reads psi, reads lambda and writes it (24
+    // bytes) and is a launch of its own.  At most kFarTerms terms' worth, so
+    // that the first pass's records stay small beside its tiles, and no group
+    // that would push the first pass past a block's shared memory.  (Keeping
+    // it below that of two blocks an SM as well costs more than the second
+    // block gives: 350 random terms over 16 qubits, complex128, energies 1795
+    // against 1503 us; 250 over 14, complex64, 189 against 170 us.)
+    constexpr int kFarTerms = 96;
+    int moved = 0;
+    for (size_t i = 1; i < plan.size();) {
+        int terms = 0;
+        for (int gi : plan[i].near) terms += h.tgroups[gi].t_end - h.tgroups[gi].t_begin;
+        if (plan[i].near.size() > 2 || !plan[i].far.empty() || moved + terms > kFarTerms) {
+            ++i;
+            continue;
+        }
+        Taken wider = plan[0];
+        wider.far.insert(wider.far.end(), plan[i].near.begin(), plan[i].near.end());
+        if (first_smem(wider) > kHSmemBlock) {
+            ++i;
+            continue;
+        }
+        moved += terms;
+        plan[0] = std::move(wider);
+        plan.erase(plan.begin() + i);
     }
+    for (const Taken &tk : plan) build(tk, out);
     out->g_begin.push_back((int)out->groups.size());
     out->c_begin.push_back((int)out->classes.size());
     out->t_begin.push_back((int)out->terms.size());

@@ -88,7 +88,8 @@ struct HostHPlan {
     std::vector<HTerm> terms;
     std::vector<HRow> rows;
 };
-std::string plan_h_passes(const HostObservable &h, int tile_bits, int coalesce_bits,
+// csz: bytes of an amplitude.
+std::string plan_h_passes(const HostObservable &h, int tile_bits, int coalesce_bits, int csz,
                           HostHPlan *out);
 
 // Returns "" on success, otherwise the reason the circuit was rejected.

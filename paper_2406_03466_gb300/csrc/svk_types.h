@@ -233,6 +233,17 @@ struct HPass {
 // threads for t >= 12 (R = 4), fewer below (at least 32 threads).
 inline int h_reg_bits(int t) { return t >= 12 ? 4 : (t == 11 ? 3 : 2); }
 
+// Shared memory of one block of the H-pass kernel, and the most a block can have.
+inline uint32_t tile_h_smem(int c128, const HPass &P) {
+    const uint32_t csz = c128 ? 16u : 8u;
+    const uint32_t row_vals = (1u << h_reg_bits(P.t)) * (P.real ? 1u : 2u);
+    return 3u * (csz << P.t) + (uint32_t)P.n_rows * (row_vals * (csz / 2u) + (uint32_t)sizeof(HRow)) +
+           (uint32_t)P.n_groups * (uint32_t)sizeof(HGroup) +
+           (uint32_t)P.n_classes * (csz + 8u + (uint32_t)sizeof(HClass)) +
+           (uint32_t)P.n_terms * (uint32_t)sizeof(HTerm) + 32u * 8u + 16u;
+}
+constexpr uint32_t kHSmemBlock = 227u * 1024u;
+
 // GF(2)-linear swizzle of a shared-memory amplitude index: the low `w` bits
 // are XORed with the fold of all higher w-bit chunks.  w = 4 for 8-byte
 // amplitudes (16 per 128-byte wavefront), 3 for 16-byte amplitudes.

@@ -905,7 +905,8 @@ sv_status tiles_forward(DeviceCtx *ctx, const PlanEntry *pe, int R, sv_dtype dt,
         const TilePass &tp = passes[i];
         const int64_t tiles = (int64_t)n_states << tp.n_tile_bits;
         const uint32_t smem = tile_fwd_smem(c128, tp);
-        if (smem > 220u * 1024u) return fail(SV_ERR_UNSUPPORTED, "tile pass needs too much shared memory");
+        if (smem - tile_table_bytes(c128, tp, false) > kPassSmem)
+            return fail(SV_ERR_UNSUPPORTED, "tile pass needs too much shared memory");
         void *out = states;
         if (ck && every > 0 && (i + 1) % every == 0 && i + 1 < passes.size())
             out = (char *)ck + ((i + 1) / every - 1) * sbytes;
@@ -1143,7 +1144,8 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
             const TilePass &tp = passes[i];
             const int64_t tiles = (int64_t)states << tp.n_tile_bits;
             const uint32_t smem = tile_rev_smem(c128, tp);
-            if (smem > 220u * 1024u) return fail(SV_ERR_UNSUPPORTED, "reverse pass needs too much shared memory");
+            if (smem - tile_table_bytes(c128, tp, true) > kPassSmem)
+                return fail(SV_ERR_UNSUPPORTED, "reverse pass needs too much shared memory");
             // psi after this pass is needed only if the next reverse pass
             // un-computes from it (it restarts from a stored state otherwise)
             const bool write_psi = i > 0 && !(i % every == 0 && i < npass);
@@ -1332,13 +1334,16 @@ sv_status multi_adjoint(DeviceCtx *ctx, const sv_problem *problems, int np,
     for (int rev = 0; rev < 2; ++rev) {
         std::vector<int> task_of(np * (size_t)max_pass, -1);
         long long tickets = 0;
+        uint32_t plain = 0;  // shared memory without phase tables
         for (int k = 0; k < max_pass; ++k)
             for (int j = 0; j < np; ++j) {
                 const MultiProblem &m = mp[j];
                 if (k >= m.npass) continue;
                 const int pi = rev ? m.npass - 1 - k : k;
                 const TilePass &tp = m.tiles[pi];
-                sw[rev].smem = std::max(sw[rev].smem, tile_sweep_smem(c128, rev != 0, tp));
+                const uint32_t need = tile_sweep_smem(c128, rev != 0, tp);
+                sw[rev].smem = std::max(sw[rev].smem, need);
+                plain = std::max(plain, need - tile_table_bytes(c128, tp, rev != 0, true));
                 SweepTask T{};
                 T.n = m.n;
                 T.n_slots = m.I;
@@ -1357,7 +1362,7 @@ sv_status multi_adjoint(DeviceCtx *ctx, const sv_problem *problems, int np,
         w.n_tasks = (int)tasks[rev].size();
         w.n_tickets = tickets;
         if (w.n_tasks == 0) continue;
-        if (w.smem > 220u * 1024u) return fail(SV_ERR_UNSUPPORTED, "uneven batch: pass needs too much shared memory");
+        if (plain > kPassSmem) return fail(SV_ERR_UNSUPPORTED, "uneven batch: pass needs too much shared memory");
         const int per_sm = tile_sweep_blocks_per_sm(c128, cfg.R, rev != 0, w.smem, threads);
         if (per_sm < 1) return fail(SV_ERR_UNSUPPORTED, "uneven batch: pass kernel does not fit an SM");
         // resident blocks only: every block that waits holds no ticket of the

@@ -1789,14 +1789,14 @@ Sparse sparse_pass(TilePass *P, uint32_t support, const int64_t *refs, bool init
     return sp;
 }
 
-// Phase tables of the split stages (kernels of kind kAny).
-static uint32_t phase_table_bytes(int c128, const TilePass &P, bool any) {
-    return any ? (uint32_t)P.n_stages * ((c128 ? 32u : 16u) << P.R) : 0u;
+uint32_t tile_table_bytes(int c128, const TilePass &P, bool rev, bool any) {
+    const bool read = any || (!pass_all_real(P) && !(rev && P.all_single));
+    return read ? (uint32_t)P.n_stages * ((c128 ? 32u : 16u) << P.R) : 0u;
 }
 
 uint32_t tile_fwd_smem(int c128, const TilePass &P, bool any) {
     const uint32_t csz = c128 ? 16u : 8u, T = 1u << (P.t - P.R);
-    const uint32_t tab = phase_table_bytes(c128, P, any || !pass_all_real(P));
+    const uint32_t tab = tile_table_bytes(c128, P, false, any);
     return 2u * (csz << P.t) + (uint32_t)P.n_stages * (T * 8u + 32u) + (uint32_t)P.n_ops * 4u * csz + tab;
 }
 
@@ -1805,7 +1805,7 @@ constexpr int kOneBufStages = 6;
 
 uint32_t tile_rev_smem(int c128, const TilePass &P, int bufs, bool any) {
     const uint32_t csz = c128 ? 16u : 8u, rsz = c128 ? 8u : 4u, T = 1u << (P.t - P.R);
-    const uint32_t tab = phase_table_bytes(c128, P, any || !pass_all_real(P));
+    const uint32_t tab = tile_table_bytes(c128, P, true, any);
     return 2u * (uint32_t)bufs * (csz << P.t) + (uint32_t)P.n_stages * (T * 8u + 32u) + (uint32_t)P.n_ops * 4u * csz +
            tab + (uint32_t)P.n_ops * T * rsz;
 }

@@ -76,6 +76,12 @@ struct Sparse {
 // The sparse form of pass P when the amplitudes' bits in `support` (an index
 // mask) are the ones that may differ from ref; sets P's tile count.
 Sparse sparse_pass(TilePass *P, uint32_t support, const int64_t *refs, bool init);
+// Phase tables of the split stages in that shared memory (reverse passes of
+// one sum a group have none): at most 4 KB, on top of kPassSmem.
+uint32_t tile_table_bytes(int c128, const TilePass &P, bool rev, bool any = false);
+// Largest shared memory of a pass without its phase tables; with them it is
+// still within the 227 KB of a block.
+constexpr uint32_t kPassSmem = 220u * 1024u;
 // Shared memory of one block of the forward / reverse kernels of pass P.
 // (any: of a kernel that takes complex and real passes alike).
 uint32_t tile_fwd_smem(int c128, const TilePass &P, bool any = false);

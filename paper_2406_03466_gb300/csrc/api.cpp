@@ -1270,6 +1270,9 @@ sv_status multi_adjoint(DeviceCtx *ctx, const sv_problem *problems, int np,
         key = mix64(key, mix64(hash_circuit(*p->circuit), hash_observable(*p->observable)));
         key = mix64(key, (uint64_t)p->n_instances);
         key = mix64(key, (uint64_t)p->cost);
+        // what the plan takes from the options beside the tile shape
+        key = mix64(key, (uint64_t)use_fusion(p->opts) | (uint64_t)use_relabel(p->opts) << 1 |
+                             (uint64_t)(p->opts && p->opts->tile_bits > 0) << 2);
         for (int i = 0; i < p->n_instances; ++i) key = mix64(key, (uint64_t)p->refs[i]);
         for (const void *ptr : {(const void *)theta[j], (const void *)(E_out ? E_out[j] : nullptr),
                                 (const void *)(L_out ? L_out[j] : nullptr), (const void *)G_out[j],
@@ -1278,7 +1281,7 @@ sv_status multi_adjoint(DeviceCtx *ctx, const sv_problem *problems, int np,
             key = mix64(key, (uint64_t)(uintptr_t)ptr);
         key = mix64(key, (uint64_t)p->input_stride);
     }
-    key = mix64(key, mix64((uint64_t)dt, (uint64_t)(cfg.t * 8 + cfg.R)));
+    key = mix64(key, mix64((uint64_t)dt, (uint64_t)((cfg.c * 32 + cfg.t) * 8 + cfg.R)));
     std::unique_ptr<MultiGraph> &g = ctx->graphs[key];
     if (g && g->exec) {
         SV_CUDA(cudaGraphLaunch(g->exec, st));

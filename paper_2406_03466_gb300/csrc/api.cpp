@@ -751,9 +751,10 @@ int *device_err(DeviceCtx *ctx) {
 constexpr int kTileEnergyKey = 10 + ONCHIP_ENERGY, kTileAdjointKey = 10 + ONCHIP_ADJOINT;
 
 // tn: a tuned tile shape (R = register bits, tpb = 2^(t - R) threads), used
-// when opts leave tile_bits and reg_bits at zero.
+// when opts leave tile_bits and reg_bits at zero.  n_def: the qubit count that
+// the default register bits go by (a batch: its smallest circuit's; 0: n).
 sv_status tile_cfg(int n, sv_dtype dt, const sv_plan_opts *o, TileCfg *cfg,
-                   const Tuned *tn = nullptr) {
+                   const Tuned *tn = nullptr, int n_def = 0) {
     if (tn && tn->R > 0 && (!o || (o->tile_bits <= 0 && o->reg_bits <= 0))) {
         sv_plan_opts t{};
         if (o) t = *o;
@@ -774,7 +775,7 @@ sv_status tile_cfg(int n, sv_dtype dt, const sv_plan_opts *o, TileCfg *cfg,
     // 8 amplitudes per thread for larger complex128 states: fewer stages, and
     // the FP64 unit, not the warps in flight, is the limit (19-qubit MC-VQE
     // adjoint 2206 against 2580 us, 16-qubit circuit learning 5474 against 6134)
-    const int r_def = dt == SV_C128 ? (n >= 16 && t >= 10 ? 3 : 2) : 4;
+    const int r_def = dt == SV_C128 ? ((n_def > 0 ? n_def : n) >= 16 && t >= 10 ? 3 : 2) : 4;
     int R = (o && o->reg_bits > 0) ? o->reg_bits : std::min(r_def, t - 5);
     if (R < 2 || R > rmax) return fail(SV_ERR_ARG, "reg_bits for tile passes must be 2..4 (2..3 complex128)");
     if (t - R > 8) R = t - 8;
@@ -1254,7 +1255,7 @@ sv_status multi_adjoint(DeviceCtx *ctx, const sv_problem *problems, int np,
     const size_t csz = c128 ? 16 : 8;
     TileCfg cfg{};
     uint64_t key = mix64(0x5e17ull, (uint64_t)np);
-    int n_min = problems[0].circuit->n_qubits;  // one default shape: the smallest circuit's
+    int n_min = problems[0].circuit->n_qubits;  // one default width for all
     for (int j = 1; j < np; ++j) n_min = std::min(n_min, problems[j].circuit->n_qubits);
     for (int j = 0; j < np; ++j) {
         const sv_problem *p = &problems[j];
@@ -1262,7 +1263,7 @@ sv_status multi_adjoint(DeviceCtx *ctx, const sv_problem *problems, int np,
         if (!wants_tiles(p->circuit->n_qubits, dt, p->opts))
             return fail(SV_ERR_UNSUPPORTED, "uneven batch: every problem must take the tile path");
         TileCfg c{};
-        sv_status s = tile_cfg(n_min, dt, p->opts, &c);
+        sv_status s = tile_cfg(p->circuit->n_qubits, dt, p->opts, &c, nullptr, n_min);
         if (s != SV_OK) return s;
         if (j == 0) cfg = c;
         else if (c.t != cfg.t || c.R != cfg.R || c.c != cfg.c)

@@ -1,6 +1,7 @@
 """Batches of circuits (sv_grad_adjoint_multi) and the options of their problems:
 a call with other options plans and records its own graph instead of replaying
-that of an earlier call on the same pointers.  Tolerances as in test_gpu_parity."""
+that of an earlier call on the same pointers, and problems whose tile shapes
+differ are refused.  Tolerances as in test_gpu_parity."""
 import numpy as np
 import pytest
 
@@ -46,3 +47,24 @@ def test_options_plan_anew(sv, opts):
         close(outs[0][1].cpu(), E, 1e-5)
     states = 2 * w.n_instances * 8 << w.n_qubits  # psi and lambda
     assert held[0] >= states and held[1] < states and held[2] >= states
+
+
+def test_mixed_tile_shapes_are_refused(sv):
+    """A fixed tile of 2^10 amplitudes is one of 2^9 for the 9-qubit problem."""
+    import torch
+    ws = [wl.mcvqe(n, 1, "nn", n_refs=2) for n in (9, 14)]
+    probs = [sv.Problem.from_spec(w, "c64", opts=sv.plan_opts(tile_bits=10, reg_bits=4)) for w in ws]
+    thetas = [torch.as_tensor(w.theta, dtype=torch.float64, device="cuda") for w in ws]
+    for k in (1, -1):
+        with pytest.raises(Exception, match="one tile shape"):
+            sv.sv_grad_adjoint_multi(probs[::k], thetas[::k])
+
+
+def test_default_shapes_of_complex128_agree(sv):
+    """14 and 17 qubits alone have different default register bits."""
+    import torch
+    ws = [wl.mcvqe(n, 1, "nn", n_refs=2) for n in (14, 17)]
+    thetas = [torch.as_tensor(w.theta, dtype=torch.float64, device="cuda") for w in ws]
+    outs = sv.sv_grad_adjoint_multi([sv.Problem.from_spec(w, "c128") for w in ws], thetas)
+    for w, (_, e_, _) in zip(ws, outs):
+        close(e_.cpu(), oracle.instance_energies(w), 1e-12)

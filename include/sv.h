@@ -453,7 +453,9 @@ sv_status sv_last_adjoint_states(int32_t *states, int32_t *passes, int64_t *forw
  * the batched parameter-shift energy kernel (kinds bit 1) and of the adjoint
  * kernel (kinds bit 2) on this problem and remembers the fastest per problem
  * structure; later calls whose opts leave reg_bits and threads_per_block at
- * zero use it.  For states in device memory (tile passes) it times tile
+ * zero use it.  An adjoint's shapes are timed against the engines that
+ * sv_grad_adjoint takes without tuning where they apply, which choose their own
+ * shapes; the fastest is remembered.  For states in device memory (tile passes) it times tile
  * shapes instead — 2^t-amplitude tiles with R register bits, t in 9..12 —
  * for the instance energies (bit 1) and the adjoint gradient (bit 2), and
  * later calls whose opts leave tile_bits and reg_bits at zero use them.

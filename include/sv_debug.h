@@ -55,6 +55,12 @@ sv_status sv_debug_h_passes(const sv_pauli_sum *h, int32_t tile_bits, int32_t co
  * SV_ERR_TIMEOUT).  limit: 1..2^20. */
 sv_status sv_debug_wait_expiry(int32_t limit, sv_stream_t stream);
 
+/* The engine of the last adjoint gradient on the current device (0 none, 1 the
+ * one-kernel on-chip engine, 2 to 4 the on-chip engine of complex, paired and
+ * single real states, 5 tile passes), its register bits and its threads per
+ * block.  Any out-pointer may be NULL. */
+sv_status sv_debug_last_adjoint(int32_t *engine, int32_t *reg_bits, int32_t *threads);
+
 /* The relabeling tile plan without the circuit's trailing CNOTs: passes kept,
  * the CNOTs left out (control, target pairs in time order; tail holds
  * 2 n_gates entries) and the layout, as sv_debug_tile_passes gives it. */

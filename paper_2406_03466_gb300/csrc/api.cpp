@@ -107,11 +107,26 @@ struct ArrayEntry {
 struct Tuned {
     int R = 0, tpb = 0, epi = 0;
     int tc = 0;  // tile passes: forward stages as tensor-core blocks
+    bool chip = false;  // on-chip sizes: the engines of chip_adjoint, of which R and tpb are
     float us = 0.f;
+};
+
+// The engine and launch shape of an adjoint gradient.
+enum AdjointEngine {
+    ADJ_NONE = 0,
+    ADJ_FUSED,    // onchip.cu
+    ADJ_COMPLEX,  // chip.cu, by kind of state
+    ADJ_PAIR,
+    ADJ_REAL,
+    ADJ_TILES     // tile passes
+};
+struct AdjointRun {
+    int engine = ADJ_NONE, R = 0, tpb = 0;
 };
 
 struct DeviceCtx {
     std::mutex mu;
+    AdjointRun last_run;  // of the last adjoint gradient
     int sms = 152;
     std::unordered_map<uint64_t, Tuned> tuned;
     std::unordered_map<uint64_t, std::unique_ptr<PlanEntry>> plans;
@@ -526,6 +541,7 @@ uint64_t tune_key(const sv_problem *p, int kind, int n_slots) {
 }
 
 const Tuned *find_tuned(DeviceCtx *ctx, const sv_problem *p, int kind, int n_slots) {
+    if (ctx->tuned.empty()) return nullptr;
     auto it = ctx->tuned.find(tune_key(p, kind, n_slots));
     return it == ctx->tuned.end() ? nullptr : &it->second;
 }
@@ -1096,6 +1112,7 @@ sv_status tiles_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta
     const CostSource cs = cost_of(p, weights);
     ctx->last_states = n_states;
     ctx->last_passes = npass;
+    ctx->last_run = {ADJ_TILES, cfg.R, 1 << (cfg.t - cfg.R)};
     int64_t moved_fwd = 0;
     ctx->moved_rev = 0;
     for (int64_t c0 = 0; c0 < I; c0 += chunk * per_state) {
@@ -2085,6 +2102,7 @@ sv_status chip_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta,
     if (e != cudaSuccess) return cuda_fail(e, "on-chip adjoint launch");
     e = launch_adjoint_combine(G, E, I, P, cs, energy_out, loss_out, grad_out, st);
     if (e != cudaSuccess) return cuda_fail(e, "adjoint combine launch");
+    ctx->last_run = {kind == 0 ? ADJ_COMPLEX : (kind == 1 ? ADJ_PAIR : ADJ_REAL), sh.R, sh.S << (n - sh.R)};
     *done = true;
     return SV_OK;
 }
@@ -2106,13 +2124,17 @@ sv_status adjoint_locked(DeviceCtx *ctx, const sv_problem *p, const double *thet
     ObsEntry *obs = nullptr;
     s = get_obs(ctx, *p->observable, p->circuit->n_qubits, p->dtype, &obs, st);
     if (s != SV_OK) return s;
-    bool done = false;
-    s = chip_adjoint(ctx, p, theta, weights, obs, energy_out, loss_out, grad_out, checkpoint_every,
-                     st, &done);
-    if (s != SV_OK || done) return s;
+    const Tuned *tn = find_tuned(ctx, p, ONCHIP_ADJOINT, I);
+    if (!tn || tn->chip) {
+        bool done = false;
+        s = chip_adjoint(ctx, p, theta, weights, obs, energy_out, loss_out, grad_out,
+                         checkpoint_every, st, &done);
+        if (s != SV_OK || done) return s;
+        tn = nullptr;
+    }
     BlockConst bc{};
-    s = plan_and_shape(ctx, ONCHIP_ADJOINT, *p->circuit, p->dtype, I, p->opts, &plan, &sh,
-                       find_tuned(ctx, p, ONCHIP_ADJOINT, I), obs, nullptr, &bc);
+    s = plan_and_shape(ctx, ONCHIP_ADJOINT, *p->circuit, p->dtype, I, p->opts, &plan, &sh, tn, obs,
+                       nullptr, &bc);
     // A deep circuit whose per-group reduced-matrix buffers leave no room for
     // one slot in shared memory runs as tile passes instead (a state of
     // n >= 7 qubits has at least two tiles' worth of amplitudes to split).
@@ -2142,6 +2164,7 @@ sv_status adjoint_locked(DeviceCtx *ctx, const sv_problem *p, const double *thet
     if (e != cudaSuccess) return cuda_fail(e, "adjoint launch");
     e = launch_adjoint_combine(G, E, I, P, cs, energy_out, loss_out, grad_out, st);
     if (e != cudaSuccess) return cuda_fail(e, "adjoint combine launch");
+    ctx->last_run = {ADJ_FUSED, sh.R, sh.S * sh.Ts};
     return SV_OK;
 }
 
@@ -2554,6 +2577,19 @@ sv_status sv_autotune(const sv_problem *p, const double *theta, int32_t kinds,
     cudaEvent_t e0, e1;
     SV_CUDA(cudaEventCreate(&e0));
     SV_CUDA(cudaEventCreate(&e1));
+    auto time_us = [&](auto &&call, float *us) -> sv_status {  // the fastest of three
+        *us = 1e30f;
+        for (int rep = 0; rep < 3; ++rep) {
+            SV_CUDA(cudaEventRecord(e0, st));
+            SV_CUDA(call());
+            SV_CUDA(cudaEventRecord(e1, st));
+            SV_CUDA(cudaEventSynchronize(e1));
+            float ms = 0.f;
+            SV_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+            *us = std::min(*us, ms * 1e3f);
+        }
+        return SV_OK;
+    };
     const int rmax = p->dtype == SV_C128 ? 3 : 4;
     const int tpbs[] = {32, 64, 128, 256, 512};
     for (int kind : {ONCHIP_ENERGY, ONCHIP_ADJOINT}) {
@@ -2591,25 +2627,49 @@ sv_status sv_autotune(const sv_problem *p, const double *theta, int32_t kinds,
                                : launch_onchip_adjoint(p->dtype == SV_C128, sh, plan->dev, obs->dev,
                                                        src, cs, G, E2, st, &bc, obs->dtab.ptr);
                 };
-                if (run() != cudaSuccess) {
+                // an adjoint candidate is a whole call: with its combination
+                auto call = [&]() {
+                    cudaError_t e = run();
+                    if (e == cudaSuccess && kind == ONCHIP_ADJOINT)
+                        e = launch_adjoint_combine(G, E2, I, P, cs, E2 + I, nullptr, E, st);
+                    return e;
+                };
+                if (call() != cudaSuccess) {
                     cudaGetLastError();
                     continue;
                 }
-                float tbest = 1e30f;
-                for (int rep = 0; rep < 3; ++rep) {
-                    SV_CUDA(cudaEventRecord(e0, st));
-                    SV_CUDA(run());
-                    SV_CUDA(cudaEventRecord(e1, st));
-                    SV_CUDA(cudaEventSynchronize(e1));
-                    float ms = 0.f;
-                    SV_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-                    if (ms < tbest) tbest = ms;
-                }
-                if (tbest * 1e3f < best.us) {
-                    best.us = tbest * 1e3f;
+                float us = 0.f;
+                s = time_us(call, &us);
+                if (s != SV_OK) return s;
+                if (us < best.us) {
+                    best.us = us;
                     best.R = sh.R;
                     best.tpb = sh.S * sh.Ts;
                     best.epi = kind == ONCHIP_ENERGY ? epi : 0;
+                }
+            }
+        }
+        if (kind == ONCHIP_ADJOINT) {  // the other engines, which choose their own shapes
+            sv_plan_opts o{};
+            if (p->opts) o = *p->opts;
+            o.reg_bits = o.threads_per_block = o.epilogue = 0;
+            sv_problem q = *p;
+            q.opts = &o;
+            bool done = false;
+            auto call = [&]() {
+                const sv_status r = chip_adjoint(ctx, &q, theta, nullptr, obs, E2 + I, E2, E, 0, st, &done);
+                return r == SV_OK ? cudaSuccess : cudaErrorUnknown;
+            };
+            float us = 0.f;
+            if (call() == cudaSuccess && done) {
+                s = time_us(call, &us);
+                if (s != SV_OK) return s;
+                if (us < best.us) {
+                    best = Tuned{};
+                    best.us = us;
+                    best.R = ctx->last_run.R;
+                    best.tpb = ctx->last_run.tpb;
+                    best.chip = true;
                 }
             }
         }
@@ -2785,6 +2845,16 @@ sv_status sv_debug_wait_expiry(int32_t limit, sv_stream_t stream) {
     if (!err) return fail(SV_ERR_CUDA, "device error word");
     cudaError_t e = launch_wait_expiry(err, (uint32_t)limit, (cudaStream_t)stream);
     return e == cudaSuccess ? SV_OK : cuda_fail(e, "wait-expiry launch");
+}
+
+sv_status sv_debug_last_adjoint(int32_t *engine, int32_t *reg_bits, int32_t *threads) {
+    DeviceCtx *ctx = context();
+    if (!ctx) return fail(SV_ERR_CUDA, "no CUDA device");
+    std::lock_guard<std::mutex> lk(ctx->mu);
+    if (engine) *engine = ctx->last_run.engine;
+    if (reg_bits) *reg_bits = ctx->last_run.R;
+    if (threads) *threads = ctx->last_run.tpb;
+    return SV_OK;
 }
 
 sv_status sv_shutdown(void) {

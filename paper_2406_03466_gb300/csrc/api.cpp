@@ -948,12 +948,14 @@ sv_status tiles_forward(DeviceCtx *ctx, const PlanEntry *pe, int R, sv_dtype dt,
 // Energies of n_slots slots (parameter-shift or instance slots) of states in
 // device memory, in groups of slots that fit the memory budget.
 sv_status tiles_energies(DeviceCtx *ctx, const sv_problem *p, const double *theta, int mode,
-                         int n_slots, double *E, cudaStream_t st, int slot_begin = 0) {
+                         int n_slots, double *E, cudaStream_t st, int slot_begin = 0,
+                         const TileCfg *forced = nullptr) {
     const sv_dtype dt = p->dtype;
     const int c128 = dt == SV_C128, n = p->circuit->n_qubits, I = p->n_instances;
     TileCfg cfg{};
-    sv_status s = tile_cfg(n, dt, p->opts, &cfg, find_tuned(ctx, p, kTileEnergyKey, p->n_instances));
+    sv_status s = forced ? SV_OK : tile_cfg(n, dt, p->opts, &cfg, find_tuned(ctx, p, kTileEnergyKey, p->n_instances));
     if (s != SV_OK) return s;
+    if (forced) cfg = *forced;
     ObsEntry *obs = nullptr;
     s = get_obs(ctx, *p->observable, n, dt, &obs, st);
     if (s != SV_OK) return s;
@@ -2481,13 +2483,16 @@ sv_status sv_grad_param_shift_plain(const sv_problem *p, const double *theta, do
 // Tile shapes (tile bits t, register bits R) for the energies of the
 // instances (kinds bit 1) and the adjoint gradient (bit 2) of a problem whose
 // states live in device memory: each candidate runs once to plan and warm,
-// then the faster of two CUDA-event-timed calls counts.
+// then the faster of two CUDA-event-timed calls counts.  The problem keeps its
+// own options, so that a candidate's plan is the one its shape gets later (a
+// tile_bits fixed in the options would keep the trailing CNOTs).
 sv_status tune_tiles(const sv_problem *p, const double *theta, int32_t kinds, cudaStream_t st) {
     DeviceCtx *ctx = context();
     if (!ctx) return fail(SV_ERR_CUDA, "no CUDA device");
     if (p->opts && (p->opts->tile_bits > 0 || p->opts->reg_bits > 0)) return SV_OK;  // fixed by the caller
     const int n = p->circuit->n_qubits, I = p->n_instances, Pp = p->circuit->n_params > 0 ? p->circuit->n_params : 1;
     const bool c128 = p->dtype == SV_C128;
+    std::lock_guard<std::mutex> lk(ctx->mu);
     // (tile bits, register bits, tensor-core blocks)
     const int cand_c64[][3] = {{11, 4, 0}, {11, 3, 0}, {12, 4, 0}, {10, 3, 0}, {10, 4, 0},
                                {11, 4, 1}, {12, 4, 1}};
@@ -2515,11 +2520,12 @@ sv_status tune_tiles(const sv_problem *p, const double *theta, int32_t kinds, cu
             o.tile_bits = t;
             o.reg_bits = R;
             o.tensor_blocks = tc;
-            sv_problem q = *p;
-            q.opts = &o;
+            TileCfg cfg{};
+            if (tile_cfg(n, p->dtype, &o, &cfg) != SV_OK) continue;
             auto run = [&]() {
-                return key == kTileEnergyKey ? sv_energies(&q, theta, E, L, st)
-                                             : sv_grad_adjoint(&q, theta, nullptr, E, L, G, 0, st);
+                return key == kTileEnergyKey
+                           ? tiles_energies(ctx, p, theta, SLOTS_INSTANCES, I, E, st, 0, &cfg)
+                           : tiles_adjoint(ctx, p, theta, nullptr, E, L, G, 0, st, nullptr, &cfg);
             };
             if (run() != SV_OK) continue;  // unsupported shape for this problem
             float tbest = 1e30f;
@@ -2539,7 +2545,6 @@ sv_status tune_tiles(const sv_problem *p, const double *theta, int32_t kinds, cu
                 best.tc = tc;
             }
         }
-        std::lock_guard<std::mutex> lk(ctx->mu);
         if (best.R > 0) ctx->tuned[tune_key(p, key, I)] = best;
     }
     cudaEventDestroy(e0);

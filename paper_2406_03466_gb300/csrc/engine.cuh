@@ -165,11 +165,14 @@ __device__ SlotInfo resolve(const SlotSource &s, int b) {
 // as a sum of two doubles; what is still beyond (past 1e18) goes without.
 __device__ __forceinline__ void half_sincos(double a, float *s, float *c) {
     double h = 0.5 * a;
-    if (fabs(h) > 512.0) {
+    float hi = (float)h;
+    if (fabsf(hi) > 512.f) {
         const double k = rint(h * 0.15915494309189535);
         h = fma(k, -2.4492935982947064e-16, fma(k, -6.283185307179586, h));
+        hi = (float)h;
+        if (fabsf(hi) > 512.f) h = (double)hi;
     }
-    const float hi = (float)h, lo = fabs(h) > 512.0 ? 0.f : (float)(h - (double)hi);
+    const float lo = (float)(h - (double)hi);
     float s0, c0;
     sincosf(hi, &s0, &c0);
     *s = __fmaf_rn(lo, c0, s0);

@@ -2047,6 +2047,9 @@ sv_status chip_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta,
     //   96; 12 qubits, 24 groups 82 / 115 (66 / 58 with 4 states)
     //   complex complex128: 7 qubits, 7 groups 71 / 62, 14 groups 104 / 101, 28
     //   groups 152 / 168; 8 qubits, 16 groups 107 / 111
+    //   real complex128, always ahead: 7 qubits, 7 groups 29 / 42 (152 states 31
+    //   / 54, 200 states 44 / 56), 14 groups 37 / 66; 12 qubits, 36 groups 285 /
+    //   909, 72 groups 308 / 449 (against tile passes)
     const int64_t groups = pe->dev.n_groups, work = groups << n;
     const bool many = I > ctx->sms;  // more than one state per SM
     const bool gain = c128   ? real || work >= 2048

@@ -1244,7 +1244,7 @@ template <typename Real> struct HCoef {
 // thread bits (the row's class coefficients times their register-bit signs,
 // built once per tile by the whole block), each row added with the sign of
 // its thread-bit mask.  Products in the state's precision, sums over the
-// block's amplitudes in FP64.  kLam = false: energies only.  kPair (with
+// block's amplitudes in FP64.  kLam = false: energies only.  kPairE (with
 // kRealH): each state holds the real states of slots 2 slot and 2 slot + 1,
 // whose energies are summed apart (those below e_rows are written).
 template <typename Real, int R, bool kLam, bool kRealH, bool kPairE>
@@ -1741,7 +1741,10 @@ cudaError_t launch_group_mats(int c128, const Program &p, const SlotSource &src,
     // lanes a group while that fits the SMs' schedulers in one wave: the
     // latency of a group's loads and sines counts then, not their number.
     const int64_t groups = (int64_t)n_states * std::max(1, p.n_groups);
-    const bool wide = !c128 && groups * 4 <= 152 * 4 * 32;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const bool wide = !c128 && groups * 4 <= (int64_t)sms * 4 * 32;
     const int g = grid_1d(wide ? groups * 4 : groups, 32);
     const bool y_only = every && kind != 0;  // (the on-chip engine's real kinds)
     cudaError_t e =

@@ -158,25 +158,22 @@ __device__ SlotInfo resolve(const SlotSource &s, int b) {
 
 // ------------------------------------------------------- gate matrices
 
-// sin and cos of a / 2.  FP32: the half angle's rounding to float is put back
-// to first order, so the pair carries the rounding of the function only.  That
-// rounding grows with the angle, and with it the pair's distance from the unit
-// circle (its square / 2): beyond 512 (3e-5) whole turns come off first, 2 pi
-// as a sum of two doubles; what is still beyond (past 1e18) goes without.
+// a / 2 without whole turns (2 pi as a sum of two doubles).
+__device__ __noinline__ float half_turn(double a) {
+    const double d = 0.5 * a, k = rint(d * 0.15915494309189535);
+    return (float)fma(k, -2.4492935982947064e-16, fma(k, -6.283185307179586, d));
+}
+// sin and cos of a / 2.  FP32: the half angle rounded to float, beyond |a| = 8,
+// where that rounding is more than the function's own, without whole turns.  No
+// FP64 here, and the reduction a call that ptxas cannot turn into predicated
+// instructions: every group of every circuit is formed, and GB300 does 2 FP64
+// instructions a clock and SM.  160 circuits of 7 qubits and 42 parameters by
+// parameter shift: 64.0 us; 72 with the reduction inlined, or with the
+// rounding put back to first order (which changed no error: 7e-7 each way).
 __device__ __forceinline__ void half_sincos(double a, float *s, float *c) {
-    double h = 0.5 * a;
-    float hi = (float)h;
-    if (fabsf(hi) > 512.f) {
-        const double k = rint(h * 0.15915494309189535);
-        h = fma(k, -2.4492935982947064e-16, fma(k, -6.283185307179586, h));
-        hi = (float)h;
-        if (fabsf(hi) > 512.f) h = (double)hi;
-    }
-    const float lo = (float)(h - (double)hi);
-    float s0, c0;
-    sincosf(hi, &s0, &c0);
-    *s = __fmaf_rn(lo, c0, s0);
-    *c = __fmaf_rn(-lo, s0, c0);
+    float h = 0.5f * (float)a;
+    if (fabsf(h) > 4.f) h = half_turn(a);
+    sincosf(h, s, c);
 }
 __device__ __forceinline__ void half_sincos(double a, double *s, double *c) { sincos(a * 0.5, s, c); }
 
@@ -194,8 +191,10 @@ __device__ __forceinline__ void rotation(int axis, Real s, Real c, C g[4]) {
 }
 
 // An encoding's input: |x| <= 1, where a complex64 problem's x counts as
-// +-1 when it rounds to that in float (beyond it the matrix is NaN).
-template <typename In> __device__ __forceinline__ double enc_input(double x) {
+// +-1 when it rounds to that in float (beyond it the matrix is NaN).  Real:
+// what it is used in (float: rounding it says it all).
+template <typename In, typename Real = double> __device__ __forceinline__ double enc_input(double x) {
+    if (std::is_same<Real, float>::value) return x;
     return fabs(x) > 1.0 && fabs((double)(In)x) <= 1.0 ? copysign(1.0, x) : x;
 }
 
@@ -224,17 +223,19 @@ __device__ void member_matrix(const Member &m, const SlotInfo &si, C g[4]) {
     // The encodings' half angles without inverse functions: with a =
     // arcsin x, cos a = sqrt(1 - x^2), cos(a/2) = sqrt((1 + cos a) / 2) and
     // sin(a/2) = x / (2 cos(a/2)); with a = arccos u, cos(a/2) =
-    // sqrt((1 + u) / 2) and sin(a/2) = sqrt((1 - u) / 2).
+    // sqrt((1 + u) / 2) and sin(a/2) = sqrt((1 - u) / 2).  1 - x^2 as a
+    // product, whose factors are exact near |x| = 1.
     case M_ENC_RY_ASIN: {
-        const double x = enc_input<In>(si.x[m.param]);
-        const Real ca = sqrtR((Real)((1.0 - x) * (1.0 + x)));
+        const Real x = (Real)enc_input<In, Real>(si.x[m.param]);
+        const Real ca = sqrtR(((Real)1 - x) * ((Real)1 + x));
         const Real cs = sqrtR((Real)0.5 * ((Real)1 + ca));
-        rotation<Real, C>(1, (Real)x / ((Real)2 * cs), cs, g);
+        rotation<Real, C>(1, x / ((Real)2 * cs), cs, g);
         break;
     }
     default: {  // M_ENC_RZ_ACOS_SQ
-        const double x = enc_input<In>(si.x[m.param]), u = x * x;
-        rotation<Real, C>(2, sqrtR((Real)(0.5 * (1.0 - u))), sqrtR((Real)(0.5 * (1.0 + u))), g);
+        const Real x = (Real)enc_input<In, Real>(si.x[m.param]);
+        rotation<Real, C>(2, sqrtR((Real)0.5 * (((Real)1 - x) * ((Real)1 + x))),
+                          sqrtR((Real)0.5 * fmaR(x, x, (Real)1)), g);
         break;
     }
     }
@@ -251,12 +252,14 @@ template <typename C> __device__ __forceinline__ void matmul2(const C A[4], cons
 template <typename Real, typename C, typename In = Real>
 __device__ void group_matrix(const Program &p, int g, const SlotInfo &si, C *out) {
     const Group grp = p.groups[g];
-    C M[4];
-    member_matrix<Real, C, In>(p.members[grp.m_begin], si, M);  // a group has a member
-    for (int m = grp.m_begin + 1; m < grp.m_end; ++m) {
+    C M[4] = {cmk<C>(1, 0), cmk<C>(0, 0), cmk<C>(0, 0), cmk<C>(1, 0)};
+    for (int m = grp.m_begin; m < grp.m_end; ++m) {
         C G[4], T[4];
         member_matrix<Real, C, In>(p.members[m], si, G);
-        matmul2(G, M, T);
+        // complex64: no branch for the first (97 parameters on 4 qubits 343 against
+        // 352 us); complex128: a product of 8 FP64 multiply-adds less
+        if (std::is_same<Real, float>::value || m > grp.m_begin) matmul2(G, M, T);
+        else T[0] = G[0], T[1] = G[1], T[2] = G[2], T[3] = G[3];
         M[0] = T[0]; M[1] = T[1]; M[2] = T[2]; M[3] = T[3];
     }
     out[0] = M[0]; out[1] = M[1]; out[2] = M[2]; out[3] = M[3];

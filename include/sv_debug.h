@@ -61,6 +61,11 @@ sv_status sv_debug_wait_expiry(int32_t limit, sv_stream_t stream);
  * block.  Any out-pointer may be NULL. */
 sv_status sv_debug_last_adjoint(int32_t *engine, int32_t *reg_bits, int32_t *threads);
 
+/* The default launch shape of the on-chip kernels (kind 0: energies, 3: the
+ * one-kernel adjoint) for n_slots states on a device of `sms` SMs: register
+ * bits and threads per block.  Host-only. */
+sv_status sv_debug_onchip_shape(int32_t kind, int32_t n_qubits, int32_t dtype, int32_t n_slots,
+                                int32_t sms, int32_t *reg_bits, int32_t *threads);
 /* The relabeling tile plan without the circuit's trailing CNOTs: passes kept,
  * the CNOTs left out (control, target pairs in time order; tail holds
  * 2 n_gates entries) and the layout, as sv_debug_tile_passes gives it. */

@@ -4,6 +4,7 @@
 #include <string>
 #include <vector>
 
+#include "kernels.h"
 #include "planner.h"
 #include "sv_debug.h"
 
@@ -79,6 +80,15 @@ sv_status sv_debug_tile_passes(const sv_circuit *c, int32_t tile_bits, int32_t r
     if (tile_passes) std::memcpy(tile_passes, tp.data(), tp.size() * sizeof(TilePass));
     if (layout)
         for (size_t q = 0; q < h.layout.size(); ++q) layout[q] = h.layout[q];
+    return SV_OK;
+}
+
+sv_status sv_debug_onchip_shape(int32_t kind, int32_t n_qubits, int32_t dtype, int32_t n_slots,
+                                int32_t sms, int32_t *reg_bits, int32_t *threads) {
+    OnchipShape sh{};
+    if (onchip_shape(kind, n_qubits, 0, 0, dtype == SV_C128, n_slots, 0, 0, &sh, sms)) return SV_ERR_ARG;
+    if (reg_bits) *reg_bits = sh.R;
+    if (threads) *threads = sh.S * sh.Ts;
     return SV_OK;
 }
 

@@ -260,8 +260,12 @@ const char *onchip_shape(int kind, int n, int n_groups, int n_params, int c128, 
         while (R > 2 && (int64_t)n_slots * (int64_t(1) << (n > R ? n - R : 0)) < want) --R;
         // complex128 issues one FP64 instruction of a warp in 16 clocks: a
         // batch that leaves most SMs without a warp halves them once more (33
-        // circuits of 4 qubits: 30.2 -> 18.4 us)
-        if (c128 && R == 2 && kind == ONCHIP_ENERGY &&
+        // circuits of 4 qubits: 30.2 -> 18.4 us), up to 8 qubits: a state of
+        // more fills its SM's issue with one register bit as well, and its
+        // longer chain of stages loses (1 to 33 circuits, one register bit
+        // against two: 8 qubits 22-57 / 26-92 us, 9 qubits 40-89 / 37-94, 10
+        // qubits 65-173 / 50-167)
+        if (c128 && R == 2 && n <= 8 && kind == ONCHIP_ENERGY &&
             ((int64_t)n_slots << (n > 2 ? n - 2 : 0)) < (int64_t)num_sms * 32)
             R = 1;
     }

@@ -767,10 +767,10 @@ int *device_err(DeviceCtx *ctx) {
 constexpr int kTileEnergyKey = 10 + ONCHIP_ENERGY, kTileAdjointKey = 10 + ONCHIP_ADJOINT;
 
 // tn: a tuned tile shape (R = register bits, tpb = 2^(t - R) threads), used
-// when opts leave tile_bits and reg_bits at zero.  n_def: the qubit count that
-// the default register bits go by (a batch: its smallest circuit's; 0: n).
+// when opts leave tile_bits and reg_bits at zero.  batch: for an uneven batch,
+// whose circuits share one default width.
 sv_status tile_cfg(int n, sv_dtype dt, const sv_plan_opts *o, TileCfg *cfg,
-                   const Tuned *tn = nullptr, int n_def = 0) {
+                   const Tuned *tn = nullptr, bool batch = false) {
     if (tn && tn->R > 0 && (!o || (o->tile_bits <= 0 && o->reg_bits <= 0))) {
         sv_plan_opts t{};
         if (o) t = *o;
@@ -790,8 +790,11 @@ sv_status tile_cfg(int n, sv_dtype dt, const sv_plan_opts *o, TileCfg *cfg,
                                         "[coalesced bits + 2, 12] and at most n_qubits");
     // 8 amplitudes per thread for larger complex128 states: fewer stages, and
     // the FP64 unit, not the warps in flight, is the limit (19-qubit MC-VQE
-    // adjoint 2206 against 2580 us, 16-qubit circuit learning 5474 against 6134)
-    const int r_def = dt == SV_C128 ? ((n_def > 0 ? n_def : n) >= 16 && t >= 10 ? 3 : 2) : 4;
+    // adjoint 2206 against 2580 us, 16-qubit circuit learning 5474 against 6134).
+    // Not the persistent sweeps of a batch (two circuits of 16 and 17 qubits,
+    // 6 instances each, 8 against 4 a thread: real 9211 / 5984 us, mixed 9230 /
+    // 5576, three rotations a group 9143 / 8902).
+    const int r_def = dt == SV_C128 ? (!batch && n >= 16 && t >= 10 ? 3 : 2) : 4;
     int R = (o && o->reg_bits > 0) ? o->reg_bits : std::min(r_def, t - 5);
     if (R < 2 || R > rmax) return fail(SV_ERR_ARG, "reg_bits for tile passes must be 2..4 (2..3 complex128)");
     if (t - R > 8) R = t - 8;
@@ -1274,15 +1277,13 @@ sv_status multi_adjoint(DeviceCtx *ctx, const sv_problem *problems, int np,
     const size_t csz = c128 ? 16 : 8;
     TileCfg cfg{};
     uint64_t key = mix64(0x5e17ull, (uint64_t)np);
-    int n_min = problems[0].circuit->n_qubits;  // one default width for all
-    for (int j = 1; j < np; ++j) n_min = std::min(n_min, problems[j].circuit->n_qubits);
     for (int j = 0; j < np; ++j) {
         const sv_problem *p = &problems[j];
         if (p->dtype != dt) return fail(SV_ERR_ARG, "uneven batch: problems differ in dtype");
         if (!wants_tiles(p->circuit->n_qubits, dt, p->opts))
             return fail(SV_ERR_UNSUPPORTED, "uneven batch: every problem must take the tile path");
         TileCfg c{};
-        sv_status s = tile_cfg(p->circuit->n_qubits, dt, p->opts, &c, nullptr, n_min);
+        sv_status s = tile_cfg(p->circuit->n_qubits, dt, p->opts, &c, nullptr, true);
         if (s != SV_OK) return s;
         if (j == 0) cfg = c;
         else if (c.t != cfg.t || c.R != cfg.R || c.c != cfg.c)

@@ -72,6 +72,7 @@ struct PlanEntry {
     bool real = false;  // every group's matrix is real
     bool y_only = false;  // every group is Y rotations and Ry encodings
     bool one_per_bit = false;  // stages: sorted, at most one group a register bit
+    int n_par = 0;  // groups with parameters
     HostProgram host;
     std::vector<TilePass> tiles;  // tile plans: one kernel descriptor per pass
     DeviceBuf buf;
@@ -273,7 +274,10 @@ sv_status get_plan(DeviceCtx *ctx, const sv_circuit &c, int R, bool fuse, sv_dty
     e->input_dim = c.input_dim;
     const HostProgram &h = e->host;
     e->real = true;
-    for (const Group &g : h.groups) e->real = e->real && g.real;
+    for (const Group &g : h.groups) {
+        e->real = e->real && g.real;
+        e->n_par += g.has_param != 0;
+    }
     e->y_only = e->one_per_bit = true;
     for (const Member &m : h.members)
         e->y_only = e->y_only && (m.kind == M_RY || m.kind == M_ENC_RY_ASIN);
@@ -2046,18 +2050,23 @@ sv_status chip_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta,
     //   66.7 / 65.9, 80 groups (82 k) 79 / 95
     //   the same with 256 states: 10 qubits, 30 groups 68 / 58, 40 groups 74 /
     //   96; 12 qubits, 24 groups 82 / 115 (66 / 58 with 4 states)
-    //   complex complex128: 7 qubits, 7 groups 71 / 62, 14 groups 104 / 101, 28
-    //   groups 152 / 168; 8 qubits, 16 groups 107 / 111
+    //   complex complex128, every group with parameters: 7 qubits, 7 groups 69 /
+    //   60, 35 groups (4.5 k) 192 / 212; 8 qubits, 8 groups 70 / 64, 16 groups
+    //   (4 k) 100 / 103; 10 qubits, 10 groups (10 k) 132 / 126 to 111 / 115, 70
+    //   groups 593 / 711; 11 qubits, 305 states, 33 groups 1397 / 1904
+    //   fewer groups with parameters (that engine sums and takes the real
+    //   path per group, chip.cu turns every amplitude of every stage): 10
+    //   qubits, 28 of 31 groups 335 / 339, 37 of 48 467 / 448; 8 qubits, 22 of
+    //   26 190 / 184, 12 of 16 and less 131 / 107, none of 56 239 / 123
     //   real complex128, always ahead: 7 qubits, 7 groups 29 / 42 (152 states 31
     //   / 54, 200 states 44 / 56), 14 groups 37 / 66; 12 qubits, 36 groups 285 /
     //   909, 72 groups 308 / 449 (against tile passes)
     const int64_t groups = pe->dev.n_groups, work = groups << n;
     const bool many = I > ctx->sms;  // more than one state per SM
-    const bool gain = c128   ? real || work >= 2048
+    const bool gain = c128   ? real || (work >= 4096 && pe->n_par * 20 >= groups * 19)
                       : real ? work >= 48 * 1024
                              : (groups >= 38 && (work >= 64 * 1024 || (n >= 10 && many))) ||
                                    (n >= 12 && many);
-    if (!gain) return SV_OK;
     // pairs of real states once single ones would share SMs
     const int kind = !real ? 0 : (many ? 1 : 2);
     const int n_states = kind == 1 ? (I + 1) / 2 : I;
@@ -2068,7 +2077,8 @@ sv_status chip_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta,
         // qubits 4 (2); tile passes spread that with a third lost and about
         // 250 us of launches.  12 qubits, 32 circuit-learning instances: 703
         // us as tile passes, 1855 us on chip; 11 qubits, 12 MC-VQE references:
-        // 281 against 235 us.
+        // 281 against 235 us; against the one-kernel engine, without parameters:
+        // 12 qubits, 36 groups 148 against 536.
         const double w = (double)(int64_t(1) << n) *
                          (pe->dev.n_groups * (real ? 5.5 : 23.0) + obs->dev.n_tgroups * (real ? 2.0 : 4.0));
         const double us = w / (2.0 * 2000.0);  // one state on its SM
@@ -2083,6 +2093,7 @@ sv_status chip_adjoint(DeviceCtx *ctx, const sv_problem *p, const double *theta,
             ctx->last_rev_bytes = 0;
         }
     }
+    if (!gain) return SV_OK;
     ChipShape sh{};
     if (chip_shape(kind, n, R, c128, pe->dev.n_groups, P, pe->dev.n_stages, n_states, ctx->sms, &sh))
         return SV_OK;

@@ -9,7 +9,7 @@ import pytest
 
 import oracle
 import workloads as wl
-from test_gpu_autotune_engines import COMPLEX, PAIR, REAL, TILES, last_adjoint
+from test_gpu_autotune_engines import COMPLEX, FUSED, PAIR, REAL, TILES, last_adjoint
 
 pytestmark = pytest.mark.gpu
 
@@ -28,12 +28,14 @@ def close(got, want, tol):
     assert float(np.max(np.abs(got - want))) <= tol * max(1.0, float(np.max(np.abs(want))))
 
 
-def workload(n, layers, instances, real, shared=False):
-    """`layers` layers of one group on every qubit, each ending in CNOTs."""
+def workload(n, layers, instances, real, shared=False, every=False):
+    """`layers` layers of one group on every qubit (every: all with parameters),
+    each ending in CNOTs."""
     rng = np.random.default_rng(100 * n + layers + instances)
     gates, p = [wl.Gate("ENC_RY_ASIN", target=0, param=0)], 0
     kinds = ([["RY"], ["RY", "RY"], ["fixed"], ["fixed", "RY"]] if real else
-             [["RX", "RZ"], ["RY"], ["H", "RZ"], ["X"], ["RZ", "RX", "RZ"], ["RY", "fixed", "H"]])
+             [["RX", "RZ"], ["RY"], ["H", "RZ"], ["X", "RZ"] if every else ["X"], ["RZ", "RX", "RZ"],
+              ["RY", "fixed", "H"]])
     for layer in range(layers):
         for q in range(n):
             for op in kinds[rng.integers(len(kinds))]:
@@ -70,7 +72,7 @@ CASES = [("c64", False, 8, 33, 2), ("c64", False, 10, 7, 3), ("c64", False, 11, 
 @pytest.mark.parametrize("dtype,real,n,layers,instances", CASES)
 def test_engine_of_the_default_route(sv, dtype, real, n, layers, instances, shared):
     import torch
-    w = workload(n, layers, instances, real, shared)
+    w = workload(n, layers, instances, real, shared, every=dtype == "c128")
     theta = torch.as_tensor(w.theta, dtype=torch.float64, device="cuda")
     _, e_, g_ = sv.sv_grad_adjoint(sv.Problem.from_spec(w, dtype), theta)
     few = dtype == "c128" and not real and n >= 11  # few large states: tile passes
@@ -94,3 +96,31 @@ def test_ladder_runs_fewer_passes(sv, dtype):
     fixed = sv.Problem.from_spec(w, dtype, opts=sv.plan_opts(tile_bits=11 if dtype == "c64" else 10))
     sv.sv_grad_adjoint(fixed, theta)
     assert passes < sv.sv_last_moved()["passes"]
+
+
+@pytest.mark.parametrize("n,layers,ops,engine", [
+    (8, 2, ("RX", "RZ"), COMPLEX), (8, 7, ("H",), FUSED), (10, 3, ("mixed",), FUSED), (8, 1, ("RX", "RZ"), FUSED)])
+def test_line_between_the_complex128_engines(sv, n, layers, ops, engine):
+    """Complex circuits go to the engine of split stages when their groups carry
+    parameters and there is enough of them."""
+    import torch
+    rng = np.random.default_rng(n + layers)
+    gates, p = [], 0
+    for layer in range(layers):
+        for q in range(n):
+            for op in (("X", "H") if (q + layer) % 3 else ("RZ", "RX")) if ops == ("mixed",) else ops:
+                rot = op in ("RX", "RY", "RZ")
+                gates.append(wl.Gate(op, target=q, param=p if rot else -1))
+                p += rot
+        gates += wl.cnot_ladder(n)
+    gates.append(wl.Gate("RZ", target=0, param=p))
+    w = wl.Workload("line", n, gates, p + 1, rng.uniform(-3, 3, p + 1),
+                    rng.choice([0, 1, 2, 3], size=(5, n)).astype(np.int8), rng.normal(size=5),
+                    rng.integers(0, 1 << n, 3).astype(np.int64), weights=np.ones(3))
+    theta = torch.as_tensor(w.theta, dtype=torch.float64, device="cuda")
+    _, e_, g_ = sv.sv_grad_adjoint(sv.Problem.from_spec(w, "c128"), theta)
+    assert last_adjoint(sv)[0] == engine
+    ks = sorted({0, w.n_params - 1})
+    _, E, g = oracle.grad_param_shift(w, params=ks)
+    close(e_.cpu(), E, 1e-12)
+    close(g_.cpu()[ks], g, 1e-12)

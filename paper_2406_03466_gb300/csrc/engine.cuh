@@ -253,13 +253,15 @@ template <typename Real, typename C, typename In = Real>
 __device__ void group_matrix(const Program &p, int g, const SlotInfo &si, C *out) {
     const Group grp = p.groups[g];
     C M[4] = {cmk<C>(1, 0), cmk<C>(0, 0), cmk<C>(0, 0), cmk<C>(1, 0)};
-    for (int m = grp.m_begin; m < grp.m_end; ++m) {
+    int m = grp.m_begin;
+    // complex128: the first member as it is (8 FP64 multiply-adds less; 160
+    // circuits of 7 qubits by parameter shift 556 against 572 us); complex64:
+    // one call of the sines (97 parameters on 4 qubits 343 against 352 us)
+    if constexpr (std::is_same<Real, double>::value) member_matrix<Real, C, In>(p.members[m++], si, M);
+    for (; m < grp.m_end; ++m) {
         C G[4], T[4];
         member_matrix<Real, C, In>(p.members[m], si, G);
-        // complex64: no branch for the first (97 parameters on 4 qubits 343 against
-        // 352 us); complex128: a product of 8 FP64 multiply-adds less
-        if (std::is_same<Real, float>::value || m > grp.m_begin) matmul2(G, M, T);
-        else T[0] = G[0], T[1] = G[1], T[2] = G[2], T[3] = G[3];
+        matmul2(G, M, T);
         M[0] = T[0]; M[1] = T[1]; M[2] = T[2]; M[3] = T[3];
     }
     out[0] = M[0]; out[1] = M[1]; out[2] = M[2]; out[3] = M[3];
